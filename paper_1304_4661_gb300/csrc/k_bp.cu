@@ -189,21 +189,44 @@ __global__ void k_bp_next_level(BpArgs a) {
     if (__any_sync(FULL, any) && lane == 0) atomicOr(a.changed, 1u);
 }
 
-// S^0 := S^0 minus S^{-1} for every (v, i)
-__global__ void k_bp_finish(size_t nt, ulonglong2 *m) {
-    for (size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x; x < nt;
-         x += (size_t)gridDim.x * blockDim.x) {
-        ulonglong2 p = m[x];
-        p.y &= ~p.x;
-        m[x] = p;
+// S^0 := S^0 minus S^{-1} for every (v, i), a warp per vertex (lanes own roots
+// lane and lane + 32); only pairs that change are written back. e (or null)
+// receives the vertex's non-empty roots: x for S^{-1}, y for either set.
+__global__ void k_bp_finish(uint32_t n, uint32_t t, ulonglong2 *m, ulonglong2 *e) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
+        uint64_t e1 = 0, e01 = 0;
+        ulonglong2 p[2];
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            p[h] = make_ulonglong2(0, 0);
+            const uint32_t i = lane + 32 * h;
+            if (i < t) p[h] = m[(size_t)v * t + i];
+        }
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t i = lane + 32 * h;
+            if (p[h].x & p[h].y) {
+                p[h].y &= ~p[h].x;
+                m[(size_t)v * t + i] = p[h];
+            }
+            e1 |= (uint64_t)__ballot_sync(FULL, p[h].x != 0) << (32 * h);
+            e01 |= (uint64_t)__ballot_sync(FULL, (p[h].x | p[h].y) != 0) << (32 * h);
+        }
+        if (e && lane == 0) e[v] = make_ulonglong2(e1, e01);
     }
+}
+
+int finish_grid(uint32_t n, int sms) {  // a warp per vertex, up to 16 blocks an SM
+    return (int)std::max<uint64_t>(1, std::min<uint64_t>(((uint64_t)n + 7) / 8, (uint64_t)sms * 16));
 }
 
 }  // namespace
 
 int bp_run(uint32_t n, uint32_t t, uint32_t graphs, const uint32_t *d_roff, const uint32_t *d_rcol,
            const uint32_t *d_root, const uint32_t *d_cnt, const uint32_t *d_S, uint8_t *d_bp_d,
-           uint64_t *d_bp_m, uint32_t *d_err, cudaStream_t s, uint32_t *levels) {
+           uint64_t *d_bp_m, ulonglong2 *d_bp_e, uint32_t *d_err, cudaStream_t s, uint32_t *levels) {
     *levels = 0;
     if (t == 0 || n == 0) return PLL_OK;
     if (t > PLL_MAX_T) return PLL_E_RANGE;
@@ -263,8 +286,7 @@ int bp_run(uint32_t n, uint32_t t, uint32_t graphs, const uint32_t *d_roff, cons
     }
     host_free(h_flag);
     if (st == PLL_OK) {
-        k_bp_finish<<<(int)std::min<size_t>((nt + 255) / 256, (size_t)sms * 32), 256, 0, s>>>(
-            nt, reinterpret_cast<ulonglong2 *>(d_bp_m));
+        k_bp_finish<<<finish_grid(n, sms), 256, 0, s>>>(n, t, reinterpret_cast<ulonglong2 *>(d_bp_m), d_bp_e);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // before the temporaries are freed
         if (e != cudaSuccess) st = cuda_status(e);
@@ -340,8 +362,7 @@ int bp_run_in(uint32_t n, uint32_t t, const uint32_t *d_roff, const uint32_t *d_
         PLL_TRY(cudaStreamSynchronize(s));
         if (h_flag == 0 && L >= 1) break;
     }
-    k_bp_finish<<<(int)std::min<size_t>((nt + 255) / 256, (size_t)sms * 32), 256, 0, s>>>(
-        nt, reinterpret_cast<ulonglong2 *>(d_bp_m));
+    k_bp_finish<<<finish_grid(n, sms), 256, 0, s>>>(n, t, reinterpret_cast<ulonglong2 *>(d_bp_m), nullptr);
     PLL_TRY(cudaGetLastError());
     PLL_TRY(cudaStreamSynchronize(s));
     return PLL_OK;

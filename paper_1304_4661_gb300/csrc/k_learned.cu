@@ -549,7 +549,7 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
         PLL_TRY(cudaMemsetAsync(m_err.p, 0, 4, s));
         PLL_CHECK(bp_run(n, t, 1, m_roff.as<uint32_t>(), m_rcol.as<uint32_t>(), m_root.as<uint32_t>(),
                          m_cnt.as<uint32_t>(), m_S.as<uint32_t>(), m_bpd.as<uint8_t>(),
-                         m_bpm.as<uint64_t>(), m_err.as<uint32_t>(), s, &levels));
+                         m_bpm.as<uint64_t>(), nullptr, m_err.as<uint32_t>(), s, &levels));
         PLL_CHECK(read_u32(m_err.as<uint32_t>(), s, &h_err));
         if (h_err) return (h_err & ERR_DEPTH) ? PLL_E_RANGE : PLL_E_CUDA;
     }

@@ -18,33 +18,27 @@
 //   init    per root: the level-0 entry (v_k, k, 0) (the root is never
 //           pruned: Query(v_k, v_k) >= 2 for v_k outside X), its visited bit,
 //           a hash table of its label L(v_k) -- the root array T of Sec.
-//           4.5.1 ("Querying"), so a prune test costs O(|L(u)|) probes -- and
-//           two 64-bit feasibility masks over the bit-parallel roots.
-//   expand  one warp per entry (u, k, d) of the level: read u's neighbours 32
-//           per step and look each one up in the root's visited row (a bitmap
-//           [B][ceil(n / 32)], one row per root of the batch: the per-root
-//           visited set of Alg. 1, one bit per vertex, so the 32 lanes of a
-//           warp, which share the root, read neighbouring words). For a
-//           neighbour w not yet visited, the lane first runs the cheap part of
-//           the prune test (it decides ~90% of them on power-law graphs) and
-//           claims w with an atomicOr only if w survives it. A vertex the
-//           bit-parallel labels prune stays unmarked: the bit-parallel bound
-//           of a pair does not depend on the level, so if it prunes w at level
-//           d + 1 it prunes w again at any later level where w is reached, and
-//           leaving the bit clear changes no label. The test: bit-parallel
-//           distances only -- with
-//           d~_i = d(v_k,r_i) + d(r_i,w), some d~_i <= d + 1 prunes (Sec. 5.3:
-//           the distance through {r_i} U S_{r_i} is at most d~_i). Rows of t
-//           bytes (padded to 16) arrive in 16-byte loads, four roots per
-//           instruction (saturating byte add, byte compare). The lane also
-//           records which roots could still reach the bound with their masks:
-//           d~_i = d + 2 needs a reduction of 1 (possible only if S^{-1}(v_k)
-//           or S^0(v_k) is non-empty), d~_i = d + 3 needs the S^{-1}
-//           intersection (S^{-1}(v_k) non-empty). The lane then checks the
-//           masks of the first QUICK roots itself: roots come in rank order,
-//           so these are the largest hubs and they decide most mask tests.
-//           Survivors are claimed; freshly claimed (slot, w) pairs and the
-//           remaining feasible roots are the next level's candidates.
+//           4.5.1 ("Querying"), so a prune test costs O(|L(u)|) probes.
+//   expand  the arcs (u, w) of the entries (u, k, d) of the level, w of rank >=
+//           k0 (lower ranks are always pruned). First the cheap part of the
+//           prune test, which decides 19 of 20 on power-law graphs: the
+//           bit-parallel distances -- with d~_i = d(v_k,r_i) + d(r_i,w), some
+//           d~_i <= d + 1 prunes (Sec. 5.3: the distance through {r_i} U S_{r_i}
+//           is at most d~_i) -- on rows of four bits a root (eight roots per
+//           instruction; bytes past level NIB_LEVEL). A w that it leaves is
+//           looked up in the root's visited row (a bitmap [B][ceil(n / 32)],
+//           one row per root of the batch: the per-root visited set of Alg.
+//           1). If unvisited: which roots could still reach the bound with
+//           their masks (d~_i = d + 2 needs a reduction of 1, d~_i = d + 3
+//           the S^{-1} intersection; neither can come from empty sets), then the
+//           masks of the first QUICK roots: roots come in rank order, so these
+//           are the largest hubs and they decide most mask tests. Survivors
+//           are claimed with an atomicOr; freshly claimed (slot, w) pairs and
+//           the remaining feasible roots are the next level's candidates. A
+//           vertex the bit-parallel labels prune stays unmarked: the
+//           bit-parallel bound of a pair does not depend on the level, so if
+//           it prunes w at level d + 1 it prunes w again at any later level
+//           where w is reached, and leaving the bit clear changes no label.
 //   test    the rest of the test, one WARP per candidate so that lanes work
 //           in parallel instead of a few lanes looping alone: each lane first
 //           loads its own candidate's label offsets (32 candidates' loads in
@@ -62,6 +56,7 @@
 // learn that the frontier is empty; sweeps over an empty range return at once.
 #include <cub/cub.cuh>
 
+#include "bp_nibble.h"
 #include "pll_internal.cuh"
 
 namespace pll {
@@ -113,6 +108,65 @@ __device__ __forceinline__ uint32_t filt_bit(uint32_t h) {
     return x >> 22;
 }
 
+// Neighbours of rank < k0 need no test: they are pruned at whatever level they
+// are reached. (A hub of a finished batch answers every distance to itself
+// exactly, Thm 4.1, and so do the bit-parallel labels for a vertex of X:
+// Query(v_k, w) = d(v_k, w) <= level.) Lists are ascending, so rstart cuts them
+// off as a prefix, unread: on power-law graphs most arcs lead to hubs. Levels
+// next to the deepest distance read the whole list, so that a vertex at depth
+// 255 is found (and is an error) exactly where it would be without the cut: a
+// vertex adjacent to one at depth 254 is at depth 253 at least.
+constexpr uint32_t WHOLE_LEVEL = 250;
+__device__ __forceinline__ uint32_t first_arc(const BatchArgs &a, uint32_t u, uint32_t nlevel) {
+    return nlevel >= WHOLE_LEVEL ? a.roff[u] : a.rstart[u];
+}
+
+__global__ void k_row_starts(uint32_t n, uint32_t k0, const uint32_t *__restrict__ roff,
+                             const uint32_t *__restrict__ rcol, uint32_t *rstart) {
+    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
+        uint32_t lo = k0 ? rstart[u] : roff[u];
+        const uint32_t first = lo, end = roff[u + 1];
+        if (lo < end && rcol[lo] < k0) {
+            // gallop, then search the last step: batches move the cut a little
+            uint32_t step = 1;
+            while (step < end - lo && rcol[lo + step] < k0) {
+                lo += step;
+                step <<= 1;
+            }
+            uint32_t hi = end - lo < step ? end : lo + step;
+            ++lo;
+            while (lo < hi) {
+                const uint32_t mid = lo + ((hi - lo) >> 1);
+                if (rcol[mid] < k0) lo = mid + 1; else hi = mid;
+            }
+        }
+        if (lo != first || k0 == 0) rstart[u] = lo;
+    }
+}
+
+// New entries (w, k) of level `level` (the lanes with keep): those of more than
+// SLICE arcs to expand leave the arcs past the first SLICE as slices.
+__device__ __forceinline__ void append_slices(const BatchArgs &a, bool keep, int lane, uint32_t w, uint32_t k,
+                                              uint32_t level) {
+    uint32_t rb = 0, deg = 0;
+    if (keep) {
+        rb = first_arc(a, w, level + 1);
+        deg = a.roff[w + 1] - rb;
+    }
+    for (unsigned m = __ballot_sync(FULL, deg > SLICE); m; m &= m - 1) {
+        const int j = __ffs(m) - 1;
+        const uint32_t b = __shfl_sync(FULL, rb, j), e = b + __shfl_sync(FULL, deg, j);
+        const uint32_t kj = __shfl_sync(FULL, k, j), cnt = (e - b - 1) / SLICE;
+        unsigned long long base = 0;
+        if (lane == j) base = atomicAdd(&a.ctr->slice_n, (unsigned long long)cnt);
+        base = __shfl_sync(FULL, base, j);
+        for (uint32_t i = lane; i < cnt; i += 32) {
+            const uint32_t x = b + (i + 1) * SLICE;
+            if (base + i < a.slice_cap) a.slices[base + i] = make_uint4(kj, x, e - x < SLICE ? e : x + SLICE, 0);
+        }
+    }
+}
+
 __global__ void k_batch_init(BatchArgs a) {
     const int lane = threadIdx.x & 31;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
@@ -125,23 +179,7 @@ __global__ void k_batch_init(BatchArgs a) {
             else atomicOr(&a.ctr->err, ERR_BUF);
             atomicOr(&a.visited[(size_t)slot * a.NW + (k >> 5)], 1u << (k & 31));
         }
-        // feasibility masks over the bit-parallel roots
-        uint64_t h1 = 0, h01 = 0;
-        for (uint32_t i0 = 0; i0 < a.t; i0 += 32) {
-            const uint32_t i = i0 + lane;
-            uint64_t k1 = 0, kz = 0;
-            if (i < a.t) {
-                const ulonglong2 m = reinterpret_cast<const ulonglong2 *>(a.bp_m)[(size_t)k * a.t + i];
-                k1 = m.x;
-                kz = m.y;
-            }
-            h1 |= (uint64_t)__ballot_sync(FULL, k1 != 0) << i0;
-            h01 |= (uint64_t)__ballot_sync(FULL, (k1 | kz) != 0) << i0;
-        }
-        if (lane == 0) {
-            a.rootbits[2 * slot] = h1;
-            a.rootbits[2 * slot + 1] = h01;
-        }
+        append_slices(a, lane == 0, lane, k, k, 0);
         // a 1024-bit filter of L(v_k)'s hubs: most hubs of a candidate's label
         // are not in the root's, and the filter tells so with one load (for
         // labels of up to FILT_MAX_LEN entries, where at most 12 % of its bits
@@ -341,42 +379,74 @@ __device__ __forceinline__ bool quick_masks(const BatchArgs &a, uint32_t k, uint
 }
 
 
-// One arc (u, w) of an entry of root ki (batch slot `slot`; kr = its row in
-// shared memory, from `rows`): look w up in the root's visited row; if
-// unvisited, the bit-parallel test and the first masks; claim w if it
-// survives. Returns true for a fresh claim (w becomes a candidate with
-// feasible roots c1 / c2). fast: the rows are the clamped ones.
-__device__ __forceinline__ bool expand_arc(const BatchArgs &a, const uint8_t *rows, uint32_t ki, uint32_t slot,
-                                           uint32_t w, const uint4 *kr, uint32_t nq, uint32_t nlevel,
-                                           bool fast, bool near, uint32_t lv, uint64_t &c1, uint64_t &c2,
-                                           uint32_t &nreach) {
-    uint32_t *word = a.visited + (size_t)slot * a.NW + (w >> 5);
-    const uint32_t wbit = 1u << (w & 31);
-    uint4 wq[PLL_MAX_T / 16];
-#pragma unroll
-    for (uint32_t c = 0; c < PLL_MAX_T / 16; ++c)
-        wq[c] = (c < nq) ? __ldg(reinterpret_cast<const uint4 *>(rows + (size_t)w * a.tp) + c)
-                         : make_uint4(0, 0, 0, 0);
-    if (*word & wbit) return false;
-    ++nreach;
-    bool pruned;
-    if (nlevel >= INF8) {
-        atomicOr(&a.ctr->err, ERR_DEPTH);
-        return false;
-    } else if (fast) {
-        pruned = bp_prunes_c(kr, wq, nq, lv);
-        if (!pruned) bp_feasible_c(kr, wq, nq, nlevel, c1, c2);
-    } else if (!near) {
-        pruned = bp_prunes(kr, wq, nq, lv);
-        if (!pruned) bp_feasible(kr, wq, nq, nlevel, c1, c2);
+// ---- nibble rows (bp_nibble.h): bp_q holds the distances clamped to 7, four
+// bits a root, for levels up to NIB_LEVEL
+__device__ __forceinline__ uint4 nib_thresholds4(uint4 q, uint32_t lv) {
+    return make_uint4(nib_thresholds(q.x, lv), nib_thresholds(q.y, lv), nib_thresholds(q.z, lv),
+                      nib_thresholds(q.w, lv));
+}
+__device__ __forceinline__ uint32_t nib_any(uint4 p, uint4 q) {
+    return nib_within(p.x, q.x) | nib_within(p.y, q.y) | nib_within(p.z, q.z) | nib_within(p.w, q.w);
+}
+__device__ __forceinline__ uint32_t nib_mask(uint4 p, uint4 q) {
+    return nib_roots(nib_within(p.x, q.x), nib_within(p.y, q.y), nib_within(p.z, q.z), nib_within(p.w, q.w));
+}
+
+// The nibble row of vertex v (qn = 1 or 2 chunks; the second chunk is zero
+// without one): one 32-byte load a lane where the row has 32 bytes. The sweep
+// is bound by the L1's rate of scattered accesses (81 % of its peak on the
+// heaviest R-MAT-19 launch), and two 16-byte loads of one sector count twice
+// there: R-MAT-20's sweeps take 51.4 ms with one load, 55.3 ms with two.
+__device__ __forceinline__ void load_row(const BatchArgs &a, uint32_t v, uint4 &q0, uint4 &q1) {
+    if (a.qn > 1) {
+        const uint4 *row = a.bp_q + 2 * (size_t)v;
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(q0.x), "=r"(q0.y), "=r"(q0.z), "=r"(q0.w), "=r"(q1.x), "=r"(q1.y), "=r"(q1.z), "=r"(q1.w)
+            : "l"(row));
     } else {
-        pruned = bp_test_plain(a, ki, w, nlevel, c1, c2);
+        q0 = __ldg(a.bp_q + v);
+        q1 = make_uint4(0, 0, 0, 0);
     }
-    if (pruned) return false;
-    c1 &= a.rootbits[2 * slot + 1];
-    c2 &= a.rootbits[2 * slot];
-    if (quick_masks(a, ki, w, c1, c2)) return false;
-    return !(atomicOr(word, wbit) & wbit);
+}
+
+// How a sweep tests the bit-parallel distances of candidates of one level.
+enum BpMode : uint32_t {
+    BP_NONE,    // t = 0, or a level past the last distance (every new vertex is an error)
+    BP_NIBBLE,  // level <= NIB_LEVEL
+    BP_CLAMP,   // level <= FAST_LEVEL: clamped bytes
+    BP_BYTES,   // saturating bytes
+    BP_PLAIN    // level + 2 would overflow a byte
+};
+__device__ __forceinline__ BpMode bp_mode(const BatchArgs &a, uint32_t nlevel) {
+    if (a.t == 0 || nlevel >= INF8) return BP_NONE;
+    if (nlevel <= NIB_LEVEL) return BP_NIBBLE;
+    if (nlevel <= FAST_LEVEL) return BP_CLAMP;
+    return nlevel + 2 < INF8 ? BP_BYTES : BP_PLAIN;
+}
+
+// Deeper levels (past NIB_LEVEL): does a bit-parallel distance prune w, and if
+// not, which roots' masks may (c1, c2)? The byte rows, 16 roots a step.
+__device__ __noinline__ bool bp_test_deep(const BatchArgs &a, BpMode mode, uint32_t k, uint32_t w,
+                                          uint32_t nlevel, uint64_t &c1, uint64_t &c2) {
+    if (mode == BP_PLAIN) return bp_test_plain(a, k, w, nlevel, c1, c2);
+    const uint32_t nq = a.tp >> 4;
+    const uint8_t *rows = mode == BP_CLAMP ? a.bp_c : a.bp_d;
+    uint4 kr[PLL_MAX_T / 16], wq[PLL_MAX_T / 16];
+#pragma unroll
+    for (uint32_t c = 0; c < PLL_MAX_T / 16; ++c) {
+        const bool in = c < nq;
+        kr[c] = in ? __ldg(reinterpret_cast<const uint4 *>(rows + (size_t)k * a.tp) + c) : make_uint4(0, 0, 0, 0);
+        wq[c] = in ? __ldg(reinterpret_cast<const uint4 *>(rows + (size_t)w * a.tp) + c) : make_uint4(0, 0, 0, 0);
+    }
+    c1 = c2 = 0;
+    if (mode == BP_CLAMP) {
+        if (bp_prunes_c(kr, wq, nq, (0x80u + nlevel) * 0x01010101u)) return true;
+        bp_feasible_c(kr, wq, nq, nlevel, c1, c2);
+    } else {
+        if (bp_prunes(kr, wq, nq, nlevel * 0x01010101u)) return true;
+        bp_feasible(kr, wq, nq, nlevel, c1, c2);
+    }
+    return false;
 }
 
 __device__ __forceinline__ void append_cand(const BatchArgs &a, bool keep, int lane, uint32_t slot, uint32_t w,
@@ -393,47 +463,202 @@ __device__ __forceinline__ void append_cand(const BatchArgs &a, bool keep, int l
         }
     }
 }
-// entries [lvl_b, lvl_e) of the current level -> candidates of the next, one
-// warp per entry, 32 consecutive arcs per step (coalesced column loads; the
-// root's row, the same for every lane, sits once per warp in shared memory).
-// 1280 threads per SM (48 registers a thread): the sweep hides the latency of
-// its row and visited-word loads with resident warps.
-// The sweep over entries [b, e) of level `level` by the warps of a grid;
-// kr: this warp's row in shared memory. Adds the arcs it scans and the
-// vertices it tests to nexp / nreach.
+
+// What a warp of the expand sweep keeps in shared memory: for each entry of
+// its chunk the nibble row of the root (q) and its prune thresholds (p), and
+// the arcs that the distances did not prune.
+struct ExpandWarp {
+    uint4 p[32][2], q[32][2];
+    uint32_t queue[64];  // w << 5 | entry of the chunk
+};
+
+// The second part of the expand sweep, for up to 32 arcs of the queue at once:
+// look w up in the root's visited row; if unvisited, which roots' masks may
+// still prune it, and the first masks; claim w if it survives.
+__device__ __forceinline__ void expand_open(const BatchArgs &a, const ExpandWarp &sw, uint32_t at, uint32_t count,
+                                            uint32_t k_lane, uint32_t nlevel, BpMode mode, uint32_t &nreach) {
+    const int lane = threadIdx.x & 31;
+    const bool act = (uint32_t)lane < count;
+    const uint32_t item = act ? sw.queue[at + lane] : 0u;
+    const uint32_t j = item & 31u, w = item >> 5;
+    const uint32_t k = __shfl_sync(FULL, k_lane, j), slot = k - a.k0;
+    bool keep = false;
+    uint64_t c1 = 0, c2 = 0;
+    if (act) {
+        uint32_t *word = a.visited + (size_t)slot * a.NW + (w >> 5);
+        const uint32_t wbit = 1u << (w & 31);
+        if (!(*word & wbit)) {
+            ++nreach;
+            bool pruned = false;
+            if (nlevel >= INF8) {
+                atomicOr(&a.ctr->err, ERR_DEPTH);
+                pruned = true;
+            } else if (mode == BP_NIBBLE) {
+                uint4 q[2];
+                load_row(a, w, q[0], q[1]);
+                uint32_t m1[2] = {0, 0}, m2[2] = {0, 0};
+#pragma unroll
+                for (uint32_t c = 0; c < 2; ++c) {
+                    if (c < a.qn) {
+                        const uint4 kq = sw.q[j][c];
+                        m1[c] = nib_mask(nib_thresholds4(kq, nlevel + 1), q[c]);
+                        m2[c] = nib_mask(nib_thresholds4(kq, nlevel + 2), q[c]) & ~m1[c];
+                    }
+                }
+                c1 = (uint64_t)m1[1] << 32 | m1[0];
+                c2 = (uint64_t)m2[1] << 32 | m2[0];
+            } else if (mode != BP_NONE) {
+                pruned = bp_test_deep(a, mode, k, w, nlevel, c1, c2);
+            }
+            if (c1 | c2) {
+                // a reduction of 2 needs S^{-1} of both ends non-empty, one of 1
+                // S^{-1} of one end and S^{-1} or S^0 of the other
+                const ulonglong2 ew = __ldg(a.bp_e + w), ek = __ldg(a.bp_e + k);
+                c1 &= (ek.x & ew.y) | (ek.y & ew.x);
+                c2 &= ek.x & ew.x;
+                pruned = quick_masks(a, k, w, c1, c2);
+            }
+            if (!pruned) keep = !(atomicOr(word, wbit) & wbit);
+        }
+    }
+    append_cand(a, keep, lane, slot, w, c1, c2);
+}
+
+#ifndef PLL_HEAVY_DEG
+#define PLL_HEAVY_DEG 64
+#endif
+#ifndef PLL_EXPAND_TPS
+#define PLL_EXPAND_TPS 1024
+#endif
+constexpr uint32_t HEAVY_DEG = PLL_HEAVY_DEG;
+constexpr int EXPAND_TPS = PLL_EXPAND_TPS;
+
+// The expand sweep: entries [b, e) of level `level` and the slices of its long
+// entries -> candidates of the next, by the warps of a grid. A warp takes a
+// chunk of up to 32 of them (fewer when the level has fewer than that for
+// every warp): lane j fetches entry j's key,
+// row bounds and nibble row, so these dependent loads are in flight for the
+// whole chunk, and then the arcs are tested: those of an entry of at least
+// HEAVY_DEG neighbours 32 at a time, the others' laid end to end over the lanes.
+//
+// An arc (u, w) is first put to the bit-parallel distances, which need one
+// 32-byte sector of w (an L2-resident table) and prune 19 of 20; only then is
+// w looked up in the root's visited row, a scattered DRAM access. (Vertices
+// that the distances prune are never marked, so the order of the two tests
+// changes nothing.) The arcs that are left go through a queue in shared
+// memory, so that the rest of the test runs with full warps.
+//
+// Bound by the L1's rate of scattered accesses (one row per arc). 1024 threads
+// per SM (64 registers; 1280 threads spill: 52.9 against 51.4 ms). All of
+// R-MAT-20's expand sweeps (t = 64; 3.15G arcs): 95.1 ms with a warp per
+// entry, 64-byte rows and the visited word first; 71.9 ms with chunks, the
+// queue and nibble rows; 55.3 ms with long lists in slices; 51.4 ms with one
+// load a row; 39.2 ms with the lists cut at rank k0 (1.64G arcs left).
 __device__ __forceinline__ void expand_body(const BatchArgs &a, unsigned long long b, unsigned long long e,
-                                            uint32_t level, uint4 *kr, uint32_t &nexp, uint32_t &nreach) {
+                                            unsigned long long slice_n, uint32_t level, ExpandWarp &sw,
+                                            uint32_t &nexp, uint32_t &nreach) {
     const int lane = threadIdx.x & 31;
     const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
     const unsigned long long gw = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nq = a.tp >> 4;
-    const uint32_t nlevel = level + 1;                // level of the candidates
-    const bool fast = nlevel <= FAST_LEVEL;           // clamped rows, plain arithmetic
-    const bool near = nlevel + 2 >= INF8;             // byte sums could overflow
-    const uint32_t lv = fast ? (0x80u + nlevel) * 0x01010101u : nlevel * 0x01010101u;
-    const uint8_t *rows = fast ? a.bp_c : a.bp_d;
-    for (unsigned long long j = b + gw; j < e; j += nwarps) {
+    const uint32_t nlevel = level + 1;  // level of the candidates
+    const BpMode mode = bp_mode(a, nlevel);
+    // slices that did not all fit: every entry is expanded whole
+    const uint32_t most = slice_n <= a.slice_cap ? SLICE : ~0u;
+    const unsigned long long ne = e - b, items = ne + (slice_n <= a.slice_cap ? slice_n : 0);
+    const unsigned long long per = (items + nwarps - 1) / nwarps;
+    const uint32_t G = per < 1 ? 1u : per < 32 ? (uint32_t)per : 32u;
+    for (unsigned long long c0 = gw * G; c0 < items; c0 += nwarps * G) {
         // entries and candidates are written by other SMs between the phases of
         // one launch (k_batch_levels): read them from L2, never from a line the
         // L1 kept from an earlier level
-        const uint64_t key = __ldcg(a.out + j);
-        const uint32_t u = (uint32_t)(key >> 32);
-        const uint32_t k = entry_hub((uint32_t)key);
-        const uint32_t slot = k - a.k0;
-        __syncwarp();
-        if ((uint32_t)lane < nq) kr[lane] = __ldg(reinterpret_cast<const uint4 *>(rows + (size_t)k * a.tp) + lane);
-        __syncwarp();
-        const uint32_t eb = a.roff[u], ee = a.roff[u + 1];
-        if (lane == 0) nexp += ee - eb;
-        for (uint32_t x = eb; x < ee; x += 32) {
-            bool keep = false;
-            uint32_t w = 0;
-            uint64_t c1 = 0, c2 = 0;
-            if (x + lane < ee) {
-                w = a.rcol[x + lane];
-                keep = expand_arc(a, rows, k, slot, w, kr, nq, nlevel, fast, near, lv, c1, c2, nreach);
+        const uint32_t cnt = items - c0 < G ? (uint32_t)(items - c0) : G;
+        uint32_t k = a.k0, eb = 0, deg = 0;
+        __syncwarp();  // the previous chunk is done with sw
+        if ((uint32_t)lane < cnt) {
+            if (c0 + lane < ne) {
+                const uint64_t key = __ldcg(a.out + b + c0 + lane);
+                const uint32_t u = (uint32_t)(key >> 32);
+                k = entry_hub((uint32_t)key);
+                eb = first_arc(a, u, nlevel);
+                deg = min(a.roff[u + 1] - eb, most);
+            } else {
+                const uint4 sl = __ldcg(a.slices + (c0 + lane - ne));
+                k = sl.x;
+                eb = sl.y;
+                deg = sl.z - sl.y;
             }
-            append_cand(a, keep, lane, slot, w, c1, c2);
+            nexp += deg;
+            if (mode == BP_NIBBLE) {
+                uint4 q[2];
+                load_row(a, k, q[0], q[1]);
+#pragma unroll
+                for (uint32_t c = 0; c < 2; ++c) {
+                    sw.q[lane][c] = q[c];
+                    sw.p[lane][c] = nib_thresholds4(q[c], nlevel);
+                }
+            }
+        }
+        __syncwarp();
+        // entries with at least HEAVY_DEG neighbours one by one (arcs [x, xe) of
+        // entry j are next), then the other entries' arcs end to end
+        uint32_t heavy = __ballot_sync(FULL, deg >= HEAVY_DEG);
+        const uint32_t len = deg < HEAVY_DEG ? deg : 0;
+        uint32_t incl = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const uint32_t total = __shfl_sync(FULL, incl, 31);
+        const uint32_t excl = incl - len;
+        uint32_t x = 0, xe = 0, j = 0, x0 = 0, nqueue = 0;
+        for (;;) {
+            bool open;
+            uint32_t arc;
+            if (x >= xe && heavy) {
+                j = __ffs(heavy) - 1;
+                heavy &= heavy - 1;
+                x = __shfl_sync(FULL, eb, j);
+                xe = x + __shfl_sync(FULL, deg, j);
+            }
+            const bool more = x < xe || x0 < total;
+            if (x < xe) {
+                arc = x + lane;
+                open = arc < xe;
+                x += 32;
+            } else {
+                const uint32_t y = x0 + lane;
+                j = 0;  // owner: the last entry whose first arc is <= y
+#pragma unroll
+                for (uint32_t step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(FULL, excl, j + step) <= y) j += step;
+                arc = __shfl_sync(FULL, eb - excl, j) + y;
+                open = y < total;
+                x0 += 32;
+            }
+            uint32_t w = 0;
+            if (open) {
+                w = a.rcol[arc];
+                if (mode == BP_NIBBLE) {
+                    uint4 q0, q1;
+                    load_row(a, w, q0, q1);
+                    uint32_t hit = nib_any(sw.p[j][0], q0);
+                    if (a.qn > 1) hit |= nib_any(sw.p[j][1], q1);
+                    open = hit == 0;
+                    nreach += hit != 0;
+                }
+            }
+            const unsigned m = __ballot_sync(FULL, open);
+            if (open) sw.queue[nqueue + __popc(m & ((1u << lane) - 1u))] = w << 5 | j;
+            nqueue += __popc(m);
+            if (nqueue >= 32 || (!more && nqueue)) {
+                __syncwarp();
+                const uint32_t take = min(nqueue, 32u);
+                nqueue -= take;
+                expand_open(a, sw, nqueue, take, k, nlevel, mode, nreach);
+                __syncwarp();
+            }
+            if (!more && nqueue == 0) break;
         }
     }
 }
@@ -449,17 +674,20 @@ __device__ __forceinline__ void flush_work(const BatchArgs &a, int w0, uint32_t 
     if ((threadIdx.x & 31) == 0 && y) atomicAdd(&a.ctr->work[w0 + 1], (unsigned long long)y);
 }
 
+__device__ __forceinline__ ExpandWarp &expand_warp(uint4 *dyn) {
+    return reinterpret_cast<ExpandWarp *>(dyn)[threadIdx.x >> 5];
+}
+
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_expand(BatchArgs a) {
-    extern __shared__ uint4 s_rows[];
+__global__ void __launch_bounds__(BLOCK, EXPAND_TPS / BLOCK) k_batch_expand(BatchArgs a) {
+    extern __shared__ uint4 s_dyn[];
     uint32_t nexp = 0, nreach = 0;
-    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->level,
-                s_rows + (size_t)(threadIdx.x >> 5) * (PLL_MAX_T / 16), nexp, nreach);
+    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->slice_n, a.desc->level, expand_warp(s_dyn), nexp, nreach);
     flush_work(a, 2, nexp, nreach);
 }
 
 template <int BLOCK>
-constexpr size_t expand_smem() { return (size_t)(BLOCK / 32) * (PLL_MAX_T / 16) * sizeof(uint4); }
+constexpr size_t expand_smem() { return (size_t)(BLOCK / 32) * sizeof(ExpandWarp); }
 
 // bp_c = min(bp_d, CLAMP) bytewise, 16 bytes per thread and step
 __global__ void k_clamp_rows(const uint4 *bp_d, uint4 *bp_c, size_t n16) {
@@ -474,6 +702,22 @@ __global__ void k_clamp_rows(const uint4 *bp_d, uint4 *bp_c, size_t n16) {
             x[j] = (x[j] & 0x3F3F3F3Fu) | (big * CLAMP);
         }
         bp_c[i] = v;
+    }
+}
+
+// Nibble rows (see expand_body): thread g of vertex v turns the 32 bytes of
+// roots 32 g .. 32 g + 31 (16 where the row ends) into four words.
+__global__ void k_nibble_rows(const uint8_t *__restrict__ bp_d, uint32_t tp, uint32_t qn, uint4 *bp_q, size_t nrows) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nrows; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t v = i / qn;
+        const uint32_t g = (uint32_t)(i - v * qn);
+        const uint4 *row = reinterpret_cast<const uint4 *>(bp_d + v * tp) + 2 * g;
+        uint32_t d[8];
+        const uint4 lo = __ldg(row);
+        const uint4 hi = 32 * g + 16 < tp ? __ldg(row + 1) : make_uint4(~0u, ~0u, ~0u, ~0u);
+        d[0] = lo.x; d[1] = lo.y; d[2] = lo.z; d[3] = lo.w;
+        d[4] = hi.x; d[5] = hi.y; d[6] = hi.z; d[7] = hi.w;
+        bp_q[i] = make_uint4(nib_pack(d, 0), nib_pack(d, 1), nib_pack(d, 2), nib_pack(d, 3));
     }
 }
 
@@ -730,6 +974,7 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
                 if (pos < a.out_cap) a.out[pos] = pack_tuple(w, a.k0 + slot, level);
                 else atomicOr(&a.ctr->err, ERR_BUF);
             }
+            append_slices(a, keep, lane, w, a.k0 + slot, level);
         }
     }
 }
@@ -766,6 +1011,7 @@ __device__ __forceinline__ bool grid_barrier(const BatchArgs &a, LoopState *ls) 
             ls->err = atomicOr(&a.ctr->err, 0u);
             ls->cand_n = atomicAdd(&a.ctr->cand_n, 0ull);
             ls->out_n = atomicAdd(&a.ctr->out_n, 0ull);
+            ls->slice_n = atomicExch(&a.ctr->slice_n, 0ull);  // the sweep before the barrier wrote or read them all
             __threadfence();
             atomicAdd(&ls->gen, 1u);
         } else {
@@ -793,19 +1039,19 @@ __device__ __forceinline__ bool grid_barrier(const BatchArgs &a, LoopState *ls) 
 // needs the host. Block 0 adds the phases' wall times to the loop state.
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs a) {
-    extern __shared__ uint4 s_rows[];
+    extern __shared__ uint4 s_dyn[];
     __shared__ TestCand s_cand[BLOCK / 32][32];
     LoopState *ls = a.loop;
-    uint4 *kr = s_rows + (size_t)(threadIdx.x >> 5) * (PLL_MAX_T / 16);
+    ExpandWarp &sw = expand_warp(s_dyn);
     TestCand *tc = s_cand[threadIdx.x >> 5];
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
-    unsigned long long lvl_b = a.desc->lvl_b, lvl_e = a.desc->lvl_e, cand_e = 0;
+    unsigned long long lvl_b = a.desc->lvl_b, lvl_e = a.desc->lvl_e, slice_n = a.desc->slice_n, cand_e = 0;
     uint32_t level = 0, nexp = 0, nreach = 0, n_scan = 0, n_mask = 0;
     unsigned long long ns_e = 0, ns_t = 0;
     constexpr uint32_t STOP = ERR_DEPTH | ERR_BUF | ERR_TIMEOUT;
     while (lvl_b < lvl_e) {
         const unsigned long long t0 = timer ? global_ns() : 0;
-        expand_body(a, lvl_b, lvl_e, level, kr, nexp, nreach);
+        expand_body(a, lvl_b, lvl_e, slice_n, level, sw, nexp, nreach);
         if (!grid_barrier(a, ls)) break;
         const unsigned long long t1 = timer ? global_ns() : 0;
         if (*(volatile uint32_t *)&ls->err & STOP) break;
@@ -823,6 +1069,7 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs 
         const unsigned long long on = *(volatile unsigned long long *)&ls->out_n;
         lvl_b = lvl_e;
         lvl_e = on < a.out_cap ? on : a.out_cap;
+        slice_n = *(volatile unsigned long long *)&ls->slice_n;
         ++level;
     }
     flush_work(a, 2, nexp, nreach);
@@ -845,6 +1092,8 @@ __device__ __forceinline__ void advance_desc(const BatchArgs &a, int phase) {
         d->level = 0;
         d->cand_b = 0;
         d->cand_e = 0;
+        d->slice_n = a.ctr->slice_n;
+        a.ctr->slice_n = 0;
         if (a.loop) a.loop->t_mark = global_ns();
     } else if (phase == 1) {   // after expand: candidates of level + 1
         d->cand_b = d->cand_e;
@@ -853,6 +1102,8 @@ __device__ __forceinline__ void advance_desc(const BatchArgs &a, int phase) {
         d->lvl_b = d->lvl_e;
         d->lvl_e = on < a.out_cap ? on : a.out_cap;
         d->level += 1;
+        d->slice_n = a.ctr->slice_n;
+        a.ctr->slice_n = 0;
     }
 }
 
@@ -875,13 +1126,12 @@ __device__ __forceinline__ const BatchArgs &args_to_shared(const BatchArgs *ap, 
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_expand_g(const BatchArgs *__restrict__ ap) {
-    extern __shared__ uint4 s_rows[];
+__global__ void __launch_bounds__(BLOCK, EXPAND_TPS / BLOCK) k_batch_expand_g(const BatchArgs *__restrict__ ap) {
+    extern __shared__ uint4 s_dyn[];
     __shared__ BatchArgs s_args;
     const BatchArgs &a = args_to_shared(ap, &s_args);
     uint32_t nexp = 0, nreach = 0;
-    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->level,
-                s_rows + (size_t)(threadIdx.x >> 5) * (PLL_MAX_T / 16), nexp, nreach);
+    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->slice_n, a.desc->level, expand_warp(s_dyn), nexp, nreach);
     flush_work(a, 2, nexp, nreach);
 }
 
@@ -983,6 +1233,22 @@ int batch_clamp_rows(const uint8_t *bp_d, uint8_t *bp_c, size_t bytes, int grid,
     if (bytes == 0) return PLL_OK;
     k_clamp_rows<<<grid > 0 ? grid : 1, 256, 0, s>>>(reinterpret_cast<const uint4 *>(bp_d),
                                                      reinterpret_cast<uint4 *>(bp_c), bytes / 16);
+    PLL_TRY(cudaGetLastError());
+    return PLL_OK;
+}
+
+int batch_row_starts(uint32_t n, uint32_t k0, const uint32_t *roff, const uint32_t *rcol, uint32_t *rstart,
+                     int grid, cudaStream_t s) {
+    const int want = (int)((n + 255) / 256);
+    k_row_starts<<<want < 4 * grid ? want : 4 * grid, 256, 0, s>>>(n, k0, roff, rcol, rstart);
+    PLL_TRY(cudaGetLastError());
+    return PLL_OK;
+}
+
+int batch_nibble_rows(const uint8_t *bp_d, uint32_t n, uint32_t tp, uint32_t qn, uint4 *bp_q, int grid,
+                      cudaStream_t s) {
+    if (n == 0 || qn == 0) return PLL_OK;
+    k_nibble_rows<<<grid > 0 ? grid : 1, 256, 0, s>>>(bp_d, tp, qn, bp_q, (size_t)n * qn);
     PLL_TRY(cudaGetLastError());
     return PLL_OK;
 }

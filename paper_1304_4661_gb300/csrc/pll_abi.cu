@@ -95,7 +95,7 @@ struct Timer {
 
 // Step 3: batched pruned BFS + cleanup + append, then step 4.
 int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, const uint8_t *inX,
-                 uint32_t bmax, uint32_t block, uint32_t flags, cudaStream_t s) {
+                 const ulonglong2 *bp_e, uint32_t bmax, uint32_t block, uint32_t flags, cudaStream_t s) {
     // how each batch's levels run: a CUDA graph whose while node loops over
     // the two sweeps (the default), one cooperative persistent launch, or
     // separate launches enqueued by the host
@@ -150,15 +150,19 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         init.timeout_ns = test_barrier_timeout_ns();
         PLL_TRY(cudaMemcpyAsync(d_loop, &init, sizeof(init), cudaMemcpyHostToDevice, s));
     }
-    // clamped copy of the bit-parallel distance rows for the expand sweep
+    // clamped copies of the bit-parallel distance rows for the expand sweep
     PoolMem m_bpc(s);
     PLL_CHECK(m_bpc.alloc(std::max<size_t>((size_t)n * ix->tp, 16)));
     PLL_CHECK(batch_clamp_rows(ix->d_bp_d, m_bpc.as<uint8_t>(), (size_t)n * ix->tp, grid[0], s));
-    ix->stats.launches += 1;
+    const uint32_t qn = (ix->t + 31) / 32;
+    PoolMem m_bpq(s);
+    PLL_CHECK(m_bpq.alloc(std::max<size_t>((size_t)n * qn * 16, 16)));
+    PLL_CHECK(batch_nibble_rows(ix->d_bp_d, n, ix->tp, qn, m_bpq.as<uint4>(), grid[0], s));
+    ix->stats.launches += ix->t ? 2 : 0;
     // visited bitmap, one row of ceil(n / 32) words per root slot; cleared once
     // here, then lazily after each batch (only the words the batch set)
     const uint32_t NW = (n + 31) / 32;
-    PoolMem m_vis(s), m_ht(s), m_htoff(s), m_itemp(s), m_bits(s), m_cand(s), m_candc(s), m_out(s),
+    PoolMem m_vis(s), m_ht(s), m_htoff(s), m_itemp(s), m_cand(s), m_candc(s), m_out(s),
         m_sorted(s), m_keep(s), m_temp(s);
     PLL_CHECK(m_vis.alloc((size_t)bmax * NW * 4));
     PLL_TRY(cudaMemsetAsync(m_vis.p, 0, (size_t)bmax * NW * 4, s));
@@ -178,7 +182,6 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PLL_CHECK(m_htoff.alloc(((size_t)bmax + 1) * 8));
     const size_t itemp_bytes = ((batch_init_temp_bytes(bmax) + 255) & ~(size_t)255) + ((size_t)bmax + 1) * 8 + 256;
     PLL_CHECK(m_itemp.alloc(itemp_bytes));
-    PLL_CHECK(m_bits.alloc((size_t)bmax * 16));
     PoolMem m_filt(s);
     PLL_CHECK(m_filt.alloc((size_t)bmax * FILT_WORDS * 4));
     uint64_t cand_cap = caps.cand ? caps.cand
@@ -207,6 +210,11 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PLL_CHECK(m_cand.alloc(cand_cap * 8));
     PLL_CHECK(m_candc.alloc(cand_cap * 16));
     PLL_CHECK(alloc_out());
+    PoolMem m_rstart(s);
+    PLL_CHECK(m_rstart.alloc((size_t)n * 4));
+    PoolMem m_slices(s);
+    const uint64_t slice_cap = caps.cand ? std::min<uint64_t>(caps.cand, SLICE_CAP) : SLICE_CAP;
+    PLL_CHECK(m_slices.alloc(slice_cap * 16));
 
     // pinned mirror of the counters and the level descriptor
     struct Mirror {
@@ -295,24 +303,26 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         }
         BatchArgs a{};
         a.n = n; a.t = ix->t; a.tp = ix->tp;
-        a.roff = roff; a.rcol = rcol;
+        a.roff = roff; a.rcol = rcol; a.rstart = m_rstart.as<uint32_t>();
         a.bp_d = ix->d_bp_d; a.bp_c = m_bpc.as<uint8_t>(); a.bp_m = ix->d_bp_m; a.inX = inX;
+        a.bp_q = m_bpq.as<uint4>(); a.qn = qn; a.bp_e = bp_e;
         a.lab_off = st.off; a.lab_len = st.len; a.pool = st.pool;
         a.k0 = k0; a.B = k1 - k0; a.NW = NW;
         a.visited = m_vis.as<uint32_t>();
         a.ht = m_ht.as<uint32_t>();
         a.ht_off = m_htoff.as<unsigned long long>();
         a.ht_cap = ht_cap;
-        a.rootbits = m_bits.as<uint64_t>();
         a.filt = m_filt.as<uint32_t>();
         a.cand = m_cand.as<uint64_t>(); a.candc = m_candc.as<uint64_t>(); a.cand_cap = cand_cap;
         a.out = m_out.as<uint64_t>(); a.out_cap = out_cap;
+        a.slices = m_slices.as<uint4>(); a.slice_cap = slice_cap;
         a.ctr = d_ctr; a.desc = d_desc; a.loop = d_loop;
         PLL_TRY(cudaEventRecord(ev0, s));
         PLL_TRY(cudaMemsetAsync(d_ctr, 0, 16, s));  // cand_n, out_n
-        PLL_TRY(cudaMemsetAsync(&d_ctr->err, 0, 4, s));
+        PLL_TRY(cudaMemsetAsync(&d_ctr->slice_n, 0, 12, s));  // slice_n, err
+        PLL_CHECK(batch_row_starts(n, k0, roff, rcol, m_rstart.as<uint32_t>(), grid[0], s));
         PLL_CHECK(batch_init(a, m_itemp.p, itemp_bytes, s));
-        ix->stats.launches += 3;
+        ix->stats.launches += 4;
         ix->stats.cub_calls += 1;
         if (device_levels) {
             // every level of the batch in one launch; events around it
@@ -602,8 +612,10 @@ int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t 
     PLL_TRY(dev_malloc(&ix->d_bp_d, std::max<size_t>((size_t)n * ix->tp, 16)));
     PLL_TRY(dev_malloc(&ix->d_bp_m, std::max<size_t>(nt, 1) * 16));
     uint32_t bp_levels = 0;
+    PoolMem m_bpe(s);  // non-empty roots of each vertex, for the pruned stage
+    if (t) PLL_CHECK(m_bpe.alloc(std::max<size_t>((size_t)n * 16, 16)));
     PLL_CHECK(bp_run(n, t, graphs, m_roff.as<uint32_t>(), m_rcol.as<uint32_t>(), ix->d_bp_root,
-                     ix->d_bp_cnt, ix->d_bp_S, ix->d_bp_d, ix->d_bp_m, d_err, s, &bp_levels));
+                     ix->d_bp_cnt, ix->d_bp_S, ix->d_bp_d, ix->d_bp_m, m_bpe.as<ulonglong2>(), d_err, s, &bp_levels));
     if (t && n) {
         ix->stats.launches += 4 + 2ull * bp_levels;  // seed, chunk counts/fill, passes, finish
         ix->stats.cub_calls += 1;
@@ -615,7 +627,7 @@ int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t 
     // ---- 3 + 4. pruned labels
     tm.start();
     PLL_CHECK(pruned_stage(ix, m_roff.as<uint32_t>(), m_rcol.as<uint32_t>(), m_inX.as<uint8_t>(),
-                           bmax, block, o.flags, s));
+                           m_bpe.as<ulonglong2>(), bmax, block, o.flags, s));
     ix->stats.ms_pruned = tm.stop_ms();
     if (spool) {
         uint64_t high = 0;

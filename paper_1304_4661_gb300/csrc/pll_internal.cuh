@@ -232,9 +232,11 @@ int prep_select_bp_graphs(uint32_t G, uint32_t t, const uint32_t *d_gs, const ui
 
 // k_bp.cu
 inline uint32_t bp_stride(uint32_t t) { return (t + 15u) & ~15u; }
+// d_bp_e (or null): per vertex the roots with S^{-1} non-empty (x) and with
+// S^{-1} or S^0 non-empty (y)
 int bp_run(uint32_t n, uint32_t t, uint32_t graphs, const uint32_t *d_roff, const uint32_t *d_rcol,
            const uint32_t *d_root, const uint32_t *d_cnt, const uint32_t *d_S, uint8_t *d_bp_d,
-           uint64_t *d_bp_m, uint32_t *d_err, cudaStream_t s, uint32_t *levels);
+           uint64_t *d_bp_m, ulonglong2 *d_bp_e, uint32_t *d_err, cudaStream_t s, uint32_t *levels);
 
 // k_bp.cu, for pll_bp_labels_noalloc: the same stage on caller scratch
 size_t bp_scratch_bytes(uint32_t n, uint64_t nnz, size_t *cub_bytes);
@@ -248,6 +250,9 @@ int bp_run_in(uint32_t n, uint32_t t, const uint32_t *d_roff, const uint32_t *d_
 // at least HT_MIN; labels longer than HT_MAX / 2 are binary-searched instead
 constexpr uint32_t FILT_WORDS = 32;     // 1024-bit hub filter per root of a batch
 constexpr uint32_t FILT_MAX_LEN = 128;  // roots with longer labels have no filter
+#ifndef PLL_SLICE
+#define PLL_SLICE 64
+#endif
 constexpr uint32_t HT_MIN = 32;
 constexpr uint32_t HT_MAX = 1u << 16;
 __host__ __device__ inline uint32_t ht_size(uint32_t len) {
@@ -257,6 +262,12 @@ __host__ __device__ inline uint32_t ht_size(uint32_t len) {
     return s;
 }
 
+// An entry of the frontier whose vertex has more than SLICE neighbours is
+// expanded in slices of SLICE arcs, so that no warp of the expand sweep is
+// left with a hub's list while the others are done.
+constexpr uint32_t SLICE = PLL_SLICE;
+constexpr uint64_t SLICE_CAP = 64ull << 20;  // slices of one level; past it entries stay whole
+
 struct BatchCounters {
     unsigned long long cand_n;    // candidates appended (all levels of the batch)
     unsigned long long out_n;     // entries (u, k, d) appended
@@ -264,6 +275,7 @@ struct BatchCounters {
                                   // claimed (cumulative)
     unsigned long long nkept;     // entries kept by the cleanup
     unsigned long long pool_top;  // label pool bump pointer
+    unsigned long long slice_n;   // slices of the next level's long entries
     uint32_t err;                 // errors of the batch's BFS (reset per batch)
     uint32_t err_post;            // errors of the appends (never reset)
 };
@@ -275,7 +287,7 @@ constexpr uint32_t ERR_TIMEOUT = 1u << 6;  // a grid barrier waited past its lim
 struct LoopState {
     unsigned int count, gen;            // barrier arrivals, generation
     unsigned int err, pad;              // snapshot of BatchCounters::err
-    unsigned long long cand_n, out_n;   // snapshots of the counts
+    unsigned long long cand_n, out_n, slice_n;  // snapshots of the counts
     unsigned long long timeout_ns;      // longest barrier wait
     unsigned long long ns_expand, ns_test;  // phase wall times (block 0)
     unsigned long long levels;          // levels run
@@ -285,6 +297,7 @@ struct LoopState {
 struct LevelDesc {
     unsigned long long lvl_b, lvl_e;    // entries of the current level
     unsigned long long cand_b, cand_e;  // candidates of the next level
+    unsigned long long slice_n;         // slices of the current level's long entries
     unsigned long long roots_n;         // level-0 entries
     uint32_t level;
     uint32_t pad;
@@ -293,31 +306,40 @@ struct LevelDesc {
 struct BatchArgs {
     uint32_t n, t, tp;
     const uint32_t *roff, *rcol;
+    const uint32_t *rstart;    // per vertex: its first neighbour of rank >= k0
     const uint8_t *bp_d;
     const uint8_t *bp_c;       // bp_d with every byte clamped to 63 (same stride)
+    const uint4 *bp_q;         // [n][qn] distances clamped to 7, four bits a root
+    const ulonglong2 *bp_e;    // [n] roots with S^{-1} non-empty, with S^{-1} or S^0 non-empty
     const uint64_t *bp_m;
     const uint8_t *inX;
     const uint64_t *lab_off;   // per-vertex start in pool
     const uint32_t *lab_len;   // per-vertex length (entries with hub < k0)
     const uint32_t *pool;
     uint32_t k0, B, NW;        // roots [k0, k0 + B), NW = ceil(n / 32)
+    uint32_t qn;               // 16-byte chunks of a bp_q row: ceil(t / 32)
     uint32_t *visited;         // [B][NW] bitmap: row of root slot s holds one bit
                                // per vertex (the per-root visited set of Alg. 1)
     uint32_t *ht;              // pool of root label hash tables
     unsigned long long *ht_off;  // [B + 1] table offsets in the pool (exclusive sums)
     unsigned long long ht_cap;   // pool capacity (entries)
-    uint64_t *rootbits;        // [B][2] feasibility masks
     uint32_t *filt;            // [B][FILT_WORDS] per-root filter of its label's hubs
     uint64_t *cand;            // (slot << 32 | vertex), all levels
     uint64_t *candc;           // [cand_cap][2] roots whose masks may still prune
     unsigned long long cand_cap;
     uint64_t *out;             // entries (u << 32 | k << 8 | d), all levels
     unsigned long long out_cap;
+    uint4 *slices;             // (hub, first arc, end arc, -) past an entry's first SLICE arcs
+    unsigned long long slice_cap;
     BatchCounters *ctr;
     LevelDesc *desc;
     LoopState *loop;           // device-side level loop (k_batch_levels)
 };
 int batch_grid(uint32_t block, int *grid);  // grid[2]: expand, test
+// rstart[u] = index of u's first neighbour of rank >= k0, from its value for an
+// earlier (smaller) k0
+int batch_row_starts(uint32_t n, uint32_t k0, const uint32_t *roff, const uint32_t *rcol, uint32_t *rstart,
+                     int grid, cudaStream_t s);
 int batch_init(const BatchArgs &a, void *temp, size_t temp_bytes, cudaStream_t s);
 size_t batch_init_temp_bytes(uint32_t bmax);
 int batch_level(const BatchArgs &a, const int *grid, uint32_t block, cudaStream_t s,
@@ -335,6 +357,10 @@ int batch_graph_build(uint32_t block, const int *grid, const BatchArgs *d_args, 
 int batch_clear(const BatchArgs &a, int grid, cudaStream_t s);
 // bp_c = min(bp_d, 63) bytewise (bytes a multiple of 16)
 int batch_clamp_rows(const uint8_t *bp_d, uint8_t *bp_c, size_t bytes, int grid, cudaStream_t s);
+
+// bp_q from bp_d (qn = ceil(t / 32) chunks a row)
+int batch_nibble_rows(const uint8_t *bp_d, uint32_t n, uint32_t tp, uint32_t qn, uint4 *bp_q, int grid,
+                      cudaStream_t s);
 
 // k_labels.cu
 struct LabelStore {

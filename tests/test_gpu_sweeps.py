@@ -1,0 +1,71 @@
+"""The pruned stage's sweeps at the sizes where their paths change, against the
+oracle's labels: row widths (t around 16, 32, 48), levels at which the distance
+test changes its rows (5 to nibbles, 60 to clamped bytes, then bytes), neighbour
+lists around the slice length, lists cut at every batch's first rank, labels
+longer than a root's table, and depths next to the 8-bit limit."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1304_4661_gb300 import graphgen as gg
+from paper_1304_4661_gb300 import pll
+
+from . import graphs
+from .gpu_util import first_label_diff, gpu_build, same_labels
+
+pytestmark = pytest.mark.gpu
+
+
+def hubs(degrees, seed):
+    """One hub of each given degree over a shared set of leaves, plus random edges among them."""
+    n = len(degrees) + max(degrees) + 40
+    e, leaf0 = [], len(degrees)
+    for h, d in enumerate(degrees):
+        e += [(h, leaf0 + (7 * h + i) % (n - leaf0)) for i in range(d)]
+    x = gg.below(seed, 4 * n, n).astype(np.int64).reshape(-1, 2)
+    e = np.concatenate([np.asarray(e, dtype=np.int64), x])
+    return gg.from_edges(n, e[:, 0], e[:, 1], f"hubs{degrees}")
+
+
+def check(g, t, **kw):
+    ref = oracle.Index(g.offsets, g.cols, t)
+    ix = gpu_build(g, t, **kw)
+    La, Lb = ix.labels(), ref.labels()
+    assert same_labels(La, Lb), first_label_diff(La, Lb, g.n)
+
+
+@pytest.mark.parametrize("t", [0, 1, 15, 17, 31, 32, 33, 48, 49, 63])
+@pytest.mark.parametrize("root_batch", [0, 3, 64])
+def test_row_widths_and_slice_lengths(t, root_batch):
+    check(hubs([63, 64, 65, 127, 128, 129, 192, 193, 257, 700], 5), t, root_batch=root_batch)
+
+
+@pytest.mark.parametrize("t", [0, 2, 33])
+@pytest.mark.parametrize("make", [lambda: graphs.grid(4, 9), lambda: graphs.grid(3, 70), lambda: graphs.grid(2, 130),
+                                  lambda: graphs.path(250), lambda: graphs.cycle(505)],
+                         ids=["grid4x9", "grid3x70", "grid2x130", "path250", "cycle505"])
+@pytest.mark.parametrize("root_batch", [1, 40, 0])
+def test_levels_across_the_row_kinds(make, t, root_batch):
+    check(make(), t, root_batch=root_batch)
+
+
+@pytest.mark.parametrize("t", [0, 1])
+@pytest.mark.parametrize("n", [300, 520])
+def test_a_depth_of_255_is_still_a_range_error(n, t):
+    g = graphs.path(n) if n == 300 else graphs.cycle(n)
+    with pytest.raises(pll.PLLError) as e:
+        gpu_build(g, t)
+    assert e.value.code == pll.PLL_E_RANGE
+
+
+def test_labels_longer_than_a_roots_table():
+    """No bit-parallel labels on a random-order high-diameter graph: labels of
+    over a thousand entries, past the largest reach table's share of four bytes
+    an entry."""
+    g = gg.ws(4000, 8, 0.5, 9)
+    order = np.argsort(gg.uniform(3, g.n)).astype(np.uint32)
+    ref = oracle.Index(g.offsets, g.cols, 0, order=order).labels()
+    assert np.diff(ref.offsets.astype(np.int64)).max() > 600
+    for root_batch in (0, 100):
+        ix = gpu_build(g, 0, order=order, root_batch=root_batch)
+        assert same_labels(ix.labels(), ref), first_label_diff(ix.labels(), ref, g.n)
