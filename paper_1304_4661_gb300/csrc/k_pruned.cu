@@ -39,13 +39,11 @@
 //           bit-parallel bound of a pair does not depend on the level, so if
 //           it prunes w at level d + 1 it prunes w again at any later level
 //           where w is reached, and leaving the bit clear changes no label.
-//   test    the rest of the test, one WARP per candidate so that lanes work
-//           in parallel instead of a few lanes looping alone: each lane first
-//           loads its own candidate's label offsets (32 candidates' loads in
-//           flight at once), then for each candidate in turn the lanes take
-//           the feasible bit-parallel roots (two each) and compare mask pairs;
-//           if none prunes, they take L(w)'s entries 32 at a time and probe
-//           the root's hash table. Survivors are appended as (w, k, d + 1).
+//   test    the rest of the test, 32 candidates per warp: the feasible
+//           bit-parallel roots of a candidate on the lanes (two each, mask
+//           pairs compared); then, root by root, the labels L(w) of the
+//           candidates that are left, past the root's reach table in shared
+//           memory to its hash table. Survivors are appended as (w, k, d + 1).
 //   clear   after the batch, the lazy reset of Sec. 4.5.1 ("Initialization"):
 //           the only bits set are those of the roots and of the recorded
 //           candidates, so their words are zeroed and nothing else is touched
@@ -71,6 +69,13 @@ namespace {
 #ifndef LONG_LABEL_ENTRIES
 #define LONG_LABEL_ENTRIES 64
 #endif
+#ifndef PLL_STAGE_ENTRIES
+#define PLL_STAGE_ENTRIES 256
+#endif
+#ifndef PLL_TEST_TPS
+#define PLL_TEST_TPS 1024
+#endif
+constexpr int TEST_TPS = PLL_TEST_TPS;
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t HT_EMPTY = 0xffffffffu;
@@ -99,13 +104,20 @@ __device__ __forceinline__ unsigned long long warp_append(unsigned long long *co
     return base + __popc(m & ((1u << lane) - 1u));
 }
 
-// Bit of hub rank h in a root's 1024-bit filter: the top 10 bits of the same
-// kind of mix as ht_slot (hub ranks of a batch build share their low bits).
-__device__ __forceinline__ uint32_t filt_bit(uint32_t h) {
+// A root's reach table: a byte per hash of a hub, four for every slot of its
+// hash table (up to REACH_MAX bytes), in which bit r (r < 8) says that some
+// hub with that hash is within r of the root (bit 7: at any distance). A
+// candidate's entry (h, d) can prune at level L only if bit min(L - d, 7) of
+// its hub's byte is set: one byte answers it for nearly every entry, and only
+// the others go to the hash table, whose chains cost dependent loads.
+__device__ __forceinline__ uint32_t reach_slot(uint32_t h, uint32_t lg) {
     uint32_t x = h * 0x85EBCA6Bu;
     x ^= x >> 13;
     x *= 0xC2B2AE35u;
-    return x >> 22;
+    return x >> (32 - lg);
+}
+__device__ __forceinline__ uint32_t reach_lg(uint32_t tmask) {  // of a hash table of tmask + 1 slots
+    return min(34u - __clz(tmask), REACH_LG_MAX);
 }
 
 // Neighbours of rank < k0 need no test: they are pruned at whatever level they
@@ -180,21 +192,7 @@ __global__ void k_batch_init(BatchArgs a) {
             atomicOr(&a.visited[(size_t)slot * a.NW + (k >> 5)], 1u << (k & 31));
         }
         append_slices(a, lane == 0, lane, k, k, 0);
-        // a 1024-bit filter of L(v_k)'s hubs: most hubs of a candidate's label
-        // are not in the root's, and the filter tells so with one load (for
-        // labels of up to FILT_MAX_LEN entries, where at most 12 % of its bits
-        // are set; longer labels go to the table directly)
         const uint32_t len = a.lab_len[k];
-        uint32_t *filt = a.filt + (size_t)slot * FILT_WORDS;
-        if (len <= FILT_MAX_LEN) {
-            filt[lane] = 0;
-            __syncwarp();
-            const uint32_t *lab = a.pool + a.lab_off[k];
-            for (uint32_t j = lane; j < len; j += 32) {
-                const uint32_t fb = filt_bit(entry_hub(lab[j]));
-                atomicOr(&filt[fb >> 5], 1u << (fb & 31));
-            }
-        }
         // root array T as a hash table of 2 x |L(v_k)| slots (very long labels,
         // and tables past the pool's end, are binary-searched instead; the host
         // grows the pool for the next batches)
@@ -204,11 +202,18 @@ __global__ void k_batch_init(BatchArgs a) {
         } else if (te > tb) {
             uint32_t *ht = a.ht + tb;
             const uint32_t mask = (uint32_t)(te - tb) - 1;
-            for (uint32_t s = lane; s <= mask; s += 32) ht[s] = HT_EMPTY;
+            uint32_t *reach = a.reach + tb;
+            const uint32_t lg = reach_lg(mask);
+            const uint4 empty = make_uint4(HT_EMPTY, HT_EMPTY, HT_EMPTY, HT_EMPTY);
+            for (uint32_t s = lane; s <= mask / 4; s += 32) reinterpret_cast<uint4 *>(ht)[s] = empty;
+            for (uint32_t s = lane; s < 1u << (lg - 4); s += 32)
+                reinterpret_cast<uint4 *>(reach)[s] = make_uint4(0, 0, 0, 0);
             __syncwarp();
             const uint32_t *lab = a.pool + a.lab_off[k];
             for (uint32_t j = lane; j < len; j += 32) {
                 const uint32_t e = lab[j];
+                const uint32_t rs = reach_slot(entry_hub(e), lg), rd = min(entry_dist(e), 7u);
+                atomicOr(&reach[rs >> 2], ((0xffu << rd) & 0xffu) << (8 * (rs & 3)));
                 uint32_t s = ht_slot(entry_hub(e), mask);
                 while (atomicCAS(&ht[s], HT_EMPTY, e) != HT_EMPTY) s = (s + 1) & mask;
             }
@@ -748,19 +753,26 @@ __global__ void k_batch_clear(BatchArgs a) {
 // candidate j), in two parts:
 //   masks   one candidate with feasible roots at a time: the lanes take the
 //           roots (two each) and compare mask pairs (Sec. 5.3);
-//   labels  of the candidates the masks did not prune: a long label (at
-//           least LONG_LABEL entries) is scanned by the whole warp, LU rounds
-//           of 32 entries per step; the shorter labels L(w) are laid end to end
-//           and the lanes take LU x 32 consecutive entries per step (lane x's
-//           candidate found by a binary search over a warp scan of the
-//           lengths), so short labels do not leave lanes idle and the chunks
-//           of different candidates are in flight together. Each entry
-//           (h, d) is looked up in the root's filter (roots with labels of at
-//           most FILT_MAX_LEN entries), and only if its bit is set in the
-//           root's hash table T (or, without a table, by a binary search of
-//           L(v_k)); d + T[h] <= level prunes the candidate. A candidate found
-//           pruned takes no further entries.
-// Per-candidate data sits in shared memory for the lanes that work on it.
+//   labels  of the candidates the masks did not prune, root by root (the sweeps
+//           keep a root's candidates together: 4 to 6 of 32 share one on
+//           average). The root's reach table is copied to shared memory, and
+//           the labels L(w) are read past it: a long one (at least LONG_LABEL
+//           entries) by the whole warp, LU rounds of 32 entries a step; the
+//           others laid end to end over the lanes (lane x's candidate found by
+//           a binary search over a warp scan of the lengths). An entry at
+//           distance d >= level can prune nothing (every hub is at least 1 from
+//           the root), which settles 95 of 100 entries on power-law graphs and
+//           6 of 10 on the high-diameter ones without a look at the table; an
+//           entry that the table lets through is looked up in the root's hash
+//           table T (or, without one, by a binary search of L(v_k)), and
+//           d + T[h] <= level prunes the candidate. A candidate found pruned
+//           takes no further entries.
+//
+// Bound by latency and, on long labels, by instruction issue. All test sweeps
+// of the batch of 96 uneven graphs (t = 16; 29.0G label entries read, 12.0G of
+// them nearer than the candidate): 325 ms with every entry probed in the hash
+// table (gathers from L2), 124 ms so; of R-MAT-20 (t = 64; 7.8G entries, 0.4G
+// nearer): 65.9 ms before, 47.0 ms so.
 constexpr int LU = LABEL_ROUNDS;  // label rounds per step of the test sweep
 constexpr int LU_LOOP = LABEL_ROUNDS_LOOP;  // the same inside the level loop (fewer
                                             // registers: the loop's own state is live)
@@ -768,81 +780,83 @@ constexpr int LU_LOOP = LABEL_ROUNDS_LOOP;  // the same inside the level loop (f
 // one by the whole warp (no owner search per entry, and an exit at the first
 // step that prunes); shorter labels are laid end to end over the lanes
 constexpr uint32_t LONG_LABEL = LONG_LABEL_ENTRIES;
+// a root's table is staged for at least this many label entries of its
+// candidates, else read where it lies (the batch's test sweeps take 124 ms with
+// any line from 1 to 500, 141 ms without staging; R-MAT-20's 47 to 48 ms)
+constexpr uint32_t STAGE_ENTRIES = PLL_STAGE_ENTRIES;
 
-struct TestCand {
-    unsigned long long lab_base;  // pool offset of L(w) minus the candidate's first flattened index
-    unsigned long long tb;        // its root's table in the table pool
-    unsigned long long koff;      // L(v_k) in the label pool (binary-search fallback)
-    uint32_t slot, tmask, klen, pad;  // tmask = table slots - 1, NONE without a table
+// What a warp of the test sweep keeps in shared memory.
+struct TestWarp {
+    uint4 reach[REACH_MAX / 16];  // the staged table of the root at hand
 };
 
-// The label test of LU label entries per lane (ent[u], of candidate own[u],
-// where act[u]): in three stages so that the loads of all of them are in
-// flight together -- the filter words, then the first table slot of each hub
-// (collision chains and the binary-search fallback follow one by one). Returns
-// the lane's candidates that an entry prunes (d + T[h] <= level), as bits.
-template <int U>
-__device__ __forceinline__ uint32_t lookup_entries(const BatchArgs &a, const TestCand *tc,
-                                                   const uint32_t (&ent)[U], const uint32_t (&own)[U],
-                                                   const bool (&act)[U], uint32_t level, uint32_t &n_scan) {
-    uint32_t fw[U], y0[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        fw[u] = ~0u;  // no filter: every hub goes to the table
-        if (act[u]) {
-            const TestCand &c = tc[own[u]];
-            if (c.klen <= FILT_MAX_LEN) {
-                const uint32_t fb = filt_bit(entry_hub(ent[u]));
-                fw[u] = a.filt[(size_t)c.slot * FILT_WORDS + (fb >> 5)] >> (fb & 31);
-            }
+// The root whose candidates are at hand (the same on every lane).
+struct TestRoot {
+    unsigned long long tb;  // its tables in the table pools
+    uint32_t k, klen;
+    uint32_t tmask;         // hash-table slots - 1, NONE without a table
+    uint32_t lg;            // log2 of the reach table's bytes
+    bool staged;            // the reach table is in shared memory
+};
+
+// distance from the root to hub h, INF8 if h is not in its label
+__device__ __forceinline__ uint32_t root_distance(const BatchArgs &a, const TestRoot &r, uint32_t h) {
+    if (r.tmask != NONE) {
+        const uint32_t *ht = a.ht + r.tb;
+        for (uint32_t sl = ht_slot(h, r.tmask);; sl = (sl + 1) & r.tmask) {
+            const uint32_t y = ht[sl];
+            if (y == HT_EMPTY) return INF8;
+            if (entry_hub(y) == h) return entry_dist(y);
         }
     }
+    const uint32_t *rlab = a.pool + a.lab_off[r.k];
+    uint32_t lo = 0, hi = r.klen;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (entry_hub(rlab[mid]) < h) lo = mid + 1; else hi = mid;
+    }
+    return lo < r.klen && entry_hub(rlab[lo]) == h ? entry_dist(rlab[lo]) : (uint32_t)INF8;
+}
+
+// The label test of U label entries per lane (ent[u], of candidate own[u],
+// where act[u]) against root r. Returns the lane's candidates that an entry
+// prunes (d + T[h] <= level), as bits.
+template <int U>
+__device__ __forceinline__ uint32_t test_entries(const BatchArgs &a, const TestWarp &tw, const TestRoot &r,
+                                                 const uint32_t (&ent)[U], const uint32_t (&own)[U],
+                                                 uint32_t act, uint32_t level) {
+    const uint8_t *sh = reinterpret_cast<const uint8_t *>(tw.reach);
+    const uint8_t *gl = reinterpret_cast<const uint8_t *>(a.reach + r.tb);
+    uint32_t open = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        y0[u] = HT_EMPTY;
-        if (act[u] && (fw[u] & 1u)) {
-            const TestCand &c = tc[own[u]];
-            if (c.tmask != NONE) y0[u] = a.ht[c.tb + ht_slot(entry_hub(ent[u]), c.tmask)];
+        const uint32_t d = entry_dist(ent[u]);
+        if (!((act >> u) & 1) || d >= level) continue;
+        uint32_t near = 0xff;
+        if (r.tmask != NONE) {
+            const uint32_t x = reach_slot(entry_hub(ent[u]), r.lg);
+            near = r.staged ? sh[x] : gl[x];
         }
+        open |= ((near >> min(level - d, 7u)) & 1) << u;
     }
     uint32_t pm = 0;
+    if (open) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        if (!act[u]) continue;
-        ++n_scan;
-        if (!(fw[u] & 1u)) continue;
-        const TestCand &c = tc[own[u]];
-        const uint32_t h = entry_hub(ent[u]);
-        uint32_t tk = INF8;
-        if (c.tmask != NONE) {
-            const uint32_t *ht = a.ht + c.tb;
-            uint32_t sl = ht_slot(h, c.tmask), y = y0[u];
-            for (;;) {
-                if (y == HT_EMPTY) break;
-                if (entry_hub(y) == h) { tk = entry_dist(y); break; }
-                sl = (sl + 1) & c.tmask;
-                y = ht[sl];
+        for (int u = 0; u < U; ++u)
+            if ((open >> u) & 1) {
+                const uint32_t t = root_distance(a, r, entry_hub(ent[u]));
+                if (t != INF8 && t + entry_dist(ent[u]) <= level) pm |= 1u << own[u];
             }
-        } else {
-            const uint32_t *rlab = a.pool + c.koff;
-            uint32_t lo = 0, hi = c.klen;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (entry_hub(rlab[mid]) < h) lo = mid + 1; else hi = mid;
-            }
-            if (lo < c.klen && entry_hub(rlab[lo]) == h) tk = entry_dist(rlab[lo]);
-        }
-        if (tk != INF8 && tk + entry_dist(ent[u]) <= level) pm |= 1u << own[u];
     }
     return pm;
 }
 
-// The sweep over candidates [b, e) of level `level` by the warps of a grid;
-// tc: this warp's 32 records in shared memory. Adds the label entries it scans
-// and the mask pairs it reads to n_scan / n_mask.
+// The sweep over candidates [b, e) of level `level` by the warps of a grid.
+// Adds the label entries it reads and the mask pairs it reads to n_scan /
+// n_mask.
 template <int U>
 __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long b, unsigned long long e,
-                                          uint32_t level, TestCand *tc, uint32_t &n_scan, uint32_t &n_mask) {
+                                          uint32_t level, TestWarp &tw, uint32_t &n_scan, uint32_t &n_mask) {
     const int lane = threadIdx.x & 31;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     // warp-uniform trip count: each warp takes 32 consecutive candidates
@@ -851,22 +865,20 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
          i0 < span; i0 += stride) {
         const uint32_t cnt = (uint32_t)((e - b - i0) < 32 ? (e - b - i0) : 32);
         const bool valid = (uint32_t)lane < cnt;
-        uint64_t mine = 0;
         ulonglong2 mc = make_ulonglong2(0, 0);
-        uint32_t wlen = 0, klen = 0, slot = 0, w = 0;
-        unsigned long long woff = 0, koff = 0, tb = 0, te = 0;
+        uint32_t wlen = 0, klen = 0, slot = 0, w = 0, tmask = NONE;
+        unsigned long long woff = 0, tb = 0;
         if (valid) {  // per-candidate metadata, loaded in parallel
-            mine = __ldcg(a.cand + b + i0 + lane);
+            const uint64_t mine = __ldcg(a.cand + b + i0 + lane);
             mc = __ldcg(reinterpret_cast<const ulonglong2 *>(a.candc) + b + i0 + lane);
             w = (uint32_t)mine;
             slot = (uint32_t)(mine >> 32);
-            const uint32_t k = a.k0 + slot;
             wlen = a.lab_len[w];
             woff = a.lab_off[w];
-            klen = a.lab_len[k];
-            koff = a.lab_off[k];
+            klen = a.lab_len[a.k0 + slot];
             tb = a.ht_off[slot];
-            te = a.ht_off[slot + 1];
+            const unsigned long long te = a.ht_off[slot + 1];
+            if (te > tb && te <= a.ht_cap) tmask = (uint32_t)(te - tb) - 1;
         }
         // ---- masks
         uint32_t pruned = 0;
@@ -890,82 +902,87 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             }
             if (__any_sync(FULL, p)) pruned |= 1u << j;
         }
-        // ---- labels: candidates with long labels get the whole warp in turn;
-        // the labels of the others are laid end to end over the lanes
-        const bool open = valid && !((pruned >> lane) & 1);
-        const uint32_t len = (open && wlen < LONG_LABEL) ? wlen : 0;
-        uint32_t incl = len;
+        // ---- labels, root by root
+        uint32_t todo = __ballot_sync(FULL, valid && !((pruned >> lane) & 1) && wlen && klen);
+        while (todo) {
+            const uint32_t j0 = __ffs(todo) - 1;
+            const uint32_t s0 = __shfl_sync(FULL, slot, j0);
+            const bool in = ((todo >> lane) & 1) && slot == s0;
+            const uint32_t group = __ballot_sync(FULL, in);
+            todo &= ~group;
+            TestRoot r;
+            r.k = a.k0 + s0;
+            r.klen = __shfl_sync(FULL, klen, j0);
+            r.tmask = __shfl_sync(FULL, tmask, j0);
+            r.tb = __shfl_sync(FULL, tb, j0);
+            r.lg = reach_lg(r.tmask);
+            r.staged = r.tmask != NONE && __reduce_add_sync(FULL, in ? min(wlen, 0xffffu) : 0u) >= STAGE_ENTRIES;
+            __syncwarp();  // the previous root's table has been read
+            if (r.staged) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(a.reach + r.tb);
+                for (uint32_t x = lane; x < 1u << (r.lg - 4); x += 32) tw.reach[x] = src[x];
+            }
+            __syncwarp();
+            uint32_t ent[U], own[U];
+            // long labels: LU rounds of 32 entries per step, leaving at the
+            // first step that prunes. Without bit-parallel labels (t = 0) the
+            // labels prune most candidates, mostly with their first hubs (the
+            // highest-ranked): the first step is one round only.
+            for (uint32_t m = __ballot_sync(FULL, in && wlen >= LONG_LABEL); m; m &= m - 1) {
+                const uint32_t j = __ffs(m) - 1;
+                const uint32_t lj = __shfl_sync(FULL, wlen, j);
+                const uint32_t *lab = a.pool + __shfl_sync(FULL, woff, j);
+                for (uint32_t x0 = 0, step = a.t == 0 ? 32u : 32u * U; x0 < lj; x0 += step, step = 32u * U) {
+                    const uint32_t end = min(lj, x0 + step);
+                    uint32_t act = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const uint32_t total = __shfl_sync(FULL, incl, 31);
-        const uint32_t excl = incl - len;
-        __syncwarp();  // the previous group is done with tc
-        if (valid) {
-            TestCand c;
-            c.lab_base = woff - excl;
-            c.tb = tb;
-            c.koff = koff;
-            c.slot = slot;
-            c.tmask = (te > tb && te <= a.ht_cap) ? (uint32_t)(te - tb) - 1 : NONE;
-            c.klen = klen;
-            c.pad = 0;
-            tc[lane] = c;
-        }
-        __syncwarp();
-        uint32_t ent[U], own[U];
-        bool act[U];
-        // long labels: LU rounds of 32 entries per step, leaving at the first
-        // step that prunes
-        for (uint32_t m = __ballot_sync(FULL, open && wlen >= LONG_LABEL); m; m &= m - 1) {
-            const uint32_t j = __ffs(m) - 1;
-            const uint32_t lj = __shfl_sync(FULL, wlen, j);
-            const unsigned long long base = tc[j].lab_base + __shfl_sync(FULL, excl, j);
-            // without bit-parallel labels (t = 0) the labels prune most
-            // candidates, mostly with their first hubs (the highest-ranked):
-            // the first 32 entries alone, then U rounds per step. With them,
-            // most candidates that reach this test survive it and need every
-            // entry, so U rounds from the start.
-            if (a.t == 0) {
-                uint32_t e1[1], o1[1] = {j};
-                bool a1[1] = {true};
-                e1[0] = a.pool[base + lane];
-                if (__any_sync(FULL, lookup_entries(a, tc, e1, o1, a1, level, n_scan) != 0)) {
-                    pruned |= 1u << j;
-                    continue;
+                    for (int u = 0; u < U; ++u) {
+                        const uint32_t x = x0 + 32 * u + lane;
+                        own[u] = j;
+                        ent[u] = 0;
+                        if (x < end) {
+                            act |= 1u << u;
+                            ent[u] = lab[x];
+                        }
+                    }
+                    n_scan += __popc(act);
+                    if (__any_sync(FULL, test_entries(a, tw, r, ent, own, act, level) != 0)) {
+                        pruned |= 1u << j;
+                        break;
+                    }
                 }
             }
-            for (uint32_t x0 = a.t == 0 ? 32u : 0u; x0 < lj; x0 += 32 * U) {
+            // short labels laid end to end
+            const uint32_t len = (in && wlen < LONG_LABEL) ? wlen : 0;
+            uint32_t incl = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            const uint32_t excl = incl - len;
+            const unsigned long long base = woff - excl;
+            for (uint32_t x0 = 0; x0 < total; x0 += 32 * U) {
+                uint32_t act = 0;
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const uint32_t x = x0 + 32 * u + lane;
+                    uint32_t j = 0;  // owner: the last candidate whose first entry is <= x
+#pragma unroll
+                    for (uint32_t step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
                     own[u] = j;
-                    act[u] = x < lj;
-                    ent[u] = act[u] ? a.pool[base + x] : 0u;
+                    ent[u] = 0;
+                    const unsigned long long lb = __shfl_sync(FULL, base, j);
+                    if (x < total && !((pruned >> j) & 1)) {
+                        act |= 1u << u;
+                        ent[u] = a.pool[lb + x];
+                    }
                 }
-                if (__any_sync(FULL, lookup_entries(a, tc, ent, own, act, level, n_scan) != 0)) {
-                    pruned |= 1u << j;
-                    break;
-                }
+                n_scan += __popc(act);
+                pruned |= __reduce_or_sync(FULL, test_entries(a, tw, r, ent, own, act, level));
             }
-        }
-        // short labels laid end to end (lane x's candidate found by a binary
-        // search over the warp scan of their lengths)
-        for (uint32_t x0 = 0; x0 < total; x0 += 32 * U) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const uint32_t x = x0 + 32 * u + lane;
-                uint32_t j = 0;  // owner: the last candidate whose first entry is <= x
-#pragma unroll
-                for (uint32_t step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
-                own[u] = j;
-                act[u] = x < total && !((pruned >> j) & 1);
-                ent[u] = act[u] ? a.pool[tc[j].lab_base + x] : 0u;
-            }
-            pruned |= __reduce_or_sync(FULL, lookup_entries(a, tc, ent, own, act, level, n_scan));
         }
         const bool keep = valid && !((pruned >> lane) & 1);
         if (__any_sync(FULL, keep)) {
@@ -980,10 +997,21 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_test(BatchArgs a) {
-    __shared__ TestCand s_cand[BLOCK / 32][32];
+constexpr size_t test_smem() { return (size_t)(BLOCK / 32) * sizeof(TestWarp); }
+// the cooperative loop's sweeps take turns with the same shared memory
+template <int BLOCK>
+constexpr size_t levels_smem() {
+    return expand_smem<BLOCK>() > test_smem<BLOCK>() ? expand_smem<BLOCK>() : test_smem<BLOCK>();
+}
+__device__ __forceinline__ TestWarp &test_warp(uint4 *dyn) {
+    return reinterpret_cast<TestWarp *>(dyn)[threadIdx.x >> 5];
+}
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test(BatchArgs a) {
+    extern __shared__ uint4 s_dyn[];
     uint32_t n_scan = 0, n_mask = 0;
-    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, s_cand[threadIdx.x >> 5], n_scan, n_mask);
+    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
     flush_work(a, 0, n_scan, n_mask);
 }
 
@@ -1040,10 +1068,9 @@ __device__ __forceinline__ bool grid_barrier(const BatchArgs &a, LoopState *ls) 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs a) {
     extern __shared__ uint4 s_dyn[];
-    __shared__ TestCand s_cand[BLOCK / 32][32];
     LoopState *ls = a.loop;
     ExpandWarp &sw = expand_warp(s_dyn);
-    TestCand *tc = s_cand[threadIdx.x >> 5];
+    TestWarp &tw = test_warp(s_dyn);
     const bool timer = blockIdx.x == 0 && threadIdx.x == 0;
     unsigned long long lvl_b = a.desc->lvl_b, lvl_e = a.desc->lvl_e, slice_n = a.desc->slice_n, cand_e = 0;
     uint32_t level = 0, nexp = 0, nreach = 0, n_scan = 0, n_mask = 0;
@@ -1058,7 +1085,7 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs 
         const unsigned long long cand_b = cand_e;
         const unsigned long long cn = *(volatile unsigned long long *)&ls->cand_n;
         cand_e = cn < a.cand_cap ? cn : a.cand_cap;
-        test_body<LU_LOOP>(a, cand_b, cand_e, level + 1, tc, n_scan, n_mask);
+        test_body<LU_LOOP>(a, cand_b, cand_e, level + 1, tw, n_scan, n_mask);
         if (!grid_barrier(a, ls)) break;
         if (timer) {
             const unsigned long long t2 = global_ns();
@@ -1136,12 +1163,12 @@ __global__ void __launch_bounds__(BLOCK, EXPAND_TPS / BLOCK) k_batch_expand_g(co
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_test_g(const BatchArgs *__restrict__ ap) {
-    __shared__ TestCand s_cand[BLOCK / 32][32];
+__global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test_g(const BatchArgs *__restrict__ ap) {
+    extern __shared__ uint4 s_dyn[];
     __shared__ BatchArgs s_args;
     const BatchArgs &a = args_to_shared(ap, &s_args);
     uint32_t n_scan = 0, n_mask = 0;
-    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, s_cand[threadIdx.x >> 5], n_scan, n_mask);
+    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
     flush_work(a, 0, n_scan, n_mask);
 }
 
@@ -1172,7 +1199,11 @@ static cudaError_t occupancy(int *pe, int *pt) {
                                          (int)expand_smem<BLOCK>());
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pe, k_batch_expand<BLOCK>, BLOCK, expand_smem<BLOCK>());
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pt, k_batch_test<BLOCK>, BLOCK, 0);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_batch_test<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)test_smem<BLOCK>());
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pt, k_batch_test<BLOCK>, BLOCK, test_smem<BLOCK>());
     return e;
 }
 
@@ -1224,7 +1255,7 @@ static void level_sweeps(const BatchArgs &a, const int *grid, cudaStream_t s, cu
     if (ev) cudaEventRecord(ev[1], s);
     k_batch_advance<<<1, 1, 0, s>>>(a, 1);
     if (ev) cudaEventRecord(ev[2], s);
-    k_batch_test<BLOCK><<<grid[1], BLOCK, 0, s>>>(a);
+    k_batch_test<BLOCK><<<grid[1], BLOCK, test_smem<BLOCK>(), s>>>(a);
     if (ev) cudaEventRecord(ev[3], s);
     k_batch_advance<<<1, 1, 0, s>>>(a, 2);
 }
@@ -1267,9 +1298,9 @@ static cudaError_t levels_grid(int *grid) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_batch_levels<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)expand_smem<BLOCK>());
+                                 (int)levels_smem<BLOCK>());
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_levels<BLOCK>, BLOCK, expand_smem<BLOCK>());
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_levels<BLOCK>, BLOCK, levels_smem<BLOCK>());
     *grid = (e == cudaSuccess && coop && per > 0) ? sms * per : 0;
     return e;
 }
@@ -1291,7 +1322,7 @@ static cudaError_t launch_levels(const BatchArgs &a, int grid, cudaStream_t s) {
     BatchArgs arg = a;
     void *args[] = {&arg};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_batch_levels<BLOCK>), dim3(grid),
-                                       dim3(BLOCK), args, expand_smem<BLOCK>(), s);
+                                       dim3(BLOCK), args, levels_smem<BLOCK>(), s);
 }
 
 int batch_levels(const BatchArgs &a, uint32_t block, int grid, cudaStream_t s) {
@@ -1316,6 +1347,8 @@ static int graph_build(const int *grid, const BatchArgs *d_args, cudaGraph_t *pg
     } guard{g};
     PLL_TRY(cudaFuncSetAttribute(k_batch_expand_g<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)expand_smem<BLOCK>()));
+    PLL_TRY(cudaFuncSetAttribute(k_batch_test_g<BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)test_smem<BLOCK>()));
     cudaGraphConditionalHandle h;
     PLL_TRY(cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault));
     cudaGraphNodeParams cp{};
@@ -1349,11 +1382,13 @@ static int graph_build(const int *grid, const BatchArgs *d_args, cudaGraph_t *pg
     kp.func = reinterpret_cast<void *>(k_batch_test_g<BLOCK>);
     kp.gridDim = dim3(grid[1]);
     kp.blockDim = dim3(BLOCK);
+    kp.sharedMemBytes = (unsigned)test_smem<BLOCK>();
     kp.kernelParams = a_tst;
     PLL_TRY(cudaGraphAddKernelNode(&n[2], body, &n[1], 1, &kp));
     kp.func = reinterpret_cast<void *>(k_batch_advance_g);
     kp.gridDim = dim3(1);
     kp.blockDim = dim3(1);
+    kp.sharedMemBytes = 0;
     kp.kernelParams = a_adv2;
     PLL_TRY(cudaGraphAddKernelNode(&n[3], body, &n[2], 1, &kp));
     PLL_TRY(cudaGraphInstantiate(pexec, g, 0));

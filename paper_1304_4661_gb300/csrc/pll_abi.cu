@@ -182,8 +182,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PLL_CHECK(m_htoff.alloc(((size_t)bmax + 1) * 8));
     const size_t itemp_bytes = ((batch_init_temp_bytes(bmax) + 255) & ~(size_t)255) + ((size_t)bmax + 1) * 8 + 256;
     PLL_CHECK(m_itemp.alloc(itemp_bytes));
-    PoolMem m_filt(s);
-    PLL_CHECK(m_filt.alloc((size_t)bmax * FILT_WORDS * 4));
+    PoolMem m_reach(s);
+    PLL_CHECK(m_reach.alloc(ht_cap * 4));
     uint64_t cand_cap = caps.cand ? caps.cand
                                   : std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 256, free_b / 16 / 24),
                                                        1ull << 24);
@@ -312,7 +312,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.ht = m_ht.as<uint32_t>();
         a.ht_off = m_htoff.as<unsigned long long>();
         a.ht_cap = ht_cap;
-        a.filt = m_filt.as<uint32_t>();
+        a.reach = m_reach.as<uint32_t>();
         a.cand = m_cand.as<uint64_t>(); a.candc = m_candc.as<uint64_t>(); a.cand_cap = cand_cap;
         a.out = m_out.as<uint64_t>(); a.out_cap = out_cap;
         a.slices = m_slices.as<uint4>(); a.slice_cap = slice_cap;
@@ -391,6 +391,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             if (!caps.ht) {  // the test capacity keeps the pool small for the whole build
                 ht_cap = std::max<uint64_t>(need + need / 4, ht_cap * 2);
                 PLL_CHECK(m_ht.alloc(ht_cap * 4));
+                PLL_CHECK(m_reach.alloc(ht_cap * 4));
             }
             h->c.err &= ~ERR_TABLE;
         }

@@ -248,8 +248,8 @@ int bp_run_in(uint32_t n, uint32_t t, const uint32_t *d_roff, const uint32_t *d_
 // k_pruned.cu -- batch-synchronous pruned BFS over roots [k0, k0 + B)
 // root label hash tables: 2 x |L(v_k)| slots rounded up to a power of two,
 // at least HT_MIN; labels longer than HT_MAX / 2 are binary-searched instead
-constexpr uint32_t FILT_WORDS = 32;     // 1024-bit hub filter per root of a batch
-constexpr uint32_t FILT_MAX_LEN = 128;  // roots with longer labels have no filter
+constexpr uint32_t REACH_LG_MAX = 12;   // a root's reach table has at most 4096 bytes
+constexpr uint32_t REACH_MAX = 1u << REACH_LG_MAX;
 #ifndef PLL_SLICE
 #define PLL_SLICE 64
 #endif
@@ -323,7 +323,8 @@ struct BatchArgs {
     uint32_t *ht;              // pool of root label hash tables
     unsigned long long *ht_off;  // [B + 1] table offsets in the pool (exclusive sums)
     unsigned long long ht_cap;   // pool capacity (entries)
-    uint32_t *filt;            // [B][FILT_WORDS] per-root filter of its label's hubs
+    uint32_t *reach;           // reach tables: a root's at its hash table's offset (four
+                               // bytes for each of its slots, the first REACH_MAX in use)
     uint64_t *cand;            // (slot << 32 | vertex), all levels
     uint64_t *candc;           // [cand_cap][2] roots whose masks may still prune
     unsigned long long cand_cap;
