@@ -60,14 +60,8 @@
 namespace pll {
 namespace {
 
-#ifndef LABEL_ROUNDS
-#define LABEL_ROUNDS 4
-#endif
-#ifndef LABEL_ROUNDS_LOOP
-#define LABEL_ROUNDS_LOOP 2
-#endif
 #ifndef LONG_LABEL_ENTRIES
-#define LONG_LABEL_ENTRIES 64
+#define LONG_LABEL_ENTRIES 128
 #endif
 #ifndef PLL_STAGE_ENTRIES
 #define PLL_STAGE_ENTRIES 256
@@ -110,12 +104,7 @@ __device__ __forceinline__ unsigned long long warp_append(unsigned long long *co
 // candidate's entry (h, d) can prune at level L only if bit min(L - d, 7) of
 // its hub's byte is set: one byte answers it for nearly every entry, and only
 // the others go to the hash table, whose chains cost dependent loads.
-__device__ __forceinline__ uint32_t reach_slot(uint32_t h, uint32_t lg) {
-    uint32_t x = h * 0x85EBCA6Bu;
-    x ^= x >> 13;
-    x *= 0xC2B2AE35u;
-    return x >> (32 - lg);
-}
+__device__ __forceinline__ uint32_t reach_slot(uint32_t h, uint32_t lg) { return (h * 0x85EBCA6Bu) >> (32 - lg); }
 __device__ __forceinline__ uint32_t reach_lg(uint32_t tmask) {  // of a hash table of tmask + 1 slots
     return min(34u - __clz(tmask), REACH_LG_MAX);
 }
@@ -212,8 +201,8 @@ __global__ void k_batch_init(BatchArgs a) {
             const uint32_t *lab = a.pool + a.lab_off[k];
             for (uint32_t j = lane; j < len; j += 32) {
                 const uint32_t e = lab[j];
-                const uint32_t rs = reach_slot(entry_hub(e), lg), rd = min(entry_dist(e), 7u);
-                atomicOr(&reach[rs >> 2], ((0xffu << rd) & 0xffu) << (8 * (rs & 3)));
+                const uint32_t rs = reach_slot(entry_hub(e), lg), within = (0xffu << min(entry_dist(e), 7u)) & 0xffu;
+                atomicOr(&reach[rs >> 2], within << (8 * (rs & 3)));
                 uint32_t s = ht_slot(entry_hub(e), mask);
                 while (atomicCAS(&ht[s], HT_EMPTY, e) != HT_EMPTY) s = (s + 1) & mask;
             }
@@ -756,10 +745,10 @@ __global__ void k_batch_clear(BatchArgs a) {
 //   labels  of the candidates the masks did not prune, root by root (the sweeps
 //           keep a root's candidates together: 4 to 6 of 32 share one on
 //           average). The root's reach table is copied to shared memory, and
-//           the labels L(w) are read past it: a long one (at least LONG_LABEL
-//           entries) by the whole warp, LU rounds of 32 entries a step; the
-//           others laid end to end over the lanes (lane x's candidate found by
-//           a binary search over a warp scan of the lengths). An entry at
+//           the labels L(w) are read past it, four entries a lane: a long one
+//           (at least LONG_LABEL entries) by the whole warp; the others' quads
+//           of entries laid end to end over the lanes (a quad's candidate found
+//           by a binary search over a warp scan of the lengths). An entry at
 //           distance d >= level can prune nothing (every hub is at least 1 from
 //           the root), which settles 95 of 100 entries on power-law graphs and
 //           6 of 10 on the high-diameter ones without a look at the table; an
@@ -768,17 +757,19 @@ __global__ void k_batch_clear(BatchArgs a) {
 //           d + T[h] <= level prunes the candidate. A candidate found pruned
 //           takes no further entries.
 //
-// Bound by latency and, on long labels, by instruction issue. All test sweeps
-// of the batch of 96 uneven graphs (t = 16; 29.0G label entries read, 12.0G of
-// them nearer than the candidate): 325 ms with every entry probed in the hash
-// table (gathers from L2), 124 ms so; of R-MAT-20 (t = 64; 7.8G entries, 0.4G
-// nearer): 65.9 ms before, 47.0 ms so.
-constexpr int LU = LABEL_ROUNDS;  // label rounds per step of the test sweep
-constexpr int LU_LOOP = LABEL_ROUNDS_LOOP;  // the same inside the level loop (fewer
-                                            // registers: the loop's own state is live)
+// Bound by instruction issue (0.57 to 0.7 of the slots on the batch's heavy
+// launches) and the latency of the labels. All test sweeps of the batch of 96
+// uneven graphs (t = 16; 33G label entries, 12G of them nearer than the
+// candidate): 325 ms with every entry probed in the hash table (gathers from
+// L2), 124 ms with the reach tables and single entries on the lanes, 106.6 ms
+// with quads. R-MAT-20 (t = 64; 7.8G entries, 0.4G nearer): 65.9, 47.0, 43.3
+// ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
+// reach table (fewer false hits): 108 ms.
 // candidates whose labels have at least this many entries are scanned one by
 // one by the whole warp (no owner search per entry, and an exit at the first
-// step that prunes); shorter labels are laid end to end over the lanes
+// step that prunes); shorter labels are laid end to end over the lanes (the
+// line at 32: 2 ms more on R-MAT-20; at 64 to 256 no difference; none: 25 ms
+// more on the batch)
 constexpr uint32_t LONG_LABEL = LONG_LABEL_ENTRIES;
 // a root's table is staged for at least this many label entries of its
 // candidates, else read where it lies (the batch's test sweeps take 124 ms with
@@ -818,43 +809,57 @@ __device__ __forceinline__ uint32_t root_distance(const BatchArgs &a, const Test
     return lo < r.klen && entry_hub(rlab[lo]) == h ? entry_dist(rlab[lo]) : (uint32_t)INF8;
 }
 
-// The label test of U label entries per lane (ent[u], of candidate own[u],
-// where act[u]) against root r. Returns the lane's candidates that an entry
-// prunes (d + T[h] <= level), as bits.
-template <int U>
-__device__ __forceinline__ uint32_t test_entries(const BatchArgs &a, const TestWarp &tw, const TestRoot &r,
-                                                 const uint32_t (&ent)[U], const uint32_t (&own)[U],
-                                                 uint32_t act, uint32_t level) {
-    const uint8_t *sh = reinterpret_cast<const uint8_t *>(tw.reach);
-    const uint8_t *gl = reinterpret_cast<const uint8_t *>(a.reach + r.tb);
-    uint32_t open = 0;
+// Label entries arrive four to a lane (every label starts on 16 bytes and owns
+// whole quads; those past its end read as distance 255, which prunes nothing).
+// Does one of the quad's entries prune at `level` against root r? The reach
+// bytes first, read as signed: shifted right by level - d (of at most 31) they
+// give bit min(level - d, 7).
+struct Quad {
+    uint32_t e[4];
+};
+__device__ __forceinline__ Quad load_quad(const uint32_t *lab, uint32_t q, uint32_t len) {
+    const uint4 v = *reinterpret_cast<const uint4 *>(lab + 4 * q);
+    Quad r{{v.x, v.y, v.z, v.w}};
+    if (4 * q + 4 > len) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t d = entry_dist(ent[u]);
-        if (!((act >> u) & 1) || d >= level) continue;
-        uint32_t near = 0xff;
-        if (r.tmask != NONE) {
-            const uint32_t x = reach_slot(entry_hub(ent[u]), r.lg);
-            near = r.staged ? sh[x] : gl[x];
+        for (uint32_t u = 1; u < 4; ++u)
+            if (4 * q + u >= len) r.e[u] = INF8;
+    }
+    return r;
+}
+__device__ __forceinline__ bool quad_prunes(const BatchArgs &a, const TestWarp &tw, const TestRoot &r, const Quad &q,
+                                            uint32_t level) {
+    const int8_t *sh = reinterpret_cast<const int8_t *>(tw.reach);
+    const int8_t *gl = reinterpret_cast<const int8_t *>(a.reach + r.tb);
+    uint32_t open = 0;  // the entries that the table lets through
+    if (r.staged) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = (int)level - (int)entry_dist(q.e[u]);
+            const int near = sh[reach_slot(entry_hub(q.e[u]), r.lg)];
+            if (t > 0) open |= (uint32_t)(near >> min(t, 31) & 1) << u;
         }
-        open |= ((near >> min(level - d, 7u)) & 1) << u;
-    }
-    uint32_t pm = 0;
-    if (open) {
+    } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if ((open >> u) & 1) {
-                const uint32_t t = root_distance(a, r, entry_hub(ent[u]));
-                if (t != INF8 && t + entry_dist(ent[u]) <= level) pm |= 1u << own[u];
+        for (int u = 0; u < 4; ++u) {
+            const int t = (int)level - (int)entry_dist(q.e[u]);
+            if (t > 0) {
+                const int near = r.tmask != NONE ? gl[reach_slot(entry_hub(q.e[u]), r.lg)] : -1;
+                open |= (uint32_t)(near >> min(t, 31) & 1) << u;
             }
+        }
     }
-    return pm;
+    for (; open; open &= open - 1) {
+        const uint32_t lo = open & 1 ? q.e[0] : q.e[1], hi = open & 4 ? q.e[2] : q.e[3], e = open & 3 ? lo : hi;
+        const uint32_t t = root_distance(a, r, entry_hub(e));
+        if (t != INF8 && t + entry_dist(e) <= level) return true;
+    }
+    return false;
 }
 
 // The sweep over candidates [b, e) of level `level` by the warps of a grid.
 // Adds the label entries it reads and the mask pairs it reads to n_scan /
 // n_mask.
-template <int U>
 __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long b, unsigned long long e,
                                           uint32_t level, TestWarp &tw, uint32_t &n_scan, uint32_t &n_mask) {
     const int lane = threadIdx.x & 31;
@@ -923,65 +928,42 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
                 for (uint32_t x = lane; x < 1u << (r.lg - 4); x += 32) tw.reach[x] = src[x];
             }
             __syncwarp();
-            uint32_t ent[U], own[U];
-            // long labels: LU rounds of 32 entries per step, leaving at the
-            // first step that prunes. Without bit-parallel labels (t = 0) the
-            // labels prune most candidates, mostly with their first hubs (the
-            // highest-ranked): the first step is one round only.
+            // long labels, 32 quads a step, leaving at the first step that prunes
             for (uint32_t m = __ballot_sync(FULL, in && wlen >= LONG_LABEL); m; m &= m - 1) {
                 const uint32_t j = __ffs(m) - 1;
-                const uint32_t lj = __shfl_sync(FULL, wlen, j);
+                const uint32_t lj = __shfl_sync(FULL, wlen, j), quads = (lj + 3) / 4;
                 const uint32_t *lab = a.pool + __shfl_sync(FULL, woff, j);
-                for (uint32_t x0 = 0, step = a.t == 0 ? 32u : 32u * U; x0 < lj; x0 += step, step = 32u * U) {
-                    const uint32_t end = min(lj, x0 + step);
-                    uint32_t act = 0;
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const uint32_t x = x0 + 32 * u + lane;
-                        own[u] = j;
-                        ent[u] = 0;
-                        if (x < end) {
-                            act |= 1u << u;
-                            ent[u] = lab[x];
-                        }
-                    }
-                    n_scan += __popc(act);
-                    if (__any_sync(FULL, test_entries(a, tw, r, ent, own, act, level) != 0)) {
+                for (uint32_t q0 = 0; q0 < quads; q0 += 32) {
+                    const uint32_t q = q0 + lane;
+                    if (__any_sync(FULL, q < quads && quad_prunes(a, tw, r, load_quad(lab, q, lj), level))) {
                         pruned |= 1u << j;
                         break;
                     }
                 }
+                n_scan += lane == 0 ? lj : 0;
             }
-            // short labels laid end to end
-            const uint32_t len = (in && wlen < LONG_LABEL) ? wlen : 0;
-            uint32_t incl = len;
+            // short labels, their quads laid end to end
+            const uint32_t len = (in && wlen < LONG_LABEL) ? wlen : 0, nq = (len + 3) / 4;
+            n_scan += len;
+            uint32_t incl = nq;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t y = __shfl_up_sync(FULL, incl, o);
                 if (lane >= o) incl += y;
             }
             const uint32_t total = __shfl_sync(FULL, incl, 31);
-            const uint32_t excl = incl - len;
-            const unsigned long long base = woff - excl;
-            for (uint32_t x0 = 0; x0 < total; x0 += 32 * U) {
-                uint32_t act = 0;
+            const uint32_t excl = incl - nq;
+            for (uint32_t x0 = 0; x0 < total; x0 += 32) {
+                const uint32_t x = x0 + lane;
+                uint32_t j = 0;  // owner: the last candidate whose first quad is <= x
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t x = x0 + 32 * u + lane;
-                    uint32_t j = 0;  // owner: the last candidate whose first entry is <= x
-#pragma unroll
-                    for (uint32_t step = 16; step > 0; step >>= 1)
-                        if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
-                    own[u] = j;
-                    ent[u] = 0;
-                    const unsigned long long lb = __shfl_sync(FULL, base, j);
-                    if (x < total && !((pruned >> j) & 1)) {
-                        act |= 1u << u;
-                        ent[u] = a.pool[lb + x];
-                    }
-                }
-                n_scan += __popc(act);
-                pruned |= __reduce_or_sync(FULL, test_entries(a, tw, r, ent, own, act, level));
+                for (uint32_t step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
+                const uint32_t *lab = a.pool + __shfl_sync(FULL, woff, j);
+                const uint32_t lj = __shfl_sync(FULL, len, j), xj = __shfl_sync(FULL, excl, j);
+                bool p = false;
+                if (x < total) p = quad_prunes(a, tw, r, load_quad(lab, x - xj, lj), level);
+                pruned |= __reduce_or_sync(FULL, p ? 1u << j : 0u);
             }
         }
         const bool keep = valid && !((pruned >> lane) & 1);
@@ -1011,7 +993,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test(BatchArgs a) {
     extern __shared__ uint4 s_dyn[];
     uint32_t n_scan = 0, n_mask = 0;
-    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
+    test_body(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
     flush_work(a, 0, n_scan, n_mask);
 }
 
@@ -1085,7 +1067,7 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs 
         const unsigned long long cand_b = cand_e;
         const unsigned long long cn = *(volatile unsigned long long *)&ls->cand_n;
         cand_e = cn < a.cand_cap ? cn : a.cand_cap;
-        test_body<LU_LOOP>(a, cand_b, cand_e, level + 1, tw, n_scan, n_mask);
+        test_body(a, cand_b, cand_e, level + 1, tw, n_scan, n_mask);
         if (!grid_barrier(a, ls)) break;
         if (timer) {
             const unsigned long long t2 = global_ns();
@@ -1168,7 +1150,7 @@ __global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test_g(const 
     __shared__ BatchArgs s_args;
     const BatchArgs &a = args_to_shared(ap, &s_args);
     uint32_t n_scan = 0, n_mask = 0;
-    test_body<LU>(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
+    test_body(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
     flush_work(a, 0, n_scan, n_mask);
 }
 
