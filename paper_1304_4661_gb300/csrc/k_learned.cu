@@ -23,7 +23,9 @@
 #include <cub/cub.cuh>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <new>
 
 #include "pll_internal.cuh"
@@ -62,108 +64,244 @@ __global__ void k_deg_twohop(uint32_t n, const uint32_t *__restrict__ off,
     }
 }
 
-struct CoreCtl {
-    unsigned long long removed;  // vertices removed by the pass
-    unsigned long long alive;    // vertices left after it
-    uint32_t min_deg;            // least remaining degree among them
-    uint32_t pad;
-};
+// Core numbers as the limit of repeated h-indices (Lu et al., Nature
+// Communications 7, 2016): every vertex starts at its degree, and its value is
+// replaced by the largest h such that h neighbours have a value of at least h,
+// until nothing changes. Values only fall and never pass the core number, so
+// they may be updated in place in any order. Only vertices that lost support
+// are looked at again: a vertex that falls to h marks the neighbours above h
+// for the next step. R-MAT-17 settles in 20 to 32 steps, most of them over a
+// few hundred vertices, where peeling by degree takes 488 dependent passes,
+// each a scan of all vertices and a read-back (pll_features with t = 64: 24.0
+// ms so, 4.7 ms with the steps, 1.3 ms of it theirs). Bound by the longest
+// lists of a step and the gathers of their neighbours' values.
+constexpr uint32_t CORE_BIG = 512;     // lists this long get a block each
+constexpr int CORE_BIG_BLOCKS = 1024;
+constexpr int CORE_CHUNK = 4;          // vertices a warp looks at together; it takes the marked
+                                       // ones in turn (32 at a time: 0.75 ms more on R-MAT-17)
 
-__global__ void k_core_init(uint32_t n, const uint32_t *__restrict__ deg, uint32_t *cur,
-                            uint8_t *alive) {
+__global__ void k_core_init(uint32_t n, const uint32_t *__restrict__ deg, uint32_t *cur, uint8_t *dirty0,
+                            uint8_t *dirty1, uint32_t *big, uint32_t *nbig) {
     for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (uint64_t)gridDim.x * blockDim.x) {
         cur[v] = deg[v];
-        alive[v] = 1;
+        dirty0[v] = deg[v] != 0;
+        dirty1[v] = 0;
+        if (deg[v] >= CORE_BIG) big[atomicAdd(nbig, 1u)] = (uint32_t)v;
     }
 }
 
-// One peeling pass at level k: every remaining vertex with at most k
-// remaining neighbours is removed with core number k and lowers its
-// remaining neighbours' degrees. The vertices left at the start of level k
-// form the k-core, so everything removed during level k has core number k; a
-// degree lowered during the pass may hide a removal until the next pass, and
-// the level ends with a pass that removes nothing.
-__global__ void k_core_pass(uint32_t n, const uint32_t *__restrict__ off,
-                            const uint32_t *__restrict__ col, uint32_t k, uint32_t *cur,
-                            uint8_t *alive, uint32_t *core, CoreCtl *ctl) {
+struct CoreArgs {
+    uint32_t n;
+    const uint32_t *off, *col;
+    uint32_t *cur;
+    uint8_t *src, *dst;  // marked vertices of this step and of the next
+    const uint32_t *big, *nbig;
+    const uint32_t *prev;  // what the step before changed (null: run)
+    uint32_t *changed;
+};
+
+// A vertex of at least CORE_BIG neighbours, one block: if fewer than c of them
+// are at c or above, the largest h in [that count, c) by histograms of 256
+// bins over the range that is left.
+__device__ void core_big(const CoreArgs &a, uint32_t v) {
+    __shared__ uint32_t hist[256], sum[8], pick;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t b = a.off[v], e = a.off[v + 1], c = a.cur[v];
+    auto block_sum = [&](uint32_t x) {
+        x = __reduce_add_sync(FULL, x);
+        __syncthreads();
+        if (lane == 0) sum[warp] = x;
+        __syncthreads();
+        uint32_t t = 0;
+        for (int w = 0; w < 8; ++w) t += sum[w];
+        return t;
+    };
+    uint32_t x = 0;
+    for (uint32_t j = b + tid; j < e; j += 256) x += a.cur[a.col[j]] >= c;
+    uint32_t above = block_sum(x);  // values past the range at hand
+    if (above >= c) return;
+    uint32_t lo = above, hi = c - 1;
+    for (;;) {
+        const uint32_t width = (hi - lo) / 256 + 1;
+        hist[tid] = 0;
+        __syncthreads();
+        for (uint32_t j = b + tid; j < e; j += 256) {
+            const uint32_t y = a.cur[a.col[j]];
+            if (y >= lo && y <= hi) atomicAdd(&hist[(y - lo) / width], 1u);
+        }
+        if (tid == 0) pick = 0;
+        __syncthreads();
+        // values of bin tid and above: a scan over the bins from the top
+        uint32_t suffix = hist[255 - tid];
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, suffix, o);
+            if (lane >= o) suffix += y;
+        }
+        if (lane == 31) sum[warp] = suffix;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w) suffix += sum[w];
+        const uint32_t bin = 255 - tid;
+        // the highest bin whose first value h has h neighbours at it or above
+        const uint64_t h = (uint64_t)lo + (uint64_t)bin * width;
+        if (h <= hi && (uint64_t)above + suffix >= h) atomicMax(&pick, bin);
+        __syncthreads();
+        const uint32_t at = pick;
+        if (width == 1) {
+            lo += at;
+            break;
+        }
+        if (tid == 255 - (int)at) hist[0] = suffix - hist[at];  // values past the chosen bin
+        __syncthreads();
+        above += hist[0];
+        lo += at * width;
+        hi = min(hi, lo + width - 1);
+        __syncthreads();
+    }
+    if (tid == 0) {
+        a.cur[v] = lo;
+        *a.changed = 1;
+    }
+    for (uint32_t j = b + tid; j < e; j += 256) {
+        const uint32_t u = a.col[j];
+        if (a.cur[u] > lo) a.dst[u] = 1;
+    }
+}
+
+// the other marked vertices, a warp each, the neighbours' values in registers
+__device__ void core_small(const CoreArgs &a, uint32_t v, uint32_t b, uint32_t d) {
+    constexpr uint32_t Q = CORE_BIG / 32;
     const int lane = threadIdx.x & 31;
-    for (uint64_t base = (uint64_t)blockIdx.x * blockDim.x; base < n;
-         base += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t v = base + threadIdx.x;
-        bool rm = false, keep = false;
-        uint32_t d = 0xffffffffu;
-        if (v < n && alive[v]) {
-            d = *reinterpret_cast<volatile uint32_t *>(&cur[v]);  // neighbours lower it concurrently
-            if (d <= k) {
-                rm = true;
-                alive[v] = 0;
-                core[v] = k;
-                for (uint32_t j = off[v]; j < off[v + 1]; ++j) {
-                    const uint32_t u = col[j];
-                    if (alive[u]) atomicSub(&cur[u], 1u);
-                }
-            } else {
-                keep = true;
-            }
-        }
-        const unsigned mr = __ballot_sync(FULL, rm), mk = __ballot_sync(FULL, keep);
-        uint32_t dm = keep ? d : 0xffffffffu;
+    const uint32_t c = a.cur[v];
+    uint32_t id[Q], val[Q], x = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dm = min(dm, __shfl_xor_sync(FULL, dm, o));
-        if (lane == 0) {
-            if (mr) atomicAdd(&ctl->removed, (unsigned long long)__popc(mr));
-            if (mk) {
-                atomicAdd(&ctl->alive, (unsigned long long)__popc(mk));
-                atomicMin(&ctl->min_deg, dm);
-            }
+    for (uint32_t q = 0; q < Q; ++q) {
+        if (32 * q >= d) break;
+        const bool in = 32 * q + lane < d;
+        id[q] = in ? a.col[b + 32 * q + lane] : v;
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < Q; ++q) {
+        if (32 * q >= d) break;
+        val[q] = 32 * q + lane < d ? min(a.cur[id[q]], c) : 0;
+        x += val[q] >= c;
+    }
+    uint32_t lo = __reduce_add_sync(FULL, x), hi = c - 1;
+    if (lo >= c) return;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) / 2;
+        x = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < Q; ++q) {
+            if (32 * q >= d) break;
+            x += val[q] >= mid;
         }
+        if (__reduce_add_sync(FULL, x) >= mid) lo = mid; else hi = mid - 1;
+    }
+    if (lane == 0) {
+        a.cur[v] = lo;
+        *a.changed = 1;
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < Q; ++q) {
+        if (32 * q >= d) break;
+        if (val[q] > lo) a.dst[id[q]] = 1;
     }
 }
 
-// Raw features of vertex v (caller id), one warp per vertex; the bit-parallel
-// rows are in rank space (row inv[v]), lanes own roots lane and lane + 32.
-__global__ void k_features_raw(uint32_t n, uint32_t t, uint32_t tp, const uint32_t *__restrict__ inv,
-                               const uint32_t *__restrict__ deg,
-                               const unsigned long long *__restrict__ two_hop,
-                               const uint32_t *__restrict__ core, const uint8_t *__restrict__ bp_d,
-                               const uint64_t *__restrict__ bp_m, float *X) {
+// One step: the marked vertices' values. Blocks below CORE_BIG_BLOCKS take the
+// long lists, the others 32 vertices a warp. Nothing to do (and nothing
+// marked) if the step before changed nothing.
+__global__ void __launch_bounds__(256) k_core_step(CoreArgs a) {
+    if (a.prev && *a.prev == 0) return;
+    if (blockIdx.x < CORE_BIG_BLOCKS) {
+        for (uint32_t i = blockIdx.x; i < *a.nbig; i += CORE_BIG_BLOCKS) {
+            const uint32_t v = a.big[i];
+            const bool marked = a.src[v];  // the same on every thread
+            __syncthreads();
+            if (!marked) continue;
+            core_big(a, v);
+            __syncthreads();
+            if (threadIdx.x == 0) a.src[v] = 0;
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const uint64_t warp = ((uint64_t)(blockIdx.x - CORE_BIG_BLOCKS) * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t warps = ((uint64_t)(gridDim.x - CORE_BIG_BLOCKS) * blockDim.x) >> 5;
+    for (uint64_t v0 = warp * CORE_CHUNK; v0 < a.n; v0 += warps * CORE_CHUNK) {
+        const uint64_t v = v0 + lane;
+        uint32_t b = 0, d = CORE_BIG;
+        if (lane < CORE_CHUNK && v < a.n && a.src[v]) {
+            b = a.off[v];
+            d = a.off[v + 1] - b;
+        }
+        for (unsigned m = __ballot_sync(FULL, d < CORE_BIG); m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            core_small(a, (uint32_t)(v0 + j), __shfl_sync(FULL, b, j), __shfl_sync(FULL, d, j));
+        }
+        if (d < CORE_BIG) a.src[v] = 0;
+    }
+}
+
+// Raw features (by caller id), a warp for 32 vertices: the bit-parallel rows
+// (in rank space, row inv[v]) one vertex after the other over the lanes (roots
+// lane and lane + 32), then a lane per vertex for the logarithms and quotients,
+// which are in double precision: the FP64 units do two lanes a cycle, so the
+// warp must not spend them on one vertex at a time (R-MAT-17, t = 64: 1173 us
+// with a warp per vertex, 102 us so).
+__global__ void __launch_bounds__(256) k_features_raw(uint32_t n, uint32_t t, uint32_t tp,
+                                                      const uint32_t *__restrict__ inv,
+                                                      const uint32_t *__restrict__ deg,
+                                                      const unsigned long long *__restrict__ two_hop,
+                                                      const uint32_t *__restrict__ core,
+                                                      const uint8_t *__restrict__ bp_d,
+                                                      const uint64_t *__restrict__ bp_m, float *X) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t v = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-        uint32_t sum = 0, mn = D_CAP, near = 0, p1 = 0, p0 = 0;
+    for (uint64_t v0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; v0 < n; v0 += warps * 32) {
+        const uint64_t v = v0 + lane;
+        uint32_t sum = 0, mn = D_CAP, near = 0, p1 = 0, p0 = 0;  // of vertex v
         if (t) {
-            const size_t r = inv[v];
-            for (uint32_t i = lane; i < t; i += 32) {
-                const uint32_t dc = min((uint32_t)bp_d[r * tp + i], D_CAP);
-                sum += dc;
-                mn = min(mn, dc);
-                near += dc <= 2;
-                p1 += __popcll(bp_m[2 * (r * t + i)]);
-                p0 += __popcll(bp_m[2 * (r * t + i) + 1]);
-            }
+            const uint32_t mine = v < n ? inv[v] : 0;
+            const int cnt = n - v0 < 32 ? (int)(n - v0) : 32;
+#pragma unroll 4
+            for (int j = 0; j < cnt; ++j) {
+                const size_t r = __shfl_sync(FULL, mine, j);
+                uint32_t dn = 0, pp = 0, m = D_CAP;  // sum | near << 16, |S^-1| | |S^0| << 16
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sum += __shfl_xor_sync(FULL, sum, o);
-                mn = min(mn, __shfl_xor_sync(FULL, mn, o));
-                near += __shfl_xor_sync(FULL, near, o);
-                p1 += __shfl_xor_sync(FULL, p1, o);
-                p0 += __shfl_xor_sync(FULL, p0, o);
+                for (uint32_t h = 0; h < 2; ++h) {
+                    const uint32_t i = lane + 32 * h;
+                    if (i < t) {
+                        const uint32_t dc = min((uint32_t)bp_d[r * tp + i], D_CAP);
+                        const ulonglong2 s = reinterpret_cast<const ulonglong2 *>(bp_m)[r * t + i];
+                        m = min(m, dc);
+                        dn += dc + ((uint32_t)(dc <= 2) << 16);
+                        pp += __popcll(s.x) + ((uint32_t)__popcll(s.y) << 16);
+                    }
+                }
+                dn = __reduce_add_sync(FULL, dn);  // at most 64 * 32 and 64
+                pp = __reduce_add_sync(FULL, pp);  // at most 64 * 64 each
+                m = __reduce_min_sync(FULL, m);
+                if (lane == j) {
+                    sum = dn & 0xffff;
+                    near = dn >> 16;
+                    p1 = pp & 0xffff;
+                    p0 = pp >> 16;
+                    mn = m;
+                }
             }
         }
-        if (lane < NF) {
-            double f = 0;
-            switch (lane) {
-                case 0: f = log1p((double)deg[v]); break;
-                case 1: f = log1p((double)two_hop[v]); break;
-                case 2: f = log1p((double)core[v]); break;
-                case 3: f = t ? (double)sum / t : 0; break;
-                case 4: f = t ? (double)mn : 0; break;
-                case 5: f = t ? (double)near / t : 0; break;
-                case 6: f = t ? (double)p1 / (64.0 * t) : 0; break;
-                default: f = t ? (double)p0 / (64.0 * t) : 0; break;
-            }
-            X[v * NF + lane] = (float)f;
+        if (v < n) {
+            float *x = X + v * NF;
+            x[0] = (float)log1p((double)deg[v]);
+            x[1] = (float)log1p((double)two_hop[v]);
+            x[2] = (float)log1p((double)core[v]);
+            x[3] = t ? (float)((double)sum / t) : 0.f;
+            x[4] = t ? (float)mn : 0.f;
+            x[5] = t ? (float)((double)near / t) : 0.f;
+            x[6] = t ? (float)((double)p1 / (64.0 * t)) : 0.f;
+            x[7] = t ? (float)((double)p0 / (64.0 * t)) : 0.f;
         }
     }
 }
@@ -203,13 +341,18 @@ __global__ void k_mean(uint32_t n, double *acc) {
     if (threadIdx.x < NF) acc[threadIdx.x] = n ? acc[threadIdx.x] / n : 0;
 }
 
-__global__ void k_standardise(uint32_t n, const double *__restrict__ mean, const double *__restrict__ ssd,
+// ssd[j] becomes the population std of column j (a square root per column, not
+// per value, in double precision)
+__global__ void k_std(uint32_t n, double *ssd) {
+    if (threadIdx.x < NF) ssd[threadIdx.x] = sqrt(ssd[threadIdx.x] / n);
+}
+
+__global__ void k_standardise(uint32_t n, const double *__restrict__ mean, const double *__restrict__ sd,
                               float *X) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (uint64_t)n * NF;
          i += (uint64_t)gridDim.x * blockDim.x) {
         const int j = (int)(i % NF);
-        const double sd = sqrt(ssd[j] / n);
-        X[i] = sd > 0 ? (float)(((double)X[i] - mean[j]) / sd) : 0.f;
+        X[i] = sd[j] > 0 ? (float)(((double)X[i] - mean[j]) / sd[j]) : 0.f;
     }
 }
 
@@ -228,154 +371,298 @@ __global__ void k_log1p_counts(uint32_t n, const uint32_t *__restrict__ counts, 
 }
 
 // ------------------------------------------------------------------ network
+// the bf16 parameters as floats (W has room for NP + 3)
 __device__ __forceinline__ void load_weights(const __nv_bfloat16 *__restrict__ w16, float *W) {
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) W[i] = __bfloat162float(w16[i]);
+    const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(w16);
+    for (int i = threadIdx.x; i < NP / 2; i += blockDim.x) {
+        const float2 f = __bfloat1622float2(p[i]);
+        W[2 * i] = f.x;
+        W[2 * i + 1] = f.y;
+    }
+    if (threadIdx.x == 0) W[NP - 1] = __bfloat162float(w16[NP - 1]);
 }
 
-// y = w3 . relu(W2 relu(W1 x + b1) + b2) + b3, one thread per row.
-__global__ void __launch_bounds__(256) k_mlp_fwd(uint64_t n, const float *__restrict__ X,
-                                                 const __nv_bfloat16 *__restrict__ w16, float *y) {
-    __shared__ float W[NP];
-    load_weights(w16, W);
-    __syncthreads();
-    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    float x[NF], h1[HID];
+// row r of the features; vec: x is 16-byte aligned
+__device__ __forceinline__ void load_features(const float *__restrict__ X, uint64_t r, bool vec, float (&x)[NF]) {
+    if (vec) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(X) + 2 * r);
+        const float4 b = __ldg(reinterpret_cast<const float4 *>(X) + 2 * r + 1);
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    } else {
 #pragma unroll
-    for (int k = 0; k < NF; ++k) x[k] = X[r * NF + k];
-#pragma unroll
-    for (int i = 0; i < HID; ++i) {
-        float z = W[O_B1 + i];
-#pragma unroll
-        for (int k = 0; k < NF; ++k) z = fmaf(W[O_W1 + i * NF + k], x[k], z);
-        h1[i] = fmaxf(z, 0.f);
+        for (int k = 0; k < NF; ++k) x[k] = X[r * NF + k];
     }
-    float out = W[O_B3];
-    for (int j = 0; j < HID; ++j) {
-        float z = W[O_B2 + j];
-#pragma unroll
-        for (int i = 0; i < HID; ++i) z = fmaf(W[O_W2 + j * HID + i], h1[i], z);
-        out = fmaf(W[O_W3 + j], fmaxf(z, 0.f), out);
-    }
-    y[r] = out;
 }
 
-constexpr int GT = 128;      // rows per block of the gradient kernel
-constexpr int RS = HID + 1;  // padded row stride of the activation tiles
-constexpr int XS = NF + 1;
-constexpr size_t GRAD_SMEM =
-    sizeof(float) * ((NP + 3) / 4 * 4 + GT * XS + 4 * GT * RS + 2 * GT);
-
-// Gradient of the mean squared error over `batch` rows (row g of the batch
-// is sample idx[g], or g without idx). Each block takes GT rows: one thread
-// per row runs the forward pass and back-propagates to dZ2 and dZ1 in shared
-// memory; then the block's threads share the 4801 parameter gradients, each a
-// sum over the block's rows, and write them as one partial per block (summed
-// in a fixed order by k_mlp_reduce, so the result is deterministic).
-__global__ void __launch_bounds__(GT) k_mlp_grad(uint32_t batch, const float *__restrict__ X,
-                                                 const float *__restrict__ target,
-                                                 const uint32_t *__restrict__ idx,
-                                                 const __nv_bfloat16 *__restrict__ w16,
-                                                 float *partial, float *ploss) {
-    extern __shared__ float sm[];
-    float *W = sm;
-    float *Xs = W + (NP + 3) / 4 * 4;
-    float *H1 = Xs + GT * XS;
-    float *H2 = H1 + GT * RS;
-    float *DZ2 = H2 + GT * RS;
-    float *DZ1 = DZ2 + GT * RS;
-    float *DY = DZ1 + GT * RS;
-    float *LS = DY + GT;
+// y = w3 . relu(W2 relu(W1 x + b1) + b2) + b3, R rows a thread (row tid + FT a
+// of the block's tile). Every output keeps one chain of multiply-adds in index
+// order. Bound by the FP32 units: with one row a thread and one output unit
+// at a time each multiply-add waited for the one before it and every four
+// took a load of weights (2.1M rows: 980 us, 20 TFLOP/s); with four units at a
+// time over two rows eight chains run together and a load of four weights
+// serves eight multiply-adds: 385 us, 51 TFLOP/s (63 % of the FMA pipe and 66 %
+// of the shared-memory bandwidth). The same with two-row multiply-adds
+// (fma.rn.f32x2): 403 us. Three blocks an SM (168 registers).
+constexpr int FT = 128;
+template <int R>
+__global__ void __launch_bounds__(FT, 3) k_mlp_fwd(uint64_t n, const float *__restrict__ X, bool vec,
+                                                const __nv_bfloat16 *__restrict__ w16, float *y) {
+    __shared__ __align__(16) float W[NP + 3];
     load_weights(w16, W);
     __syncthreads();
-
-    const int s = threadIdx.x;
-    const uint32_t g = blockIdx.x * GT + s;
-    const bool valid = g < batch;
-    const uint64_t row = valid ? (idx ? idx[g] : g) : 0;
-    float x[NF], h1[HID];
+    for (uint64_t base = (uint64_t)blockIdx.x * FT * R; base < n; base += (uint64_t)gridDim.x * FT * R) {
+        float x[R][NF], h1[R][HID];
 #pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        x[k] = valid ? X[row * NF + k] : 0.f;
-        Xs[s * XS + k] = x[k];
-    }
-#pragma unroll
-    for (int i = 0; i < HID; ++i) {
-        float z = W[O_B1 + i];
-#pragma unroll
-        for (int k = 0; k < NF; ++k) z = fmaf(W[O_W1 + i * NF + k], x[k], z);
-        h1[i] = fmaxf(z, 0.f);
-        H1[s * RS + i] = h1[i];
-    }
-    float y = W[O_B3];
-    for (int j = 0; j < HID; ++j) {
-        float z = W[O_B2 + j];
-#pragma unroll
-        for (int i = 0; i < HID; ++i) z = fmaf(W[O_W2 + j * HID + i], h1[i], z);
-        const float h2 = fmaxf(z, 0.f);
-        H2[s * RS + j] = h2;
-        y = fmaf(W[O_W3 + j], h2, y);
-    }
-    const float res = valid ? y - target[row] : 0.f;
-    const float dy = 2.f * res / (float)batch;
-    DY[s] = dy;
-    LS[s] = res * res;
-    float dh[HID];
-#pragma unroll
-    for (int i = 0; i < HID; ++i) dh[i] = 0.f;
-    for (int j = 0; j < HID; ++j) {
-        const float dz = H2[s * RS + j] > 0.f ? dy * W[O_W3 + j] : 0.f;
-        DZ2[s * RS + j] = dz;
-#pragma unroll
-        for (int i = 0; i < HID; ++i) dh[i] = fmaf(W[O_W2 + j * HID + i], dz, dh[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < HID; ++i) DZ1[s * RS + i] = h1[i] > 0.f ? dh[i] : 0.f;
-    __syncthreads();
-
-    float *out = partial + (size_t)blockIdx.x * NP;
-    for (int o = threadIdx.x; o < NP; o += GT) {
-        float acc = 0.f;
-        if (o < O_B1) {
-            const int i = o / NF, k = o % NF;
-            for (int r = 0; r < GT; ++r) acc = fmaf(DZ1[r * RS + i], Xs[r * XS + k], acc);
-        } else if (o < O_W2) {
-            const int i = o - O_B1;
-            for (int r = 0; r < GT; ++r) acc += DZ1[r * RS + i];
-        } else if (o < O_B2) {
-            const int j = (o - O_W2) / HID, i = (o - O_W2) % HID;
-            for (int r = 0; r < GT; ++r) acc = fmaf(DZ2[r * RS + j], H1[r * RS + i], acc);
-        } else if (o < O_W3) {
-            const int j = o - O_B2;
-            for (int r = 0; r < GT; ++r) acc += DZ2[r * RS + j];
-        } else if (o < O_B3) {
-            const int j = o - O_W3;
-            for (int r = 0; r < GT; ++r) acc = fmaf(DY[r], H2[r * RS + j], acc);
-        } else {
-            for (int r = 0; r < GT; ++r) acc += DY[r];
+        for (int a = 0; a < R; ++a) {
+            const uint64_t r = base + FT * a + threadIdx.x;
+            load_features(X, r < n ? r : n - 1, vec, x[a]);
         }
-        out[o] = acc;
+#pragma unroll
+        for (int i = 0; i < HID; ++i) {
+            float z[R];
+#pragma unroll
+            for (int a = 0; a < R; ++a) z[a] = W[O_B1 + i];
+#pragma unroll
+            for (int k = 0; k < NF; ++k) {
+                const float w = W[O_W1 + i * NF + k];
+#pragma unroll
+                for (int a = 0; a < R; ++a) z[a] = fmaf(w, x[a][k], z[a]);
+            }
+#pragma unroll
+            for (int a = 0; a < R; ++a) h1[a][i] = fmaxf(z[a], 0.f);
+        }
+        float out[R];
+#pragma unroll
+        for (int a = 0; a < R; ++a) out[a] = W[O_B3];
+#pragma unroll 1
+        for (int j = 0; j < HID; j += 4) {
+            float z[4][R];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int a = 0; a < R; ++a) z[c][a] = W[O_B2 + j + c];
+#pragma unroll
+            for (int i = 0; i < HID; i += 4) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float4 w = *reinterpret_cast<const float4 *>(&W[O_W2 + (j + c) * HID + i]);
+#pragma unroll
+                    for (int a = 0; a < R; ++a) {
+                        z[c][a] = fmaf(w.x, h1[a][i], z[c][a]);
+                        z[c][a] = fmaf(w.y, h1[a][i + 1], z[c][a]);
+                        z[c][a] = fmaf(w.z, h1[a][i + 2], z[c][a]);
+                        z[c][a] = fmaf(w.w, h1[a][i + 3], z[c][a]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int a = 0; a < R; ++a) out[a] = fmaf(W[O_W3 + j + c], fmaxf(z[c][a], 0.f), out[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < R; ++a) {
+            const uint64_t r = base + FT * a + threadIdx.x;
+            if (r < n) y[r] = out[a];
+        }
     }
-    if (threadIdx.x == 0) {
-        float l = 0.f;
-        for (int r = 0; r < GT; ++r) l += LS[r];
+}
+
+constexpr int GT = 64;       // rows per block of the gradient kernel
+constexpr int GTH = 256;     // its threads: 16 x 16, each 4 x 4 outputs of a 64 x 64 product
+constexpr int RS = HID + 4;  // padded row stride of its tiles: 16-byte loads of 16 rows without conflicts
+struct GradSmem {
+    float W2[HID * RS], W2t[HID * RS];    // [j][i], [i][j]
+    float H1[GT * RS], H1t[HID * RS];     // [row][i] (later dZ1), [i][row]
+    float D2[GT * RS], D2t[HID * RS];     // [row][j] (first H2, then dZ2), [j][row]
+    float X[GT * NF], W1[HID * NF], b1[HID], b2[HID], w3[HID], dy[GT], sq[GT];
+    float b3;
+};
+
+// acc[a][b] += sum over k of A[r0 + 16 a][k] B[c0 + 16 b][k], k ascending: a 4 x 4
+// register tile of a product of two 64 x 64 tiles, both read along k
+__device__ __forceinline__ void tile_product(const float *A, const float *B, int r0, int c0, float (&acc)[4][4]) {
+#pragma unroll 4
+    for (int k = 0; k < HID; k += 4) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) x[a] = *reinterpret_cast<const float4 *>(&A[(r0 + 16 * a) * RS + k]);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) y[b] = *reinterpret_cast<const float4 *>(&B[(c0 + 16 * b) * RS + k]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                acc[a][b] = fmaf(x[a].x, y[b].x, acc[a][b]);
+                acc[a][b] = fmaf(x[a].y, y[b].y, acc[a][b]);
+                acc[a][b] = fmaf(x[a].z, y[b].z, acc[a][b]);
+                acc[a][b] = fmaf(x[a].w, y[b].w, acc[a][b]);
+            }
+    }
+}
+
+// Gradient of the mean squared error over `batch` rows (row g of the batch is
+// sample idx[g], or g without idx). Each block takes GT rows: the forward pass
+// and the back-propagation to dZ2 and dZ1 as products of 64 x 64 tiles in
+// shared memory (each in both layouts that its products read along), then
+// the sums over the rows for the 4801 parameters, written as one partial per
+// block (summed in a fixed order by k_mlp_reduce, so the result is
+// deterministic). Bound by shared-memory loads (8 for 64 multiply-adds) and,
+// at a batch of 16,384, by one wave of 256 blocks, two an SM: with a thread
+// per row and 128 rows a block each SM had four warps. 50.6 -> 21.7 us there.
+__global__ void __launch_bounds__(GTH) k_mlp_grad(uint32_t batch, const float *__restrict__ X, bool vec,
+                                                  const float *__restrict__ target,
+                                                  const uint32_t *__restrict__ idx,
+                                                  const __nv_bfloat16 *__restrict__ w16,
+                                                  float *partial, float *ploss) {
+    extern __shared__ float4 grad_dyn[];
+    GradSmem &s = *reinterpret_cast<GradSmem *>(grad_dyn);
+    const int tid = threadIdx.x, r0 = tid >> 4, c0 = tid & 15;
+    for (int o = tid; o < NP; o += GTH) {
+        const float w = __bfloat162float(w16[o]);
+        if (o < O_B1) s.W1[o] = w;
+        else if (o < O_W2) s.b1[o - O_B1] = w;
+        else if (o < O_B2) {
+            const int j = (o - O_W2) / HID, i = (o - O_W2) % HID;
+            s.W2[j * RS + i] = w;
+            s.W2t[i * RS + j] = w;
+        } else if (o < O_W3) s.b2[o - O_B2] = w;
+        else if (o < O_B3) s.w3[o - O_W3] = w;
+        else s.b3 = w;
+    }
+    uint64_t row = 0;  // of thread tid < GT
+    bool valid = false;
+    if (tid < GT) {
+        const uint32_t g = blockIdx.x * GT + tid;
+        valid = g < batch;
+        row = valid ? (idx ? idx[g] : g) : 0;
+        float x[NF];
+        load_features(X, row, vec, x);
+#pragma unroll
+        for (int k = 0; k < NF; ++k) s.X[tid * NF + k] = valid ? x[k] : 0.f;
+    }
+    __syncthreads();
+
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int r = r0 + 16 * a, i = c0 + 16 * b;
+            float z = s.b1[i];
+#pragma unroll
+            for (int k = 0; k < NF; ++k) z = fmaf(s.W1[i * NF + k], s.X[r * NF + k], z);
+            z = fmaxf(z, 0.f);
+            s.H1[r * RS + i] = z;
+            s.H1t[i * RS + r] = z;
+        }
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[a][b] = s.b2[c0 + 16 * b];
+    tile_product(s.H1, s.W2, r0, c0, acc);  // Z2
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            acc[a][b] = fmaxf(acc[a][b], 0.f);
+            s.D2[(r0 + 16 * a) * RS + c0 + 16 * b] = acc[a][b];  // H2
+        }
+    __syncthreads();
+    if (tid < GT) {
+        float y = s.b3;
+#pragma unroll
+        for (int j = 0; j < HID; j += 4) {
+            const float4 h = *reinterpret_cast<const float4 *>(&s.D2[tid * RS + j]);
+            y = fmaf(s.w3[j], h.x, y);
+            y = fmaf(s.w3[j + 1], h.y, y);
+            y = fmaf(s.w3[j + 2], h.z, y);
+            y = fmaf(s.w3[j + 3], h.w, y);
+        }
+        const float res = valid ? y - target[row] : 0.f;
+        s.dy[tid] = 2.f * res / (float)batch;
+        s.sq[tid] = res * res;
+    }
+    __syncthreads();
+    float *out = partial + (size_t)blockIdx.x * NP;
+    if (tid < HID) {  // dw3, from H2
+        float a = 0.f;
+#pragma unroll 8
+        for (int r = 0; r < GT; ++r) a = fmaf(s.dy[r], s.D2[r * RS + tid], a);
+        out[O_W3 + tid] = a;
+    } else if (tid == HID) {
+        float a = 0.f, l = 0.f;
+        for (int r = 0; r < GT; ++r) {
+            a += s.dy[r];
+            l += s.sq[r];
+        }
+        out[O_B3] = a;
         ploss[blockIdx.x] = l;
     }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int r = r0 + 16 * a, j = c0 + 16 * b;
+            const float dz = acc[a][b] > 0.f ? s.dy[r] * s.w3[j] : 0.f;
+            s.D2[r * RS + j] = dz;
+            s.D2t[j * RS + r] = dz;
+            acc[a][b] = 0.f;
+        }
+    __syncthreads();
+    tile_product(s.D2, s.W2t, r0, c0, acc);  // dH1
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            float *h = &s.H1[(r0 + 16 * a) * RS + c0 + 16 * b];  // read and replaced by this thread only
+            *h = *h > 0.f ? acc[a][b] : 0.f;
+            acc[a][b] = 0.f;
+        }
+    tile_product(s.D2t, s.H1t, r0, c0, acc);  // dW2[j][i]
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) out[O_W2 + (r0 + 16 * a) * HID + c0 + 16 * b] = acc[a][b];
+    __syncthreads();
+    float w0 = 0.f, w1 = 0.f, bs = 0.f;  // dW1[i][k], dW1[i + 32][k]; db1 or db2
+    const int i1 = tid / NF, k1 = tid % NF;
+    const float *bsrc = tid < HID ? &s.H1[tid] : &s.D2[tid - HID];
+#pragma unroll 8
+    for (int r = 0; r < GT; ++r) {
+        const float x = s.X[r * NF + k1];
+        w0 = fmaf(s.H1[r * RS + i1], x, w0);
+        w1 = fmaf(s.H1[r * RS + i1 + 32], x, w1);
+        if (tid < 2 * HID) bs += bsrc[r * RS];
+    }
+    out[O_W1 + i1 * NF + k1] = w0;
+    out[O_W1 + (i1 + 32) * NF + k1] = w1;
+    if (tid < HID) out[O_B1 + tid] = bs;
+    else if (tid < 2 * HID) out[O_B2 + tid - HID] = bs;
 }
 
-// grad[o] = sum over blocks of partial[b][o], in block order; grad[NP] = loss.
-__global__ void k_mlp_reduce(uint32_t blocks, uint32_t batch, const float *__restrict__ partial,
-                             const float *__restrict__ ploss, float *grad) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o < NP) {
-        float a = 0.f;
-        for (uint32_t b = 0; b < blocks; ++b) a += partial[(size_t)b * NP + o];
-        grad[o] = a;
-    } else if (o == NP) {
-        float a = 0.f;
-        for (uint32_t b = 0; b < blocks; ++b) a += ploss[b];
-        grad[NP] = a / (float)batch;
+// grad[o] = sum over blocks of partial[b][o], eight interleaved runs of blocks
+// in block order, then the runs in order; grad[NP] = loss.
+__global__ void __launch_bounds__(256) k_mlp_reduce(uint32_t blocks, uint32_t batch, const float *__restrict__ partial,
+                                                    const float *__restrict__ ploss, float *grad) {
+    __shared__ float part[8][32];
+    const int lane = threadIdx.x & 31, run = threadIdx.x >> 5, o = blockIdx.x * 32 + lane;
+    float a = 0.f;
+    if (o <= NP) {
+        const float *src = o < NP ? partial + o : ploss;
+        const size_t step = o < NP ? NP : 1;
+#pragma unroll 4
+        for (uint32_t b = run; b < blocks; b += 8) a += src[(size_t)b * step];
     }
+    part[run][lane] = a;
+    __syncthreads();
+    if (run != 0 || o > NP) return;
+#pragma unroll
+    for (int r = 1; r < 8; ++r) a += part[r][lane];
+    grad[o] = o < NP ? a : a / (float)batch;
 }
 
 // Adam (Kingma and Ba, 2015) on the float32 master parameters; c1, c2 are
@@ -441,39 +728,42 @@ int read_u32(const uint32_t *d, cudaStream_t s, uint32_t *h) {
 
 }  // namespace
 
-// Core numbers of the caller-space graph (deg already computed).
+// Core numbers of the caller-space graph (deg already computed). The steps are
+// enqueued several at a time; a step that finds nothing changed before it
+// returns at once.
 int core_numbers(const Graph &g, const uint32_t *d_deg, uint32_t *d_core, cudaStream_t s) {
     const uint32_t n = g.n;
     if (n == 0) return PLL_OK;
-    DevMem m_cur, m_alive, m_ctl;
-    PLL_CHECK(m_cur.alloc((size_t)n * 4));
-    PLL_CHECK(m_alive.alloc(n));
-    PLL_CHECK(m_ctl.alloc(sizeof(CoreCtl)));
-    CoreCtl *h = nullptr;
-    PLL_TRY(cudaMallocHost(&h, sizeof(CoreCtl)));
-    struct HostFree {
-        CoreCtl *p;
-        ~HostFree() { cudaFreeHost(p); }
-    } hf{h};
-    k_core_init<<<grid_for(n, 256), 256, 0, s>>>(n, d_deg, m_cur.as<uint32_t>(), m_alive.as<uint8_t>());
+    constexpr int AHEAD = 8;
+    PoolMem m_d0(s), m_d1(s), m_big(s), m_ctl(s);
+    PLL_CHECK(m_d0.alloc(n));
+    PLL_CHECK(m_d1.alloc(n));
+    PLL_CHECK(m_big.alloc(std::max<uint64_t>(g.nnz / CORE_BIG, 1) * 4));
+    PLL_CHECK(m_ctl.alloc((AHEAD + 1) * 4));
+    uint32_t *nbig = m_ctl.as<uint32_t>(), *changed = nbig + 1;
+    PLL_TRY(cudaMemsetAsync(nbig, 0, 4, s));
+    k_core_init<<<grid_for(n, 256), 256, 0, s>>>(n, d_deg, d_core, m_d0.as<uint8_t>(), m_d1.as<uint8_t>(),
+                                                 m_big.as<uint32_t>(), nbig);
     PLL_TRY(cudaGetLastError());
-    uint32_t k = 0;
-    // every pass removes a vertex or raises k past a degree, so the loop is finite
-    const uint64_t max_passes = 2ull * n + 2;
-    for (uint64_t pass = 0;; ++pass) {
-        if (pass > max_passes) return PLL_E_CUDA;
-        const CoreCtl init{0, 0, 0xffffffffu, 0};
-        PLL_TRY(cudaMemcpyAsync(m_ctl.p, &init, sizeof(CoreCtl), cudaMemcpyHostToDevice, s));
-        k_core_pass<<<grid_for(n, 256), 256, 0, s>>>(n, g.off, g.col, k, m_cur.as<uint32_t>(),
-                                                     m_alive.as<uint8_t>(), d_core, m_ctl.as<CoreCtl>());
+    CoreArgs a{n, g.off, g.col, d_core, m_d0.as<uint8_t>(), m_d1.as<uint8_t>(), m_big.as<uint32_t>(), nbig,
+               nullptr, nullptr};
+    const int grid = CORE_BIG_BLOCKS + grid_for((uint64_t)n * 32 / CORE_CHUNK, 256);
+    uint32_t h[AHEAD];
+    // every step but the last lowers a value, so the loop is finite
+    for (uint64_t step = 0; step <= g.nnz + AHEAD; step += AHEAD) {
+        PLL_TRY(cudaMemsetAsync(changed, 0, AHEAD * 4, s));
+        for (int i = 0; i < AHEAD; ++i) {
+            a.prev = i ? changed + i - 1 : nullptr;
+            a.changed = changed + i;
+            k_core_step<<<grid, 256, 0, s>>>(a);
+            std::swap(a.src, a.dst);
+        }
         PLL_TRY(cudaGetLastError());
-        PLL_TRY(cudaMemcpyAsync(h, m_ctl.p, sizeof(CoreCtl), cudaMemcpyDeviceToHost, s));
+        PLL_TRY(cudaMemcpyAsync(h, changed, AHEAD * 4, cudaMemcpyDeviceToHost, s));
         PLL_TRY(cudaStreamSynchronize(s));
-        if (h->removed) continue;
-        if (h->alive == 0) break;
-        k = h->min_deg;
+        if (h[AHEAD - 1] == 0) return PLL_OK;
     }
-    return PLL_OK;
+    return PLL_E_CUDA;
 }
 
 }  // namespace pll
@@ -504,7 +794,7 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
     if (n == 0) return PLL_OK;
     Graph g;
     g.n = n; g.nnz = nnz; g.off = offsets; g.col = cols;
-    DevMem m_err;
+    PoolMem m_err(s);
     PLL_CHECK(m_err.alloc(4));
     PLL_TRY(cudaMemsetAsync(m_err.p, 0, 4, s));
     PLL_CHECK(prep_validate_csr(g, m_err.as<uint32_t>(), s));
@@ -512,7 +802,7 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
     PLL_CHECK(read_u32(m_err.as<uint32_t>(), s, &h_err));
     if (h_err) return PLL_E_INVAL;
 
-    DevMem m_deg, m_two, m_core;
+    PoolMem m_deg(s), m_two(s), m_core(s);
     PLL_CHECK(m_deg.alloc((size_t)n * 4));
     uint64_t *d_two = two_hop;
     uint32_t *d_core = core;
@@ -525,7 +815,7 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
 
     // bit-parallel labels of the Degree order (rank space)
     const uint32_t tp = bp_stride(t);
-    DevMem m_order, m_inv, m_roff, m_rcol, m_inX, m_root, m_cnt, m_S, m_bpd, m_bpm;
+    PoolMem m_order(s), m_inv(s), m_roff(s), m_rcol(s), m_inX(s), m_root(s), m_cnt(s), m_S(s), m_bpd(s), m_bpm(s);
     if (t) {
         PLL_CHECK(m_order.alloc((size_t)n * 4));
         PLL_CHECK(m_inv.alloc((size_t)n * 4));
@@ -553,18 +843,19 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
         PLL_CHECK(read_u32(m_err.as<uint32_t>(), s, &h_err));
         if (h_err) return (h_err & ERR_DEPTH) ? PLL_E_RANGE : PLL_E_CUDA;
     }
-    k_features_raw<<<grid_for((uint64_t)n * 32, 256), 256, 0, s>>>(
+    k_features_raw<<<grid_for(n, 256), 256, 0, s>>>(
         n, t, tp, m_inv.as<uint32_t>(), m_deg.as<uint32_t>(),
         reinterpret_cast<const unsigned long long *>(d_two), d_core, m_bpd.as<uint8_t>(),
         m_bpm.as<uint64_t>(), feat);
     PLL_TRY(cudaGetLastError());
-    DevMem m_mom;
+    PoolMem m_mom(s);
     PLL_CHECK(m_mom.alloc(2 * NF * sizeof(double)));
     double *mean = m_mom.as<double>(), *ssd = mean + NF;
     PLL_TRY(cudaMemsetAsync(m_mom.p, 0, 2 * NF * sizeof(double), s));
     k_col_moments<<<grid_for(n, 256), 256, 0, s>>>(n, feat, mean, 0, mean);
     k_mean<<<1, 32, 0, s>>>(n, mean);
     k_col_moments<<<grid_for(n, 256), 256, 0, s>>>(n, feat, mean, 1, ssd);
+    k_std<<<1, 32, 0, s>>>(n, ssd);
     k_standardise<<<grid_for((uint64_t)n * NF, 256), 256, 0, s>>>(n, mean, ssd, feat);
     PLL_TRY(cudaGetLastError());
     PLL_TRY(cudaStreamSynchronize(s));
@@ -594,7 +885,7 @@ PLL_API int pll_order_from_scores(const float *scores, uint32_t n, uint32_t *ord
     if (n && (!scores || !order)) return PLL_E_INVAL;
     if (n == 0) return PLL_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    DevMem m_keys, m_sorted, m_temp;
+    PoolMem m_keys(s), m_sorted(s), m_temp(s);
     PLL_CHECK(m_keys.alloc((size_t)n * 8));
     PLL_CHECK(m_sorted.alloc((size_t)n * 8));
     k_score_keys<<<grid_for(n, 256), 256, 0, s>>>(n, scores, m_keys.as<uint64_t>());
@@ -622,7 +913,7 @@ PLL_API int pll_mlp_create(uint32_t max_batch, pll_mlp **out) {
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess) e = cudaMalloc(&p->mem, nf * sizeof(float));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GRAD_SMEM);
+        e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         if (p->mem) cudaFree(p->mem);
@@ -676,7 +967,13 @@ PLL_API int pll_mlp_forward(const pll_mlp *p, const float *x, uint64_t n, float 
     if (!p || (n && (!x || !y))) return PLL_E_INVAL;
     if (n == 0) return PLL_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    k_mlp_fwd<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, x, p->w16, y);
+    // two rows a thread where that still fills the GPU (three blocks an SM)
+    const bool vec = reinterpret_cast<uintptr_t>(x) % 16 == 0;
+    const uint64_t wide = 152ull * 3;
+    if (n >= wide * FT * 2)
+        k_mlp_fwd<2><<<(unsigned)wide, FT, 0, s>>>(n, x, vec, p->w16, y);
+    else
+        k_mlp_fwd<1><<<(unsigned)((n + FT - 1) / FT), FT, 0, s>>>(n, x, vec, p->w16, y);
     PLL_TRY(cudaGetLastError());
     return PLL_OK;
 }
@@ -687,9 +984,10 @@ PLL_API int pll_mlp_grad(pll_mlp *p, const float *x, const float *target, const 
     if (batch > p->max_batch) return PLL_E_RANGE;
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t blocks = (batch + GT - 1) / GT;
-    k_mlp_grad<<<blocks, GT, GRAD_SMEM, s>>>(batch, x, target, idx, p->w16, p->partial, p->ploss);
+    const bool vec = reinterpret_cast<uintptr_t>(x) % 16 == 0;
+    k_mlp_grad<<<blocks, GTH, sizeof(GradSmem), s>>>(batch, x, vec, target, idx, p->w16, p->partial, p->ploss);
     PLL_TRY(cudaGetLastError());
-    k_mlp_reduce<<<(NP + 1 + 255) / 256, 256, 0, s>>>(blocks, batch, p->partial, p->ploss, p->grad);
+    k_mlp_reduce<<<(NP + 1 + 31) / 32, 256, 0, s>>>(blocks, batch, p->partial, p->ploss, p->grad);
     PLL_TRY(cudaGetLastError());
     return PLL_OK;
 }
@@ -697,9 +995,25 @@ PLL_API int pll_mlp_grad(pll_mlp *p, const float *x, const float *target, const 
 PLL_API int pll_mlp_read_grad(const pll_mlp *p, float *host_grad, float *host_loss, void *stream) {
     if (!p || (!host_grad && !host_loss)) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    if (host_grad) PLL_TRY(cudaMemcpyAsync(host_grad, p->grad, NP * sizeof(float), cudaMemcpyDeviceToHost, s));
-    if (host_loss) PLL_TRY(cudaMemcpyAsync(host_loss, p->grad + NP, sizeof(float), cudaMemcpyDeviceToHost, s));
+    // gradient and loss in one copy into pinned memory (two into the caller's
+    // pageable arrays are staged ones, a wait each); one buffer per thread, as
+    // the call is synchronous. It lives as long as the thread.
+    static thread_local float *pinned = nullptr;
+    if (!pinned && cudaMallocHost(&pinned, (NP + 1) * sizeof(float)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        pinned = nullptr;
+    }
+    if (!pinned) {
+        if (host_grad) PLL_TRY(cudaMemcpyAsync(host_grad, p->grad, NP * sizeof(float), cudaMemcpyDeviceToHost, s));
+        if (host_loss) PLL_TRY(cudaMemcpyAsync(host_loss, p->grad + NP, sizeof(float), cudaMemcpyDeviceToHost, s));
+        PLL_TRY(cudaStreamSynchronize(s));
+        return PLL_OK;
+    }
+    const size_t first = host_grad ? 0 : NP, last = host_loss ? NP + 1 : NP;
+    PLL_TRY(cudaMemcpyAsync(pinned + first, p->grad + first, (last - first) * sizeof(float), cudaMemcpyDeviceToHost, s));
     PLL_TRY(cudaStreamSynchronize(s));
+    if (host_grad) std::memcpy(host_grad, pinned, NP * sizeof(float));
+    if (host_loss) *host_loss = pinned[NP];
     return PLL_OK;
 }
 
@@ -728,7 +1042,7 @@ PLL_API int pll_learned_order(const uint32_t *offsets, const uint32_t *cols, uin
     if (!p || (n && !order)) return PLL_E_INVAL;
     if (n == 0) return PLL_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    DevMem m_x, m_y;
+    PoolMem m_x(s), m_y(s);
     PLL_CHECK(m_x.alloc((size_t)n * NF * 4));
     PLL_CHECK(m_y.alloc((size_t)n * 4));
     PLL_CHECK(pll_features(offsets, cols, n, nnz, t, stream, m_x.as<float>(), nullptr, nullptr));
