@@ -118,46 +118,72 @@ __global__ void k_relabel(uint32_t n, const uint32_t *__restrict__ order,
 
 __global__ void k_set_last(uint32_t *a, uint32_t idx, uint32_t val) { a[idx] = val; }
 
-// Sec. 5.4 greedy choice, one warp. inX doubles as the "used" mark.
-__global__ void k_select_bp(uint32_t n, uint32_t t, const uint32_t *__restrict__ roff,
-                            const uint32_t *__restrict__ rcol, uint8_t *inX, uint32_t *root,
-                            uint32_t *cnt, uint32_t *S) {
-    const int lane = threadIdx.x;
+// Sec. 5.4 greedy choice, one block (a hub's members may lie behind thousands
+// of used neighbours: 512 at a step; R-MAT-20, t = 64: 568 us with one warp, 156
+// so, a chain of 64 dependent choices). inX doubles as the "used" mark.
+constexpr int SELECT_THREADS = 512;
+__global__ void __launch_bounds__(SELECT_THREADS) k_select_bp(uint32_t n, uint32_t t, const uint32_t *__restrict__ roff,
+                                                              const uint32_t *__restrict__ rcol, uint8_t *inX,
+                                                              uint32_t *root, uint32_t *cnt, uint32_t *S) {
+    __shared__ uint32_t s_count[SELECT_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    volatile uint8_t *used = inX;  // written and read by this block only
+    // this thread's place among those with ok set, and how many there are
+    auto place = [&](bool ok, uint32_t *total) -> uint32_t {
+        const unsigned m = __ballot_sync(FULL, ok);
+        __syncthreads();
+        if (lane == 0) s_count[warp] = __popc(m);
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+        for (int w = 0; w < SELECT_THREADS / 32; ++w) {
+            const uint32_t c = s_count[w];
+            if (w < warp) before += c;
+            all += c;
+        }
+        *total = all;
+        return before + __popc(m & ((1u << lane) - 1u));
+    };
+    __shared__ uint32_t s_root;
     uint32_t next = 0;
     for (uint32_t i = 0; i < t; ++i) {
         // lowest unused rank >= next
-        uint32_t r = NONE;
+        bool found = false;
         while (next < n) {
-            uint32_t c = next + lane;
-            bool ok = c < n && !inX[c];
-            unsigned m = __ballot_sync(FULL, ok);
-            if (m) { r = next + __ffs(m) - 1; break; }
-            next += 32;
+            const uint32_t c = next + tid;
+            const bool ok = c < n && !used[c];
+            uint32_t all = 0;
+            const uint32_t p = place(ok, &all);
+            if (ok && p == 0) s_root = c;
+            __syncthreads();
+            if (all) {
+                found = true;
+                break;
+            }
+            next += SELECT_THREADS;
         }
-        if (r == NONE) {
-            if (lane == 0) { root[i] = NONE; cnt[i] = 0; }
+        if (!found) {
+            if (tid == 0) { root[i] = NONE; cnt[i] = 0; }
             continue;
         }
-        if (lane == 0) { inX[r] = 1; root[i] = r; }
+        const uint32_t r = s_root;
+        if (tid == 0) { used[r] = 1; root[i] = r; }
         next = r + 1;
-        __syncwarp();
+        __syncthreads();
         uint32_t c = 0;
         const uint32_t b = roff[r], e = roff[r + 1];
-        for (uint32_t x = b; x < e && c < BPW; x += 32) {
-            uint32_t w = (x + lane < e) ? rcol[x + lane] : NONE;
-            bool ok = (w != NONE) && !inX[w];
-            unsigned m = __ballot_sync(FULL, ok);
-            uint32_t pos = c + __popc(m & ((1u << lane) - 1u));
-            __syncwarp();
+        for (uint32_t x = b; x < e && c < BPW; x += SELECT_THREADS) {
+            const uint32_t w = e - x > (uint32_t)tid ? rcol[x + tid] : NONE;
+            const bool ok = w != NONE && !used[w];
+            uint32_t all = 0;
+            const uint32_t pos = c + place(ok, &all);
             if (ok && pos < BPW) {
                 S[(size_t)i * BPW + pos] = w;
-                inX[w] = 1;
+                used[w] = 1;
             }
-            c += __popc(m);
-            __syncwarp();
+            c += all;
         }
-        if (lane == 0) cnt[i] = c < BPW ? c : BPW;
-        __syncwarp();
+        if (tid == 0) cnt[i] = c < BPW ? c : BPW;
+        __syncthreads();
     }
 }
 
@@ -351,7 +377,7 @@ int prep_select_bp_roots(uint32_t n, uint32_t t, const uint32_t *d_roff, const u
                          uint8_t *d_inX, uint32_t *d_root, uint32_t *d_cnt, uint32_t *d_S,
                          cudaStream_t s) {
     if (t == 0) return PLL_OK;
-    k_select_bp<<<1, 32, 0, s>>>(n, t, d_roff, d_rcol, d_inX, d_root, d_cnt, d_S);
+    k_select_bp<<<1, SELECT_THREADS, 0, s>>>(n, t, d_roff, d_rcol, d_inX, d_root, d_cnt, d_S);
     PLL_TRY(cudaGetLastError());
     return PLL_OK;
 }
