@@ -558,7 +558,7 @@ PLL_API void pll_paths_free(pll_paths *p);
  *                  undirected labels (t = 0) in both sets.
  *   order          device or NULL: rank -> vertex; NULL = descending in- plus
  *                  out-degree, ties by ascending id.
- *   opts           t = 0; root_batch as for pll_build (0 = 1024, halved while
+ *   opts           t = 0; root_batch as for pll_build (0 = 16384, halved while
  *                  n x root_batch / 8 bytes of visited bits pass 2 GiB); block,
  *                  flags, reserved: 0. NULL = defaults.
  *   out            receives the index; free it with pll_dfree.

@@ -53,9 +53,10 @@ __global__ void k_root_segments(const uint64_t *__restrict__ T, uint64_t P, uint
 // and (v_k, h, b) with a + b <= d (the lowest such h lies on a shortest
 // v_k-u path). u's tuples with hub < k are [lo_u, x): the run of u ends at x,
 // and its start is found by galloping back from x (runs are short). v_k's
-// come from seg (or, without it, a binary search).
-__global__ void k_cleanup(const uint64_t *__restrict__ T, uint64_t P, const uint64_t *__restrict__ seg,
-                          uint32_t k0, uint8_t *keep) {
+// come from R (T itself; for directed graphs the other direction's tuples), at
+// the range seg gives (or, without it, a binary search).
+__global__ void k_cleanup(const uint64_t *__restrict__ T, uint64_t P, const uint64_t *__restrict__ R, uint64_t PR,
+                          const uint64_t *__restrict__ seg, uint32_t k0, uint8_t *keep) {
     for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < P;
          x += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t key = T[x];
@@ -75,13 +76,13 @@ __global__ void k_cleanup(const uint64_t *__restrict__ T, uint64_t P, const uint
             lo_k = seg[2 * (k - k0)];
             hi_k = seg[2 * (k - k0) + 1];
         } else {
-            lo_k = lower_bound_u64(T, 0, P, (uint64_t)k << 32);
-            hi_k = lower_bound_u64(T, lo_k, P, pack_tuple(k, k, 0));
+            lo_k = lower_bound_u64(R, 0, PR, (uint64_t)k << 32);
+            hi_k = lower_bound_u64(R, lo_k, PR, pack_tuple(k, k, 0));
         }
         uint64_t i = lo_u, j = lo_k;
         bool drop = false;
         while (i < x && j < hi_k) {
-            const uint32_t ei = (uint32_t)T[i], ej = (uint32_t)T[j];
+            const uint32_t ei = (uint32_t)T[i], ej = (uint32_t)R[j];
             const uint32_t hi = entry_hub(ei), hj = entry_hub(ej);
             if (hi == hj) {
                 if (entry_dist(ei) + entry_dist(ej) <= d) { drop = true; break; }
@@ -171,16 +172,16 @@ int labels_sort_tuples(uint64_t *d_in, uint64_t *d_out, uint64_t count, int begi
     return PLL_OK;
 }
 
-int labels_cleanup(const uint64_t *d_sorted, uint64_t count, uint8_t *d_keep, uint32_t k0, uint32_t B,
-                   void *scratch, size_t scratch_bytes, cudaStream_t s) {
+int labels_cleanup(const uint64_t *d_sorted, uint64_t count, const uint64_t *d_roots, uint64_t root_count,
+                   uint8_t *d_keep, uint32_t k0, uint32_t B, void *scratch, size_t scratch_bytes, cudaStream_t s) {
     if (count == 0) return PLL_OK;
     uint64_t *seg = nullptr;
     if (scratch && scratch_bytes >= (size_t)B * 16) {
         seg = static_cast<uint64_t *>(scratch);
-        k_root_segments<<<(B + 255) / 256, 256, 0, s>>>(d_sorted, count, k0, B, seg);
+        k_root_segments<<<(B + 255) / 256, 256, 0, s>>>(d_roots, root_count, k0, B, seg);
         PLL_TRY(cudaGetLastError());
     }
-    k_cleanup<<<grid_for(count, 256), 256, 0, s>>>(d_sorted, count, seg, k0, d_keep);
+    k_cleanup<<<grid_for(count, 256), 256, 0, s>>>(d_sorted, count, d_roots, root_count, seg, k0, d_keep);
     PLL_TRY(cudaGetLastError());
     return PLL_OK;
 }

@@ -878,8 +878,8 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             mc = __ldcg(reinterpret_cast<const ulonglong2 *>(a.candc) + b + i0 + lane);
             w = (uint32_t)mine;
             slot = (uint32_t)(mine >> 32);
-            wlen = a.lab_len[w];
-            woff = a.lab_off[w];
+            wlen = a.vis_len[w];
+            woff = a.vis_off[w];
             klen = a.lab_len[a.k0 + slot];
             tb = a.ht_off[slot];
             const unsigned long long te = a.ht_off[slot + 1];
@@ -932,7 +932,7 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             for (uint32_t m = __ballot_sync(FULL, in && wlen >= LONG_LABEL); m; m &= m - 1) {
                 const uint32_t j = __ffs(m) - 1;
                 const uint32_t lj = __shfl_sync(FULL, wlen, j), quads = (lj + 3) / 4;
-                const uint32_t *lab = a.pool + __shfl_sync(FULL, woff, j);
+                const uint32_t *lab = a.vis_pool + __shfl_sync(FULL, woff, j);
                 for (uint32_t q0 = 0; q0 < quads; q0 += 32) {
                     const uint32_t q = q0 + lane;
                     if (__any_sync(FULL, q < quads && quad_prunes(a, tw, r, load_quad(lab, q, lj), level))) {
@@ -959,7 +959,7 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
 #pragma unroll
                 for (uint32_t step = 16; step > 0; step >>= 1)
                     if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
-                const uint32_t *lab = a.pool + __shfl_sync(FULL, woff, j);
+                const uint32_t *lab = a.vis_pool + __shfl_sync(FULL, woff, j);
                 const uint32_t lj = __shfl_sync(FULL, len, j), xj = __shfl_sync(FULL, excl, j);
                 bool p = false;
                 if (x < total) p = quad_prunes(a, tw, r, load_quad(lab, x - xj, lj), level);

@@ -306,7 +306,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.roff = roff; a.rcol = rcol; a.rstart = m_rstart.as<uint32_t>();
         a.bp_d = ix->d_bp_d; a.bp_c = m_bpc.as<uint8_t>(); a.bp_m = ix->d_bp_m; a.inX = inX;
         a.bp_q = m_bpq.as<uint4>(); a.qn = qn; a.bp_e = bp_e;
-        a.lab_off = st.off; a.lab_len = st.len; a.pool = st.pool;
+        a.lab_off = a.vis_off = st.off; a.lab_len = a.vis_len = st.len; a.pool = a.vis_pool = st.pool;
         a.k0 = k0; a.B = k1 - k0; a.NW = NW;
         a.visited = m_vis.as<uint32_t>();
         a.ht = m_ht.as<uint32_t>();
@@ -430,7 +430,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             PLL_CHECK(labels_sort_tuples(m_out.as<uint64_t>(), m_sorted.as<uint64_t>(), P, SORT_BEGIN_BIT, end_bit,
                                          m_temp.p, &tb, s));
             // the sort is done with the temporary space; the cleanup borrows it
-            PLL_CHECK(labels_cleanup(m_sorted.as<uint64_t>(), P, m_keep.as<uint8_t>(), k0, k1 - k0,
+            PLL_CHECK(labels_cleanup(m_sorted.as<uint64_t>(), P, m_sorted.as<uint64_t>(), P,
+                                     m_keep.as<uint8_t>(), k0, k1 - k0,
                                      m_temp.p, temp_bytes, s));
             tb = temp_bytes;
             PLL_CHECK(labels_compact(m_sorted.as<uint64_t>(), m_keep.as<uint8_t>(), P,

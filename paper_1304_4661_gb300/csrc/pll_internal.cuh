@@ -313,9 +313,12 @@ struct BatchArgs {
     const ulonglong2 *bp_e;    // [n] roots with S^{-1} non-empty, with S^{-1} or S^0 non-empty
     const uint64_t *bp_m;
     const uint8_t *inX;
-    const uint64_t *lab_off;   // per-vertex start in pool
+    const uint64_t *lab_off;   // labels of the roots: per-vertex start in pool
     const uint32_t *lab_len;   // per-vertex length (entries with hub < k0)
     const uint32_t *pool;
+    const uint64_t *vis_off;   // labels of the visited vertices: the same arrays, or
+    const uint32_t *vis_len;   // (directed graphs) those of the other label set
+    const uint32_t *vis_pool;
     uint32_t k0, B, NW;        // roots [k0, k0 + B), NW = ceil(n / 32)
     uint32_t qn;               // 16-byte chunks of a bp_q row: ceil(t / 32)
     uint32_t *visited;         // [B][NW] bitmap: row of root slot s holds one bit
@@ -377,9 +380,11 @@ struct LabelStore {
 // radix sort of packed tuples by their bits [begin_bit, end_bit)
 int labels_sort_tuples(uint64_t *d_in, uint64_t *d_out, uint64_t count, int begin_bit, int end_bit,
                        void *d_temp, size_t *temp_bytes, cudaStream_t s);
-// scratch (>= 16 B bytes, may be NULL) holds each root's own tuple range
-int labels_cleanup(const uint64_t *d_sorted, uint64_t count, uint8_t *d_keep, uint32_t k0, uint32_t B,
-                   void *scratch, size_t scratch_bytes, cudaStream_t s);
+// d_roots: the sorted tuples that hold the roots' own entries (d_sorted, or the
+// other direction's of a directed batch). scratch (>= 16 B bytes, may be NULL)
+// holds each root's own tuple range
+int labels_cleanup(const uint64_t *d_sorted, uint64_t count, const uint64_t *d_roots, uint64_t root_count,
+                   uint8_t *d_keep, uint32_t k0, uint32_t B, void *scratch, size_t scratch_bytes, cudaStream_t s);
 int labels_compact(const uint64_t *d_in, const uint8_t *d_keep, uint64_t count, uint64_t *d_out,
                    unsigned long long *d_nout, void *d_temp, size_t *temp_bytes, cudaStream_t s);
 int labels_append(const LabelStore &st, const uint64_t *d_kept,

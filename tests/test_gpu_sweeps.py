@@ -69,3 +69,22 @@ def test_labels_longer_than_a_roots_table():
     for root_batch in (0, 100):
         ix = gpu_build(g, 0, order=order, root_batch=root_batch)
         assert same_labels(ix.labels(), ref), first_label_diff(ix.labels(), ref, g.n)
+
+
+def two_way_ladder(n):
+    """A directed path of n vertices with arcs back from everywhere to the first few: deep forward
+    BFSs whose vertices reach low ranks at every level."""
+    arcs = [(i, i + 1) for i in range(n - 1)] + [(i, j) for i in range(5, n) for j in range(0, 4)]
+    return gg.digraph(n, arcs, f"ladder{n}")
+
+
+@pytest.mark.parametrize("n", [240, 250, 254])
+@pytest.mark.parametrize("root_batch", [0, 1, 30])
+def test_directed_depths_next_to_the_limit(n, root_batch):
+    """Arcs to finished hubs at every depth: the cut lists must give the labels of whole ones, and
+    a depth of 255 must be an error only where whole lists make it one."""
+    from .gpu_util import dev_u32
+    d = two_way_ladder(n)
+    ref = oracle.DirectedIndex(d.offsets, d.cols)
+    ix = pll.DirectedIndex(dev_u32(d.offsets), dev_u32(d.cols), root_batch=root_batch)
+    assert same_labels(ix.labels_in(), ref.labels_in()) and same_labels(ix.labels_out(), ref.labels_out())
