@@ -3,7 +3,9 @@
 // d(s, t) = min( bit-parallel query (Sec. 5.3), Query(s, t, L) (Sec. 3.3) ).
 //
 // A persistent grid (a few CTAs per SM) walks the pairs; one warp answers one
-// pair. A launch too small to fill the GPU that way (up to 4 pairs per
+// pair, the bit-parallel part first, which bounds what the labels can add
+// (pair_bounded). Pairs with an end that nothing reaches are settled by one
+// lane each (lone_pair). A launch too small to fill the GPU that way (up to 4 pairs per
 // resident block) gives each pair 2, 4 or 8 warps instead, which split the
 // label scan and meet in shared memory. Lanes own bit-parallel roots (lane, lane + 32): the t distance bytes
 // of s and of t arrive in one coalesced load each, and d~_i = d(s,r_i) +
@@ -25,6 +27,7 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t BIG = 1u << 20;
+constexpr int QUERY_BLOCKS = 8;
 
 struct QueryArgs {
     uint32_t n, t, tp;
@@ -162,7 +165,7 @@ __device__ __forceinline__ uint32_t label_min_merge_at(const QueryArgs &a, uint3
 }
 
 // The bit-parallel answer, fetching masks only where they can beat `best`
-// (the normal-label answer), then the final byte.
+// (a label answer, or BIG).
 __device__ __forceinline__ uint32_t finish_pair(const QueryArgs &a, uint32_t s, uint32_t t, int lane,
                                                 uint32_t td0, uint32_t td1, uint32_t dstar,
                                                 uint32_t best) {
@@ -194,51 +197,192 @@ __device__ __forceinline__ void store_answer(const QueryArgs &a, uint64_t qi, ui
     a.out[qi] = (uint8_t)answer_byte(a, best);
 }
 
+// An open pair: the ends' ranks, and where their labels are.
+struct OpenPair {
+    uint64_t os, ot;
+    uint32_t s, t, ls, lt;
+};
+
+// v's bit-parallel row holds no distance (nothing reaches v from any root)
+__device__ __forceinline__ bool row_empty(const QueryArgs &a, uint32_t v) {
+    const uint4 *row = reinterpret_cast<const uint4 *>(a.bp_d + (size_t)v * a.tp);
+    for (uint32_t c = 0; c < a.tp / 16; ++c) {
+        const uint4 r = row[c];
+        if ((r.x & r.y & r.z & r.w) != 0xffffffffu) return false;
+    }
+    return true;
+}
+
+// One thread: a pair with an end x that no bit-parallel root reaches and whose
+// label has at most one entry (h, d), on power-law graphs mostly an isolated
+// vertex, 4 of 10 on R-MAT-20 and so 6 of 10 uniform pairs. The pair's distance
+// is d + d(h, y) if h is in the label of the other end y, none otherwise;
+// a label's hubs are at most its vertex's own rank.
+__device__ __forceinline__ bool lone_pair(const QueryArgs &a, uint32_t s, uint64_t os, uint32_t ls, uint32_t t,
+                                          uint64_t ot, uint32_t lt, uint32_t *dist) {
+    if (ls > 1 && lt > 1) return false;
+    const bool at_s = ls <= 1 && row_empty(a, s);
+    if (!at_s && !(lt <= 1 && row_empty(a, t))) return false;
+    *dist = BIG;
+    if ((at_s ? ls : lt) == 0) return true;
+    const uint32_t e = a.lab[at_s ? os : ot], h = entry_hub(e), y = at_s ? t : s;
+    if (h > y) return true;
+    const uint32_t *B = a.lab + (at_s ? ot : os);
+    const uint32_t lb = at_s ? lt : ls;
+    uint32_t lo = 0, hi = lb;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (entry_hub(B[mid]) < h) lo = mid + 1; else hi = mid;
+    }
+    if (lo < lb && entry_hub(B[lo]) == h) *dist = entry_dist(e) + entry_dist(B[lo]);
+    return true;
+}
+
+// Entries of L(v) that can be part of a distance below ub through a hub that is
+// neither end, compacted into `keep` (KEEP places): at most ub - 2 from v, as
+// the other end is at least 1 from such a hub. *direct: the distance of v to
+// `other`, if that is one of its hubs. AHEAD windows of 32 entries are loaded
+// together. Returns how many are kept (over KEEP: too many, not all looked at).
+constexpr uint32_t KEEP = 32;
+constexpr int AHEAD = 2;
+__device__ __forceinline__ uint32_t keep_near(const uint32_t *__restrict__ lab, uint32_t len, uint32_t v,
+                                              uint32_t ub, uint32_t other, int lane, uint32_t *keep,
+                                              uint32_t *direct) {
+    uint32_t cnt = 0;
+    for (uint32_t x0 = 0; x0 < len && cnt <= KEEP; x0 += 32 * AHEAD) {
+        uint32_t e[AHEAD];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            const uint32_t x = x0 + 32 * u + lane;
+            e[u] = x < len ? lab[x] : NONE;
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            const uint32_t h = entry_hub(e[u]), d = entry_dist(e[u]);
+            if (h == other) *direct = d;
+            const bool in = e[u] != NONE && d + 2 <= ub && h != v;
+            const unsigned m = __ballot_sync(FULL, in);
+            const uint32_t pos = cnt + __popc(m & ((1u << lane) - 1u));
+            if (in && pos < KEEP) keep[pos] = e[u];
+            cnt += __popc(m);
+        }
+    }
+    return cnt;
+}
+
+// The distance of an open pair, one warp. The bit-parallel answer ub comes
+// first: a common hub of the labels matters only below it. A label's hubs are
+// at most its vertex's own rank, so of the two ends only the one of lower rank,
+// h, can be a hub of the other, v: L(v) is read first, for h itself and for the
+// near entries that can be on a path through a third hub (on power-law graphs,
+// with ub 3 or 4, 1 entry in 20, often none), and L(h) only if there are some.
+// The reads are one pass of independent loads; the merge join's windows wait
+// for one another. (Bounded by the least d~ alone, with the masks after the
+// labels, twice as many entries stay: 0.6 ms more on the 10M pairs of
+// R-MAT-20; with both labels loaded along with the rows: 1 ms more.) Without a
+// bound (t = 0, or ends that no root reaches), with too many near entries or
+// where one label is long against the other, the merge join or its binary
+// searches decide.
+constexpr uint32_t LONG_LABEL = 256;
+__device__ __forceinline__ uint32_t pair_bounded(const QueryArgs &a, const OpenPair &p, int lane, uint32_t *keep) {
+    uint32_t td0, td1, dstar;
+    bp_tilde(a, p.s, p.t, lane, &td0, &td1, &dstar);
+    if (dstar >= BIG) return label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane);
+    uint32_t ub = finish_pair(a, p.s, p.t, lane, td0, td1, dstar, BIG);
+    const bool low = p.s < p.t;  // h = s, v = t
+    const uint32_t h = low ? p.s : p.t, v = low ? p.t : p.s, lh = low ? p.ls : p.lt, lv = low ? p.lt : p.ls;
+    if (ub <= 1 || lv == 0) return ub;
+    if (lv > LONG_LABEL && lv > PLL_MERGE_RATIO * lh) return min(ub, label_min(a, p.s, p.t, lane, 0, 32));
+    uint32_t direct = BIG;
+    const uint32_t cv = keep_near(a.lab + (low ? p.ot : p.os), lv, v, ub, h, lane, keep, &direct);
+    if (cv > KEEP) return min(ub, label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane));
+    ub = min(ub, warp_min(direct));
+    if (cv == 0 || ub <= 2) return ub;
+    __syncwarp();
+    const uint32_t *H = a.lab + (low ? p.os : p.ot);
+    uint32_t best = ub;
+    if (lh > LONG_LABEL) {  // a lane for each kept entry
+        if ((uint32_t)lane < cv) {
+            const uint32_t e = keep[lane];
+            uint32_t lo = 0, hi = lh;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (entry_hub(H[mid]) < entry_hub(e)) lo = mid + 1; else hi = mid;
+            }
+            if (lo < lh && entry_hub(H[lo]) == entry_hub(e)) best = min(best, entry_dist(e) + entry_dist(H[lo]));
+        }
+    } else {
+        const uint32_t e = (uint32_t)lane < cv ? keep[lane] : NONE;
+        __syncwarp();
+        const uint32_t ch = keep_near(H, lh, h, ub, NONE, lane, keep, &direct);
+        if (ch > KEEP) return min(ub, label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane));
+        __syncwarp();
+        for (uint32_t i = 0; i < ch; ++i) {
+            const uint32_t f = keep[i];
+            if (entry_hub(f) == entry_hub(e)) best = min(best, entry_dist(e) + entry_dist(f));
+        }
+    }
+    best = warp_min(best);
+    __syncwarp();  // the next pair writes keep
+    return best;
+}
+
 // One warp per pair, PG pairs at a time: lane j < PG first fetches pair j's
 // ids, ranks and label offsets (three dependent loads, in flight for PG pairs
-// at once instead of one after another), and answers the trivial pairs; the
-// warp then answers the others one by one from the lanes' registers. PG is
-// 32 for launches that fill the GPU that way and smaller for launches that
-// would otherwise leave warps idle. Eight CTAs per SM (32 registers a
-// thread): the kernel is bound by the latency of its loads, so it wants every
-// resident warp it can get.
+// at once instead of one after another), and answers the trivial and the lone
+// pairs; the warp then answers the others one by one, their ranks and offsets
+// in shared memory. PG is 32 for launches that fill the GPU that way and smaller
+// for launches that would otherwise leave warps idle. Bound by the traffic and
+// the latency of scattered loads, so it wants resident warps: eight blocks an
+// SM, 32 registers a thread (six blocks: 10 % slower). 10M uniform pairs of
+// R-MAT-20, t = 64: 5.02 ms with the merge join for every pair, 3.22 ms so, of
+// which (by leaving steps out) 0.3 ms for ranks, offsets and lone pairs, 0.3
+// for the rows, 1.0 for the masks and 0.8 for each end's label.
 template <int PG>
-__global__ void __launch_bounds__(256, 8) k_query(QueryArgs a) {
+__global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
+    __shared__ uint32_t s_keep[8][KEEP];
+    __shared__ OpenPair s_pair[8][PG];
     const int lane = threadIdx.x & 31;
+    uint32_t *keep = s_keep[threadIdx.x >> 5];
+    OpenPair *pair = s_pair[threadIdx.x >> 5];
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t q0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PG; q0 < a.q;
          q0 += warps * PG) {
         const uint64_t qi = q0 + lane;
         const bool mine = lane < PG && qi < a.q;
-        uint32_t s = 0, t = 0, ans = 0;
-        bool bad = false, open = false;
-        uint64_t os = 0, ot = 0;
-        uint32_t ls = 0, lt = 0;
+        uint32_t ans = 0;
+        bool open = false;
         if (mine) {
-            open = !trivial_pair(a, a.src[qi * a.stride], a.dst[qi * a.stride], &s, &t, &ans, &bad);
+            OpenPair p;
+            bool bad = false;
+            open = !trivial_pair(a, a.src[qi * a.stride], a.dst[qi * a.stride], &p.s, &p.t, &ans, &bad);
             if (open) {
-                os = a.lab_off[s];
-                ot = a.lab_off[t];
-                ls = (uint32_t)(a.lab_off[s + 1] - os);
-                lt = (uint32_t)(a.lab_off[t + 1] - ot);
+                p.os = a.lab_off[p.s];
+                p.ot = a.lab_off[p.t];
+                p.ls = (uint32_t)(a.lab_off[p.s + 1] - p.os);
+                p.lt = (uint32_t)(a.lab_off[p.t + 1] - p.ot);
+                uint32_t d;
+                if (lone_pair(a, p.s, p.os, p.ls, p.t, p.ot, p.lt, &d)) {
+                    ans = answer_byte(a, d);
+                    open = false;
+                } else {
+                    pair[lane] = p;
+                }
             } else if (bad) {
                 atomicAdd(a.err + 1, 1ull);
             }
         }
+        __syncwarp();
         for (uint32_t m = __ballot_sync(FULL, open); m; m &= m - 1) {
             const int j = __ffs(m) - 1;
-            const uint32_t sj = __shfl_sync(FULL, s, j), tj = __shfl_sync(FULL, t, j);
-            const uint64_t osj = __shfl_sync(FULL, os, j), otj = __shfl_sync(FULL, ot, j);
-            const uint32_t lsj = __shfl_sync(FULL, ls, j), ltj = __shfl_sync(FULL, lt, j);
-            uint32_t td0, td1, dstar;
-            bp_tilde(a, sj, tj, lane, &td0, &td1, &dstar);
-            const uint32_t best = finish_pair(a, sj, tj, lane, td0, td1, dstar,
-                                              label_min_merge_at(a, sj, tj, osj, lsj, otj, ltj, lane));
+            const OpenPair p = pair[j];
+            const uint32_t best = pair_bounded(a, p, lane, keep);
             if (lane == j) ans = answer_byte(a, best);  // best is the same on every lane
         }
         // the group's answers in one coalesced store (the output may be host
         // memory that the GPU writes directly)
         if (mine) a.out[qi] = (uint8_t)ans;
+        __syncwarp();  // the next group writes pair
     }
 }
 
