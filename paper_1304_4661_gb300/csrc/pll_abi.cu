@@ -718,26 +718,38 @@ namespace {
 // temporary device copy of a host array, stream ordered
 using AsyncBuf = PoolMem;
 
-int query_status(const pll_index *ix, cudaStream_t s) {
-    // the two counters come back into pinned memory (a pageable target makes
-    // the copy a staged one); one buffer per thread: pll_query is synchronous,
-    // so a thread has one in flight at a time. It lives as long as the thread.
-    static thread_local unsigned long long *pinned = nullptr;
-    unsigned long long stack_h[2] = {0, 0};
-    if (!pinned && cudaMallocHost(&pinned, 16) != cudaSuccess) {
-        (void)cudaGetLastError();
-        pinned = nullptr;
+// status of a synchronous call's launch once the stream is waited for: from the
+// thread's counters, or (without them) from the index's own
+int query_status(const pll_index *ix, const unsigned long long *err, cudaStream_t s) {
+    if (err != ix->d_qerr) {
+        PLL_TRY(cudaStreamSynchronize(s));
+        return error_status(err);
     }
-    unsigned long long *h = pinned ? pinned : stack_h;
+    unsigned long long h[2] = {0, 0};
     PLL_TRY(cudaMemcpyAsync(h, ix->d_qerr, 16, cudaMemcpyDeviceToHost, s));
     PLL_TRY(cudaStreamSynchronize(s));
     if (h[0] == 0 && h[1] == 0) return PLL_OK;
     PLL_TRY(cudaMemsetAsync(ix->d_qerr, 0, 16, s));
     PLL_TRY(cudaStreamSynchronize(s));
-    return h[1] ? PLL_E_INVAL : PLL_E_RANGE;
+    return error_status(h);
+}
+
+unsigned long long *query_errors_of(const pll_index *ix) {
+    unsigned long long *e = thread_errors();
+    return e ? e : ix->d_qerr;
 }
 
 }  // namespace
+
+unsigned long long *thread_errors() {
+    static thread_local unsigned long long *pinned = nullptr;
+    if (!pinned && cudaMallocHost(&pinned, 32) != cudaSuccess) {
+        (void)cudaGetLastError();
+        pinned = nullptr;
+    }
+    if (pinned) pinned[0] = pinned[1] = 0;
+    return pinned;
+}
 
 void index_release(pll_index *ix) { free_index(ix); }
 
@@ -898,7 +910,7 @@ PLL_API int pll_query_async(const pll_index *idx, const uint32_t *src, const uin
     if (!idx) return PLL_E_INVAL;
     if (q == 0) return PLL_OK;
     if (!src || !dst || !out) return PLL_E_INVAL;
-    return query_launch(idx, src, dst, q, out, (cudaStream_t)stream);
+    return query_launch(idx, src, dst, q, out, idx->d_qerr, (cudaStream_t)stream);
 }
 
 PLL_API int pll_query_errors(const pll_index *idx, void *stream, uint64_t *count) {
@@ -918,8 +930,9 @@ PLL_API int pll_query(const pll_index *idx, const uint32_t *src, const uint32_t 
     if (q == 0) return PLL_OK;
     if (!src || !dst || !out) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    PLL_CHECK(query_launch(idx, src, dst, q, out, s));
-    return query_status(idx, s);
+    unsigned long long *err = query_errors_of(idx);
+    PLL_CHECK(query_launch(idx, src, dst, q, out, err, s));
+    return query_status(idx, err, s);
 }
 
 PLL_API int pll_query_host(const pll_index *idx, const uint32_t *src, const uint32_t *dst,
@@ -936,10 +949,11 @@ PLL_API int pll_query_host(const pll_index *idx, const uint32_t *src, const uint
         PLL_CHECK(dout.alloc(q));
         PLL_TRY(cudaMemcpyAsync(ds.p, src, q * 4, cudaMemcpyHostToDevice, s));
         PLL_TRY(cudaMemcpyAsync(dd.p, dst, q * 4, cudaMemcpyHostToDevice, s));
+        unsigned long long *err = query_errors_of(idx);
         PLL_CHECK(query_launch(idx, (const uint32_t *)ds.p, (const uint32_t *)dd.p, q,
-                               (uint8_t *)dout.p, s));
+                               (uint8_t *)dout.p, err, s));
         PLL_TRY(cudaMemcpyAsync(out, dout.p, q, cudaMemcpyDeviceToHost, s));
-        st = query_status(idx, s);
+        st = query_status(idx, err, s);
     }
     PLL_TRY(cudaStreamSynchronize(s));
     return st;

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) k_dquery(DQueryArgs a) {
         if (sid >= a.n || tid >= a.n) {
             if (lane == 0) {
                 a.out[qi] = INF8;
-                atomicAdd(a.err + 1, 1ull);
+                atomicAdd_system(a.err + 1, 1ull);
             }
             continue;
         }
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) k_dquery(DQueryArgs a) {
                 a.out[qi] = INF8;
             } else if (best >= INF8) {
                 a.out[qi] = INF8;
-                atomicAdd(a.err, 1ull);
+                atomicAdd_system(a.err, 1ull);
             } else {
                 a.out[qi] = (uint8_t)best;
             }
@@ -563,13 +563,19 @@ PLL_API int pll_dquery(const pll_dindex *idx, const uint32_t *src, const uint32_
     if (!src || !dst || !out) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
     DQueryArgs a{idx->n, idx->d_inv, idx->d_off[0], idx->d_off[1], idx->d_lab[0], idx->d_lab[1],
-                 src, dst, q, out, idx->d_qerr};
+                 src, dst, q, out, thread_errors()};
+    const bool own = a.err != nullptr;
+    if (!own) a.err = idx->d_qerr;
     int dev = 0, sms = 0;
     PLL_TRY(cudaGetDevice(&dev));
     PLL_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const uint64_t want = (q + 7) / 8, most = (uint64_t)(sms > 0 ? sms : 1) * 8;
     k_dquery<<<(unsigned)std::min(want, most), 256, 0, s>>>(a);
     PLL_TRY(cudaGetLastError());
+    if (own) {
+        PLL_TRY(cudaStreamSynchronize(s));
+        return error_status(a.err);
+    }
     unsigned long long h[2] = {0, 0};
     PLL_TRY(cudaMemcpyAsync(h, idx->d_qerr, 16, cudaMemcpyDeviceToHost, s));
     PLL_TRY(cudaStreamSynchronize(s));

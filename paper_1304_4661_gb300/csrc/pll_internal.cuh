@@ -397,10 +397,22 @@ int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_t
                     size_t *temp_bytes, cudaStream_t s, uint32_t round);
 
 // k_query.cu
+// err: two counters the launch adds its errors to (ix->d_qerr, or a
+// synchronous caller's own), [0] finite distances >= 255, [1] ids >= n
 int query_launch(const pll_index *ix, const uint32_t *d_src, const uint32_t *d_dst, uint64_t q,
-                 uint8_t *d_out, cudaStream_t s);
+                 uint8_t *d_out, unsigned long long *err, cudaStream_t s);
 // as query_launch with pair i at (d_src[i * stride], d_dst[i * stride])
 int query_launch_strided(const pll_index *ix, const uint32_t *d_src, const uint32_t *d_dst,
-                         uint32_t stride, uint64_t q, uint8_t *d_out, cudaStream_t s);
+                         uint32_t stride, uint64_t q, uint8_t *d_out, unsigned long long *err,
+                         cudaStream_t s);
+// The calling thread's own pair of error counters, zeroed (with room for two more
+// words behind them): pinned host memory
+// that kernels add to directly (only where there is an error), so that a
+// synchronous call needs no copy to learn its status, only its wait. Null if it
+// cannot be had. One in use at a time per thread; it lives as long as the thread.
+unsigned long long *thread_errors();
+inline int error_status(const unsigned long long *h) {
+    return h[1] ? PLL_E_INVAL : h[0] ? PLL_E_RANGE : PLL_OK;
+}
 
 }  // namespace pll

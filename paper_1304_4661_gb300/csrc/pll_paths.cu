@@ -19,19 +19,23 @@
 // taken here.
 //
 // Kernels: k_parents (a warp per vertex, lanes per label entry, each lane
-// binary-searching the labels of the vertex's neighbours), k_path_lengths and
-// k_paths (a warp per pair: lanes split the label join and the bit-parallel
-// slots; the two climbs run on lanes 0 and 1; bit-parallel walks scan 32
-// neighbours per step and take the first by ballot).
+// binary-searching the labels of the vertex's neighbours); path lengths come
+// from the distance query; k_paths (a warp for up to 32 pairs: ranks, offsets and
+// lone pairs on the lanes, the witnesses of the others one by one by the whole
+// warp, then all climbs, a lane each, and all bit-parallel walks, eight lanes
+// each, side by side).
 #include <algorithm>
 #include <new>
 #include <vector>
 
 #include <cub/device/device_scan.cuh>
+#include <thrust/iterator/counting_iterator.h>
+#include <thrust/iterator/transform_iterator.h>
 
-#include "pll_internal.cuh"
+#include "pair_device.cuh"
 
 using namespace pll;
+using namespace pll::pairs;
 
 // Shortest-path support over a built index (borrowed: it must outlive this).
 struct pll_paths {
@@ -43,9 +47,8 @@ struct pll_paths {
 
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
-constexpr uint32_t BIG = 1u << 20;
 constexpr uint64_t NOPOS = ~0ull;
+constexpr int PATH_BLOCKS = 8;  // of k_paths on an SM
 
 // error bits of the path kernels
 enum : uint32_t {
@@ -103,27 +106,14 @@ __global__ void __launch_bounds__(256) k_parents(ParentArgs a) {
 }
 
 struct PathArgs {
-    uint32_t n, t, tp;
-    const uint32_t *inv, *order, *graph;
-    const uint8_t *bp_d;
-    const uint64_t *bp_m;
-    const uint64_t *lab_off;
-    const uint32_t *lab, *par;
+    QueryArgs x;               // the index and the pairs
+    const uint32_t *order, *par;
     const uint32_t *roff, *rcol;
-    const uint32_t *src, *dst;
-    uint64_t q;
-    uint64_t *len;             // k_path_lengths: vertices of each path
-    const uint64_t *path_off;  // k_paths: slot of pair i is [path_off[i], path_off[i + 1])
+    const uint64_t *path_off;  // slot of pair i is [path_off[i], path_off[i + 1])
     uint64_t cap;
     uint32_t *path;
     uint32_t *err;
 };
-
-__device__ __forceinline__ uint32_t warp_min(uint32_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(FULL, v, o));
-    return v;
-}
 
 __device__ __forceinline__ uint64_t warp_min64(uint64_t v) {
 #pragma unroll
@@ -137,12 +127,10 @@ __device__ __forceinline__ uint64_t warp_min64(uint64_t v) {
 // The common hub of L(s) and L(t) with the least distance sum (lowest rank
 // among equals), as (sum << 32) | (hub << 8) | d(hub, s); NOPOS if none.
 // Lanes take entries of the shorter label and binary-search the longer.
-__device__ __forceinline__ uint64_t best_hub(const PathArgs &a, uint32_t s, uint32_t t, int lane) {
-    const uint64_t os = a.lab_off[s], ot = a.lab_off[t];
-    const uint32_t ls = (uint32_t)(a.lab_off[s + 1] - os), lt = (uint32_t)(a.lab_off[t + 1] - ot);
-    const bool sa = ls <= lt;
-    const uint32_t *A = a.lab + (sa ? os : ot), *B = a.lab + (sa ? ot : os);
-    const uint32_t la = sa ? ls : lt, lb = sa ? lt : ls;
+__device__ __forceinline__ uint64_t best_hub(const QueryArgs &a, const OpenPair &p, int lane) {
+    const bool sa = p.ls <= p.lt;
+    const uint32_t *A = a.lab + (sa ? p.os : p.ot), *B = a.lab + (sa ? p.ot : p.os);
+    const uint32_t la = sa ? p.ls : p.lt, lb = sa ? p.lt : p.ls;
     uint64_t best = NOPOS;
     for (uint32_t j = lane; j < la; j += 32) {
         const uint32_t ea = A[j], h = entry_hub(ea);
@@ -160,54 +148,88 @@ __device__ __forceinline__ uint64_t best_hub(const PathArgs &a, uint32_t s, uint
     return warp_min64(best);
 }
 
-// The bit-parallel slot with the least distance (lowest slot among equals) as
-// (distance << 16) | (slot << 8) | (kind << 6) | bit: kind 0 meets in
-// S^{-1} of both ends (d~ - 2), kind 1 in S^{-1} of one and S^0 of the other
-// (d~ - 1), kind 2 at r_i (d~); bit = the lowest member where they meet.
-// NONE if no slot reaches both.
-__device__ __forceinline__ uint32_t best_bp(const PathArgs &a, uint32_t s, uint32_t t, int lane) {
-    uint32_t best = NONE;
-    for (uint32_t i = lane; i < a.t; i += 32) {
-        const uint32_t x = a.bp_d[(size_t)s * a.tp + i], y = a.bp_d[(size_t)t * a.tp + i];
-        if (x == INF8 || y == INF8) continue;
-        const uint64_t *ms = a.bp_m + 2 * ((size_t)s * a.t + i);
-        const uint64_t *mt = a.bp_m + 2 * ((size_t)t * a.t + i);
-        const uint64_t s1 = ms[0], s0 = ms[1], t1 = mt[0], t0 = mt[1];
-        uint32_t val = x + y, kind = 2, bit = 0;
-        if (s1 & t1) {
-            val -= 2; kind = 0; bit = __ffsll((long long)(s1 & t1)) - 1;
-        } else if ((s1 & t0) | (s0 & t1)) {
-            val -= 1; kind = 1; bit = __ffsll((long long)((s1 & t0) | (s0 & t1))) - 1;
+// The common hub with the least distance sum if that is at most ub (a key of
+// best_hub's, or a larger one), from the near entries of both labels as in
+// pair_bounded; hubs that only reach ub count here, so entries up to ub - 1 do.
+constexpr uint32_t PATH_KEEP = 64;
+__device__ __forceinline__ uint64_t near_hub(const QueryArgs &a, const OpenPair &p, uint32_t ub, int lane,
+                                             uint32_t *keep) {
+    const bool low = p.s < p.t;  // h = s, v = t
+    const uint32_t h = low ? p.s : p.t, v = low ? p.t : p.s, lh = low ? p.ls : p.lt, lv = low ? p.lt : p.ls;
+    if (max(lh, lv) > LONG_LABEL && max(lh, lv) > PLL_MERGE_RATIO * min(lh, lv)) return best_hub(a, p, lane);
+    uint32_t direct = BIG;
+    const uint32_t cv = keep_near<PATH_KEEP>(a.lab + (low ? p.ot : p.os), lv, v, ub + 1, h, lane, keep, &direct);
+    if (cv > PATH_KEEP) return best_hub(a, p, lane);
+    direct = warp_min(direct);
+    uint64_t best = direct < BIG ? ((uint64_t)direct << 32) | ((uint64_t)h << 8) | (low ? 0u : direct) : NOPOS;
+    if (cv == 0) return best;
+    __syncwarp();
+    const uint32_t e0 = (uint32_t)lane < cv ? keep[lane] : NONE, e1 = lane + 32u < cv ? keep[lane + 32] : NONE;
+    __syncwarp();
+    const uint32_t ch = keep_near<PATH_KEEP>(a.lab + (low ? p.os : p.ot), lh, h, ub + 1, NONE, lane, keep, &direct);
+    if (ch > PATH_KEEP) return best_hub(a, p, lane);
+    __syncwarp();
+    for (uint32_t i = 0; i < ch; ++i) {
+        const uint32_t f = keep[i];
+        if (entry_hub(f) == entry_hub(e0) || entry_hub(f) == entry_hub(e1)) {
+            const uint32_t e = entry_hub(f) == entry_hub(e0) ? e0 : e1;
+            const uint64_t key = ((uint64_t)(entry_dist(e) + entry_dist(f)) << 32) | ((uint64_t)entry_hub(f) << 8) |
+                                 (low ? entry_dist(f) : entry_dist(e));
+            best = key < best ? key : best;
         }
-        best = min(best, (val << 16) | (i << 8) | (kind << 6) | bit);
+    }
+    __syncwarp();  // the next pair writes keep
+    return warp_min64(best);
+}
+
+// The lowest bit-parallel slot that gives the bit-parallel distance ub, as
+// (slot << 8) | (kind << 6) | bit: kind 0 meets in S^{-1} of both ends (d~ - 2),
+// kind 1 in S^{-1} of one and S^0 of the other (d~ - 1), kind 2 at r_i (d~); bit
+// = the lowest member where they meet. No slot gives less than ub, so a slot
+// with d~ = ub meets at r_i, one with d~ = ub + 1 or ub + 2 reaches ub only by
+// the matching reduction.
+__device__ __forceinline__ uint32_t bp_slot(const QueryArgs &a, uint32_t s, uint32_t t, uint32_t ub, uint32_t td0,
+                                            uint32_t td1, int lane) {
+    uint32_t best = NONE;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t td = h ? td1 : td0, i = lane + 32 * h;
+        if (td == ub) {
+            best = min(best, i << 8 | 2u << 6);
+        } else if (td == ub + 1 || td == ub + 2) {
+            const ulonglong2 ms = reinterpret_cast<const ulonglong2 *>(a.bp_m)[(size_t)s * a.t + i];
+            const ulonglong2 mt = reinterpret_cast<const ulonglong2 *>(a.bp_m)[(size_t)t * a.t + i];
+            const uint64_t meet = td == ub + 2 ? ms.x & mt.x : (ms.x & mt.y) | (ms.y & mt.x);
+            if (meet) best = min(best, i << 8 | (td == ub + 2 ? 0u : 1u << 6) | (uint32_t)(__ffsll((long long)meet) - 1));
+        }
     }
     return warp_min(best);
 }
 
-// d(s, t) of two distinct vertices of one graph (BIG if unreachable), with
-// its witnesses: hk from best_hub, bk from best_bp.
+// How a pair's path runs: through hub `at` (by >= 0: `by` from s), or through
+// the bit-parallel vertex at = bp_slot's value (by < 0). d = BIG: there is none.
 struct Witness {
-    uint64_t hk;
-    uint32_t bk, d;
+    uint32_t d, at;
+    int by;
 };
-__device__ __forceinline__ Witness pair_witness(const PathArgs &a, uint32_t s, uint32_t t, int lane) {
-    Witness w;
-    w.hk = best_hub(a, s, t, lane);
-    w.bk = best_bp(a, s, t, lane);
-    const uint32_t dn = w.hk == NOPOS ? BIG : (uint32_t)(w.hk >> 32);
-    const uint32_t db = w.bk == NONE ? BIG : (w.bk >> 16);
-    w.d = min(dn, db);
-    return w;
+__device__ __forceinline__ Witness pair_witness(const QueryArgs &a, const OpenPair &p, int lane, uint32_t *keep) {
+    uint32_t td0 = BIG, td1 = BIG, dstar = BIG;
+    if (a.t) bp_tilde(a, p.s, p.t, lane, &td0, &td1, &dstar);
+    const uint32_t ub = finish_pair(a, p.s, p.t, lane, td0, td1, dstar, BIG);
+    const uint64_t hk = ub < BIG ? near_hub(a, p, ub, lane, keep) : best_hub(a, p, lane);
+    const uint32_t dn = hk == NOPOS ? BIG : (uint32_t)(hk >> 32);
+    if (dn <= ub) return Witness{dn, (uint32_t)(hk >> 8) & 0xffffffu, (int)((uint32_t)hk & 0xffu)};
+    return Witness{ub, bp_slot(a, p.s, p.t, ub, td0, td1, lane), -1};
 }
 
 // Distance from the bit-parallel vertex of slot i (r_i for kind 2, else member
 // `bit` of S_{r_i}) to v; BIG if unreachable.
 __device__ __forceinline__ uint32_t bp_dist_to(const PathArgs &a, uint32_t i, uint32_t kind,
                                                uint32_t bit, uint32_t v) {
-    const uint32_t d = a.bp_d[(size_t)v * a.tp + i];
+    const uint32_t d = a.x.bp_d[(size_t)v * a.x.tp + i];
     if (d == INF8) return BIG;
     if (kind == 2) return d;
-    const uint64_t *m = a.bp_m + 2 * ((size_t)v * a.t + i);
+    const uint64_t *m = a.x.bp_m + 2 * ((size_t)v * a.x.t + i);
     const uint64_t b = 1ull << bit;
     if (m[0] & b) return d - 1;
     if (m[1] & b) return d;
@@ -215,24 +237,26 @@ __device__ __forceinline__ uint32_t bp_dist_to(const PathArgs &a, uint32_t i, ui
 }
 
 // Walks from v (at distance dv) down to the bit-parallel vertex, writing the
-// dv + 1 vertices at path[pos], path[pos + step], ... (lane 0 writes). Every
-// lane returns the same value: false if some vertex has no nearer neighbour.
+// dv + 1 vertices at path[pos], path[pos + step], ...; by the WALK lanes of
+// `group` (lane g of them), each step to the first neighbour one hop nearer.
+// Every lane returns the same value: false if some vertex has no nearer neighbour.
+constexpr int WALK = 8;  // 4 or 16 lanes: 3 % slower
 __device__ bool bp_walk(const PathArgs &a, uint32_t i, uint32_t kind, uint32_t bit, uint32_t v,
-                        uint32_t dv, int64_t pos, int step, int lane) {
-    if (lane == 0) a.path[pos] = a.order[v];
+                        uint32_t dv, int64_t pos, int step, unsigned group, int g) {
+    if (g == 0) a.path[pos] = a.order[v];
     while (dv > 0) {
         const uint32_t b = a.roff[v], e = a.roff[v + 1];
         uint32_t next = NONE;
-        for (uint32_t x = b; x < e; x += 32) {
-            const bool ok = x + lane < e && bp_dist_to(a, i, kind, bit, a.rcol[x + lane]) == dv - 1;
-            const unsigned m = __ballot_sync(FULL, ok);
-            if (m) { next = a.rcol[x + __ffs(m) - 1]; break; }
+        for (uint32_t x = b; x < e; x += WALK) {
+            const uint32_t w = x + g < e ? a.rcol[x + g] : NONE;
+            const unsigned m = __ballot_sync(group, w != NONE && bp_dist_to(a, i, kind, bit, w) == dv - 1) & group;
+            if (m) { next = __shfl_sync(group, w, __ffs(m) - 1); break; }
         }
         if (next == NONE) return false;
         v = next;
         --dv;
         pos += step;
-        if (lane == 0) a.path[pos] = a.order[v];
+        if (g == 0) a.path[pos] = a.order[v];
     }
     return true;
 }
@@ -243,119 +267,187 @@ __device__ bool climb(const PathArgs &a, uint32_t h, uint32_t v, uint32_t d, int
     for (uint32_t k = d;; --k) {
         a.path[pos] = a.order[v];
         if (k == 0) return v == h;
-        const uint64_t j = find_entry(a.lab, a.lab_off[v], a.lab_off[v + 1], pack_entry(h, k));
+        const uint64_t j = find_entry(a.x.lab, a.x.lab_off[v], a.x.lab_off[v + 1], pack_entry(h, k));
         if (j == NOPOS) return false;
         v = a.par[j];
-        if (v >= a.n) return false;
+        if (v >= a.x.n) return false;
         pos += step;
     }
 }
 
-// Vertices on the path of each pair: d + 1, 0 if unreachable (and for a bad
-// id or an out-of-range distance, which raise their error bits).
-__global__ void __launch_bounds__(256) k_path_lengths(PathArgs a) {
-    const int lane = threadIdx.x & 31;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t qi = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; qi < a.q; qi += warps) {
-        const uint32_t sid = a.src[qi], tid = a.dst[qi];
-        uint64_t len = 0;
-        if (sid >= a.n || tid >= a.n) {
-            if (lane == 0) atomicOr(a.err, PERR_ID);
-        } else {
-            const uint32_t s = a.inv[sid], t = a.inv[tid];
-            if (s == t) {
-                len = 1;
-            } else if (!a.graph || a.graph[s] == a.graph[t]) {
-                const uint32_t d = pair_witness(a, s, t, lane).d;
-                if (d < INF8) len = d + 1;
-                else if (d < BIG && lane == 0) atomicOr(a.err, PERR_RANGE);
-            }
-        }
-        if (lane == 0) a.len[qi] = len;
+// Vertices on pair i's path, from its distance byte: d + 1, 0 if unreachable (and
+// for a bad id or an out-of-range distance); 0 past the last pair.
+struct PathLength {
+    const uint8_t *dist;
+    uint64_t q;
+    __host__ __device__ uint64_t operator()(uint64_t i) const {
+        return i < q && dist[i] != INF8 ? (uint64_t)dist[i] + 1 : 0;
     }
-}
+};
 
 // One shortest path per pair into its slot; the rest of the slot (all of it
-// for an unreachable pair) is filled with NONE.
-__global__ void __launch_bounds__(256) k_paths(PathArgs a) {
-    const int lane = threadIdx.x & 31;
+// for an unreachable pair) is filled with NONE. A warp takes up to G pairs:
+// what each lane can settle about its own pair, then the witnesses of the open
+// ones one by one, then the climbs and walks of all of them side by side (two
+// ends each; a climb is a chain of dependent searches, and a walk's steps wait
+// for one another too). Bound by the latency of those chains: eight blocks an
+// SM (32 registers; five blocks of 47 registers 10 % slower). 1M uniform pairs of
+// R-MAT-20, t = 64, with the lengths: 2.90 ms with a warp per pair, binary
+// searches for every witness and the climbs on two lanes; 1.72 ms so, of which
+// (by leaving steps out) 0.6 ms is the witnesses, 0.5 the walks, 0.05 the climbs.
+__global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t G) {
+    __shared__ uint32_t s_keep[8][PATH_KEEP];
+    __shared__ OpenPair s_pair[8][32];
+    __shared__ Witness s_wit[8][32];
+    __shared__ uint64_t s_slot[8][32];
+    __shared__ uint8_t s_item[8][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    OpenPair *pair = s_pair[warp];
+    Witness *wit = s_wit[warp];
+    uint64_t *slot = s_slot[warp];
+    uint8_t *item = s_item[warp];
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t qi = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; qi < a.q; qi += warps) {
-        const uint64_t o0 = a.path_off[qi], o1 = a.path_off[qi + 1];
-        if (o1 < o0 || o1 > a.cap) {
-            if (lane == 0) atomicOr(a.err, PERR_SLOT);
-            continue;
-        }
-        const uint32_t sid = a.src[qi], tid = a.dst[qi];
-        uint64_t len = 0;
-        if (sid >= a.n || tid >= a.n) {
-            if (lane == 0) atomicOr(a.err, PERR_ID);
-        } else {
-            const uint32_t s = a.inv[sid], t = a.inv[tid];
-            if (s == t) {
-                if (o1 > o0) {
-                    if (lane == 0) a.path[o0] = sid;
-                    len = 1;
-                } else if (lane == 0) {
-                    atomicOr(a.err, PERR_SLOT);
-                }
-            } else if (!a.graph || a.graph[s] == a.graph[t]) {
-                const Witness w = pair_witness(a, s, t, lane);
-                const uint64_t hk = w.hk;
-                const uint32_t bk = w.bk, d = w.d;
-                if (d >= BIG) {
-                    // unreachable: an empty path
-                } else if (d >= INF8) {
-                    if (lane == 0) atomicOr(a.err, PERR_RANGE);
-                } else if (o1 - o0 < (uint64_t)d + 1) {
-                    if (lane == 0) atomicOr(a.err, PERR_SLOT);
-                } else {
-                    bool ok;
-                    const uint32_t dn = hk == NOPOS ? BIG : (uint32_t)(hk >> 32);
-                    if (dn == d) {  // a common hub: climb its tree from both ends
-                        const uint32_t h = (uint32_t)(hk >> 8) & 0xffffffu, ds = (uint32_t)hk & 0xffu;
-                        bool mine = true;
-                        if (lane == 0) mine = climb(a, h, s, ds, (int64_t)o0, 1);
-                        else if (lane == 1) mine = climb(a, h, t, d - ds, (int64_t)(o0 + d), -1);
-                        ok = __all_sync(FULL, mine);
-                    } else {        // through r_i or a member of S_{r_i}
-                        const uint32_t i = (bk >> 8) & 0xffu, kind = (bk >> 6) & 3u, bit = bk & 63u;
-                        const uint32_t ds = bp_dist_to(a, i, kind, bit, s), dt = bp_dist_to(a, i, kind, bit, t);
-                        ok = ds + dt == d && bp_walk(a, i, kind, bit, s, ds, (int64_t)o0, 1, lane) &&
-                             bp_walk(a, i, kind, bit, t, dt, (int64_t)(o0 + d), -1, lane);
+    for (uint64_t q0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * G; q0 < a.x.q; q0 += warps * G) {
+        const uint64_t qi = q0 + lane;
+        uint64_t o0 = 0, o1 = 0, len = 0;
+        bool open = false, routed = false;  // needs a witness; has one
+        if ((uint32_t)lane < G && qi < a.x.q) {
+            o0 = a.path_off[qi];
+            o1 = a.path_off[qi + 1];
+            if (o1 < o0 || o1 > a.cap) {
+                atomicOr_system(a.err, PERR_SLOT);
+                o1 = o0;  // nothing is written
+            } else {
+                OpenPair p;
+                uint32_t ans = 0;
+                bool bad = false;
+                const uint32_t sid = a.x.src[qi];
+                if (trivial_pair(a.x, sid, a.x.dst[qi], &p.s, &p.t, &ans, &bad)) {
+                    if (bad) {
+                        atomicOr_system(a.err, PERR_ID);
+                    } else if (ans == 0) {  // s = t
+                        if (o1 > o0) {
+                            a.path[o0] = sid;
+                            len = 1;
+                        } else {
+                            atomicOr_system(a.err, PERR_SLOT);
+                        }
                     }
-                    if (ok) len = (uint64_t)d + 1;
-                    else if (lane == 0) atomicOr(a.err, PERR_WALK);
+                } else {
+                    p.os = a.x.lab_off[p.s];
+                    p.ot = a.x.lab_off[p.t];
+                    p.ls = (uint32_t)(a.x.lab_off[p.s + 1] - p.os);
+                    p.lt = (uint32_t)(a.x.lab_off[p.t + 1] - p.ot);
+                    pair[lane] = p;
+                    uint32_t d, hub, ds;
+                    if (lone_pair(a.x, p.s, p.os, p.ls, p.t, p.ot, p.lt, &d, &hub, &ds)) {
+                        if (d < BIG) {
+                            wit[lane] = Witness{d, hub, (int)ds};
+                            routed = true;
+                        }
+                    } else {
+                        open = true;
+                    }
                 }
             }
         }
-        __syncwarp();  // the walk's writes come before the fill that may cover them
-        for (uint64_t x = o0 + len + lane; x < o1; x += 32) a.path[x] = NONE;
+        __syncwarp();
+        for (unsigned m = __ballot_sync(FULL, open); m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            const Witness w = pair_witness(a.x, pair[j], lane, s_keep[warp]);
+            if (lane == j) {
+                wit[j] = w;
+                routed = w.d < BIG;
+            }
+        }
+        bool climbs = false, walks = false;
+        if (routed) {
+            const Witness w = wit[lane];
+            if (w.d >= INF8) {
+                atomicOr_system(a.err, PERR_RANGE);
+            } else if (o1 - o0 < (uint64_t)w.d + 1) {
+                atomicOr_system(a.err, PERR_SLOT);
+            } else {
+                climbs = w.by >= 0;
+                walks = !climbs;
+                slot[lane] = o0;
+            }
+        }
+        __syncwarp();
+        // a common hub: climb its tree from both ends
+        uint32_t failed = 0;
+        unsigned m = __ballot_sync(FULL, climbs);
+        if (climbs) {
+            const int at = 2 * __popc(m & ((1u << lane) - 1u));
+            item[at] = (uint8_t)lane;
+            item[at + 1] = (uint8_t)(lane | 32);
+        }
+        __syncwarp();
+        for (int x = lane; x < 2 * __popc(m); x += 32) {
+            const int j = item[x] & 31;
+            const Witness w = wit[j];
+            const bool from_t = item[x] & 32;
+            const bool ok = from_t ? climb(a, w.at, pair[j].t, w.d - w.by, (int64_t)(slot[j] + w.d), -1)
+                                   : climb(a, w.at, pair[j].s, w.by, (int64_t)slot[j], 1);
+            if (!ok) failed |= 1u << j;
+        }
+        __syncwarp();
+        // through r_i or a member of S_{r_i}: walk to it from both ends
+        m = __ballot_sync(FULL, walks);
+        if (walks) {
+            const int at = 2 * __popc(m & ((1u << lane) - 1u));
+            item[at] = (uint8_t)lane;
+            item[at + 1] = (uint8_t)(lane | 32);
+        }
+        __syncwarp();
+        const unsigned group = ((1u << WALK) - 1u) << (lane & ~(WALK - 1));
+        for (int x = lane / WALK; x < 2 * __popc(m); x += 32 / WALK) {
+            const int j = item[x] & 31;
+            const Witness w = wit[j];
+            const bool from_t = item[x] & 32;
+            const uint32_t i = w.at >> 8, kind = (w.at >> 6) & 3u, bit = w.at & 63u;
+            const uint32_t ds = bp_dist_to(a, i, kind, bit, pair[j].s), dt = bp_dist_to(a, i, kind, bit, pair[j].t);
+            const bool ok = ds + dt == w.d &&
+                            (from_t ? bp_walk(a, i, kind, bit, pair[j].t, dt, (int64_t)(slot[j] + w.d), -1, group,
+                                              lane & (WALK - 1))
+                                    : bp_walk(a, i, kind, bit, pair[j].s, ds, (int64_t)slot[j], 1, group,
+                                              lane & (WALK - 1)));
+            if (!ok) failed |= 1u << j;
+        }
+        failed = __reduce_or_sync(FULL, failed);
+        if (climbs || walks) {
+            if ((failed >> lane) & 1) atomicOr_system(a.err, PERR_WALK);
+            else len = (uint64_t)wit[lane].d + 1;
+        }
+        __syncwarp();  // the walks' writes come before the fill that may cover them
+        for (m = __ballot_sync(FULL, o0 + len < o1); m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            const uint64_t b = __shfl_sync(FULL, o0 + len, j), e = __shfl_sync(FULL, o1, j);
+            for (uint64_t x = b + lane; x < e; x += 32) a.path[x] = NONE;
+        }
+        __syncwarp();  // the next group writes the shared arrays
     }
 }
 
-int warp_grid(uint64_t items, int *blocks) {
+int warp_grid(uint64_t items, int per_sm, int *blocks) {
     int dev = 0, sms = 0;
     PLL_TRY(cudaGetDevice(&dev));
     PLL_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const uint64_t want = (items + 7) / 8;  // 8 warps per block
-    const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * 8;
+    const uint64_t most = (uint64_t)(sms > 0 ? sms : 1) * per_sm;
     *blocks = (int)(want < most ? (want > 0 ? want : 1) : most);
     return PLL_OK;
 }
 
 // stream-ordered 4-byte error word, one per call
 struct ErrWord {
+    PoolMem m;
     uint32_t *p = nullptr;
     cudaStream_t s;
-    explicit ErrWord(cudaStream_t st) : s(st) {}
-    ~ErrWord() { if (p) cudaFreeAsync(p, s); }
+    explicit ErrWord(cudaStream_t st) : m(st), s(st) {}
     int alloc() {
-        if (cudaMallocAsync(reinterpret_cast<void **>(&p), 4, s) != cudaSuccess) {
-            p = nullptr;
-            (void)cudaGetLastError();
-            return PLL_E_NOMEM;
-        }
+        PLL_CHECK(m.alloc(4));
+        p = m.as<uint32_t>();
         PLL_TRY(cudaMemsetAsync(p, 0, 4, s));
         return PLL_OK;
     }
@@ -378,20 +470,6 @@ void paths_release(pll_paths *p) {
     dev_free(p->d_rcol);
     dev_free(p->d_par);
     delete p;
-}
-
-PathArgs path_args(const pll_paths *p, const uint32_t *src, const uint32_t *dst, uint64_t q,
-                   uint32_t *err) {
-    const pll_index *ix = p->ix;
-    PathArgs a{};
-    a.n = ix->n; a.t = ix->t; a.tp = ix->tp;
-    a.inv = ix->d_inv; a.order = ix->d_order; a.graph = ix->d_graph;
-    a.bp_d = ix->d_bp_d; a.bp_m = ix->d_bp_m;
-    a.lab_off = ix->d_lab_off; a.lab = ix->d_lab; a.par = p->d_par;
-    a.roff = p->d_roff; a.rcol = p->d_rcol;
-    a.src = src; a.dst = dst; a.q = q;
-    a.err = err;
-    return a;
 }
 
 }  // namespace
@@ -424,14 +502,14 @@ PLL_API int pll_paths_create(const pll_index *idx, const uint32_t *offsets, cons
     PLL_TRY(dev_malloc(&p->d_rcol, std::max<uint64_t>(nnz, 1) * 4));
     PLL_TRY(dev_malloc(&p->d_par, std::max<uint64_t>(idx->entries, 1) * 4));
     {
-        DevMem inv;  // relabel writes an inverse order; the index keeps its own
+        PoolMem inv(s);  // relabel writes an inverse order; the index keeps its own
         PLL_CHECK(inv.alloc(std::max<size_t>((size_t)n * 4, 4)));
         PLL_CHECK(prep_relabel(g, idx->d_order, inv.as<uint32_t>(), p->d_roff, p->d_rcol, s));
     }
     if (n > 0 && idx->entries > 0) {
         ParentArgs a{n, p->d_roff, p->d_rcol, idx->d_lab_off, idx->d_lab, p->d_par, err.p};
         int blocks = 0;
-        PLL_CHECK(warp_grid(n, &blocks));
+        PLL_CHECK(warp_grid(n, 8, &blocks));
         k_parents<<<blocks, 256, 0, s>>>(a);
         PLL_TRY(cudaGetLastError());
     }
@@ -471,27 +549,23 @@ PLL_API int pll_path_offsets(const pll_paths *p, const uint32_t *src, const uint
     if (q > 0 && (!src || !dst)) return PLL_E_INVAL;
     if (q >= 0x7fffffffull) return PLL_E_RANGE;
     cudaStream_t s = (cudaStream_t)stream;
-    ErrWord err(s);
-    PLL_CHECK(err.alloc());
-    DevMem len, temp;
-    PLL_CHECK(len.alloc((q + 1) * 8));
-    PLL_TRY(cudaMemsetAsync(len.p, 0, (q + 1) * 8, s));
-    if (q > 0) {
-        PathArgs a = path_args(p, src, dst, q, err.p);
-        a.len = len.as<uint64_t>();
-        int blocks = 0;
-        PLL_CHECK(warp_grid(q, &blocks));
-        k_path_lengths<<<blocks, 256, 0, s>>>(a);
-        PLL_TRY(cudaGetLastError());
-    }
+    // the pairs' distances, then one scan of the lengths they stand for; the
+    // errors and the total come back in the thread's pinned counters
+    unsigned long long *h = thread_errors();
+    if (!h) return PLL_E_NOMEM;
+    PoolMem dist(s), temp(s);
+    PLL_CHECK(dist.alloc(q));
+    PLL_CHECK(query_launch(p->ix, src, dst, q, dist.as<uint8_t>(), h, s));
+    auto lengths = thrust::make_transform_iterator(thrust::counting_iterator<uint64_t>(0),
+                                                   PathLength{dist.as<uint8_t>(), q});
     size_t tb = 0;
-    PLL_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, len.as<uint64_t>(), path_off, (int)(q + 1), s));
+    PLL_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, lengths, path_off, (int)(q + 1), s));
     PLL_CHECK(temp.alloc(tb));
-    PLL_TRY(cub::DeviceScan::ExclusiveSum(temp.p, tb, len.as<uint64_t>(), path_off, (int)(q + 1), s));
-    PLL_TRY(cudaMemcpyAsync(total, path_off + q, 8, cudaMemcpyDeviceToHost, s));
-    uint32_t h = 0;
-    PLL_CHECK(err.read(&h));  // synchronises: the scan is done before temp and len go
-    return path_status(h);
+    PLL_TRY(cub::DeviceScan::ExclusiveSum(temp.p, tb, lengths, path_off, (int)(q + 1), s));
+    PLL_TRY(cudaMemcpyAsync(h + 2, path_off + q, 8, cudaMemcpyDeviceToHost, s));
+    PLL_TRY(cudaStreamSynchronize(s));
+    *total = h[2];
+    return error_status(h);
 }
 
 PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32_t *dst, uint64_t q,
@@ -500,19 +574,24 @@ PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32
     if (q == 0) return PLL_OK;
     if (!src || !dst || !path_off || (cap > 0 && !path)) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    ErrWord err(s);
-    PLL_CHECK(err.alloc());
-    PathArgs a = path_args(p, src, dst, q, err.p);
+    unsigned long long *h = thread_errors();  // pinned: its first word takes the error bits
+    if (!h) return PLL_E_NOMEM;
+    PathArgs a{};
+    a.x = query_args(p->ix, src, dst, 1, q, nullptr, h);
+    a.order = p->ix->d_order; a.par = p->d_par;
+    a.roff = p->d_roff; a.rcol = p->d_rcol;
     a.path_off = path_off;
     a.cap = cap;
     a.path = path;
+    a.err = reinterpret_cast<uint32_t *>(h);
     int blocks = 0;
-    PLL_CHECK(warp_grid(q, &blocks));
-    k_paths<<<blocks, 256, 0, s>>>(a);
+    PLL_CHECK(warp_grid(q, PATH_BLOCKS, &blocks));
+    // pairs a warp takes at once: up to 32, fewer while warps would be left idle
+    const uint64_t per = q / ((uint64_t)blocks * 8);
+    k_paths<<<blocks, 256, 0, s>>>(a, per >= 32 ? 32u : per > 1 ? (uint32_t)per : 1u);
     PLL_TRY(cudaGetLastError());
-    uint32_t h = 0;
-    PLL_CHECK(err.read(&h));
-    return path_status(h);
+    PLL_TRY(cudaStreamSynchronize(s));
+    return path_status(*reinterpret_cast<const uint32_t *>(h));
 }
 
 PLL_API void pll_paths_free(pll_paths *p) { paths_release(p); }

@@ -195,7 +195,8 @@ int launch_run(pll_server *sv, const Run &r) {
     const Slot &sl = sv->slots[r.slot];
     const uint32_t *gp = sv->g_pairs + 2 * r.off;
     PLL_TRY(cudaEventRecord(sl.start, sl.stream));
-    PLL_CHECK(pll::query_launch_strided(sv->ix, gp, gp + 1, 2, r.pairs, sv->g_out + r.off, sl.stream));
+    PLL_CHECK(pll::query_launch_strided(sv->ix, gp, gp + 1, 2, r.pairs, sv->g_out + r.off,
+                                              sv->ix->d_qerr, sl.stream));
     PLL_TRY(cudaEventRecord(sl.done, sl.stream));
     return PLL_OK;
 }
