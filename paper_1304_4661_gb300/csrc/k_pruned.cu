@@ -52,8 +52,6 @@
 // Level boundaries live in a device descriptor advanced by a one-thread
 // kernel, so the host enqueues several levels ahead and reads back only to
 // learn that the frontier is empty; sweeps over an empty range return at once.
-#include <cub/cub.cuh>
-
 #include "bp_nibble.h"
 #include "pll_internal.cuh"
 
@@ -181,16 +179,21 @@ __global__ void k_batch_init(BatchArgs a) {
             atomicOr(&a.visited[(size_t)slot * a.NW + (k >> 5)], 1u << (k & 31));
         }
         append_slices(a, lane == 0, lane, k, k, 0);
-        const uint32_t len = a.lab_len[k];
+        const uint32_t len = a.lab_len[k], slots = ht_size(len);
         // root array T as a hash table of 2 x |L(v_k)| slots (very long labels,
         // and tables past the pool's end, are binary-searched instead; the host
         // grows the pool for the next batches)
-        const unsigned long long tb = a.ht_off[slot], te = a.ht_off[slot + 1];
-        if (te > a.ht_cap) {
-            if (lane == 0) atomicOr(&a.ctr->err, ERR_TABLE);
-        } else if (te > tb) {
+        unsigned long long tb = 0;
+        if (slots && lane == 0) tb = atomicAdd(&a.ctr->ht_top, (unsigned long long)slots);
+        tb = __shfl_sync(FULL, tb, 0);
+        const bool fits = slots && tb + slots <= a.ht_cap;
+        if (lane == 0) {
+            a.tab[slot] = make_uint2((uint32_t)(tb / HT_MIN), fits ? slots - 1 : NONE);
+            if (slots && !fits) atomicOr(&a.ctr->err, ERR_TABLE);
+        }
+        if (fits) {
             uint32_t *ht = a.ht + tb;
-            const uint32_t mask = (uint32_t)(te - tb) - 1;
+            const uint32_t mask = slots - 1;
             uint32_t *reach = a.reach + tb;
             const uint32_t lg = reach_lg(mask);
             const uint4 empty = make_uint4(HT_EMPTY, HT_EMPTY, HT_EMPTY, HT_EMPTY);
@@ -207,18 +210,6 @@ __global__ void k_batch_init(BatchArgs a) {
                 while (atomicCAS(&ht[s], HT_EMPTY, e) != HT_EMPTY) s = (s + 1) & mask;
             }
         }
-    }
-}
-
-// table sizes of the batch's roots (0 for bit-parallel vertices)
-__global__ void k_ht_sizes(BatchArgs a, unsigned long long *sizes) {
-    for (uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x; slot <= a.B; slot += gridDim.x * blockDim.x) {
-        uint32_t sz = 0;
-        if (slot < a.B) {
-            const uint32_t k = a.k0 + slot;
-            if (!a.inX[k]) sz = ht_size(a.lab_len[k]);
-        }
-        sizes[slot] = sz;
     }
 }
 
@@ -863,16 +854,18 @@ __device__ __forceinline__ bool quad_prunes(const BatchArgs &a, const TestWarp &
 __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long b, unsigned long long e,
                                           uint32_t level, TestWarp &tw, uint32_t &n_scan, uint32_t &n_mask) {
     const int lane = threadIdx.x & 31;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    // warp-uniform trip count: each warp takes 32 consecutive candidates
-    const unsigned long long span = ((e - b + 31) / 32) * 32;
-    for (unsigned long long i0 = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
-         i0 < span; i0 += stride) {
-        const uint32_t cnt = (uint32_t)((e - b - i0) < 32 ? (e - b - i0) : 32);
+    // each warp takes up to 32 consecutive candidates, fewer when the level has
+    // fewer than that for every warp (a warp tests them one root after another)
+    const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
+    const unsigned long long gw = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const unsigned long long total_c = e - b, per = (total_c + nwarps - 1) / nwarps;
+    const uint32_t G = per < 1 ? 1u : per < 32 ? (uint32_t)per : 32u;
+    for (unsigned long long i0 = gw * G; i0 < total_c; i0 += nwarps * G) {
+        const uint32_t cnt = total_c - i0 < G ? (uint32_t)(total_c - i0) : G;
         const bool valid = (uint32_t)lane < cnt;
         ulonglong2 mc = make_ulonglong2(0, 0);
-        uint32_t wlen = 0, klen = 0, slot = 0, w = 0, tmask = NONE;
-        unsigned long long woff = 0, tb = 0;
+        uint32_t wlen = 0, klen = 0, slot = 0, w = 0, tb = 0, tmask = NONE;
+        unsigned long long woff = 0;
         if (valid) {  // per-candidate metadata, loaded in parallel
             const uint64_t mine = __ldcg(a.cand + b + i0 + lane);
             mc = __ldcg(reinterpret_cast<const ulonglong2 *>(a.candc) + b + i0 + lane);
@@ -881,9 +874,9 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             wlen = a.vis_len[w];
             woff = a.vis_off[w];
             klen = a.lab_len[a.k0 + slot];
-            tb = a.ht_off[slot];
-            const unsigned long long te = a.ht_off[slot + 1];
-            if (te > tb && te <= a.ht_cap) tmask = (uint32_t)(te - tb) - 1;
+            const uint2 t = a.tab[slot];
+            tb = t.x;
+            tmask = t.y;
         }
         // ---- masks
         uint32_t pruned = 0;
@@ -919,7 +912,7 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             r.k = a.k0 + s0;
             r.klen = __shfl_sync(FULL, klen, j0);
             r.tmask = __shfl_sync(FULL, tmask, j0);
-            r.tb = __shfl_sync(FULL, tb, j0);
+            r.tb = (unsigned long long)__shfl_sync(FULL, tb, j0) * HT_MIN;
             r.lg = reach_lg(r.tmask);
             r.staged = r.tmask != NONE && __reduce_add_sync(FULL, in ? min(wlen, 0xffffu) : 0u) >= STAGE_ENTRIES;
             __syncwarp();  // the previous root's table has been read
@@ -1093,7 +1086,9 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs 
 // descriptor steps between sweeps (one thread)
 __device__ __forceinline__ void advance_desc(const BatchArgs &a, int phase) {
     LevelDesc *d = a.desc;
-    const unsigned long long cn = a.ctr->cand_n, on = a.ctr->out_n;
+    const unsigned long long cn = *(volatile unsigned long long *)&a.ctr->cand_n;
+    const unsigned long long on = *(volatile unsigned long long *)&a.ctr->out_n;
+    const unsigned long long sn = *(volatile unsigned long long *)&a.ctr->slice_n;
     if (phase == 0) {          // after init: level 0 = the roots
         d->lvl_b = 0;
         d->lvl_e = on < a.out_cap ? on : a.out_cap;
@@ -1101,7 +1096,7 @@ __device__ __forceinline__ void advance_desc(const BatchArgs &a, int phase) {
         d->level = 0;
         d->cand_b = 0;
         d->cand_e = 0;
-        d->slice_n = a.ctr->slice_n;
+        d->slice_n = sn;
         a.ctr->slice_n = 0;
         if (a.loop) a.loop->t_mark = global_ns();
     } else if (phase == 1) {   // after expand: candidates of level + 1
@@ -1111,18 +1106,18 @@ __device__ __forceinline__ void advance_desc(const BatchArgs &a, int phase) {
         d->lvl_b = d->lvl_e;
         d->lvl_e = on < a.out_cap ? on : a.out_cap;
         d->level += 1;
-        d->slice_n = a.ctr->slice_n;
+        d->slice_n = sn;
         a.ctr->slice_n = 0;
     }
 }
 
 __global__ void k_batch_advance(BatchArgs a, int phase) { advance_desc(a, phase); }
 
-// ---- the level loop as a CUDA graph: a while node whose body is expand,
-// advance(1), test, advance(2); the second advance sets the loop condition.
-// The kernels read the batch's arguments from device memory (the host writes
-// them before each launch of the graph), so one instantiated graph serves
-// every batch of a build.
+// ---- the level loop as a CUDA graph: a while node whose body is expand, then
+// test; the last block of each takes the step to the next phase, the second of
+// which sets the loop condition. The kernels read the batch's arguments from
+// device memory (the host writes them before each launch of the graph), so one
+// instantiated graph serves every batch of a build.
 // the batch's arguments, copied once per CTA from device memory into shared
 // memory (read there as cheaply as kernel parameters)
 __device__ __forceinline__ const BatchArgs &args_to_shared(const BatchArgs *ap, BatchArgs *sa) {
@@ -1134,43 +1129,55 @@ __device__ __forceinline__ const BatchArgs &args_to_shared(const BatchArgs *ap, 
     return *sa;
 }
 
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, EXPAND_TPS / BLOCK) k_batch_expand_g(const BatchArgs *__restrict__ ap) {
-    extern __shared__ uint4 s_dyn[];
-    __shared__ BatchArgs s_args;
-    const BatchArgs &a = args_to_shared(ap, &s_args);
-    uint32_t nexp = 0, nreach = 0;
-    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->slice_n, a.desc->level, expand_warp(s_dyn), nexp, nreach);
-    flush_work(a, 2, nexp, nreach);
-}
-
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test_g(const BatchArgs *__restrict__ ap) {
-    extern __shared__ uint4 s_dyn[];
-    __shared__ BatchArgs s_args;
-    const BatchArgs &a = args_to_shared(ap, &s_args);
-    uint32_t n_scan = 0, n_mask = 0;
-    test_body(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
-    flush_work(a, 0, n_scan, n_mask);
-}
-
-// phase 1 / 2 of advance_desc, plus the phases' wall times; phase 2 sets the
-// loop's condition: another level while the frontier is not empty and no
-// buffer overflowed and no depth reached 255
-__global__ void k_batch_advance_g(const BatchArgs *__restrict__ ap, int phase, cudaGraphConditionalHandle h) {
-    const BatchArgs &a = *ap;
-    advance_desc(a, phase);
+// The step after a sweep of the graph loop, by the block that finishes last (a
+// kernel of its own costs a launch gap, 2.5 us a step): phase 1 / 2 of
+// advance_desc, plus the phases' wall times; phase 2 sets the loop's condition:
+// another level while the frontier is not empty and no buffer overflowed and no
+// depth reached 255.
+__device__ __forceinline__ void last_block_step(const BatchArgs &a, int phase, cudaGraphConditionalHandle h) {
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     LoopState *ls = a.loop;
+    __threadfence();
+    if (atomicAdd(&ls->done, 1u) != gridDim.x - 1) return;
+    __threadfence();  // every block's appends are behind its arrival
+    ls->done = 0;
+    advance_desc(a, phase);
     const unsigned long long now = global_ns();
     if (phase == 1) {
         ls->ns_expand += now - ls->t_mark;
     } else {
         ls->ns_test += now - ls->t_mark;
         ls->levels += 1;
-        const bool more = a.desc->lvl_b < a.desc->lvl_e && !(a.ctr->err & (ERR_DEPTH | ERR_BUF));
+        const bool more = a.desc->lvl_b < a.desc->lvl_e &&
+                          !(*(volatile uint32_t *)&a.ctr->err & (ERR_DEPTH | ERR_BUF));
         cudaGraphSetConditional(h, more ? 1u : 0u);
     }
     ls->t_mark = now;
+}
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, EXPAND_TPS / BLOCK) k_batch_expand_g(const BatchArgs *__restrict__ ap,
+                                                                               cudaGraphConditionalHandle h) {
+    extern __shared__ uint4 s_dyn[];
+    __shared__ BatchArgs s_args;
+    const BatchArgs &a = args_to_shared(ap, &s_args);
+    uint32_t nexp = 0, nreach = 0;
+    expand_body(a, a.desc->lvl_b, a.desc->lvl_e, a.desc->slice_n, a.desc->level, expand_warp(s_dyn), nexp, nreach);
+    flush_work(a, 2, nexp, nreach);
+    last_block_step(a, 1, h);
+}
+
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK, TEST_TPS / BLOCK) k_batch_test_g(const BatchArgs *__restrict__ ap,
+                                                                           cudaGraphConditionalHandle h) {
+    extern __shared__ uint4 s_dyn[];
+    __shared__ BatchArgs s_args;
+    const BatchArgs &a = args_to_shared(ap, &s_args);
+    uint32_t n_scan = 0, n_mask = 0;
+    test_body(a, a.desc->cand_b, a.desc->cand_e, a.desc->level + 1, test_warp(s_dyn), n_scan, n_mask);
+    flush_work(a, 0, n_scan, n_mask);
+    last_block_step(a, 2, h);
 }
 
 }  // namespace
@@ -1207,22 +1214,7 @@ int batch_grid(uint32_t block, int *grid) {
     return PLL_OK;
 }
 
-size_t batch_init_temp_bytes(uint32_t bmax) {
-    size_t tb = 0;
-    cub::DeviceScan::ExclusiveSum(nullptr, tb, (unsigned long long *)nullptr,
-                                  (unsigned long long *)nullptr, (int)bmax + 1);
-    return tb;
-}
-
-// temp: CUB scratch of batch_init_temp_bytes(B) bytes followed by B + 1
-// 64-bit sizes
-int batch_init(const BatchArgs &a, void *temp, size_t temp_bytes, cudaStream_t s) {
-    unsigned long long *sizes = reinterpret_cast<unsigned long long *>(
-        static_cast<unsigned char *>(temp) + ((temp_bytes - ((size_t)a.B + 1) * 8) & ~(size_t)255));
-    const size_t cub_bytes = (size_t)((unsigned char *)sizes - (unsigned char *)temp);
-    k_ht_sizes<<<(int)((a.B + 256) / 256), 256, 0, s>>>(a, sizes);
-    size_t tb = cub_bytes;
-    PLL_TRY(cub::DeviceScan::ExclusiveSum(temp, tb, sizes, a.ht_off, (int)a.B + 1, s));
+int batch_init(const BatchArgs &a, cudaStream_t s) {
     const int g = (int)((a.B * 32ull + 255) / 256);
     k_batch_init<<<g > 0 ? g : 1, 256, 0, s>>>(a);
     k_batch_advance<<<1, 1, 0, s>>>(a, 0);
@@ -1342,37 +1334,19 @@ static int graph_build(const int *grid, const BatchArgs *d_args, cudaGraph_t *pg
     PLL_TRY(cudaGraphAddNode(&cnode, g, nullptr, nullptr, 0, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     const BatchArgs *ap = d_args;
-    int ph1 = 1, ph2 = 2;
-    void *a_exp[] = {&ap};
-    void *a_adv1[] = {&ap, &ph1, &h};
-    void *a_tst[] = {&ap};
-    void *a_adv2[] = {&ap, &ph2, &h};
+    void *args[] = {&ap, &h};
     cudaKernelNodeParams kp{};
-    cudaGraphNode_t n[4];
+    cudaGraphNode_t n[2];
     kp.func = reinterpret_cast<void *>(k_batch_expand_g<BLOCK>);
     kp.gridDim = dim3(grid[0]);
     kp.blockDim = dim3(BLOCK);
     kp.sharedMemBytes = (unsigned)expand_smem<BLOCK>();
-    kp.kernelParams = a_exp;
+    kp.kernelParams = args;
     PLL_TRY(cudaGraphAddKernelNode(&n[0], body, nullptr, 0, &kp));
-    kp.func = reinterpret_cast<void *>(k_batch_advance_g);
-    kp.gridDim = dim3(1);
-    kp.blockDim = dim3(1);
-    kp.sharedMemBytes = 0;
-    kp.kernelParams = a_adv1;
-    PLL_TRY(cudaGraphAddKernelNode(&n[1], body, &n[0], 1, &kp));
     kp.func = reinterpret_cast<void *>(k_batch_test_g<BLOCK>);
     kp.gridDim = dim3(grid[1]);
-    kp.blockDim = dim3(BLOCK);
     kp.sharedMemBytes = (unsigned)test_smem<BLOCK>();
-    kp.kernelParams = a_tst;
-    PLL_TRY(cudaGraphAddKernelNode(&n[2], body, &n[1], 1, &kp));
-    kp.func = reinterpret_cast<void *>(k_batch_advance_g);
-    kp.gridDim = dim3(1);
-    kp.blockDim = dim3(1);
-    kp.sharedMemBytes = 0;
-    kp.kernelParams = a_adv2;
-    PLL_TRY(cudaGraphAddKernelNode(&n[3], body, &n[2], 1, &kp));
+    PLL_TRY(cudaGraphAddKernelNode(&n[1], body, &n[0], 1, &kp));
     PLL_TRY(cudaGraphInstantiate(pexec, g, 0));
     *pg = g;
     guard.g = nullptr;

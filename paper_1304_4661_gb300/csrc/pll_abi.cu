@@ -162,7 +162,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     // visited bitmap, one row of ceil(n / 32) words per root slot; cleared once
     // here, then lazily after each batch (only the words the batch set)
     const uint32_t NW = (n + 31) / 32;
-    PoolMem m_vis(s), m_ht(s), m_htoff(s), m_itemp(s), m_cand(s), m_candc(s), m_out(s),
+    PoolMem m_vis(s), m_ht(s), m_tab(s), m_cand(s), m_candc(s), m_out(s),
         m_sorted(s), m_keep(s), m_temp(s);
     PLL_CHECK(m_vis.alloc((size_t)bmax * NW * 4));
     PLL_TRY(cudaMemsetAsync(m_vis.p, 0, (size_t)bmax * NW * 4, s));
@@ -179,9 +179,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     }
     uint64_t ht_cap = caps.ht ? caps.ht : std::max<uint64_t>((uint64_t)bmax * 2048, 1ull << 20);
     PLL_CHECK(m_ht.alloc(ht_cap * 4));
-    PLL_CHECK(m_htoff.alloc(((size_t)bmax + 1) * 8));
-    const size_t itemp_bytes = ((batch_init_temp_bytes(bmax) + 255) & ~(size_t)255) + ((size_t)bmax + 1) * 8 + 256;
-    PLL_CHECK(m_itemp.alloc(itemp_bytes));
+    PLL_CHECK(m_tab.alloc((size_t)bmax * 8));
     PoolMem m_reach(s);
     PLL_CHECK(m_reach.alloc(ht_cap * 4));
     uint64_t cand_cap = caps.cand ? caps.cand
@@ -310,7 +308,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.k0 = k0; a.B = k1 - k0; a.NW = NW;
         a.visited = m_vis.as<uint32_t>();
         a.ht = m_ht.as<uint32_t>();
-        a.ht_off = m_htoff.as<unsigned long long>();
+        a.tab = m_tab.as<uint2>();
         a.ht_cap = ht_cap;
         a.reach = m_reach.as<uint32_t>();
         a.cand = m_cand.as<uint64_t>(); a.candc = m_candc.as<uint64_t>(); a.cand_cap = cand_cap;
@@ -319,11 +317,10 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.ctr = d_ctr; a.desc = d_desc; a.loop = d_loop;
         PLL_TRY(cudaEventRecord(ev0, s));
         PLL_TRY(cudaMemsetAsync(d_ctr, 0, 16, s));  // cand_n, out_n
-        PLL_TRY(cudaMemsetAsync(&d_ctr->slice_n, 0, 12, s));  // slice_n, err
+        PLL_TRY(cudaMemsetAsync(&d_ctr->slice_n, 0, 20, s));  // slice_n, ht_top, err
         PLL_CHECK(batch_row_starts(n, k0, roff, rcol, m_rstart.as<uint32_t>(), grid[0], s));
-        PLL_CHECK(batch_init(a, m_itemp.p, itemp_bytes, s));
-        ix->stats.launches += 4;
-        ix->stats.cub_calls += 1;
+        PLL_CHECK(batch_init(a, s));
+        ix->stats.launches += 3;
         if (device_levels) {
             // every level of the batch in one launch; events around it
             PLL_TRY(cudaMemsetAsync(&d_loop->count, 0, 4, s));
@@ -383,10 +380,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         if (h->c.err & ERR_DEPTH) return PLL_E_RANGE;
         if (h->c.err & ERR_TABLE) {  // some root tables did not fit: those roots were
             // binary-searched (same answers); grow the pool for later batches
-            unsigned long long need = 0;
-            PLL_TRY(cudaMemcpyAsync(&need, m_htoff.as<unsigned long long>() + a.B, 8,
-                                    cudaMemcpyDeviceToHost, s));
-            PLL_TRY(cudaStreamSynchronize(s));
+            const uint64_t need = h->c.ht_top;
             ix->stats.table_fallbacks += 1;
             if (!caps.ht) {  // the test capacity keeps the pool small for the whole build
                 ht_cap = std::max<uint64_t>(need + need / 4, ht_cap * 2);
@@ -459,8 +453,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         ix->stats.ms_test = ls.ns_test * 1e-6;
         ix->stats.expand_launches = ls.levels;
         ix->stats.test_launches = ls.levels;
-        // the graph's body runs four kernels a level (expand, step, test, step)
-        if (graph_levels) ix->stats.launches += 4ull * ls.levels;
+        // the graph's body runs two kernels a level (expand, test)
+        if (graph_levels) ix->stats.launches += 2ull * ls.levels;
     }
     ix->stats.pruned_scanned = h->c.work[0];
     ix->stats.pruned_masks = h->c.work[1];

@@ -337,7 +337,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     // buffers shared by the directions (candidates, tables, the visited rows) or
     // one each (tuples and their sorted copy, needed together by the cleanup);
     // a batch that overflows one runs again with a larger one
-    PoolMem vis(s), ht(s), reach(s), htoff(s), itemp(s), cand(s), candc(s), slices(s), inX(s), keep(s), temp(s);
+    PoolMem vis(s), ht(s), reach(s), tab(s), cand(s), candc(s), slices(s), inX(s), keep(s), temp(s);
     PoolMem rstart[2] = {PoolMem(s), PoolMem(s)}, out[2] = {PoolMem(s), PoolMem(s)},
             sorted[2] = {PoolMem(s), PoolMem(s)};
     PLL_CHECK(vis.alloc((size_t)bmax * NW * 4));
@@ -347,9 +347,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     uint64_t ht_cap = std::max<uint64_t>((uint64_t)bmax * 1024, 1ull << 18);
     PLL_CHECK(ht.alloc(ht_cap * 4));
     PLL_CHECK(reach.alloc(ht_cap * 4));
-    PLL_CHECK(htoff.alloc(((size_t)bmax + 1) * 8));
-    const size_t itemp_bytes = ((batch_init_temp_bytes(bmax) + 255) & ~(size_t)255) + ((size_t)bmax + 1) * 8 + 256;
-    PLL_CHECK(itemp.alloc(itemp_bytes));
+    PLL_CHECK(tab.alloc((size_t)bmax * 8));
     const uint64_t slice_cap = std::min<uint64_t>(std::max<uint64_t>(ix->nnz, 1ull << 16), SLICE_CAP);
     PLL_CHECK(slices.alloc(slice_cap * 16));
     size_t free_b = 0, total_b = 0;
@@ -398,16 +396,16 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         a.vis_off = to.off; a.vis_len = to.len; a.vis_pool = to.pool;
         a.k0 = k0; a.B = B; a.NW = NW;
         a.visited = vis.as<uint32_t>();
-        a.ht = ht.as<uint32_t>(); a.ht_off = htoff.as<unsigned long long>(); a.ht_cap = ht_cap;
+        a.ht = ht.as<uint32_t>(); a.tab = tab.as<uint2>(); a.ht_cap = ht_cap;
         a.reach = reach.as<uint32_t>();
         a.cand = cand.as<uint64_t>(); a.candc = candc.as<uint64_t>(); a.cand_cap = cand_cap;
         a.out = out[dir].as<uint64_t>(); a.out_cap = out_cap;
         a.slices = slices.as<uint4>(); a.slice_cap = slice_cap;
         a.ctr = &d->c[dir]; a.desc = &d->d[dir]; a.loop = m_loop.as<LoopState>();
         PLL_TRY(cudaMemsetAsync(a.ctr, 0, 16, s));             // cand_n, out_n
-        PLL_TRY(cudaMemsetAsync(&a.ctr->slice_n, 0, 12, s));   // slice_n, err
+        PLL_TRY(cudaMemsetAsync(&a.ctr->slice_n, 0, 20, s));   // slice_n, ht_top, err
         if (cut) PLL_CHECK(batch_row_starts(n, k0, a.roff, a.rcol, rstart[dir].as<uint32_t>(), grid[0], s));
-        PLL_CHECK(batch_init(a, itemp.p, itemp_bytes, s));
+        PLL_CHECK(batch_init(a, s));
         PLL_TRY(cudaMemcpyAsync(m_args.p, &a, sizeof(BatchArgs), cudaMemcpyHostToDevice, s));
         PLL_TRY(cudaGraphLaunch(loop.e, s));
         return batch_clear(a, grid[0], s);
@@ -438,7 +436,8 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         PLL_CHECK(settle());
         const uint32_t err = h->d.c[0].err | h->d.c[1].err;
         if (err & ERR_TABLE) {  // those roots were binary-searched; grow for later batches
-            ht_cap *= 4;
+            const uint64_t need = std::max(h->d.c[0].ht_top, h->d.c[1].ht_top);
+            ht_cap = std::max<uint64_t>(need + need / 4, ht_cap * 2);
             PLL_CHECK(ht.alloc(ht_cap * 4));
             PLL_CHECK(reach.alloc(ht_cap * 4));
         }

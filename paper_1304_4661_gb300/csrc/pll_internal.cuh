@@ -276,6 +276,7 @@ struct BatchCounters {
     unsigned long long nkept;     // entries kept by the cleanup
     unsigned long long pool_top;  // label pool bump pointer
     unsigned long long slice_n;   // slices of the next level's long entries
+    unsigned long long ht_top;    // table pool bump pointer (reset per batch)
     uint32_t err;                 // errors of the batch's BFS (reset per batch)
     uint32_t err_post;            // errors of the appends (never reset)
 };
@@ -286,7 +287,8 @@ constexpr uint32_t ERR_TIMEOUT = 1u << 6;  // a grid barrier waited past its lim
 // the snapshots its last CTA takes; phase times summed over the build.
 struct LoopState {
     unsigned int count, gen;            // barrier arrivals, generation
-    unsigned int err, pad;              // snapshot of BatchCounters::err
+    unsigned int err;                   // snapshot of BatchCounters::err
+    unsigned int done;                  // graph loop: blocks done with the current sweep
     unsigned long long cand_n, out_n, slice_n;  // snapshots of the counts
     unsigned long long timeout_ns;      // longest barrier wait
     unsigned long long ns_expand, ns_test;  // phase wall times (block 0)
@@ -324,7 +326,8 @@ struct BatchArgs {
     uint32_t *visited;         // [B][NW] bitmap: row of root slot s holds one bit
                                // per vertex (the per-root visited set of Alg. 1)
     uint32_t *ht;              // pool of root label hash tables
-    unsigned long long *ht_off;  // [B + 1] table offsets in the pool (exclusive sums)
+    uint2 *tab;                // per root slot: its table's place in the pool (in units of
+                               // HT_MIN slots) and its slots - 1 (NONE: no table)
     unsigned long long ht_cap;   // pool capacity (entries)
     uint32_t *reach;           // reach tables: a root's at its hash table's offset (four
                                // bytes for each of its slots, the first REACH_MAX in use)
@@ -344,8 +347,7 @@ int batch_grid(uint32_t block, int *grid);  // grid[2]: expand, test
 // earlier (smaller) k0
 int batch_row_starts(uint32_t n, uint32_t k0, const uint32_t *roff, const uint32_t *rcol, uint32_t *rstart,
                      int grid, cudaStream_t s);
-int batch_init(const BatchArgs &a, void *temp, size_t temp_bytes, cudaStream_t s);
-size_t batch_init_temp_bytes(uint32_t bmax);
+int batch_init(const BatchArgs &a, cudaStream_t s);
 int batch_level(const BatchArgs &a, const int *grid, uint32_t block, cudaStream_t s,
                 cudaEvent_t *ev);
 // all levels of a batch in one cooperative launch (grid from
