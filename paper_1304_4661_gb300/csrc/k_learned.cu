@@ -823,7 +823,7 @@ PLL_API int pll_features(const uint32_t *offsets, const uint32_t *cols, uint32_t
         PLL_CHECK(m_roff.alloc(((size_t)n + 1) * 4));
         PLL_CHECK(m_rcol.alloc(std::max<uint64_t>(nnz, 1) * 4));
         PLL_CHECK(prep_relabel(g, m_order.as<uint32_t>(), m_inv.as<uint32_t>(), m_roff.as<uint32_t>(),
-                               m_rcol.as<uint32_t>(), s));
+                               m_rcol.as<uint32_t>(), nullptr, nullptr, s));
         PLL_CHECK(m_inX.alloc(n));
         PLL_TRY(cudaMemsetAsync(m_inX.p, 0, n, s));
         PLL_CHECK(m_root.alloc((size_t)t * 4));

@@ -102,17 +102,21 @@ __global__ void k_inverse_and_degree(uint32_t n, const uint32_t *__restrict__ or
     }
 }
 
-// One warp per rank r: rcol[roff[r] + j] = inv[col[off[v] + j]], v = order[r].
-__global__ void k_relabel(uint32_t n, const uint32_t *__restrict__ order,
-                          const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
-                          const uint32_t *__restrict__ inv, const uint32_t *__restrict__ roff,
-                          uint32_t *rcol) {
+// The arcs in rank order, one warp per rank r: from[roff[r] + j] = r, to[...] =
+// inv[col[off[v] + j]], v = order[r].
+__global__ void k_rank_arcs(uint32_t n, const uint32_t *__restrict__ order,
+                            const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
+                            const uint32_t *__restrict__ inv, const uint32_t *__restrict__ roff,
+                            uint32_t *from, uint32_t *to) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t r = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n; r += warps) {
         uint32_t v = order[r];
         uint32_t b = off[v], e = off[v + 1], o = roff[r];
-        for (uint32_t x = b + lane; x < e; x += 32) rcol[o + (x - b)] = inv[col[x]];
+        for (uint32_t x = b + lane; x < e; x += 32) {
+            from[o + (x - b)] = (uint32_t)r;
+            to[o + (x - b)] = inv[col[x]];
+        }
     }
 }
 
@@ -338,13 +342,36 @@ int prep_check_order(const Graph &g, const uint32_t *d_order, uint32_t *d_err, c
     return PLL_OK;
 }
 
+// Stable radix sort of the nnz arcs (keys, vals) by their keys, which are below
+// n; temp grows as needed. On return the Current() buffers hold them.
+static int sort_arcs(uint64_t nnz, uint32_t n, cub::DoubleBuffer<uint32_t> &keys, cub::DoubleBuffer<uint32_t> &vals,
+                     PoolMem &temp, cudaStream_t s) {
+    int bits = 1;
+    while (bits < 32 && ((n - 1) >> bits)) ++bits;
+    size_t tb = 0;
+    PLL_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tb, keys, vals, (int64_t)nnz, 0, bits, s));
+    if (tb > temp.bytes) PLL_CHECK(temp.alloc(tb));
+    PLL_TRY(cub::DeviceRadixSort::SortPairs(temp.p, tb, keys, vals, (int64_t)nnz, 0, bits, s));
+    return PLL_OK;
+}
+
+static int land(uint32_t *dst, const uint32_t *src, uint64_t count, cudaStream_t s) {
+    if (dst != src) PLL_TRY(cudaMemcpyAsync(dst, src, count * 4, cudaMemcpyDeviceToDevice, s));
+    return PLL_OK;
+}
+
+// The rank-space lists without a sort of each: the arcs listed by ascending rank
+// of one end, sorted stably by the other end, leave every list of that end
+// ascending. A radix sort of the arcs by as many bits as a rank has is three
+// passes over them; sorting list by list was held up by the hubs' lists.
+// Preparation of R-MAT-20 (31.4M arcs, long lists): 7.0 -> 3.8 ms.
 int prep_relabel(const Graph &g, const uint32_t *d_order, uint32_t *d_inv, uint32_t *d_roff,
-                 uint32_t *d_rcol, cudaStream_t s) {
+                 uint32_t *d_rcol, uint32_t *d_heads, uint32_t *d_tails, cudaStream_t s) {
     if (g.n == 0) {
         PLL_TRY(cudaMemsetAsync(d_roff, 0, 4, s));
         return PLL_OK;
     }
-    PoolMem rdeg(s), tmpcol(s), temp(s);
+    PoolMem rdeg(s), m_a(s), m_b(s), m_c(s), temp(s);
     PLL_CHECK(rdeg.alloc((size_t)g.n * 4));
     k_inverse_and_degree<<<grid_for(g.n, 256), 256, 0, s>>>(g.n, d_order, g.off, d_inv,
                                                             rdeg.as<uint32_t>());
@@ -359,16 +386,27 @@ int prep_relabel(const Graph &g, const uint32_t *d_order, uint32_t *d_inv, uint3
         PLL_TRY(cudaStreamSynchronize(s));
         return PLL_OK;
     }
-    PLL_CHECK(tmpcol.alloc(g.nnz * 4));
-    k_relabel<<<grid_for((uint64_t)g.n * 32, 256), 256, 0, s>>>(g.n, d_order, g.off, g.col, d_inv,
-                                                                d_roff, tmpcol.as<uint32_t>());
+    PLL_CHECK(m_a.alloc(g.nnz * 4));
+    PLL_CHECK(m_b.alloc(g.nnz * 4));
+    uint32_t *a = m_a.as<uint32_t>(), *b = m_b.as<uint32_t>();
+    if (!d_heads) {
+        PLL_CHECK(m_c.alloc(g.nnz * 4));
+        d_heads = m_c.as<uint32_t>();
+        d_tails = d_rcol;
+    }
+    k_rank_arcs<<<grid_for((uint64_t)g.n * 32, 256), 256, 0, s>>>(g.n, d_order, g.off, g.col, d_inv, d_roff, a, b);
     PLL_TRY(cudaGetLastError());
-    size_t tb2 = 0;
-    PLL_TRY(cub::DeviceSegmentedSort::SortKeys(nullptr, tb2, tmpcol.as<uint32_t>(), d_rcol,
-                                               (int64_t)g.nnz, (int64_t)g.n, d_roff, d_roff + 1, s));
-    if (tb2 > temp.bytes) PLL_CHECK(temp.alloc(tb2));
-    PLL_TRY(cub::DeviceSegmentedSort::SortKeys(temp.p, tb2, tmpcol.as<uint32_t>(), d_rcol,
-                                               (int64_t)g.nnz, (int64_t)g.n, d_roff, d_roff + 1, s));
+    cub::DoubleBuffer<uint32_t> heads(b, d_heads), tails(a, d_tails);
+    PLL_CHECK(sort_arcs(g.nnz, g.n, heads, tails, temp, s));
+    PLL_CHECK(land(d_tails, tails.Current(), g.nnz, s));
+    if (d_tails != d_rcol) {
+        // directed: those are the reverse lists; by tails they give the forward ones
+        PLL_CHECK(land(d_heads, heads.Current(), g.nnz, s));
+        PLL_CHECK(land(a, d_tails, g.nnz, s));
+        cub::DoubleBuffer<uint32_t> keys(a, b), vals(d_heads, d_rcol);
+        PLL_CHECK(sort_arcs(g.nnz, g.n, keys, vals, temp, s));
+        PLL_CHECK(land(d_rcol, vals.Current(), g.nnz, s));
+    }
     PLL_TRY(cudaStreamSynchronize(s));
     return PLL_OK;
 }

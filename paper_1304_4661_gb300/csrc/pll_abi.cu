@@ -575,7 +575,8 @@ int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t 
     PoolMem m_roff(s), m_rcol(s), m_inX(s);
     PLL_CHECK(m_roff.alloc(((size_t)n + 1) * 4));
     PLL_CHECK(m_rcol.alloc(std::max<uint64_t>(nnz, 1) * 4));
-    PLL_CHECK(prep_relabel(g, ix->d_order, ix->d_inv, m_roff.as<uint32_t>(), m_rcol.as<uint32_t>(), s));
+    PLL_CHECK(prep_relabel(g, ix->d_order, ix->d_inv, m_roff.as<uint32_t>(), m_rcol.as<uint32_t>(), nullptr,
+                           nullptr, s));
     PLL_CHECK(m_inX.alloc(std::max<size_t>(n, 1)));
     PLL_TRY(cudaMemsetAsync(m_inX.p, 0, std::max<size_t>(n, 1), s));
     const uint32_t t = o.t;

@@ -26,8 +26,8 @@
 // labels read from the other; so are sorting, cleanup (each direction's tuples
 // against the other's), compaction and the label store (k_labels.cu). The host
 // reads back once a batch. Kernels of their own: k_dvalidate (CSR checks),
-// k_dindeg / k_ddeg (in- plus out-degree for the Degree order), k_dcount_in /
-// k_dfill_in (the reverse CSR; a warp per vertex) and k_dquery (warp per pair).
+// k_dindeg / k_ddeg (in- plus out-degree for the Degree order and the reverse
+// lists' offsets; a warp per vertex) and k_dquery (warp per pair).
 // R-MAT-15, arcs one way or both (1.2M): 49.3 ms for the build and 1M queries
 // with a thread-serial merge of two labels per frontier entry, two read-backs a
 // level and batches of 1024; 14.3 ms so. What is left is launches: ten root
@@ -100,14 +100,6 @@ __global__ void k_dindeg(uint32_t n, const uint32_t *__restrict__ off, const uin
 __global__ void k_ddeg(uint32_t n, const uint32_t *__restrict__ off, uint32_t *deg) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
         deg[v] += off[v + 1] - off[v];
-}
-
-// the reverse CSR's columns, unsorted within a row
-__global__ void k_dfill_in(uint32_t n, const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
-                           uint32_t *cursor, uint32_t *icol) {
-    const uint32_t lane = threadIdx.x & 31, warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < n; u += warps)
-        for (uint32_t x = off[u] + lane, e = off[u + 1]; x < e; x += 32) icol[atomicAdd(&cursor[col[x]], 1u)] = u;
 }
 
 // ------------------------------------------------------------- query
@@ -233,17 +225,16 @@ int directed_prep(pll_dindex *ix, const uint32_t *off, const uint32_t *col, cons
     }
     PLL_CHECK(adj_off[0].alloc(((size_t)n + 1) * 4));
     PLL_CHECK(adj_col[0].alloc(std::max<uint64_t>(nnz, 1) * 4));
-    PLL_CHECK(prep_relabel(g, ix->d_order, ix->d_inv, adj_off[0].as<uint32_t>(), adj_col[0].as<uint32_t>(), s));
-    // reverse CSR: count, scan, scatter, then sort each row
     PLL_CHECK(adj_off[1].alloc(((size_t)n + 1) * 4));
     PLL_CHECK(adj_col[1].alloc(std::max<uint64_t>(nnz, 1) * 4));
-    PoolMem cnt(s), cursor(s), unsorted(s), temp(s);
+    PoolMem heads(s), cnt(s), temp(s);
+    PLL_CHECK(heads.alloc(std::max<uint64_t>(nnz, 1) * 4));
+    PLL_CHECK(prep_relabel(g, ix->d_order, ix->d_inv, adj_off[0].as<uint32_t>(), adj_col[0].as<uint32_t>(),
+                           heads.as<uint32_t>(), adj_col[1].as<uint32_t>(), s));
+    // the reverse lists' offsets: arcs into each rank, counted and scanned
     PLL_CHECK(cnt.alloc(((size_t)n + 1) * 4));
-    PLL_CHECK(cursor.alloc(((size_t)n + 1) * 4));
-    PLL_CHECK(unsorted.alloc(std::max<uint64_t>(nnz, 1) * 4));
     PLL_TRY(cudaMemsetAsync(cnt.p, 0, ((size_t)n + 1) * 4, s));
-    const uint32_t *ro = adj_off[0].as<uint32_t>(), *rc = adj_col[0].as<uint32_t>();
-    k_dindeg<<<warp_blocks, 256, 0, s>>>(n, ro, rc, cnt.as<uint32_t>());
+    k_dindeg<<<warp_blocks, 256, 0, s>>>(n, adj_off[0].as<uint32_t>(), adj_col[0].as<uint32_t>(), cnt.as<uint32_t>());
     PLL_TRY(cudaGetLastError());
     size_t tb = 0;
     PLL_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt.as<uint32_t>(), adj_off[1].as<uint32_t>(),
@@ -251,19 +242,6 @@ int directed_prep(pll_dindex *ix, const uint32_t *off, const uint32_t *col, cons
     PLL_CHECK(temp.alloc(tb));
     PLL_TRY(cub::DeviceScan::ExclusiveSum(temp.p, tb, cnt.as<uint32_t>(), adj_off[1].as<uint32_t>(),
                                           (int64_t)n + 1, s));
-    PLL_TRY(cudaMemcpyAsync(cursor.p, adj_off[1].p, ((size_t)n + 1) * 4, cudaMemcpyDeviceToDevice, s));
-    k_dfill_in<<<warp_blocks, 256, 0, s>>>(n, ro, rc, cursor.as<uint32_t>(), unsorted.as<uint32_t>());
-    PLL_TRY(cudaGetLastError());
-    if (nnz) {
-        size_t tb2 = 0;
-        PLL_TRY(cub::DeviceSegmentedSort::SortKeys(nullptr, tb2, unsorted.as<uint32_t>(), adj_col[1].as<uint32_t>(),
-                                                   (int64_t)nnz, (int64_t)n, adj_off[1].as<uint32_t>(),
-                                                   adj_off[1].as<uint32_t>() + 1, s));
-        if (tb2 > temp.bytes) PLL_CHECK(temp.alloc(tb2));
-        PLL_TRY(cub::DeviceSegmentedSort::SortKeys(temp.p, tb2, unsorted.as<uint32_t>(), adj_col[1].as<uint32_t>(),
-                                                   (int64_t)nnz, (int64_t)n, adj_off[1].as<uint32_t>(),
-                                                   adj_off[1].as<uint32_t>() + 1, s));
-    }
     return PLL_OK;
 }
 

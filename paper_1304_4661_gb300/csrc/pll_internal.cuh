@@ -215,8 +215,11 @@ struct Graph {
 int prep_validate_csr(const Graph &g, uint32_t *d_err, cudaStream_t s);
 int prep_degree_order(const Graph &g, uint32_t *d_order, cudaStream_t s);
 int prep_check_order(const Graph &g, const uint32_t *d_order, uint32_t *d_err, cudaStream_t s);
+// d_heads, d_tails: null for a symmetric graph. For a directed one d_tails receives
+// the reverse lists (the arcs' tails by head, ascending); d_heads is scratch (nnz
+// each).
 int prep_relabel(const Graph &g, const uint32_t *d_order, uint32_t *d_inv, uint32_t *d_roff,
-                 uint32_t *d_rcol, cudaStream_t s);
+                 uint32_t *d_rcol, uint32_t *d_heads, uint32_t *d_tails, cudaStream_t s);
 int prep_select_bp_roots(uint32_t n, uint32_t t, const uint32_t *d_roff, const uint32_t *d_rcol,
                          uint8_t *d_inX, uint32_t *d_root, uint32_t *d_cnt, uint32_t *d_S,
                          cudaStream_t s);

@@ -504,7 +504,7 @@ PLL_API int pll_paths_create(const pll_index *idx, const uint32_t *offsets, cons
     {
         PoolMem inv(s);  // relabel writes an inverse order; the index keeps its own
         PLL_CHECK(inv.alloc(std::max<size_t>((size_t)n * 4, 4)));
-        PLL_CHECK(prep_relabel(g, idx->d_order, inv.as<uint32_t>(), p->d_roff, p->d_rcol, s));
+        PLL_CHECK(prep_relabel(g, idx->d_order, inv.as<uint32_t>(), p->d_roff, p->d_rcol, nullptr, nullptr, s));
     }
     if (n > 0 && idx->entries > 0) {
         ParentArgs a{n, p->d_roff, p->d_rcol, idx->d_lab_off, idx->d_lab, p->d_par, err.p};

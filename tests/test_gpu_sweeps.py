@@ -11,7 +11,7 @@ from paper_1304_4661_gb300 import graphgen as gg
 from paper_1304_4661_gb300 import pll
 
 from . import graphs
-from .gpu_util import first_label_diff, gpu_build, same_labels
+from .gpu_util import dev_u32, first_label_diff, gpu_build, same_labels
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +88,14 @@ def test_directed_depths_next_to_the_limit(n, root_batch):
     ref = oracle.DirectedIndex(d.offsets, d.cols)
     ix = pll.DirectedIndex(dev_u32(d.offsets), dev_u32(d.cols), root_batch=root_batch)
     assert same_labels(ix.labels_in(), ref.labels_in()) and same_labels(ix.labels_out(), ref.labels_out())
+
+
+@pytest.mark.parametrize("n", [2, 256, 257, 65536, 65537])
+def test_rank_space_lists_at_the_sort_widths(n):
+    """The lists come from a radix sort over as many bits as a rank has: one, two and three passes."""
+    g = graphs.path(2) if n == 2 else gg.ba(n, 2, n)
+    check(g, 16)
+    d = gg.oriented(g, 3, both=0.3)
+    ix, ref = pll.DirectedIndex(dev_u32(d.offsets), dev_u32(d.cols)), oracle.DirectedIndex(d.offsets, d.cols)
+    for a, b in ((ix.labels_in(), ref.labels_in()), (ix.labels_out(), ref.labels_out())):
+        assert same_labels(a, b), first_label_diff(a, b, d.n)
