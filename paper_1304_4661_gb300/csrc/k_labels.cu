@@ -130,6 +130,67 @@ __global__ void k_append(LabelStore st, const uint64_t *__restrict__ K,
     }
 }
 
+// The near copy, one warp per vertex: the label's entries (whole quads of them)
+// counted by class, then dealt out; the lanes with the same class are found by
+// four ballots. Reads each label twice (the second time from L1) and writes it
+// once: all rebuilds of R-MAT-20 together add 1.1 ms to its build.
+constexpr int NEAR_THREADS = 256;
+__device__ __forceinline__ unsigned same_class(uint32_t q, bool on) {
+    unsigned m = __ballot_sync(0xffffffffu, on);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const unsigned bal = __ballot_sync(0xffffffffu, (q >> b) & 1);
+        m &= (q >> b) & 1 ? bal : ~bal;
+    }
+    return m;
+}
+__global__ void __launch_bounds__(NEAR_THREADS) k_near(LabelStore st) {
+    static_assert(NEAR_CLASSES == 15, "sixteen classes, four bits");
+    __shared__ uint32_t s_cnt[NEAR_THREADS / 32][16];
+    const int lane = threadIdx.x & 31;
+    uint32_t *cnt = s_cnt[threadIdx.x >> 5];
+    const unsigned below = (1u << lane) - 1;
+    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t v = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < st.n; v += warps) {
+        const uint32_t base = st.len[v] & ~3u;
+        const uint64_t off = st.off[v];
+        const uint32_t *src = st.pool + off;
+        if (lane < 16) cnt[lane] = 0;
+        __syncwarp();
+        for (uint32_t x = 0; x < base; x += 32) {
+            const bool on = x + lane < base;
+            const uint32_t q = on ? min(entry_dist(src[x + lane]), NEAR_CLASSES) : 0u;
+            const unsigned m = same_class(q, on);
+            if (on && !(m & below)) cnt[q] += __popc(m);
+            __syncwarp();
+        }
+        // cnt[q] becomes the class's start
+        uint32_t c = lane < 16 ? cnt[lane] : 0, incl = c;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane < 16) cnt[lane] = incl - c;
+        if (lane < (int)NEAR_CLASSES) st.near_end[(size_t)lane * st.n + v] = incl;
+        if (lane == 0) st.near_lab[v] = NearLabel{off, base, 0};
+        __syncwarp();
+        for (uint32_t x = 0; x < base; x += 32) {
+            const bool on = x + lane < base;
+            const uint32_t e = on ? src[x + lane] : 0u;
+            const uint32_t q = on ? min(entry_dist(e), NEAR_CLASSES) : 0u;
+            const unsigned m = same_class(q, on);
+            uint32_t at = on ? cnt[q] : 0;
+            __syncwarp();
+            if (on) {
+                st.near[off + at + __popc(m & below)] = e;
+                if (!(m & below)) cnt[q] = at + __popc(m);
+            }
+            __syncwarp();
+        }
+    }
+}
+
 // One warp per vertex: dst[doff[v] + j] = src[soff[v] + j], j < len[v].
 __global__ void k_gather_labels(uint32_t n, const uint64_t *__restrict__ soff,
                                 const uint32_t *__restrict__ len, const uint32_t *__restrict__ src,
@@ -215,6 +276,54 @@ int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_t
     PLL_TRY(cudaGetLastError());
     PLL_TRY(cub::DeviceScan::ExclusiveSum(d_temp, *temp_bytes, d_out, (int64_t)n, s));
     return PLL_OK;
+}
+
+// The near copy is rebuilt when the store has grown by a quarter since the last
+// time, so all rebuilds together rewrite five times the final labels (growth of
+// 10, 25, 50 %: builds of 129.6, 129.0, 128.7 ms on R-MAT-20, 156.0, 156.9, 158.0
+// on the batch of 96 graphs; keeping every label in order on each append instead
+// costs 33 and 41 ms more in the append). A store of fewer than NEAR_MIN entries
+// has none: builds that small are launches (BA-10k, R-MAT-15 both ways: no
+// difference with a line at 65536 or none). It doubles the store's memory: it is
+// kept up while it takes at most an eighth of the memory that is free (an older
+// copy stays good, and without one the test sweep reads whole labels).
+constexpr uint64_t NEAR_MIN = 1 << 18, NEAR_GROWTH_PCT = 25;
+int labels_near(LabelStore &st, uint64_t total, cudaStream_t s) {
+    if (total < NEAR_MIN || total < st.near_total + st.near_total / 100 * NEAR_GROWTH_PCT) return PLL_OK;
+    if (st.near_cap < st.pool_cap) {
+        const uint64_t per_vertex = (uint64_t)st.n * (sizeof(NearLabel) + NEAR_CLASSES * 4);
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return PLL_OK;
+        }
+        if (st.pool_cap * 4 + per_vertex > free_b / 8) return PLL_OK;
+        pool_free(st.near, s);
+        st.near = nullptr;
+        PoolMem near(s), lab(s), end(s);
+        PLL_CHECK(near.alloc(st.pool_cap * 4));
+        if (!st.near_lab) {
+            PLL_CHECK(lab.alloc((size_t)st.n * sizeof(NearLabel)));
+            PLL_CHECK(end.alloc((size_t)st.n * NEAR_CLASSES * 4));
+            st.near_lab = static_cast<NearLabel *>(lab.release());
+            st.near_end = static_cast<uint32_t *>(end.release());
+        }
+        st.near = static_cast<uint32_t *>(near.release());
+        st.near_cap = st.pool_cap;
+    }
+    k_near<<<grid_for((uint64_t)st.n * 32, NEAR_THREADS), NEAR_THREADS, 0, s>>>(st);
+    PLL_TRY(cudaGetLastError());
+    st.near_total = total;
+    return PLL_OK;
+}
+
+void labels_near_free(LabelStore &st, cudaStream_t s) {
+    pool_free(st.near, s);
+    pool_free(st.near_lab, s);
+    pool_free(st.near_end, s);
+    st.near = nullptr;
+    st.near_lab = nullptr;
+    st.near_end = nullptr;
 }
 
 // Rewrites the pool (capacity = length rounded up to 4 entries, so arrays

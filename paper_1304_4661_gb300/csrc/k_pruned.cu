@@ -741,8 +741,10 @@ __global__ void k_batch_clear(BatchArgs a) {
 //           of entries laid end to end over the lanes (a quad's candidate found
 //           by a binary search over a warp scan of the lengths). An entry at
 //           distance d >= level can prune nothing (every hub is at least 1 from
-//           the root), which settles 95 of 100 entries on power-law graphs and
-//           6 of 10 on the high-diameter ones without a look at the table; an
+//           the root): 95 of 100 entries on power-law graphs and 6 of 10 on the
+//           high-diameter ones, most of which are not even read (the labels are
+//           read from their near copy, k_labels.cu, up to distance level - 1,
+//           and from the store past what the copy holds); an
 //           entry that the table lets through is looked up in the root's hash
 //           table T (or, without one, by a binary search of L(v_k)), and
 //           d + T[h] <= level prunes the candidate. A candidate found pruned
@@ -754,7 +756,8 @@ __global__ void k_batch_clear(BatchArgs a) {
 // candidate): 325 ms with every entry probed in the hash table (gathers from
 // L2), 124 ms with the reach tables and single entries on the lanes, 106.6 ms
 // with quads. R-MAT-20 (t = 64; 7.8G entries, 0.4G nearer): 65.9, 47.0, 43.3
-// ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
+// ms; with the near copy, which leaves the near entries and those of the last
+// batches (16G and 1.05G), 68.9 and 32.8 ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
 // reach table (fewer false hits): 108 ms.
 // candidates whose labels have at least this many entries are scanned one by
 // one by the whole warp (no owner search per entry, and an exit at the first
@@ -767,9 +770,19 @@ constexpr uint32_t LONG_LABEL = LONG_LABEL_ENTRIES;
 // any line from 1 to 500, 141 ms without staging; R-MAT-20's 47 to 48 ms)
 constexpr uint32_t STAGE_ENTRIES = PLL_STAGE_ENTRIES;
 
+// Where the label entries of a candidate lie that a test reads: the near copy's
+// entries of distance < level, then those appended since its last rebuild (all
+// of them without a near copy).
+struct Spans {
+    const uint32_t *near, *rest;
+    uint32_t near_n, rest_n;  // entries
+    uint32_t first, near_q;   // the candidate's first quad of those laid end to end; near_n in quads
+};
+
 // What a warp of the test sweep keeps in shared memory.
 struct TestWarp {
     uint4 reach[REACH_MAX / 16];  // the staged table of the root at hand
+    Spans spans[32];              // the candidates' labels
 };
 
 // The root whose candidates are at hand (the same on every lane).
@@ -818,6 +831,10 @@ __device__ __forceinline__ Quad load_quad(const uint32_t *lab, uint32_t q, uint3
     }
     return r;
 }
+// quad q of a candidate's spans
+__device__ __forceinline__ Quad span_quad(const Spans &sp, uint32_t q) {
+    return q < sp.near_q ? load_quad(sp.near, q, sp.near_n) : load_quad(sp.rest, q - sp.near_q, sp.rest_n);
+}
 __device__ __forceinline__ bool quad_prunes(const BatchArgs &a, const TestWarp &tw, const TestRoot &r, const Quad &q,
                                             uint32_t level) {
     const int8_t *sh = reinterpret_cast<const int8_t *>(tw.reach);
@@ -864,15 +881,25 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
         const uint32_t cnt = total_c - i0 < G ? (uint32_t)(total_c - i0) : G;
         const bool valid = (uint32_t)lane < cnt;
         ulonglong2 mc = make_ulonglong2(0, 0);
-        uint32_t wlen = 0, klen = 0, slot = 0, w = 0, tb = 0, tmask = NONE;
-        unsigned long long woff = 0;
+        uint32_t wlen = 0, klen = 0, slot = 0, w = 0, tb = 0, tmask = NONE, wquads = 0;
+        __syncwarp();  // the previous candidates' spans have been read
         if (valid) {  // per-candidate metadata, loaded in parallel
             const uint64_t mine = __ldcg(a.cand + b + i0 + lane);
             mc = __ldcg(reinterpret_cast<const ulonglong2 *>(a.candc) + b + i0 + lane);
             w = (uint32_t)mine;
             slot = (uint32_t)(mine >> 32);
-            wlen = a.vis_len[w];
-            woff = a.vis_off[w];
+            Spans sp{nullptr, a.vis_pool + a.vis_off[w], 0, a.vis_len[w], 0, 0};
+            if (a.near) {
+                const NearLabel nl = a.near_lab[w];
+                sp.near = a.near + nl.off;
+                sp.near_n = level <= NEAR_CLASSES ? a.near_end[(size_t)(level - 1) * a.n + w] : nl.base;
+                sp.near_q = (sp.near_n + 3) / 4;
+                sp.rest += nl.base;
+                sp.rest_n -= nl.base;
+            }
+            wlen = sp.near_n + sp.rest_n;
+            wquads = sp.near_q + (sp.rest_n + 3) / 4;
+            tw.spans[lane] = sp;
             klen = a.lab_len[a.k0 + slot];
             const uint2 t = a.tab[slot];
             tb = t.x;
@@ -924,20 +951,21 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             // long labels, 32 quads a step, leaving at the first step that prunes
             for (uint32_t m = __ballot_sync(FULL, in && wlen >= LONG_LABEL); m; m &= m - 1) {
                 const uint32_t j = __ffs(m) - 1;
-                const uint32_t lj = __shfl_sync(FULL, wlen, j), quads = (lj + 3) / 4;
-                const uint32_t *lab = a.vis_pool + __shfl_sync(FULL, woff, j);
+                const Spans sp = tw.spans[j];
+                const uint32_t quads = __shfl_sync(FULL, wquads, j);
                 for (uint32_t q0 = 0; q0 < quads; q0 += 32) {
                     const uint32_t q = q0 + lane;
-                    if (__any_sync(FULL, q < quads && quad_prunes(a, tw, r, load_quad(lab, q, lj), level))) {
+                    if (__any_sync(FULL, q < quads && quad_prunes(a, tw, r, span_quad(sp, q), level))) {
                         pruned |= 1u << j;
                         break;
                     }
                 }
-                n_scan += lane == 0 ? lj : 0;
+                n_scan += lane == 0 ? sp.near_n + sp.rest_n : 0;
             }
             // short labels, their quads laid end to end
-            const uint32_t len = (in && wlen < LONG_LABEL) ? wlen : 0, nq = (len + 3) / 4;
-            n_scan += len;
+            const bool mine_short = in && wlen < LONG_LABEL;
+            const uint32_t nq = mine_short ? wquads : 0;
+            n_scan += mine_short ? wlen : 0;
             uint32_t incl = nq;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -946,16 +974,19 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             }
             const uint32_t total = __shfl_sync(FULL, incl, 31);
             const uint32_t excl = incl - nq;
+            tw.spans[lane].first = excl;
+            __syncwarp();
             for (uint32_t x0 = 0; x0 < total; x0 += 32) {
                 const uint32_t x = x0 + lane;
                 uint32_t j = 0;  // owner: the last candidate whose first quad is <= x
 #pragma unroll
                 for (uint32_t step = 16; step > 0; step >>= 1)
                     if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
-                const uint32_t *lab = a.vis_pool + __shfl_sync(FULL, woff, j);
-                const uint32_t lj = __shfl_sync(FULL, len, j), xj = __shfl_sync(FULL, excl, j);
                 bool p = false;
-                if (x < total) p = quad_prunes(a, tw, r, load_quad(lab, x - xj, lj), level);
+                if (x < total) {
+                    const Spans sp = tw.spans[j];
+                    p = quad_prunes(a, tw, r, span_quad(sp, x - sp.first), level);
+                }
                 pruned |= __reduce_or_sync(FULL, p ? 1u << j : 0u);
             }
         }

@@ -130,7 +130,10 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     struct PoolGuard {
         LabelStore *st;
         cudaStream_t s;
-        ~PoolGuard() { pool_free(st->pool, s); }
+        ~PoolGuard() {
+            pool_free(st->pool, s);
+            labels_near_free(*st, s);
+        }
     } pool_guard{&st, s};
 
     int grid[2] = {0, 0};
@@ -305,6 +308,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.bp_d = ix->d_bp_d; a.bp_c = m_bpc.as<uint8_t>(); a.bp_m = ix->d_bp_m; a.inX = inX;
         a.bp_q = m_bpq.as<uint4>(); a.qn = qn; a.bp_e = bp_e;
         a.lab_off = a.vis_off = st.off; a.lab_len = a.vis_len = st.len; a.pool = a.vis_pool = st.pool;
+        a.near = st.near; a.near_lab = st.near_lab; a.near_end = st.near_end;
         a.k0 = k0; a.B = k1 - k0; a.NW = NW;
         a.visited = m_vis.as<uint32_t>();
         a.ht = m_ht.as<uint32_t>();
@@ -433,6 +437,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             PLL_CHECK(labels_append(st, m_out.as<uint64_t>(), &d_ctr->nkept, P, &d_ctr->err_post, s));
             ix->stats.launches += 2;   // cleanup, append
             ix->stats.cub_calls += 2;  // sort, select
+            // (the builds with small test tables run without the near copy)
+            if (!caps.ht) PLL_CHECK(labels_near(st, total, s));
             PLL_TRY(cudaEventRecord(ev[3], s));
             post_pending = true;
         }

@@ -250,7 +250,10 @@ struct Store {
     PoolMem off, len, cap;
     cudaStream_t s;
     explicit Store(cudaStream_t st_) : off(st_), len(st_), cap(st_), s(st_) {}
-    ~Store() { pool_free(st.pool, s); }
+    ~Store() {
+        pool_free(st.pool, s);
+        labels_near_free(st, s);
+    }
     int init(uint32_t n, unsigned long long *top) {
         st.n = n;
         PLL_CHECK(off.alloc((size_t)n * 8));
@@ -372,6 +375,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         a.inX = inX.as<uint8_t>();
         a.lab_off = from.off; a.lab_len = from.len; a.pool = from.pool;
         a.vis_off = to.off; a.vis_len = to.len; a.vis_pool = to.pool;
+        a.near = to.near; a.near_lab = to.near_lab; a.near_end = to.near_end;
         a.k0 = k0; a.B = B; a.NW = NW;
         a.visited = vis.as<uint32_t>();
         a.ht = ht.as<uint32_t>(); a.tab = tab.as<uint2>(); a.ht_cap = ht_cap;
@@ -459,6 +463,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
             PLL_CHECK(labels_compact(sorted[dir].as<uint64_t>(), keep.as<uint8_t>(), P[dir], out[dir].as<uint64_t>(),
                                      &d->c[dir].nkept, temp.p, &tb, s));
             PLL_CHECK(labels_append(st, out[dir].as<uint64_t>(), &d->c[dir].nkept, P[dir], &d->c[dir].err_post, s));
+            PLL_CHECK(labels_near(st, total[dir], s));
             pending[dir] = true;
         }
         ++ix->batches;

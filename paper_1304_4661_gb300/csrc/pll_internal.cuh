@@ -308,6 +308,17 @@ struct LevelDesc {
     uint32_t pad;
 };
 
+// The near copy of a store: every label as it was at the last rebuild, ordered by
+// distance (classes 0, 1, ..., NEAR_CLASSES - 1 and one of all that is farther), so
+// that a reader who wants the entries nearer than some distance reads a prefix and
+// the entries appended since. It is rebuilt as the store grows (labels_near).
+constexpr uint32_t NEAR_CLASSES = 15;
+struct NearLabel {
+    uint64_t off;    // in the near copy
+    uint32_t base;   // entries it holds (a multiple of 4): the label's first `base`
+    uint32_t pad;
+};
+
 struct BatchArgs {
     uint32_t n, t, tp;
     const uint32_t *roff, *rcol;
@@ -324,6 +335,9 @@ struct BatchArgs {
     const uint64_t *vis_off;   // labels of the visited vertices: the same arrays, or
     const uint32_t *vis_len;   // (directed graphs) those of the other label set
     const uint32_t *vis_pool;
+    const uint32_t *near;      // their near copy, or null
+    const NearLabel *near_lab;
+    const uint32_t *near_end;
     uint32_t k0, B, NW;        // roots [k0, k0 + B), NW = ceil(n / 32)
     uint32_t qn;               // 16-byte chunks of a bp_q row: ceil(t / 32)
     uint32_t *visited;         // [B][NW] bitmap: row of root slot s holds one bit
@@ -380,6 +394,10 @@ struct LabelStore {
     uint32_t *pool = nullptr;
     uint64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
+    uint32_t *near = nullptr;        // [near_cap] the near copy, or null
+    uint64_t near_cap = 0, near_total = 0;
+    NearLabel *near_lab = nullptr;   // [n]
+    uint32_t *near_end = nullptr;    // [NEAR_CLASSES][n] its entries of distance <= c
     bool pooled = false;  // `pool` comes from pool_malloc (else dev_malloc)
 };
 // radix sort of packed tuples by their bits [begin_bit, end_bit)
@@ -396,6 +414,9 @@ int labels_append(const LabelStore &st, const uint64_t *d_kept,
                   const unsigned long long *d_nkept, uint64_t max_count, uint32_t *d_err,
                   cudaStream_t s);
 int labels_regrow(LabelStore &st, uint64_t new_cap, cudaStream_t s);
+// rebuilds the near copy if the store (of `total` entries) has outgrown it
+int labels_near(LabelStore &st, uint64_t total, cudaStream_t s);
+void labels_near_free(LabelStore &st, cudaStream_t s);
 int labels_finalize(const LabelStore &st, uint64_t total, uint64_t *d_off, uint32_t *d_lab,
                     void *d_temp, size_t *temp_bytes, cudaStream_t s);
 int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_temp,

@@ -99,3 +99,19 @@ def test_rank_space_lists_at_the_sort_widths(n):
     ix, ref = pll.DirectedIndex(dev_u32(d.offsets), dev_u32(d.cols)), oracle.DirectedIndex(d.offsets, d.cols)
     for a, b in ((ix.labels_in(), ref.labels_in()), (ix.labels_out(), ref.labels_out())):
         assert same_labels(a, b), first_label_diff(a, b, d.n)
+
+
+@pytest.mark.parametrize("name,make,t", [("ba", lambda: gg.ba(20000, 6, 7), 0), ("ws", lambda: gg.ws(12000, 6, 0.02, 2), 0),
+                                         ("ws8", lambda: gg.ws(12000, 6, 0.05, 2), 8)])
+@pytest.mark.parametrize("root_batch", [0, 500])
+def test_stores_that_outgrow_their_near_copy(name, make, t, root_batch):
+    """Two to three million entries, at distances on both sides of the last distance class."""
+    check(make(), t, root_batch=root_batch)
+
+
+def test_directed_stores_that_outgrow_their_near_copy():
+    d = gg.oriented(gg.ba(20000, 6, 7), 3, both=0.3)
+    ref = oracle.DirectedIndex(d.offsets, d.cols)
+    ix = pll.DirectedIndex(dev_u32(d.offsets), dev_u32(d.cols), root_batch=1000)
+    for a, b in ((ix.labels_in(), ref.labels_in()), (ix.labels_out(), ref.labels_out())):
+        assert same_labels(a, b), first_label_diff(a, b, d.n)
