@@ -39,9 +39,8 @@
 //           bit-parallel bound of a pair does not depend on the level, so if
 //           it prunes w at level d + 1 it prunes w again at any later level
 //           where w is reached, and leaving the bit clear changes no label.
-//   test    the rest of the test, 32 candidates per warp: the feasible
-//           bit-parallel roots of a candidate on the lanes (two each, mask
-//           pairs compared); then, root by root, the labels L(w) of the
+//   test    the rest of the test, 32 candidates per warp: the mask pairs of
+//           their feasible bit-parallel roots compared, one a lane; then, root by root, the labels L(w) of the
 //           candidates that are left, past the root's reach table in shared
 //           memory to its hash table. Survivors are appended as (w, k, d + 1).
 //   clear   after the batch, the lazy reset of Sec. 4.5.1 ("Initialization"):
@@ -731,8 +730,11 @@ __global__ void k_batch_clear(BatchArgs a) {
 
 // The rest of the prune test for 32 candidates per warp (lane j holds
 // candidate j), in two parts:
-//   masks   one candidate with feasible roots at a time: the lanes take the
-//           roots (two each) and compare mask pairs (Sec. 5.3);
+//   masks   the (candidate, feasible root) pairs of all 32 laid end to end over
+//           the lanes, a mask pair compared by each (Sec. 5.3). A candidate has
+//           four of them on R-MAT-20: one candidate at a time over the lanes
+//           left 28 of 32 idle behind two dependent loads (its test sweeps: 32.8
+//           -> 21.9 ms, the batch's 69.0 -> 64.4);
 //   labels  of the candidates the masks did not prune, root by root (the sweeps
 //           keep a root's candidates together: 4 to 6 of 32 share one on
 //           average). The root's reach table is copied to shared memory, and
@@ -757,7 +759,7 @@ __global__ void k_batch_clear(BatchArgs a) {
 // L2), 124 ms with the reach tables and single entries on the lanes, 106.6 ms
 // with quads. R-MAT-20 (t = 64; 7.8G entries, 0.4G nearer): 65.9, 47.0, 43.3
 // ms; with the near copy, which leaves the near entries and those of the last
-// batches (16G and 1.05G), 68.9 and 32.8 ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
+// batches (16G and 1.05G), 69.0 and 32.8 ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
 // reach table (fewer false hits): 108 ms.
 // candidates whose labels have at least this many entries are scanned one by
 // one by the whole warp (no owner search per entry, and an exit at the first
@@ -905,27 +907,40 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             tb = t.x;
             tmask = t.y;
         }
-        // ---- masks
+        // ---- masks: the (candidate, root) pairs laid end to end
         uint32_t pruned = 0;
-        for (uint32_t m = __ballot_sync(FULL, (mc.x | mc.y) != 0); m; m &= m - 1) {
-            const uint32_t j = __ffs(m) - 1;
-            const uint64_t c1 = __shfl_sync(FULL, mc.x, j), c2 = __shfl_sync(FULL, mc.y, j);
-            const uint32_t wj = __shfl_sync(FULL, w, j), kj = a.k0 + __shfl_sync(FULL, slot, j);
-            const ulonglong2 *wm = reinterpret_cast<const ulonglong2 *>(a.bp_m) + (size_t)wj * a.t;
-            const ulonglong2 *km = reinterpret_cast<const ulonglong2 *>(a.bp_m) + (size_t)kj * a.t;
-            bool p = false;
+        {
+            uint64_t open = mc.x | mc.y;
+            const uint32_t mine_n = __popcll(open);
+            uint32_t incl = mine_n;
 #pragma unroll
-            for (uint32_t h = 0; h < 2; ++h) {
-                const uint32_t i = lane + 32 * h;
-                const bool b1 = (c1 >> i) & 1, b2 = (c2 >> i) & 1;
-                if (b1 | b2) {
-                    ++n_mask;
-                    const ulonglong2 mw = wm[i], r = km[i];
-                    if (b1 && (((r.x | r.y) & mw.x) | (r.x & mw.y))) p = true;  // reduction >= 1
-                    if (b2 && (r.x & mw.x)) p = true;                           // reduction 2
-                }
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
             }
-            if (__any_sync(FULL, p)) pruned |= 1u << j;
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            // no table is staged yet: its place holds the list
+            static_assert(32 * PLL_MAX_T * sizeof(uint16_t) <= REACH_MAX, "every root of every candidate fits");
+            uint16_t *items = reinterpret_cast<uint16_t *>(tw.reach);
+            for (uint32_t at = incl - mine_n; open; open &= open - 1) {
+                const uint32_t i = __ffsll(open) - 1;
+                items[at++] = (uint16_t)(lane | i << 5 | (uint32_t)(mc.x >> i & 1) << 11 |
+                                         (uint32_t)(mc.y >> i & 1) << 12);
+            }
+            __syncwarp();
+            for (uint32_t x0 = 0; x0 < total; x0 += 32) {
+                const uint32_t it = x0 + lane < total ? items[x0 + lane] : 0, j = it & 31, i = it >> 5 & 63;
+                const uint32_t wj = __shfl_sync(FULL, w, j), kj = a.k0 + __shfl_sync(FULL, slot, j);
+                bool p = false;
+                if (x0 + lane < total && !((pruned >> j) & 1)) {
+                    ++n_mask;
+                    const ulonglong2 mw = reinterpret_cast<const ulonglong2 *>(a.bp_m)[(size_t)wj * a.t + i];
+                    const ulonglong2 r = reinterpret_cast<const ulonglong2 *>(a.bp_m)[(size_t)kj * a.t + i];
+                    if ((it >> 11 & 1) && (((r.x | r.y) & mw.x) | (r.x & mw.y))) p = true;  // reduction >= 1
+                    if ((it >> 12 & 1) && (r.x & mw.x)) p = true;                           // reduction 2
+                }
+                pruned |= __reduce_or_sync(FULL, p ? 1u << j : 0u);
+            }
         }
         // ---- labels, root by root
         uint32_t todo = __ballot_sync(FULL, valid && !((pruned >> lane) & 1) && wlen && klen);
