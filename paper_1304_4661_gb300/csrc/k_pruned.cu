@@ -768,8 +768,10 @@ __global__ void k_batch_clear(BatchArgs a) {
 // more on the batch)
 constexpr uint32_t LONG_LABEL = LONG_LABEL_ENTRIES;
 // a root's table is staged for at least this many label entries of its
-// candidates, else read where it lies (the batch's test sweeps take 124 ms with
-// any line from 1 to 500, 141 ms without staging; R-MAT-20's 47 to 48 ms)
+// candidates; the others' candidates are taken together, each lane reading its
+// candidate's table where it lies (128, 256, 512: 60.3, 60.1, 63.1 ms of test
+// sweeps on the batch, 19.1, 18.9, 19.1 on R-MAT-20; root by root without
+// staging 64.4 and 21.9)
 constexpr uint32_t STAGE_ENTRIES = PLL_STAGE_ENTRIES;
 
 // Where the label entries of a candidate lie that a test reads: the near copy's
@@ -943,7 +945,7 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             }
         }
         // ---- labels, root by root
-        uint32_t todo = __ballot_sync(FULL, valid && !((pruned >> lane) & 1) && wlen && klen);
+        uint32_t todo = __ballot_sync(FULL, valid && !((pruned >> lane) & 1) && wlen && klen), loose = 0;
         while (todo) {
             const uint32_t j0 = __ffs(todo) - 1;
             const uint32_t s0 = __shfl_sync(FULL, slot, j0);
@@ -956,7 +958,12 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
             r.tmask = __shfl_sync(FULL, tmask, j0);
             r.tb = (unsigned long long)__shfl_sync(FULL, tb, j0) * HT_MIN;
             r.lg = reach_lg(r.tmask);
-            r.staged = r.tmask != NONE && __reduce_add_sync(FULL, in ? min(wlen, 0xffffu) : 0u) >= STAGE_ENTRIES;
+            r.staged = __reduce_add_sync(FULL, in ? min(wlen, 0xffffu) : 0u) >= STAGE_ENTRIES;
+            if (r.tmask != NONE && !r.staged) {
+                loose |= group;
+                continue;
+            }
+            r.staged = r.tmask != NONE;
             __syncwarp();  // the previous root's table has been read
             if (r.staged) {
                 const uint4 *src = reinterpret_cast<const uint4 *>(a.reach + r.tb);
@@ -997,6 +1004,40 @@ __device__ __forceinline__ void test_body(const BatchArgs &a, unsigned long long
 #pragma unroll
                 for (uint32_t step = 16; step > 0; step >>= 1)
                     if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
+                bool p = false;
+                if (x < total) {
+                    const Spans sp = tw.spans[j];
+                    p = quad_prunes(a, tw, r, span_quad(sp, x - sp.first), level);
+                }
+                pruned |= __reduce_or_sync(FULL, p ? 1u << j : 0u);
+            }
+        }
+        // the groups with few entries, together: each lane reads its candidate's table where it lies
+        if (loose) {
+            const uint32_t nq = (loose >> lane) & 1 ? wquads : 0;
+            n_scan += nq ? wlen : 0;
+            uint32_t incl = nq;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            const uint32_t excl = incl - nq;
+            __syncwarp();
+            tw.spans[lane].first = excl;
+            __syncwarp();
+            for (uint32_t x0 = 0; x0 < total; x0 += 32) {
+                const uint32_t x = x0 + lane;
+                uint32_t j = 0;
+#pragma unroll
+                for (uint32_t step = 16; step > 0; step >>= 1)
+                    if (__shfl_sync(FULL, excl, j + step) <= x) j += step;
+                TestRoot r{};
+                r.tmask = __shfl_sync(FULL, tmask, j);
+                r.tb = (unsigned long long)__shfl_sync(FULL, tb, j) * HT_MIN;
+                r.lg = reach_lg(r.tmask);
+                r.staged = false;
                 bool p = false;
                 if (x < total) {
                     const Spans sp = tw.spans[j];
