@@ -88,10 +88,11 @@ typedef struct pll_index pll_index;
 typedef struct pll_build_opts {
     uint32_t t;          /* bit-parallel roots, 0..PLL_MAX_T (Sec. 5.4). */
     uint32_t root_batch; /* largest number of pruned-BFS roots processed in
-                            one batch (batches double from 64 up to it); 0 =
-                            16384, halved while n * root_batch / 8 bytes of
-                            visited bitmap would exceed 8 GiB. Any value
-                            gives the same labels. */
+                            one batch (batches grow from 64 up to it, 65536
+                            at most); 0 = 65536, halved while n * root_batch
+                            / 8 bytes of visited bitmap would exceed 8 GiB
+                            or, above 16384, a sixteenth of the free memory.
+                            Any value gives the same labels. */
     uint32_t block;      /* threads per CTA of the pruned-BFS kernel: 128,
                             256, 512 or 1024; 0 = library default (256). */
     uint32_t flags;      /* 0 or one of PLL_BUILD_*_LEVELS (below). */
@@ -558,8 +559,8 @@ PLL_API void pll_paths_free(pll_paths *p);
  *                  undirected labels (t = 0) in both sets.
  *   order          device or NULL: rank -> vertex; NULL = descending in- plus
  *                  out-degree, ties by ascending id.
- *   opts           t = 0; root_batch as for pll_build (0 = 16384, halved while
- *                  n x root_batch / 8 bytes of visited bits pass 2 GiB); block,
+ *   opts           t = 0; root_batch as for pll_build (with 2 GiB of visited
+ *                  bits for the 8, whoever names it); block,
  *                  flags, reserved: 0. NULL = defaults.
  *   out            receives the index; free it with pll_dfree.
  * The labels are the unique ones the sequential method gives for this order.

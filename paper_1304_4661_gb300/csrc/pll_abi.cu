@@ -8,8 +8,8 @@
 //   3. Alg. 2 over batches of roots [k0, k1): the BFSs of all roots of a
 //      batch advance level by level as bulk-synchronous sweeps (Alg. 1 per
 //      root, pruned with hubs < k0 and the bit-parallel labels), then sort +
-//      redundancy cleanup + append of the batch's entries; batch sizes double
-//      from 64 up to root_batch;
+//      redundancy cleanup + append of the batch's entries; batch sizes grow
+//      from 64 up to root_batch (next_batch, pll_internal.cuh);
 //   4. compaction of the labels into one hub-sorted CSR for queries.
 // Level boundaries stay on the device; the host reads a small counter block
 // every few levels (to see an empty frontier) and once after the append.
@@ -168,7 +168,6 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PoolMem m_vis(s), m_ht(s), m_tab(s), m_cand(s), m_candc(s), m_out(s),
         m_sorted(s), m_keep(s), m_temp(s);
     PLL_CHECK(m_vis.alloc((size_t)bmax * NW * 4));
-    PLL_TRY(cudaMemsetAsync(m_vis.p, 0, (size_t)bmax * NW * 4, s));
     const TestCaps caps = test_caps();
     // Initial sizes generous enough that the first large root batches do not
     // overflow (a batch that overflows runs again; roots whose tables do not
@@ -180,7 +179,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         (void)cudaGetLastError();
         free_b = 0;
     }
-    uint64_t ht_cap = caps.ht ? caps.ht : std::max<uint64_t>((uint64_t)bmax * 2048, 1ull << 20);
+    uint64_t ht_cap = caps.ht ? caps.ht : std::max<uint64_t>({(uint64_t)std::min(bmax, BATCH_FULL) * 2048,
+                                                                (uint64_t)bmax * 512, 1ull << 20});
     PLL_CHECK(m_ht.alloc(ht_cap * 4));
     PLL_CHECK(m_tab.alloc((size_t)bmax * 8));
     PoolMem m_reach(s);
@@ -283,7 +283,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         ix->stats.ms_post += ms;
         return PLL_OK;
     };
-    uint32_t k0 = 0, B = std::min<uint32_t>(64, bmax);
+    uint32_t k0 = 0, B = next_batch(0, 0, bmax), zeroed = 0;
     uint64_t last_cand = 0, last_out = 0, last_B = 1;
     unsigned long long work0[4] = {0, 0, 0, 0};
     while (k0 < n) {
@@ -301,6 +301,10 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
                 out_cap = (uint64_t)((double)last_out * f);
                 PLL_CHECK(alloc_out());
             }
+        }
+        if (k1 - k0 > zeroed) {  // rows used for the first time
+            PLL_TRY(cudaMemsetAsync(m_vis.as<uint32_t>() + (size_t)zeroed * NW, 0, (size_t)(k1 - k0 - zeroed) * NW * 4, s));
+            zeroed = k1 - k0;
         }
         BatchArgs a{};
         a.n = n; a.t = ix->t; a.tp = ix->tp;
@@ -445,7 +449,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         for (int w = 0; w < 4; ++w) work0[w] = h->c.work[w];  // the sweeps' counts so far
         ++batches;
         k0 = k1;
-        B = std::min<uint32_t>(B * 2, bmax);
+        B = next_batch(k0, P, bmax);
     }
     if (post_pending) {
         PLL_CHECK(read_back());
@@ -506,15 +510,7 @@ int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t 
     if (n == 0 && nnz != 0) return PLL_E_INVAL;
     uint32_t block = o.block ? o.block : 256;
     if (block != 128 && block != 256 && block != 512 && block != 1024) return PLL_E_INVAL;
-    // default: 16384 roots per batch (fewer, larger batches: one R-MAT-20 build
-    // is ~10% faster than at 4096), halved while the batch's visited bitmap
-    // (n x batch / 8 bytes) would pass 8 GiB
-    uint32_t bmax = o.root_batch;
-    if (!bmax) {
-        bmax = 16384;
-        while (bmax > 1024 && (uint64_t)n * bmax / 8 > (8ull << 30)) bmax >>= 1;
-    }
-    if (bmax > (1u << 16)) bmax = 1u << 16;
+    const uint32_t bmax = std::max(1u, std::min({n, o.root_batch ? o.root_batch : default_batch(n, 8ull << 30, 1024), BATCH_MAX}));
     const bool batch = graph_start != nullptr;
     if (!batch) graphs = 1;
     if (batch) {

@@ -322,7 +322,6 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     PoolMem rstart[2] = {PoolMem(s), PoolMem(s)}, out[2] = {PoolMem(s), PoolMem(s)},
             sorted[2] = {PoolMem(s), PoolMem(s)};
     PLL_CHECK(vis.alloc((size_t)bmax * NW * 4));
-    PLL_TRY(cudaMemsetAsync(vis.p, 0, (size_t)bmax * NW * 4, s));
     PLL_CHECK(inX.alloc(n));
     PLL_TRY(cudaMemsetAsync(inX.p, 0, n, s));
     uint64_t ht_cap = std::max<uint64_t>((uint64_t)bmax * 1024, 1ull << 18);
@@ -409,10 +408,14 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         }
         return PLL_OK;
     };
-    uint32_t B = std::min<uint32_t>(64, bmax);
+    uint32_t B = next_batch(0, 0, bmax), zeroed = 0;
     bool cut = true;
     for (uint32_t k0 = 0; k0 < n;) {
         const uint32_t k1 = (uint32_t)std::min<uint64_t>((uint64_t)k0 + B, n), Bc = k1 - k0;
+        if (Bc > zeroed) {  // rows used for the first time
+            PLL_TRY(cudaMemsetAsync(vis.as<uint32_t>() + (size_t)zeroed * NW, 0, (size_t)(Bc - zeroed) * NW * 4, s));
+            zeroed = Bc;
+        }
         for (int dir = 0; dir < 2; ++dir) PLL_CHECK(run_dir(dir, k0, Bc, cut));
         PLL_CHECK(read_back());
         PLL_CHECK(settle());
@@ -468,7 +471,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         }
         ++ix->batches;
         k0 = k1;
-        B = std::min<uint32_t>(B * 2, bmax);
+        B = next_batch(k0, P[0] + P[1], bmax);
     }
     PLL_CHECK(read_back());
     PLL_CHECK(settle());
@@ -500,10 +503,9 @@ PLL_API int pll_build_directed(const uint32_t *offsets, const uint32_t *cols, ui
     if (n > MAX_N || nnz >= 0xffffffffull) return PLL_E_RANGE;
     if ((n > 0 && !offsets) || (nnz > 0 && !cols) || (n == 0 && nnz != 0)) return PLL_E_INVAL;
     // default batch: as large as the undirected build's (R-MAT-17: 104 ms at
-    // 1024 roots, 60 ms at 16384; R-MAT-15: 22.0 and 13.6 ms), halved below while
-    // the visited bits would pass 2 GiB
-    uint32_t bmax = o.root_batch ? o.root_batch : 16384;
-    if (bmax > (1u << 16)) bmax = 1u << 16;
+    // 1024 roots, 60 ms at 16384; R-MAT-15: 22.0 and 13.6 ms); the visited bits
+    // of any batch stay within 2 GiB
+    uint32_t bmax = std::max(1u, std::min({n, o.root_batch ? o.root_batch : default_batch(n, 2ull << 30, 64), BATCH_MAX}));
     while (bmax > 64 && (uint64_t)n * bmax / 8 > (2ull << 30)) bmax >>= 1;
     cudaStream_t s = (cudaStream_t)stream;
     pll_dindex *ix = new (std::nothrow) pll_dindex();

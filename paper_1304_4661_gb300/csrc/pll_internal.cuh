@@ -21,6 +21,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "pll.h"
 
 namespace pll {
@@ -318,6 +320,47 @@ struct NearLabel {
     uint32_t base;   // entries it holds (a multiple of 4): the label's first `base`
     uint32_t pad;
 };
+
+// Size of the next root batch, after `roots_done` roots and a batch that emitted
+// `last_entries` entries. A batch costs its launches, about 0.35 ms (0.5 with its
+// host round trip); roots in one batch do not prune with each other, so a larger
+// one labels, expands and drops again more surplus entries, about 0.75 ns each.
+// While batches are small (their launches are what they cost) the roots done
+// quadruple with each, then double; a batch with more than a million entries
+// fills the device, and its successors are held to two fifths of the roots done
+// and to BATCH_FULL. Late batches emit little again and grow up to the largest
+// size. Builds of R-MAT-20, the batch of 96 graphs, BA-10k and R-MAT-15 both ways:
+//   doubling from 64 to 16384               115.2  147.1  4.19  12.5 ms
+//   this rule                                91.0  143.0  3.44  12.2
+//   with at most 16384 / 32768 roots        +9.4 / +2.5, +6.1 / +0.2 ms on the
+//                                           first two (the late batches' launches)
+//   shares of 0.25, 0.33, 0.5 for 0.4       R-MAT-20 90.6 90.9 93.4, batch 143.4 142.6 140.6
+//   lines at 64K entries (for 256K)         BA-10k 3.7 to 4.0; at 512K R-MAT-15 15.2
+//   the first batches five times the roots done   R-MAT-20 98.9
+constexpr uint32_t BATCH_MAX = 1u << 16, BATCH_FULL = 16384;
+inline uint32_t next_batch(uint64_t roots_done, uint64_t last_entries, uint32_t bmax) {
+    uint64_t b = roots_done;
+    if (last_entries < (256u << 10)) b = 3 * roots_done;
+    else if (last_entries >= (1u << 20)) b = std::min<uint64_t>(roots_done * 2 / 5, BATCH_FULL);
+    return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(b, 64), bmax);
+}
+
+// The largest batch a build uses when the caller names none: its visited bits,
+// n * batch / 8 bytes, stay within `limit`, and past the BATCH_FULL roots that
+// every build is given also within a sixteenth of the free memory.
+inline uint32_t default_batch(uint32_t n, uint64_t limit, uint32_t least) {
+    uint32_t b = BATCH_MAX;
+    while (b > least && (uint64_t)n * b / 8 > limit) b >>= 1;
+    if (b > BATCH_FULL && (uint64_t)n * b / 8 > (256u << 20)) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+            (void)cudaGetLastError();
+            free_b = 0;
+        }
+        while (b > BATCH_FULL && (uint64_t)n * b / 8 > free_b / 16) b >>= 1;
+    }
+    return b;
+}
 
 struct BatchArgs {
     uint32_t n, t, tp;
