@@ -40,33 +40,27 @@
 //           it prunes w at level d + 1 it prunes w again at any later level
 //           where w is reached, and leaving the bit clear changes no label.
 //   test    the rest of the test, 32 candidates per warp: the mask pairs of
-//           their feasible bit-parallel roots compared, one a lane; then, root by root, the labels L(w) of the
-//           candidates that are left, past the root's reach table in shared
-//           memory to its hash table. Survivors are appended as (w, k, d + 1).
+//           their feasible bit-parallel roots compared, one a lane; then, root
+//           by root, the near entries of the labels L(w) of the candidates that
+//           are left, past the root's reach table to its hash table. Survivors
+//           are appended as (w, k, d + 1).
 //   clear   after the batch, the lazy reset of Sec. 4.5.1 ("Initialization"):
 //           the only bits set are those of the roots and of the recorded
 //           candidates, so their words are zeroed and nothing else is touched
 //           (instead of clearing B * n / 8 bytes per batch).
 //
-// Level boundaries live in a device descriptor advanced by a one-thread
-// kernel, so the host enqueues several levels ahead and reads back only to
-// learn that the frontier is empty; sweeps over an empty range return at once.
+// Level boundaries live in a device descriptor, advanced by the last block of
+// each sweep of the graph loop (by a one-thread kernel where the host enqueues
+// the levels, several ahead); sweeps over an empty range return at once.
 #include "bp_nibble.h"
 #include "pll_internal.cuh"
 
 namespace pll {
 namespace {
 
-#ifndef LONG_LABEL_ENTRIES
-#define LONG_LABEL_ENTRIES 128
-#endif
-#ifndef PLL_STAGE_ENTRIES
-#define PLL_STAGE_ENTRIES 256
-#endif
-#ifndef PLL_TEST_TPS
-#define PLL_TEST_TPS 1024
-#endif
-constexpr int TEST_TPS = PLL_TEST_TPS;
+// threads an SM of the test sweep (64 registers each; at 1280 it spills: R-MAT-20's
+// test sweeps 41.6 ms against 32.8, the batch's 74.2 against 69.0)
+constexpr int TEST_TPS = 1024;
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr uint32_t HT_EMPTY = 0xffffffffu;
@@ -508,14 +502,11 @@ __device__ __forceinline__ void expand_open(const BatchArgs &a, const ExpandWarp
     append_cand(a, keep, lane, slot, w, c1, c2);
 }
 
-#ifndef PLL_HEAVY_DEG
-#define PLL_HEAVY_DEG 64
-#endif
-#ifndef PLL_EXPAND_TPS
-#define PLL_EXPAND_TPS 1024
-#endif
-constexpr uint32_t HEAVY_DEG = PLL_HEAVY_DEG;
-constexpr int EXPAND_TPS = PLL_EXPAND_TPS;
+// entries of at least this many neighbours are taken 32 arcs at a time (32 to 1000:
+// no difference), and threads an SM of the expand sweep (builds of R-MAT-20 and of
+// the batch of 96 graphs: 144.9 and 176.4 ms at 1280, 138.5 and 170.6 at 1024)
+constexpr uint32_t HEAVY_DEG = 64;
+constexpr int EXPAND_TPS = 1024;
 
 // The expand sweep: entries [b, e) of level `level` and the slices of its long
 // entries -> candidates of the next, by the warps of a grid. A warp takes a
@@ -766,13 +757,13 @@ __global__ void k_batch_clear(BatchArgs a) {
 // step that prunes); shorter labels are laid end to end over the lanes (the
 // line at 32: 2 ms more on R-MAT-20; at 64 to 256 no difference; none: 25 ms
 // more on the batch)
-constexpr uint32_t LONG_LABEL = LONG_LABEL_ENTRIES;
+constexpr uint32_t LONG_LABEL = 128;
 // a root's table is staged for at least this many label entries of its
 // candidates; the others' candidates are taken together, each lane reading its
 // candidate's table where it lies (128, 256, 512: 60.3, 60.1, 63.1 ms of test
 // sweeps on the batch, 19.1, 18.9, 19.1 on R-MAT-20; root by root without
 // staging 64.4 and 21.9)
-constexpr uint32_t STAGE_ENTRIES = PLL_STAGE_ENTRIES;
+constexpr uint32_t STAGE_ENTRIES = 256;
 
 // Where the label entries of a candidate lie that a test reads: the near copy's
 // entries of distance < level, then those appended since its last rebuild (all
