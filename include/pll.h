@@ -72,8 +72,8 @@ typedef struct pll_index pll_index;
  * labels every way).
  *   PLL_BUILD_GRAPH_LEVELS (the default, also with flags 0): one CUDA graph
  *     launch per batch, a conditional while node over the expand and test
- *     sweeps (separate kernels); a device-side step after each level stops it
- *     when the frontier is empty. No host read-back within a batch.
+ *     sweeps (separate kernels); the last block of a level stops it when the
+ *     frontier is empty. No host read-back within a batch.
  *   PLL_BUILD_COOP_LEVELS: one cooperative launch per batch that runs every
  *     level itself, with grid barriers whose waits are bounded (a wait that
  *     runs out is PLL_E_TIMEOUT); falls back to the graph where the device
@@ -106,7 +106,8 @@ typedef struct pll_stats {
     uint64_t label_entries;      /* sum over v of |L(v)| (normal labels) */
     uint64_t pre_cleanup;        /* entries emitted by batched pruned BFSs
                                     before the redundancy cleanup */
-    uint64_t visited;            /* vertices dequeued by pruned BFSs */
+    uint64_t visited;            /* (root, vertex) pairs that pruned BFSs reached
+                                    and the bit-parallel distances left */
     uint64_t batches;            /* root batches */
     uint64_t index_bytes;        /* device bytes held by the index */
     double ms_prep;              /* order, relabel, root selection */
@@ -142,8 +143,8 @@ typedef struct pll_stats {
        phases. */
     uint64_t levels_launches;
     double ms_levels;
-    /* CUDA-event time of each root batch's sort, cleanup, compaction and
-       append, summed (ms_pruned less ms_pruned_kernel, ms_post and
+    /* CUDA-event time of each root batch's sort, cleanup, compaction, append
+       and near copy, summed (ms_pruned less ms_pruned_kernel, ms_post and
        ms_finalize is the time the GPU waited on the host between batches) */
     double ms_post;
     /* most scratch memory the build held at once (its temporaries, from the
