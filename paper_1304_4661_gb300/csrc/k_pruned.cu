@@ -528,7 +528,8 @@ constexpr int EXPAND_TPS = 1024;
 // R-MAT-20's expand sweeps (t = 64; 3.15G arcs): 95.1 ms with a warp per
 // entry, 64-byte rows and the visited word first; 71.9 ms with chunks, the
 // queue and nibble rows; 55.3 ms with long lists in slices; 51.4 ms with one
-// load a row; 39.2 ms with the lists cut at rank k0 (1.64G arcs left).
+// load a row; 39.2 ms with the lists cut at rank k0 (1.64G arcs left);
+// 32.9 ms with the batch sizes of next_batch (1.3G).
 __device__ __forceinline__ void expand_body(const BatchArgs &a, unsigned long long b, unsigned long long e,
                                             unsigned long long slice_n, uint32_t level, ExpandWarp &sw,
                                             uint32_t &nexp, uint32_t &nreach) {
@@ -750,8 +751,11 @@ __global__ void k_batch_clear(BatchArgs a) {
 // L2), 124 ms with the reach tables and single entries on the lanes, 106.6 ms
 // with quads. R-MAT-20 (t = 64; 7.8G entries, 0.4G nearer): 65.9, 47.0, 43.3
 // ms; with the near copy, which leaves the near entries and those of the last
-// batches (16G and 1.05G), 69.0 and 32.8 ms. Two quads a lane in flight: 113 ms on the batch; a second hash of the
-// reach table (fewer false hits): 108 ms.
+// batches (16G and 1.05G), 69.0 and 32.8 ms; with the masks end to end and the
+// small groups together 60.1 and 18.9; with the batch sizes of next_batch 62.2 and
+// 16.2 (170M and 106M candidates). Without effect or slower: two quads a lane in
+// flight, a second hash of the reach table, the entries it lets through queued
+// and looked up 32 at a time (64 to 67 ms on the batch, 15.8 on R-MAT-20).
 // candidates whose labels have at least this many entries are scanned one by
 // one by the whole warp (no owner search per entry, and an exit at the first
 // step that prunes); shorter labels are laid end to end over the lanes (the
