@@ -325,7 +325,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         a.ctr = d_ctr; a.desc = d_desc; a.loop = d_loop;
         PLL_TRY(cudaEventRecord(ev0, s));
         PLL_TRY(cudaMemsetAsync(d_ctr, 0, 16, s));  // cand_n, out_n
-        PLL_TRY(cudaMemsetAsync(&d_ctr->slice_n, 0, 20, s));  // slice_n, ht_top, err
+        PLL_TRY(cudaMemsetAsync(&d_ctr->slice_n, 0, 28, s));  // slice_n, ht_top, taken, err
         PLL_CHECK(batch_row_starts(n, k0, roff, rcol, m_rstart.as<uint32_t>(), grid[0], s));
         PLL_CHECK(batch_init(a, s));
         ix->stats.launches += 3;

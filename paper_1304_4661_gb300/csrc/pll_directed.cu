@@ -384,7 +384,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         a.slices = slices.as<uint4>(); a.slice_cap = slice_cap;
         a.ctr = &d->c[dir]; a.desc = &d->d[dir]; a.loop = m_loop.as<LoopState>();
         PLL_TRY(cudaMemsetAsync(a.ctr, 0, 16, s));             // cand_n, out_n
-        PLL_TRY(cudaMemsetAsync(&a.ctr->slice_n, 0, 20, s));   // slice_n, ht_top, err
+        PLL_TRY(cudaMemsetAsync(&a.ctr->slice_n, 0, 28, s));   // slice_n, ht_top, taken, err
         if (cut) PLL_CHECK(batch_row_starts(n, k0, a.roff, a.rcol, rstart[dir].as<uint32_t>(), grid[0], s));
         PLL_CHECK(batch_init(a, s));
         PLL_TRY(cudaMemcpyAsync(m_args.p, &a, sizeof(BatchArgs), cudaMemcpyHostToDevice, s));

@@ -280,6 +280,7 @@ struct BatchCounters {
     unsigned long long pool_top;  // label pool bump pointer
     unsigned long long slice_n;   // slices of the next level's long entries
     unsigned long long ht_top;    // table pool bump pointer (reset per batch)
+    unsigned long long taken;     // items of the current sweep handed out past each warp's first chunk
     uint32_t err;                 // errors of the batch's BFS (reset per batch)
     uint32_t err_post;            // errors of the appends (never reset)
 };
