@@ -51,7 +51,7 @@ WORKLOADS = {
 # 24 launches, 4.955 GB of DRAM against 6.953 GB of algorithmic bytes.
 PROFILED = {
     "level-loop graph (k_batch_expand_g + k_batch_test_g)": {
-        "src_sha": "6b6e2f9ed2813426", "dram_per_alg_byte": 0.292},
+        "src_sha": "2f8ca0172ddd4fd8", "dram_per_alg_byte": 0.289},
 }
 
 

@@ -30,7 +30,7 @@
 // lists' offsets; a warp per vertex) and k_dquery (warp per pair).
 // R-MAT-15, arcs one way or both (1.2M): 49.3 ms for the build and 1M queries
 // with a thread-serial merge of two labels per frontier entry, two read-backs a
-// level and batches of 1024; 12.2 ms so. What is left is launches: two
+// level and batches of 1024; 11.9 ms so. What is left is launches: two
 // directions of up to ten levels a batch, and a sort and a cleanup each.
 #include <algorithm>
 #include <new>
