@@ -996,24 +996,21 @@ PLL_API int pll_mlp_read_grad(const pll_mlp *p, float *host_grad, float *host_lo
     if (!p || (!host_grad && !host_loss)) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
     // gradient and loss in one copy into pinned memory (two into the caller's
-    // pageable arrays are staged ones, a wait each); one buffer per thread, as
-    // the call is synchronous. It lives as long as the thread.
-    static thread_local float *pinned = nullptr;
-    if (!pinned && cudaMallocHost(&pinned, (NP + 1) * sizeof(float)) != cudaSuccess) {
-        (void)cudaGetLastError();
-        pinned = nullptr;
-    }
-    if (!pinned) {
+    // pageable arrays are staged ones, a wait each)
+    static_assert((NP + 1) * sizeof(float) <= HOST_BLOCK_BYTES, "the gradient fits a host block");
+    HostBlock block(s);
+    if (!block.p) {
         if (host_grad) PLL_TRY(cudaMemcpyAsync(host_grad, p->grad, NP * sizeof(float), cudaMemcpyDeviceToHost, s));
         if (host_loss) PLL_TRY(cudaMemcpyAsync(host_loss, p->grad + NP, sizeof(float), cudaMemcpyDeviceToHost, s));
         PLL_TRY(cudaStreamSynchronize(s));
         return PLL_OK;
     }
+    float *h = block.as<float>();
     const size_t first = host_grad ? 0 : NP, last = host_loss ? NP + 1 : NP;
-    PLL_TRY(cudaMemcpyAsync(pinned + first, p->grad + first, (last - first) * sizeof(float), cudaMemcpyDeviceToHost, s));
-    PLL_TRY(cudaStreamSynchronize(s));
-    if (host_grad) std::memcpy(host_grad, pinned, NP * sizeof(float));
-    if (host_loss) *host_loss = pinned[NP];
+    PLL_TRY(cudaMemcpyAsync(h + first, p->grad + first, (last - first) * sizeof(float), cudaMemcpyDeviceToHost, s));
+    PLL_CHECK(block.wait());
+    if (host_grad) std::memcpy(host_grad, h, NP * sizeof(float));
+    if (host_loss) *host_loss = h[NP];
     return PLL_OK;
 }
 

@@ -664,6 +664,8 @@ namespace {
 std::mutex g_pool_mu;
 struct PoolEntry { unsigned long long ctx_id; cudaMemPool_t pool; };
 std::vector<PoolEntry> g_pools;
+struct BlockEntry { unsigned long long ctx_id; void *p; };
+std::vector<BlockEntry> g_blocks;  // host blocks not in use
 
 // unique id of the current context (false if there is none or the driver
 // cannot say)
@@ -712,43 +714,53 @@ cudaMemPool_t scratch_pool() {
     return pool;
 }
 
+// The host blocks are kept by context like the pools: a context destroyed by a
+// device reset takes its blocks with it, and no later call is given one of them.
+void *host_block_take(unsigned long long *ctx_id) {
+    *ctx_id = 0;
+    if (alloc_should_fail()) return nullptr;
+    void *p = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        if (current_ctx_id(ctx_id))
+            for (size_t i = g_blocks.size(); i-- > 0;)
+                if (g_blocks[i].ctx_id == *ctx_id) {
+                    p = g_blocks[i].p;
+                    g_blocks.erase(g_blocks.begin() + i);
+                    break;
+                }
+    }
+    if (!p && cudaMallocHost(&p, HOST_BLOCK_BYTES) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    alloc_note(1);
+    return p;
+}
+
+void host_block_give(void *p, unsigned long long ctx_id) {
+    alloc_note(-1);
+    if (ctx_id) {
+        std::lock_guard<std::mutex> lock(g_pool_mu);
+        size_t kept = 0;
+        for (const BlockEntry &e : g_blocks) kept += e.ctx_id == ctx_id;
+        if (kept < HOST_BLOCKS_KEPT) {
+            try {
+                g_blocks.push_back({ctx_id, p});
+                return;
+            } catch (const std::bad_alloc &) {
+            }
+        }
+    }
+    if (cudaFreeHost(p) != cudaSuccess) (void)cudaGetLastError();
+}
+
 namespace {
 
 // temporary device copy of a host array, stream ordered
 using AsyncBuf = PoolMem;
 
-// status of a synchronous call's launch once the stream is waited for: from the
-// thread's counters, or (without them) from the index's own
-int query_status(const pll_index *ix, const unsigned long long *err, cudaStream_t s) {
-    if (err != ix->d_qerr) {
-        PLL_TRY(cudaStreamSynchronize(s));
-        return error_status(err);
-    }
-    unsigned long long h[2] = {0, 0};
-    PLL_TRY(cudaMemcpyAsync(h, ix->d_qerr, 16, cudaMemcpyDeviceToHost, s));
-    PLL_TRY(cudaStreamSynchronize(s));
-    if (h[0] == 0 && h[1] == 0) return PLL_OK;
-    PLL_TRY(cudaMemsetAsync(ix->d_qerr, 0, 16, s));
-    PLL_TRY(cudaStreamSynchronize(s));
-    return error_status(h);
-}
-
-unsigned long long *query_errors_of(const pll_index *ix) {
-    unsigned long long *e = thread_errors();
-    return e ? e : ix->d_qerr;
-}
-
 }  // namespace
-
-unsigned long long *thread_errors() {
-    static thread_local unsigned long long *pinned = nullptr;
-    if (!pinned && cudaMallocHost(&pinned, 32) != cudaSuccess) {
-        (void)cudaGetLastError();
-        pinned = nullptr;
-    }
-    if (pinned) pinned[0] = pinned[1] = 0;
-    return pinned;
-}
 
 void index_release(pll_index *ix) { free_index(ix); }
 
@@ -801,6 +813,11 @@ PLL_API int pll_release_cached(void) {
     std::lock_guard<std::mutex> lock(g_pool_mu);
     unsigned long long id = 0;
     if (!current_ctx_id(&id)) return PLL_OK;
+    for (size_t i = g_blocks.size(); i-- > 0;)
+        if (g_blocks[i].ctx_id == id) {
+            cudaFreeHost(g_blocks[i].p);
+            g_blocks.erase(g_blocks.begin() + i);
+        }
     for (const PoolEntry &pe : g_pools)
         if (pe.ctx_id == id && (e = cudaMemPoolTrimTo(pe.pool, 0)) != cudaSuccess) return cuda_status(e);
     return PLL_OK;
@@ -929,9 +946,10 @@ PLL_API int pll_query(const pll_index *idx, const uint32_t *src, const uint32_t 
     if (q == 0) return PLL_OK;
     if (!src || !dst || !out) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long *err = query_errors_of(idx);
-    PLL_CHECK(query_launch(idx, src, dst, q, out, err, s));
-    return query_status(idx, err, s);
+    CallErrors err(s);
+    PLL_CHECK(err.begin(idx->d_qerr));
+    PLL_CHECK(query_launch(idx, src, dst, q, out, err.p, s));
+    return err.finish();
 }
 
 PLL_API int pll_query_host(const pll_index *idx, const uint32_t *src, const uint32_t *dst,
@@ -948,11 +966,12 @@ PLL_API int pll_query_host(const pll_index *idx, const uint32_t *src, const uint
         PLL_CHECK(dout.alloc(q));
         PLL_TRY(cudaMemcpyAsync(ds.p, src, q * 4, cudaMemcpyHostToDevice, s));
         PLL_TRY(cudaMemcpyAsync(dd.p, dst, q * 4, cudaMemcpyHostToDevice, s));
-        unsigned long long *err = query_errors_of(idx);
+        CallErrors err(s);
+        PLL_CHECK(err.begin(idx->d_qerr));
         PLL_CHECK(query_launch(idx, (const uint32_t *)ds.p, (const uint32_t *)dd.p, q,
-                               (uint8_t *)dout.p, err, s));
+                               (uint8_t *)dout.p, err.p, s));
         PLL_TRY(cudaMemcpyAsync(out, dout.p, q, cudaMemcpyDeviceToHost, s));
-        st = query_status(idx, err, s);
+        st = err.finish();
     }
     PLL_TRY(cudaStreamSynchronize(s));
     return st;

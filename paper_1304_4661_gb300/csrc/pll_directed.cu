@@ -546,27 +546,17 @@ PLL_API int pll_dquery(const pll_dindex *idx, const uint32_t *src, const uint32_
     if (q == 0) return PLL_OK;
     if (!src || !dst || !out) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    DQueryArgs a{idx->n, idx->d_inv, idx->d_off[0], idx->d_off[1], idx->d_lab[0], idx->d_lab[1],
-                 src, dst, q, out, thread_errors()};
-    const bool own = a.err != nullptr;
-    if (!own) a.err = idx->d_qerr;
+    CallErrors err(s);
+    PLL_CHECK(err.begin(idx->d_qerr));
+    const DQueryArgs a{idx->n, idx->d_inv, idx->d_off[0], idx->d_off[1], idx->d_lab[0], idx->d_lab[1],
+                       src, dst, q, out, err.p};
     int dev = 0, sms = 0;
     PLL_TRY(cudaGetDevice(&dev));
     PLL_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const uint64_t want = (q + 7) / 8, most = (uint64_t)(sms > 0 ? sms : 1) * 8;
     k_dquery<<<(unsigned)std::min(want, most), 256, 0, s>>>(a);
     PLL_TRY(cudaGetLastError());
-    if (own) {
-        PLL_TRY(cudaStreamSynchronize(s));
-        return error_status(a.err);
-    }
-    unsigned long long h[2] = {0, 0};
-    PLL_TRY(cudaMemcpyAsync(h, idx->d_qerr, 16, cudaMemcpyDeviceToHost, s));
-    PLL_TRY(cudaStreamSynchronize(s));
-    if (h[0] == 0 && h[1] == 0) return PLL_OK;
-    PLL_TRY(cudaMemsetAsync(idx->d_qerr, 0, 16, s));
-    PLL_TRY(cudaStreamSynchronize(s));
-    return h[1] ? PLL_E_INVAL : PLL_E_RANGE;
+    return err.finish();
 }
 
 PLL_API int pll_dlabel_entries(const pll_dindex *idx, uint64_t *in_entries, uint64_t *out_entries) {

@@ -205,6 +205,40 @@ struct DevMem {
     void *release() { void *q = p; p = nullptr; bytes = 0; return q; }
 };
 
+// Pinned host memory of one synchronous call: the words its kernels add errors to
+// directly, or the target of its copy back (a pageable target makes the copy a
+// staged one). Blocks of one size are kept per CUDA context (pll_abi.cu) for the
+// calls after it, at most HOST_BLOCKS_KEPT of them, until pll_release_cached; they
+// belong to no thread. A block goes back only once the call's stream has been
+// waited for, also where the call ends early, so nothing in flight can write to
+// another call's words. p is null if no block can be had.
+constexpr size_t HOST_BLOCK_BYTES = 20480;
+constexpr size_t HOST_BLOCKS_KEPT = 16;
+void *host_block_take(unsigned long long *ctx_id);
+void host_block_give(void *p, unsigned long long ctx_id);
+struct HostBlock {
+    void *p = nullptr;
+    cudaStream_t s;
+    explicit HostBlock(cudaStream_t st) : s(st) { p = host_block_take(&ctx_id); }
+    HostBlock(const HostBlock &) = delete;
+    HostBlock &operator=(const HostBlock &) = delete;
+    // waits for the stream: what the call's work wrote to the block can be read
+    int wait() {
+        const cudaError_t e = cudaStreamSynchronize(s);
+        waited = e == cudaSuccess;
+        return waited ? PLL_OK : cuda_status(e);
+    }
+    ~HostBlock() {
+        // a stream that cannot be waited for (a lost context, a capture): freed, not kept
+        if (p) host_block_give(p, waited || wait() == PLL_OK ? ctx_id : 0);
+    }
+    template <class T> T *as() const { return static_cast<T *>(p); }
+
+private:
+    unsigned long long ctx_id = 0;
+    bool waited = false;
+};
+
 // ---- launchers (one translation unit each) ----
 struct Graph {
     uint32_t n = 0;
@@ -473,14 +507,47 @@ int query_launch(const pll_index *ix, const uint32_t *d_src, const uint32_t *d_d
 int query_launch_strided(const pll_index *ix, const uint32_t *d_src, const uint32_t *d_dst,
                          uint32_t stride, uint64_t q, uint8_t *d_out, unsigned long long *err,
                          cudaStream_t s);
-// The calling thread's own pair of error counters, zeroed (with room for two more
-// words behind them): pinned host memory
-// that kernels add to directly (only where there is an error), so that a
-// synchronous call needs no copy to learn its status, only its wait. Null if it
-// cannot be had. One in use at a time per thread; it lives as long as the thread.
-unsigned long long *thread_errors();
 inline int error_status(const unsigned long long *h) {
     return h[1] ? PLL_E_INVAL : h[0] ? PLL_E_RANGE : PLL_OK;
 }
+// The error counters of one synchronous call (and two words more that it may copy
+// to): a host block that kernels add to directly (only where there is an error), so
+// that the call needs no copy to learn its status, only its wait.
+struct CallErrors {
+    HostBlock host;
+    cudaStream_t s;
+    unsigned long long *p = nullptr;
+    explicit CallErrors(cudaStream_t st) : host(st), s(st) {}
+    // `shared`: counters on the device that serve where there is no host block
+    int begin(unsigned long long *shared) {
+        p = host.as<unsigned long long>();
+        if (p) {
+            for (int i = 0; i < 4; ++i) p[i] = 0;
+            return PLL_OK;
+        }
+        p = shared;
+        return p ? PLL_OK : PLL_E_NOMEM;
+    }
+    // waits for the stream and reads the words; shared counters are cleared
+    int finish(unsigned long long (&h)[4]) {
+        if (host.p) {
+            PLL_CHECK(host.wait());
+            for (int i = 0; i < 4; ++i) h[i] = p[i];
+            return PLL_OK;
+        }
+        h[0] = h[1] = h[2] = h[3] = 0;
+        PLL_TRY(cudaMemcpyAsync(h, p, 16, cudaMemcpyDeviceToHost, s));
+        PLL_TRY(cudaStreamSynchronize(s));
+        if (h[0] == 0 && h[1] == 0) return PLL_OK;
+        PLL_TRY(cudaMemsetAsync(p, 0, 16, s));
+        PLL_TRY(cudaStreamSynchronize(s));
+        return PLL_OK;
+    }
+    int finish() {
+        unsigned long long h[4];
+        PLL_CHECK(finish(h));
+        return error_status(h);
+    }
+};
 
 }  // namespace pll

@@ -550,20 +550,21 @@ PLL_API int pll_path_offsets(const pll_paths *p, const uint32_t *src, const uint
     if (q >= 0x7fffffffull) return PLL_E_RANGE;
     cudaStream_t s = (cudaStream_t)stream;
     // the pairs' distances, then one scan of the lengths they stand for; the
-    // errors and the total come back in the thread's pinned counters
-    unsigned long long *h = thread_errors();
-    if (!h) return PLL_E_NOMEM;
+    // total comes back behind the call's error counters
+    CallErrors err(s);
+    PLL_CHECK(err.begin(nullptr));
     PoolMem dist(s), temp(s);
     PLL_CHECK(dist.alloc(q));
-    PLL_CHECK(query_launch(p->ix, src, dst, q, dist.as<uint8_t>(), h, s));
+    PLL_CHECK(query_launch(p->ix, src, dst, q, dist.as<uint8_t>(), err.p, s));
     auto lengths = thrust::make_transform_iterator(thrust::counting_iterator<uint64_t>(0),
                                                    PathLength{dist.as<uint8_t>(), q});
     size_t tb = 0;
     PLL_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, lengths, path_off, (int)(q + 1), s));
     PLL_CHECK(temp.alloc(tb));
     PLL_TRY(cub::DeviceScan::ExclusiveSum(temp.p, tb, lengths, path_off, (int)(q + 1), s));
-    PLL_TRY(cudaMemcpyAsync(h + 2, path_off + q, 8, cudaMemcpyDeviceToHost, s));
-    PLL_TRY(cudaStreamSynchronize(s));
+    PLL_TRY(cudaMemcpyAsync(err.p + 2, path_off + q, 8, cudaMemcpyDeviceToHost, s));
+    unsigned long long h[4];
+    PLL_CHECK(err.finish(h));
     *total = h[2];
     return error_status(h);
 }
@@ -574,24 +575,25 @@ PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32
     if (q == 0) return PLL_OK;
     if (!src || !dst || !path_off || (cap > 0 && !path)) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long *h = thread_errors();  // pinned: its first word takes the error bits
-    if (!h) return PLL_E_NOMEM;
+    CallErrors err(s);  // the first word takes the error bits
+    PLL_CHECK(err.begin(nullptr));
     PathArgs a{};
-    a.x = query_args(p->ix, src, dst, 1, q, nullptr, h);
+    a.x = query_args(p->ix, src, dst, 1, q, nullptr, err.p);
     a.order = p->ix->d_order; a.par = p->d_par;
     a.roff = p->d_roff; a.rcol = p->d_rcol;
     a.path_off = path_off;
     a.cap = cap;
     a.path = path;
-    a.err = reinterpret_cast<uint32_t *>(h);
+    a.err = reinterpret_cast<uint32_t *>(err.p);
     int blocks = 0;
     PLL_CHECK(warp_grid(q, PATH_BLOCKS, &blocks));
     // pairs a warp takes at once: up to 32, fewer while warps would be left idle
     const uint64_t per = q / ((uint64_t)blocks * 8);
     k_paths<<<blocks, 256, 0, s>>>(a, per >= 32 ? 32u : per > 1 ? (uint32_t)per : 1u);
     PLL_TRY(cudaGetLastError());
-    PLL_TRY(cudaStreamSynchronize(s));
-    return path_status(*reinterpret_cast<const uint32_t *>(h));
+    unsigned long long h[4];
+    PLL_CHECK(err.finish(h));
+    return path_status((uint32_t)h[0]);
 }
 
 PLL_API void pll_paths_free(pll_paths *p) { paths_release(p); }
