@@ -512,23 +512,28 @@ inline int error_status(const unsigned long long *h) {
 }
 // The error counters of one synchronous call (and two words more that it may copy
 // to): a host block that kernels add to directly (only where there is an error), so
-// that the call needs no copy to learn its status, only its wait.
+// that the call needs no copy to learn its status, only its wait. Where there is no
+// host block, words on the device: `shared` counters, or (without them) its own.
 struct CallErrors {
     HostBlock host;
+    PoolMem dev;
     cudaStream_t s;
     unsigned long long *p = nullptr;
-    explicit CallErrors(cudaStream_t st) : host(st), s(st) {}
-    // `shared`: counters on the device that serve where there is no host block
+    explicit CallErrors(cudaStream_t st) : host(st), dev(st), s(st) {}
     int begin(unsigned long long *shared) {
         p = host.as<unsigned long long>();
         if (p) {
             for (int i = 0; i < 4; ++i) p[i] = 0;
-            return PLL_OK;
+        } else if (shared) {
+            p = shared;
+        } else {
+            PLL_CHECK(dev.alloc(32));
+            p = dev.as<unsigned long long>();
+            PLL_TRY(cudaMemsetAsync(p, 0, 32, s));
         }
-        p = shared;
-        return p ? PLL_OK : PLL_E_NOMEM;
+        return PLL_OK;
     }
-    // waits for the stream and reads the words; shared counters are cleared
+    // waits for the stream and reads the words; shared counters (two) are cleared
     int finish(unsigned long long (&h)[4]) {
         if (host.p) {
             PLL_CHECK(host.wait());
@@ -536,9 +541,9 @@ struct CallErrors {
             return PLL_OK;
         }
         h[0] = h[1] = h[2] = h[3] = 0;
-        PLL_TRY(cudaMemcpyAsync(h, p, 16, cudaMemcpyDeviceToHost, s));
+        PLL_TRY(cudaMemcpyAsync(h, p, dev.p ? 32 : 16, cudaMemcpyDeviceToHost, s));
         PLL_TRY(cudaStreamSynchronize(s));
-        if (h[0] == 0 && h[1] == 0) return PLL_OK;
+        if (dev.p || (h[0] == 0 && h[1] == 0)) return PLL_OK;
         PLL_TRY(cudaMemsetAsync(p, 0, 16, s));
         PLL_TRY(cudaStreamSynchronize(s));
         return PLL_OK;

@@ -562,7 +562,7 @@ PLL_API int pll_path_offsets(const pll_paths *p, const uint32_t *src, const uint
     PLL_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, lengths, path_off, (int)(q + 1), s));
     PLL_CHECK(temp.alloc(tb));
     PLL_TRY(cub::DeviceScan::ExclusiveSum(temp.p, tb, lengths, path_off, (int)(q + 1), s));
-    PLL_TRY(cudaMemcpyAsync(err.p + 2, path_off + q, 8, cudaMemcpyDeviceToHost, s));
+    PLL_TRY(cudaMemcpyAsync(err.p + 2, path_off + q, 8, cudaMemcpyDefault, s));
     unsigned long long h[4];
     PLL_CHECK(err.finish(h));
     *total = h[2];

@@ -114,3 +114,40 @@ def test_many_threads_keep_their_statuses_apart():
     assert lib.pll_test_live_allocs() == live
     pll.release_cached()
     assert int(ix.query(good[:1], good[:1]).cpu()[0]) == 0
+
+
+def test_calls_without_a_block_of_host_memory():
+    """The first allocation of each call, its block, fails: the status comes back from device words."""
+    g = gg.ba(3000, 3, 4)
+    ix = gpu_build(g, 16)
+    off, col = dev_u32(g.offsets), dev_u32(g.cols)
+    paths, dix = pll.Paths(ix, off, col), pll.DirectedIndex(off, col)
+    net = pll.MLP(64)
+    net.set_params(gg.mlp_init(3))
+    x, t = dev_u32(np.ones((64, 8))).float(), dev_u32(np.zeros(64)).float()
+    s, d = (dev_u32(a) for a in gg.pairs(g.n, 5000, 9))
+    bad = dev_u32(np.full(5000, g.n, np.uint32))
+    room = paths.offsets(s, d)[0]
+    lib = pll.load()
+
+    def without(call, *args):
+        lib.pll_test_fail_alloc(0)
+        try:
+            r = call(*args)
+        except pll.PLLError as e:
+            return e.code
+        finally:
+            lib.pll_test_fail_alloc(-1)
+        r = r if isinstance(r, tuple) else (r,)
+        return [a.cpu().numpy().tolist() if hasattr(a, "cpu") else np.asarray(a).tolist() for a in r]
+
+    for call, good, wrong in ((ix.query, (s, d), (bad, d)), (dix.query, (s, d), (s, bad)),
+                              (paths.offsets, (s, d), (bad, d)), (paths.query, (s, d, room), (s, bad, room)),
+                              (net.grad, (x, t), None)):
+        want = call(*good)
+        want = want if isinstance(want, tuple) else (want,)
+        want = [a.cpu().numpy().tolist() if hasattr(a, "cpu") else np.asarray(a).tolist() for a in want]
+        for _ in range(2):
+            if wrong:
+                assert without(call, *wrong) == pll.PLL_E_INVAL
+            assert without(call, *good) == want
