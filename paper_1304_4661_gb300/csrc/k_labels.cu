@@ -285,11 +285,13 @@ int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_t
 // costs 33 and 41 ms more in the append). A store of fewer than NEAR_MIN entries
 // has none: builds that small are launches (BA-10k, R-MAT-15 both ways: no
 // difference with a line at 65536 or none). It doubles the store's memory: it is
-// kept up while it takes at most an eighth of the memory that is free (an older
-// copy stays good, and without one the test sweep reads whole labels).
+// kept up while it takes at most an eighth of the memory that is free and can be
+// had (an older copy stays good, and without one the test sweep reads whole
+// labels; it is asked for again when the store has grown by another quarter).
 constexpr uint64_t NEAR_MIN = 1 << 18, NEAR_GROWTH_PCT = 25;
 int labels_near(LabelStore &st, uint64_t total, cudaStream_t s) {
-    if (total < NEAR_MIN || total < st.near_total + st.near_total / 100 * NEAR_GROWTH_PCT) return PLL_OK;
+    if (total < NEAR_MIN || total < st.near_asked + st.near_asked / 100 * NEAR_GROWTH_PCT) return PLL_OK;
+    st.near_asked = total;
     if (st.near_cap < st.pool_cap) {
         const uint64_t per_vertex = (uint64_t)st.n * (sizeof(NearLabel) + NEAR_CLASSES * 4);
         size_t free_b = 0, total_b = 0;
@@ -300,11 +302,12 @@ int labels_near(LabelStore &st, uint64_t total, cudaStream_t s) {
         if (st.pool_cap * 4 + per_vertex > free_b / 8) return PLL_OK;
         pool_free(st.near, s);
         st.near = nullptr;
+        st.near_cap = 0;
         PoolMem near(s), lab(s), end(s);
-        PLL_CHECK(near.alloc(st.pool_cap * 4));
+        if (near.alloc(st.pool_cap * 4) != PLL_OK) return PLL_OK;
         if (!st.near_lab) {
-            PLL_CHECK(lab.alloc((size_t)st.n * sizeof(NearLabel)));
-            PLL_CHECK(end.alloc((size_t)st.n * NEAR_CLASSES * 4));
+            if (lab.alloc((size_t)st.n * sizeof(NearLabel)) != PLL_OK) return PLL_OK;
+            if (end.alloc((size_t)st.n * NEAR_CLASSES * 4) != PLL_OK) return PLL_OK;
             st.near_lab = static_cast<NearLabel *>(lab.release());
             st.near_end = static_cast<uint32_t *>(end.release());
         }
@@ -313,7 +316,7 @@ int labels_near(LabelStore &st, uint64_t total, cudaStream_t s) {
     }
     k_near<<<grid_for((uint64_t)st.n * 32, NEAR_THREADS), NEAR_THREADS, 0, s>>>(st);
     PLL_TRY(cudaGetLastError());
-    st.near_total = total;
+    ++st.near_rebuilds;
     return PLL_OK;
 }
 

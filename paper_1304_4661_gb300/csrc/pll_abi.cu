@@ -442,9 +442,9 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             ix->stats.launches += 2;   // cleanup, append
             ix->stats.cub_calls += 2;  // sort, select
             // (the builds with small test tables run without the near copy)
-            const uint64_t near_before = st.near_total;
+            const uint64_t near_before = st.near_rebuilds;
             if (!caps.ht) PLL_CHECK(labels_near(st, total, s));
-            ix->stats.launches += st.near_total != near_before;
+            ix->stats.launches += st.near_rebuilds - near_before;
             PLL_TRY(cudaEventRecord(ev[3], s));
             post_pending = true;
         }

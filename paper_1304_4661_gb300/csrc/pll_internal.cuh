@@ -471,7 +471,9 @@ struct LabelStore {
     uint64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
     uint32_t *near = nullptr;        // [near_cap] the near copy, or null
-    uint64_t near_cap = 0, near_total = 0;
+    uint64_t near_cap = 0;
+    uint64_t near_asked = 0;         // entries of the store when a copy was last asked for
+    uint64_t near_rebuilds = 0;
     NearLabel *near_lab = nullptr;   // [n]
     uint32_t *near_end = nullptr;    // [NEAR_CLASSES][n] its entries of distance <= c
     bool pooled = false;  // `pool` comes from pool_malloc (else dev_malloc)
@@ -490,7 +492,8 @@ int labels_append(const LabelStore &st, const uint64_t *d_kept,
                   const unsigned long long *d_nkept, uint64_t max_count, uint32_t *d_err,
                   cudaStream_t s);
 int labels_regrow(LabelStore &st, uint64_t new_cap, cudaStream_t s);
-// rebuilds the near copy if the store (of `total` entries) has outgrown it
+// rebuilds the near copy if the store (of `total` entries) has outgrown it; a
+// store that no memory can be had for goes without one
 int labels_near(LabelStore &st, uint64_t total, cudaStream_t s);
 void labels_near_free(LabelStore &st, cudaStream_t s);
 int labels_finalize(const LabelStore &st, uint64_t total, uint64_t *d_off, uint32_t *d_lab,

@@ -1,0 +1,61 @@
+"""Memory that a build can do without: every allocation of a build is made to fail
+in turn. Those that only save time must not fail the build, and whatever the
+build then goes without, its labels are the same."""
+import gc
+
+import numpy as np
+import pytest
+
+from paper_1304_4661_gb300 import graphgen as gg
+from paper_1304_4661_gb300 import pll
+
+from .gpu_util import dev_u32, same_labels
+
+pytestmark = pytest.mark.gpu
+
+OK, NOMEM = pll.PLL_OK, pll.PLL_E_NOMEM
+
+
+def outcomes(build, labels, most):
+    """The status of the build with its k-th allocation failing, up to the last one that ends it."""
+    lib = pll.load()
+    ix = build()
+    want = labels(ix)
+    ix.close()
+    gc.collect()
+    base, codes = lib.pll_test_live_allocs(), []
+    for k in range(most):
+        lib.pll_test_fail_alloc(k)
+        try:
+            ix = build()
+        except pll.PLLError as e:
+            codes.append(e.code)
+        else:
+            codes.append(OK)
+            lib.pll_test_fail_alloc(-1)
+            assert all(same_labels(a, b) for a, b in zip(labels(ix), want)), k
+            ix.close()
+        finally:
+            lib.pll_test_fail_alloc(-1)
+        assert lib.pll_test_live_allocs() == base, k
+    assert set(codes) == {OK, NOMEM} and codes[-1] == OK  # the last ones fail nothing
+    return codes[:len(codes) - codes[::-1].index(NOMEM)]
+
+
+def undirected(g, t, **kw):
+    off, col = dev_u32(g.offsets), dev_u32(g.cols)
+    return lambda: pll.Index.build(off, col, t=t, **kw), lambda ix: [ix.labels()]
+
+
+def directed(g, **kw):
+    off, col = dev_u32(g.offsets), dev_u32(g.cols)
+    return lambda: pll.DirectedIndex(off, col, **kw), lambda ix: [ix.labels_in(), ix.labels_out()]
+
+
+@pytest.mark.parametrize("make", [lambda: undirected(gg.ba(20000, 6, 7), 0), lambda: undirected(gg.ba(20000, 6, 7), 0, root_batch=500),
+                                  lambda: directed(gg.oriented(gg.ba(20000, 6, 7), 3, both=0.3))],
+                         ids=["default", "batches-of-500", "directed"])
+def test_a_store_without_its_near_copy(make):
+    """Over 2M entries: the near copy is rebuilt several times, and each of its allocations may fail."""
+    codes = outcomes(*make(), most=160)
+    assert codes.count(OK) >= 3
