@@ -181,10 +181,13 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     }
     uint64_t ht_cap = caps.ht ? caps.ht : std::max<uint64_t>({(uint64_t)std::min(bmax, BATCH_FULL) * 2048,
                                                                 (uint64_t)bmax * 512, 1ull << 20});
-    PLL_CHECK(m_ht.alloc(ht_cap * 4));
-    PLL_CHECK(m_tab.alloc((size_t)bmax * 8));
     PoolMem m_reach(s);
-    PLL_CHECK(m_reach.alloc(ht_cap * 4));
+    auto alloc_tables = [&]() -> int {
+        PLL_CHECK(m_ht.alloc(ht_cap * 4));
+        return m_reach.alloc(ht_cap * 4);
+    };
+    PLL_CHECK(alloc_tables());
+    PLL_CHECK(m_tab.alloc((size_t)bmax * 8));
     uint64_t cand_cap = caps.cand ? caps.cand
                                   : std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 256, free_b / 16 / 24),
                                                        1ull << 24);
@@ -208,8 +211,11 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         PLL_CHECK(m_temp.alloc(temp_bytes));
         return PLL_OK;
     };
-    PLL_CHECK(m_cand.alloc(cand_cap * 8));
-    PLL_CHECK(m_candc.alloc(cand_cap * 16));
+    auto alloc_cand = [&]() -> int {
+        PLL_CHECK(m_cand.alloc(cand_cap * 8));
+        return m_candc.alloc(cand_cap * 16);
+    };
+    PLL_CHECK(alloc_cand());
     PLL_CHECK(alloc_out());
     PoolMem m_rstart(s);
     PLL_CHECK(m_rstart.alloc((size_t)n * 4));
@@ -292,15 +298,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         // not under the test capacities, which exist to make batches overflow)
         if (!caps.cand && !caps.out) {
             const double f = 1.5 * (double)(k1 - k0) / (double)last_B;
-            if ((double)last_cand * f > (double)cand_cap) {
-                cand_cap = (uint64_t)((double)last_cand * f);
-                PLL_CHECK(m_cand.alloc(cand_cap * 8));
-                PLL_CHECK(m_candc.alloc(cand_cap * 16));
-            }
-            if ((double)last_out * f > (double)out_cap) {
-                out_cap = (uint64_t)((double)last_out * f);
-                PLL_CHECK(alloc_out());
-            }
+            PLL_CHECK(grow_if_possible(cand_cap, (uint64_t)((double)last_cand * f), alloc_cand));
+            PLL_CHECK(grow_if_possible(out_cap, (uint64_t)((double)last_out * f), alloc_out));
         }
         if (k1 - k0 > zeroed) {  // rows used for the first time
             PLL_TRY(cudaMemsetAsync(m_vis.as<uint32_t>() + (size_t)zeroed * NW, 0, (size_t)(k1 - k0 - zeroed) * NW * 4, s));
@@ -390,11 +389,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             // binary-searched (same answers); grow the pool for later batches
             const uint64_t need = h->c.ht_top;
             ix->stats.table_fallbacks += 1;
-            if (!caps.ht) {  // the test capacity keeps the pool small for the whole build
-                ht_cap = std::max<uint64_t>(need + need / 4, ht_cap * 2);
-                PLL_CHECK(m_ht.alloc(ht_cap * 4));
-                PLL_CHECK(m_reach.alloc(ht_cap * 4));
-            }
+            if (!caps.ht)  // the test capacity keeps the pool small for the whole build
+                PLL_CHECK(grow_if_possible(ht_cap, std::max<uint64_t>(need + need / 4, ht_cap * 2), alloc_tables));
             h->c.err &= ~ERR_TABLE;
         }
         if (h->c.err & ERR_BUF) {  // a buffer overflowed: grow and redo the batch
@@ -402,8 +398,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             PLL_TRY(cudaMemcpyAsync(d_ctr->work, work0, sizeof(work0), cudaMemcpyHostToDevice, s));
             if (h->c.cand_n > cand_cap) {
                 cand_cap = std::max<uint64_t>(cand_cap * 2, h->c.cand_n + h->c.cand_n / 4);
-                PLL_CHECK(m_cand.alloc(cand_cap * 8));
-                PLL_CHECK(m_candc.alloc(cand_cap * 16));
+                PLL_CHECK(alloc_cand());
             }
             if (h->c.out_n > out_cap) {
                 out_cap = std::max<uint64_t>(out_cap * 2, h->c.out_n + h->c.out_n / 4);

@@ -325,8 +325,11 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     PLL_CHECK(inX.alloc(n));
     PLL_TRY(cudaMemsetAsync(inX.p, 0, n, s));
     uint64_t ht_cap = std::max<uint64_t>((uint64_t)bmax * 1024, 1ull << 18);
-    PLL_CHECK(ht.alloc(ht_cap * 4));
-    PLL_CHECK(reach.alloc(ht_cap * 4));
+    auto alloc_tables = [&]() -> int {
+        PLL_CHECK(ht.alloc(ht_cap * 4));
+        return reach.alloc(ht_cap * 4);
+    };
+    PLL_CHECK(alloc_tables());
     PLL_CHECK(tab.alloc((size_t)bmax * 8));
     const uint64_t slice_cap = std::min<uint64_t>(std::max<uint64_t>(ix->nnz, 1ull << 16), SLICE_CAP);
     PLL_CHECK(slices.alloc(slice_cap * 16));
@@ -422,9 +425,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         const uint32_t err = h->d.c[0].err | h->d.c[1].err;
         if (err & ERR_TABLE) {  // those roots were binary-searched; grow for later batches
             const uint64_t need = std::max(h->d.c[0].ht_top, h->d.c[1].ht_top);
-            ht_cap = std::max<uint64_t>(need + need / 4, ht_cap * 2);
-            PLL_CHECK(ht.alloc(ht_cap * 4));
-            PLL_CHECK(reach.alloc(ht_cap * 4));
+            PLL_CHECK(grow_if_possible(ht_cap, std::max<uint64_t>(need + need / 4, ht_cap * 2), alloc_tables));
         }
         if (err & ERR_BUF) {
             const uint64_t nc = std::max(h->d.c[0].cand_n, h->d.c[1].cand_n), no = std::max(h->d.c[0].out_n, h->d.c[1].out_n);

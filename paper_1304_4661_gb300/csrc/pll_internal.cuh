@@ -395,6 +395,19 @@ inline uint32_t default_batch(uint32_t n, uint64_t limit, uint32_t least) {
     return b;
 }
 
+// A buffer that would serve better with `want` entries than with the `cap` it has,
+// but need not grow (batches that overflow run again, roots without a table are
+// searched): where the memory for more cannot be had it keeps its size. `alloc`
+// allocates it at `cap`.
+template <class F> int grow_if_possible(uint64_t &cap, uint64_t want, F &&alloc) {
+    if (want <= cap) return PLL_OK;
+    const uint64_t had = cap;
+    cap = want;
+    if (alloc() == PLL_OK) return PLL_OK;
+    cap = had;
+    return alloc();
+}
+
 struct BatchArgs {
     uint32_t n, t, tp;
     const uint32_t *roff, *rcol;

@@ -9,6 +9,7 @@ import pytest
 from paper_1304_4661_gb300 import graphgen as gg
 from paper_1304_4661_gb300 import pll
 
+from . import graphs
 from .gpu_util import dev_u32, same_labels
 
 pytestmark = pytest.mark.gpu
@@ -59,3 +60,10 @@ def test_a_store_without_its_near_copy(make):
     """Over 2M entries: the near copy is rebuilt several times, and each of its allocations may fail."""
     codes = outcomes(*make(), most=160)
     assert codes.count(OK) >= 3
+
+
+def test_buffers_grown_ahead_of_demand():
+    """Every root of the first batch labels every vertex (3.84M tuples, all but 120,000 dropped again);
+    the tuple buffers are grown for the second, which would have fitted."""
+    codes = outcomes(*undirected(graphs.star(60000), 0), most=120)
+    assert codes.count(OK) >= 4  # the tuples, sorted, their marks, the sort's space
