@@ -290,7 +290,7 @@ int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_t
 // labels; it is asked for again when the store has grown by another quarter).
 constexpr uint64_t NEAR_MIN = 1 << 18, NEAR_GROWTH_PCT = 25;
 int labels_near(LabelStore &st, uint64_t total, cudaStream_t s) {
-    if (total < NEAR_MIN || total < st.near_asked + st.near_asked / 100 * NEAR_GROWTH_PCT) return PLL_OK;
+    if (st.near_given_back || total < NEAR_MIN || total < st.near_asked + st.near_asked / 100 * NEAR_GROWTH_PCT) return PLL_OK;
     st.near_asked = total;
     if (st.near_cap < st.pool_cap) {
         const uint64_t per_vertex = (uint64_t)st.n * (sizeof(NearLabel) + NEAR_CLASSES * 4);
@@ -327,6 +327,21 @@ void labels_near_free(LabelStore &st, cudaStream_t s) {
     st.near = nullptr;
     st.near_lab = nullptr;
     st.near_end = nullptr;
+}
+
+bool labels_near_give_back(LabelStore *const *st, int count, cudaStream_t s) {
+    bool any = false;
+    for (int i = 0; i < count; ++i) {
+        any |= st[i]->near_lab != nullptr || st[i]->near != nullptr;
+        labels_near_free(*st[i], s);
+        st[i]->near_given_back = true;
+    }
+    if (!any) return false;
+    const cudaMemPool_t pool = scratch_pool();
+    // the index's arrays are not the pool's: unmap what the pool no longer uses
+    if (cudaStreamSynchronize(s) != cudaSuccess || (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess))
+        (void)cudaGetLastError();
+    return true;
 }
 
 // Rewrites the pool (capacity = length rounded up to 4 entries, so arrays

@@ -273,6 +273,9 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
         PLL_CHECK(batch_graph_build(block, grid, m_args.as<BatchArgs>(), &lgraph, &lexec));
     }
 
+    // allocations past this point that the build cannot do without
+    LabelStore *const stores[] = {&st};
+    auto needed = [&](auto &&alloc) { return alloc_needed(stores, 1, s, alloc); };
     uint64_t total = 0, pre = 0, batches = 0;
     // A batch's sort, cleanup, compaction and append are not waited for: the
     // next batch is enqueued right behind them, and its first read-back
@@ -398,11 +401,11 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             PLL_TRY(cudaMemcpyAsync(d_ctr->work, work0, sizeof(work0), cudaMemcpyHostToDevice, s));
             if (h->c.cand_n > cand_cap) {
                 cand_cap = std::max<uint64_t>(cand_cap * 2, h->c.cand_n + h->c.cand_n / 4);
-                PLL_CHECK(alloc_cand());
+                PLL_CHECK(needed(alloc_cand));
             }
             if (h->c.out_n > out_cap) {
                 out_cap = std::max<uint64_t>(out_cap * 2, h->c.out_n + h->c.out_n / 4);
-                PLL_CHECK(alloc_out());
+                PLL_CHECK(needed(alloc_out));
             }
             continue;
         }
@@ -417,7 +420,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
             const uint64_t need = h->c.pool_top + 2 * (total + P) + 12 * P;
             if (need > st.pool_cap) {
                 uint64_t nc = std::max<uint64_t>(st.pool_cap * 2, 3 * (total + P) + 12 * P);
-                PLL_CHECK(labels_regrow(st, nc, s));
+                PLL_CHECK(needed([&] { return labels_regrow(st, nc, s); }));
                 ix->stats.pool_regrows += 1;
                 ix->stats.launches += 3;
                 ix->stats.cub_calls += 1;
@@ -473,12 +476,12 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     ix->entries = total;
 
     // step 4: compact CSR
-    PLL_TRY(dev_malloc(&ix->d_lab_off, ((size_t)n + 1) * 8));
-    PLL_TRY(dev_malloc(&ix->d_lab, std::max<uint64_t>(total, 1) * 4));
+    PLL_CHECK(needed([&]() -> int { PLL_TRY(dev_malloc(&ix->d_lab_off, ((size_t)n + 1) * 8)); return PLL_OK; }));
+    PLL_CHECK(needed([&]() -> int { PLL_TRY(dev_malloc(&ix->d_lab, std::max<uint64_t>(total, 1) * 4)); return PLL_OK; }));
     size_t ftb = 0;
     PLL_CHECK(labels_finalize(st, total, ix->d_lab_off, ix->d_lab, nullptr, &ftb, s));
     PoolMem ftemp(s);
-    PLL_CHECK(ftemp.alloc(ftb));
+    PLL_CHECK(needed([&] { return ftemp.alloc(ftb); }));
     Timer tf(s);
     tf.start();
     PLL_CHECK(labels_finalize(st, total, ix->d_lab_off, ix->d_lab, ftemp.p, &ftb, s));

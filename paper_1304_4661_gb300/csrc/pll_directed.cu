@@ -400,6 +400,9 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         return PLL_OK;
     };
     // the kept counts of a batch arrive with the next batch's read-back
+    // allocations past this point that the build cannot do without
+    LabelStore *const stores[] = {&store[0].st, &store[1].st};
+    auto needed = [&](auto &&alloc) { return alloc_needed(stores, 2, s, alloc); };
     uint64_t total[2] = {0, 0};
     bool pending[2] = {false, false};
     auto settle = [&]() -> int {
@@ -431,11 +434,11 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
             const uint64_t nc = std::max(h->d.c[0].cand_n, h->d.c[1].cand_n), no = std::max(h->d.c[0].out_n, h->d.c[1].out_n);
             if (nc > cand_cap) {
                 cand_cap = std::max<uint64_t>(cand_cap * 2, nc + nc / 4);
-                PLL_CHECK(alloc_cand());
+                PLL_CHECK(needed(alloc_cand));
             }
             if (no > out_cap) {
                 out_cap = std::max<uint64_t>(out_cap * 2, no + no / 4);
-                PLL_CHECK(alloc_out());
+                PLL_CHECK(needed(alloc_out));
             }
             continue;
         }
@@ -460,7 +463,9 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
             // worst-case pool growth of one append: 2 x (entries + new) + 8 per run
             const uint64_t need = h->d.c[dir].pool_top + 2 * (total[dir] + P[dir]) + 12 * P[dir];
             if (need > st.pool_cap)
-                PLL_CHECK(labels_regrow(st, std::max<uint64_t>(st.pool_cap * 2, 3 * (total[dir] + P[dir]) + 12 * P[dir]), s));
+                PLL_CHECK(needed([&] {
+                    return labels_regrow(st, std::max<uint64_t>(st.pool_cap * 2, 3 * (total[dir] + P[dir]) + 12 * P[dir]), s);
+                }));
             PLL_CHECK(labels_cleanup(sorted[dir].as<uint64_t>(), P[dir], sorted[1 - dir].as<uint64_t>(), P[1 - dir],
                                      keep.as<uint8_t>(), k0, Bc, temp.p, temp.bytes, s));
             size_t tb = temp.bytes;
@@ -477,11 +482,11 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     PLL_CHECK(read_back());
     PLL_CHECK(settle());
     for (int dir = 0; dir < 2; ++dir) {
-        PLL_TRY(dev_malloc(&ix->d_off[dir], ((size_t)n + 1) * 8));
-        PLL_TRY(dev_malloc(&ix->d_lab[dir], std::max<uint64_t>(total[dir], 1) * 4));
+        PLL_CHECK(needed([&]() -> int { PLL_TRY(dev_malloc(&ix->d_off[dir], ((size_t)n + 1) * 8)); return PLL_OK; }));
+        PLL_CHECK(needed([&]() -> int { PLL_TRY(dev_malloc(&ix->d_lab[dir], std::max<uint64_t>(total[dir], 1) * 4)); return PLL_OK; }));
         size_t ftb = 0;
         PLL_CHECK(labels_finalize(store[dir].st, total[dir], ix->d_off[dir], ix->d_lab[dir], nullptr, &ftb, s));
-        PLL_CHECK(temp.alloc(std::max<size_t>(ftb, 16)));
+        PLL_CHECK(needed([&] { return temp.alloc(std::max<size_t>(ftb, 16)); }));
         PLL_CHECK(labels_finalize(store[dir].st, total[dir], ix->d_off[dir], ix->d_lab[dir], temp.p, &ftb, s));
         ix->entries[dir] = total[dir];
     }

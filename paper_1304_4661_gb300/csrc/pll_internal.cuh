@@ -487,6 +487,7 @@ struct LabelStore {
     uint64_t near_cap = 0;
     uint64_t near_asked = 0;         // entries of the store when a copy was last asked for
     uint64_t near_rebuilds = 0;
+    bool near_given_back = false;    // its memory was needed: no copy any more
     NearLabel *near_lab = nullptr;   // [n]
     uint32_t *near_end = nullptr;    // [NEAR_CLASSES][n] its entries of distance <= c
     bool pooled = false;  // `pool` comes from pool_malloc (else dev_malloc)
@@ -509,6 +510,15 @@ int labels_regrow(LabelStore &st, uint64_t new_cap, cudaStream_t s);
 // store that no memory can be had for goes without one
 int labels_near(LabelStore &st, uint64_t total, cudaStream_t s);
 void labels_near_free(LabelStore &st, cudaStream_t s);
+// The near copies of `count` stores, handed back to the device for good (where
+// there are any: false if there were none).
+bool labels_near_give_back(LabelStore *const *st, int count, cudaStream_t s);
+// `alloc` allocates what the build cannot do without: where that fails the near
+// copies make room for it.
+template <class F> int alloc_needed(LabelStore *const *st, int count, cudaStream_t s, F &&alloc) {
+    const int status = alloc();
+    return status == PLL_E_NOMEM && labels_near_give_back(st, count, s) ? alloc() : status;
+}
 int labels_finalize(const LabelStore &st, uint64_t total, uint64_t *d_off, uint32_t *d_lab,
                     void *d_temp, size_t *temp_bytes, cudaStream_t s);
 int scan_u32_to_u64(const uint32_t *d_in, uint64_t *d_out, uint32_t n, void *d_temp,
