@@ -220,7 +220,7 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PoolMem m_rstart(s);
     PLL_CHECK(m_rstart.alloc((size_t)n * 4));
     PoolMem m_slices(s);
-    const uint64_t slice_cap = caps.cand ? std::min<uint64_t>(caps.cand, SLICE_CAP) : SLICE_CAP;
+    const uint64_t slice_cap = caps.cand ? std::min<uint64_t>(caps.cand, SLICE_CAP) : slice_entries(ix->nnz, free_b);
     PLL_CHECK(m_slices.alloc(slice_cap * 16));
 
     // pinned mirror of the counters and the level descriptor

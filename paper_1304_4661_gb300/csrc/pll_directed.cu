@@ -331,13 +331,13 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     };
     PLL_CHECK(alloc_tables());
     PLL_CHECK(tab.alloc((size_t)bmax * 8));
-    const uint64_t slice_cap = std::min<uint64_t>(std::max<uint64_t>(ix->nnz, 1ull << 16), SLICE_CAP);
-    PLL_CHECK(slices.alloc(slice_cap * 16));
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         (void)cudaGetLastError();
         free_b = 0;
     }
+    const uint64_t slice_cap = slice_entries(ix->nnz, free_b);
+    PLL_CHECK(slices.alloc(slice_cap * 16));
     uint64_t cand_cap = std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 128, free_b / 16 / 24), 1ull << 16);
     uint64_t out_cap = std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 64, free_b / 16 / 33), 1ull << 16);
     const int end_bit = 32 + [&] { int b = 1; while (b < 24 && ((n - 1) >> b)) ++b; return b; }();

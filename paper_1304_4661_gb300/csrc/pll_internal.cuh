@@ -303,7 +303,14 @@ __host__ __device__ inline uint32_t ht_size(uint32_t len) {
 // left with a hub's list while the others are done (R-MAT-20's expand sweeps: 55.3,
 // 57.0, 59.1, 64 ms with slices of 64, 128, 256, 512).
 constexpr uint32_t SLICE = 64;
-constexpr uint64_t SLICE_CAP = 64ull << 20;  // slices of one level; past it entries stay whole
+// Slices of one level that a build has room for (16 bytes each; a level with more
+// expands its entries whole): one for every arc, which a first batch's 64 roots do
+// not exceed, between 1 MiB and 1 GiB, and at most a sixteenth of the free memory.
+constexpr uint64_t SLICE_CAP = 64ull << 20;
+inline uint64_t slice_entries(uint64_t nnz, uint64_t free_b) {
+    const uint64_t most = std::min<uint64_t>(SLICE_CAP, free_b / 16 / 16);
+    return std::max<uint64_t>(std::min(nnz, most), 1ull << 16);
+}
 
 struct BatchCounters {
     unsigned long long cand_n;    // candidates appended (all levels of the batch)

@@ -96,3 +96,12 @@ def test_the_near_copy_makes_room_for_what_the_build_needs(make, after):
     `after`: one of them failing costs the near copy, not the build."""
     codes = outcomes(*make())
     assert codes[len(codes) - after - 3:len(codes) - after] == [OK, OK, OK]
+
+
+def test_a_small_graph_needs_little_scratch():
+    """2000 vertices: the least candidate, tuple and label buffers are 0.55 GB, and nothing else that a
+    build holds has a fixed size of more than a few MB."""
+    g = gg.ba(2000, 3, 1)
+    with_roots = undirected(g, 16)[0]()
+    assert 0 < with_roots.stats()["scratch_peak_bytes"] < 0.8e9
+    with_roots.close()
