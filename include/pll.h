@@ -207,8 +207,9 @@ PLL_API int pll_build_batch(const uint32_t *offsets, const uint32_t *cols, uint3
 /*
  * pll_autotune -- pick the pruned-stage batch size and block shape for a
  * graph (or, with graph_start, a batch of graphs as for pll_build_batch) by
- * timing trial builds: root_batch in {1024, 2048, 4096, 8192, 16384} at block
- * 256, then block in {128, 512} at the best root_batch (7 builds, CUDA-event
+ * timing trial builds: root_batch in {1024, 2048, 4096, 8192, 16384}, and in
+ * {32768, 65536} up to the library's default and the graph's size, at block
+ * 256, then block in {128, 512} at the best root_batch (7 to 9 builds, CUDA-event
  * timed on the stream). Writes the fastest options (t included) to *best and
  * their build time to *best_ms (may be NULL). The labels are the same for
  * every choice; only the time differs. Synchronous.

@@ -491,6 +491,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     return PLL_OK;
 }
 
+uint32_t undirected_batch(uint32_t n) { return default_batch(n, 8ull << 30, 1024); }
+
 // graph_start: null for one graph; else host uint32[graphs + 1] vertex ranges
 // of graphs built together as one disjoint union.
 int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t nnz,
@@ -510,7 +512,7 @@ int build_device(const uint32_t *off, const uint32_t *col, uint32_t n, uint64_t 
     if (n == 0 && nnz != 0) return PLL_E_INVAL;
     uint32_t block = o.block ? o.block : 256;
     if (block != 128 && block != 256 && block != 512 && block != 1024) return PLL_E_INVAL;
-    const uint32_t bmax = std::max(1u, std::min({n, o.root_batch ? o.root_batch : default_batch(n, 8ull << 30, 1024), BATCH_MAX}));
+    const uint32_t bmax = std::max(1u, std::min({n, o.root_batch ? o.root_batch : undirected_batch(n), BATCH_MAX}));
     const bool batch = graph_start != nullptr;
     if (!batch) graphs = 1;
     if (batch) {
@@ -909,8 +911,9 @@ PLL_API int pll_autotune(const uint32_t *offsets, const uint32_t *cols, uint32_t
         return PLL_OK;
     };
     // root-batch sizes at the default block, then block shapes at the best size
-    static const uint32_t batches[] = {1024, 2048, 4096, 8192, 16384};
-    for (uint32_t rb : batches) PLL_CHECK(trial(rb, 256));
+    uint32_t sizes[7];
+    const int count = autotune_batches(n, undirected_batch(n), sizes);
+    for (int i = 0; i < count; ++i) PLL_CHECK(trial(sizes[i], 256));
     const uint32_t rb = bo.root_batch;
     static const uint32_t blocks[] = {128, 512};
     for (uint32_t bl : blocks) PLL_CHECK(trial(rb, bl));
