@@ -43,6 +43,9 @@ template <int PG>
 __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
     __shared__ uint32_t s_keep[8][KEEP];
     __shared__ OpenPair s_pair[8][PG];
+    __shared__ uint32_t s_errors[2];
+    if (threadIdx.x < 2) s_errors[threadIdx.x] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     uint32_t *keep = s_keep[threadIdx.x >> 5];
     OpenPair *pair = s_pair[threadIdx.x >> 5];
@@ -64,13 +67,13 @@ __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
                 p.lt = (uint32_t)(a.lab_off[p.t + 1] - p.ot);
                 uint32_t d, hub, ds;
                 if (lone_pair(a, p.s, p.os, p.ls, p.t, p.ot, p.lt, &d, &hub, &ds)) {
-                    ans = answer_byte(a, d);
+                    ans = pair_answer(d);
                     open = false;
                 } else {
                     pair[lane] = p;
                 }
             } else if (bad) {
-                atomicAdd_system(a.err + 1, 1ull);
+                ans |= ANS_BAD;
             }
         }
         __syncwarp();
@@ -78,13 +81,19 @@ __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
             const int j = __ffs(m) - 1;
             const OpenPair p = pair[j];
             const uint32_t best = pair_bounded(a, p, lane, keep);
-            if (lane == j) ans = answer_byte(a, best);  // best is the same on every lane
+            if (lane == j) ans = pair_answer(best);  // best is the same on every lane
         }
         // the group's answers in one coalesced store (the output may be host
         // memory that the GPU writes directly)
         if (mine) a.out[qi] = (uint8_t)ans;
+        count_errors(s_errors, ans, lane);
         __syncwarp();  // the next group writes pair
     }
+    // the block's errors at once: the counters may be host memory, where an addition
+    // costs 12 ns (10M pairs, every id out of range: 3.6 ms with one a group, 0.07 so)
+    __syncthreads();
+    if (threadIdx.x < 2 && s_errors[threadIdx.x])
+        atomicAdd_system(a.err + threadIdx.x, (unsigned long long)s_errors[threadIdx.x]);
 }
 
 // G warps of a block per pair, for launches too small to fill the GPU with
@@ -110,7 +119,7 @@ __global__ void __launch_bounds__(256) k_query_wide(QueryArgs a) {
     if (decided) {
         if (lane == 0) {
             a.out[qi] = (uint8_t)ans;
-            if (bad) atomicAdd_system(a.err + 1, 1ull);
+            if (bad) atomicAdd_system(a.err + 1, 1ull);  // at most four times R in a launch
         }
         return;
     }
@@ -118,7 +127,11 @@ __global__ void __launch_bounds__(256) k_query_wide(QueryArgs a) {
 #pragma unroll
     for (int g = 0; g < G; ++g) best = min(best, part[warp + g]);
     best = finish_pair(a, s, t, lane, td0, td1, dstar, best);
-    if (lane == 0) store_answer(a, qi, best);
+    if (lane == 0) {
+        ans = pair_answer(best);
+        a.out[qi] = (uint8_t)ans;
+        if (ans & ANS_FAR) atomicAdd_system(a.err, 1ull);
+    }
 }
 
 }  // namespace

@@ -168,19 +168,21 @@ __device__ __forceinline__ uint32_t finish_pair(const QueryArgs &a, uint32_t s, 
     return min(best, bpb);
 }
 
-// the answer byte of a pair's minimum (255 for none or for a finite distance
-// of 255 or more; the latter is counted as an error)
-__device__ __forceinline__ uint32_t answer_byte(const QueryArgs &a, uint32_t best) {
-    if (best >= BIG) return INF8;
-    if (best >= INF8) {
-        atomicAdd_system(a.err, 1ull);  // the counters may be host memory
-        return INF8;
-    }
-    return best;
+// the answer of a pair's minimum: its byte (255 for none or for a finite distance
+// of 255 or more), and a bit above it for an error
+constexpr uint32_t ANS_FAR = 1u << 8, ANS_BAD = 1u << 9;  // a finite distance >= 255, an id >= n
+__device__ __forceinline__ uint32_t pair_answer(uint32_t best) {
+    return best >= BIG ? INF8 : best >= INF8 ? INF8 | ANS_FAR : best;
 }
 
-__device__ __forceinline__ void store_answer(const QueryArgs &a, uint64_t qi, uint32_t best) {
-    a.out[qi] = (uint8_t)answer_byte(a, best);
+// Adds the errors among a warp's answers to its block's counts (in shared memory).
+__device__ __forceinline__ void count_errors(uint32_t *count, uint32_t ans, int lane) {
+    if (!__any_sync(FULL, ans > INF8)) return;
+    const unsigned far = __ballot_sync(FULL, ans & ANS_FAR), bad = __ballot_sync(FULL, ans & ANS_BAD);
+    if (lane == 0) {
+        atomicAdd(&count[0], __popc(far));
+        atomicAdd(&count[1], __popc(bad));
+    }
 }
 
 // An open pair: the ends' ranks, and where their labels are.

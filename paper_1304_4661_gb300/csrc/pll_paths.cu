@@ -50,12 +50,13 @@ namespace {
 constexpr uint64_t NOPOS = ~0ull;
 constexpr int PATH_BLOCKS = 8;  // of k_paths on an SM
 
-// error bits of the path kernels
+// errors of the path kernels, a bit each of their error word
 enum : uint32_t {
-    PERR_ID = 1u << 0,      // vertex id >= n
-    PERR_SLOT = 1u << 1,    // path_off not non-decreasing, past cap, or a slot too short
-    PERR_RANGE = 1u << 2,   // finite distance >= 255
-    PERR_WALK = 1u << 3,    // a climb or a walk found no next vertex (graph is not the index's)
+    PERR_ID,      // vertex id >= n
+    PERR_SLOT,    // path_off not non-decreasing, past cap, or a slot too short
+    PERR_RANGE,   // finite distance >= 255
+    PERR_WALK,    // a climb or a walk found no next vertex (graph is not the index's)
+    PERR_KINDS
 };
 
 // position of the packed entry `key` in the hub-sorted label lab[lo, hi)
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(256) k_parents(ParentArgs a) {
                     if (find_entry(a.lab, a.lab_off[w], a.lab_off[w + 1], key) != NOPOS) { p = w; break; }
                 }
             }
-            if (p == NONE) atomicOr(a.err, PERR_WALK);
+            if (p == NONE) atomicOr(a.err, 1u << PERR_WALK);
             a.par[j] = p;
         }
     }
@@ -301,6 +302,9 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
     __shared__ Witness s_wit[8][32];
     __shared__ uint64_t s_slot[8][32];
     __shared__ uint8_t s_item[8][64];
+    __shared__ uint8_t s_err[PERR_KINDS];  // what errors the block met
+    if (threadIdx.x < PERR_KINDS) s_err[threadIdx.x] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     OpenPair *pair = s_pair[warp];
     Witness *wit = s_wit[warp];
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
             o0 = a.path_off[qi];
             o1 = a.path_off[qi + 1];
             if (o1 < o0 || o1 > a.cap) {
-                atomicOr_system(a.err, PERR_SLOT);
+                s_err[PERR_SLOT] = 1;
                 o1 = o0;  // nothing is written
             } else {
                 OpenPair p;
@@ -324,13 +328,13 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
                 const uint32_t sid = a.x.src[qi];
                 if (trivial_pair(a.x, sid, a.x.dst[qi], &p.s, &p.t, &ans, &bad)) {
                     if (bad) {
-                        atomicOr_system(a.err, PERR_ID);
+                        s_err[PERR_ID] = 1;
                     } else if (ans == 0) {  // s = t
                         if (o1 > o0) {
                             a.path[o0] = sid;
                             len = 1;
                         } else {
-                            atomicOr_system(a.err, PERR_SLOT);
+                            s_err[PERR_SLOT] = 1;
                         }
                     }
                 } else {
@@ -364,9 +368,9 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
         if (routed) {
             const Witness w = wit[lane];
             if (w.d >= INF8) {
-                atomicOr_system(a.err, PERR_RANGE);
+                s_err[PERR_RANGE] = 1;
             } else if (o1 - o0 < (uint64_t)w.d + 1) {
-                atomicOr_system(a.err, PERR_SLOT);
+                s_err[PERR_SLOT] = 1;
             } else {
                 climbs = w.by >= 0;
                 walks = !climbs;
@@ -416,7 +420,7 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
         }
         failed = __reduce_or_sync(FULL, failed);
         if (climbs || walks) {
-            if ((failed >> lane) & 1) atomicOr_system(a.err, PERR_WALK);
+            if ((failed >> lane) & 1) s_err[PERR_WALK] = 1;
             else len = (uint64_t)wit[lane].d + 1;
         }
         __syncwarp();  // the walks' writes come before the fill that may cover them
@@ -427,6 +431,9 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
         }
         __syncwarp();  // the next group writes the shared arrays
     }
+    __syncthreads();
+    // written once: a.err may be host memory
+    if (threadIdx.x < PERR_KINDS && s_err[threadIdx.x]) atomicOr_system(a.err, 1u << threadIdx.x);
 }
 
 int warp_grid(uint64_t items, int per_sm, int *blocks) {
@@ -459,8 +466,8 @@ struct ErrWord {
 };
 
 int path_status(uint32_t e) {
-    if (e & (PERR_ID | PERR_SLOT | PERR_WALK)) return PLL_E_INVAL;
-    if (e & PERR_RANGE) return PLL_E_RANGE;
+    if (e & (1u << PERR_ID | 1u << PERR_SLOT | 1u << PERR_WALK)) return PLL_E_INVAL;
+    if (e & (1u << PERR_RANGE)) return PLL_E_RANGE;
     return PLL_OK;
 }
 
