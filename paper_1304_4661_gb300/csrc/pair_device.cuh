@@ -235,13 +235,16 @@ __device__ __forceinline__ bool lone_pair(const QueryArgs &a, uint32_t s, uint64
 // neither end, compacted into `keep` (KEEP places): at most ub - 2 from v, as
 // the other end is at least 1 from such a hub. *direct: the distance of v to
 // `other`, if that is one of its hubs. AHEAD windows of 32 entries are loaded
-// together. Returns how many are kept (over KEEP: too many, not all looked at).
+// together. Returns how many are kept (over KEEP: too many, not all looked at). What
+// other lanes wrote to or read from `keep` before (for the last pair, which may have
+// ended early) is done first; the caller waits before it reads other lanes' places.
 constexpr int AHEAD = 2;
 template <uint32_t KEEP>
 __device__ __forceinline__ uint32_t keep_near(const uint32_t *__restrict__ lab, uint32_t len, uint32_t v,
                                               uint32_t ub, uint32_t other, int lane, uint32_t *keep,
                                               uint32_t *direct) {
     uint32_t cnt = 0;
+    __syncwarp();
     for (uint32_t x0 = 0; x0 < len && cnt <= KEEP; x0 += 32 * AHEAD) {
         uint32_t e[AHEAD];
 #pragma unroll
@@ -307,7 +310,6 @@ __device__ __forceinline__ uint32_t pair_bounded(const QueryArgs &a, const OpenP
         }
     } else {
         const uint32_t e = (uint32_t)lane < cv ? keep[lane] : NONE;
-        __syncwarp();
         const uint32_t ch = keep_near<KEEP>(H, lh, h, ub, NONE, lane, keep, &direct);
         if (ch > KEEP) return min(ub, label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane));
         __syncwarp();
@@ -316,9 +318,7 @@ __device__ __forceinline__ uint32_t pair_bounded(const QueryArgs &a, const OpenP
             if (entry_hub(f) == entry_hub(e)) best = min(best, entry_dist(e) + entry_dist(f));
         }
     }
-    best = warp_min(best);
-    __syncwarp();  // the next pair writes keep
-    return best;
+    return warp_min(best);
 }
 
 }  // namespace pairs

@@ -166,7 +166,6 @@ __device__ __forceinline__ uint64_t near_hub(const QueryArgs &a, const OpenPair 
     if (cv == 0) return best;
     __syncwarp();
     const uint32_t e0 = (uint32_t)lane < cv ? keep[lane] : NONE, e1 = lane + 32u < cv ? keep[lane + 32] : NONE;
-    __syncwarp();
     const uint32_t ch = keep_near<PATH_KEEP>(a.lab + (low ? p.os : p.ot), lh, h, ub + 1, NONE, lane, keep, &direct);
     if (ch > PATH_KEEP) return best_hub(a, p, lane);
     __syncwarp();
@@ -179,7 +178,6 @@ __device__ __forceinline__ uint64_t near_hub(const QueryArgs &a, const OpenPair 
             best = key < best ? key : best;
         }
     }
-    __syncwarp();  // the next pair writes keep
     return warp_min64(best);
 }
 
