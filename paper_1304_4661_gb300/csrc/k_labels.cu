@@ -349,16 +349,9 @@ bool labels_near_give_back(LabelStore *const *st, int count, cudaStream_t s) {
 // bump pointer would run past the pool.
 int labels_regrow(LabelStore &st, uint64_t new_cap, cudaStream_t s) {
     const uint32_t n = st.n;
-    DevMem dpool;
-    PoolMem ppool(s), noff(s), temp(s);
-    uint32_t *np = nullptr;
-    if (st.pooled) {
-        PLL_CHECK(ppool.alloc(new_cap * 4));
-        np = ppool.as<uint32_t>();
-    } else {
-        PLL_CHECK(dpool.alloc(new_cap * 4));
-        np = dpool.as<uint32_t>();
-    }
+    PoolMem pool(s), noff(s), temp(s);
+    PLL_CHECK(pool.alloc(new_cap * 4));
+    uint32_t *np = pool.as<uint32_t>();
     PLL_CHECK(noff.alloc(((size_t)n + 1) * 8));
     size_t tb = 0;
     PLL_CHECK(scan_u32_to_u64(st.len, noff.as<uint64_t>(), n, nullptr, &tb, s, 4));
@@ -381,11 +374,9 @@ int labels_regrow(LabelStore &st, uint64_t new_cap, cudaStream_t s) {
     unsigned long long top = last_off + ((last_len + 3u) & ~3u);
     PLL_TRY(cudaMemcpyAsync(st.pool_top, &top, 8, cudaMemcpyHostToDevice, s));
     PLL_TRY(cudaStreamSynchronize(s));
-    if (st.pooled) pool_free(st.pool, s);
-    else dev_free(st.pool);
+    pool_free(st.pool, s);
     st.pool = np;
-    ppool.release();
-    dpool.release();
+    pool.release();
     st.pool_cap = new_cap;
     return PLL_OK;
 }

@@ -124,7 +124,6 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     st.pool_cap = test_caps().pool ? test_caps().pool : std::max<uint64_t>((uint64_t)n * 64, 1ull << 22);
     PLL_CHECK(m_pool.alloc(st.pool_cap * 4));
     st.pool = m_pool.as<uint32_t>();
-    st.pooled = true;
     m_pool.release();  // owned through st.pool from here on (regrow swaps it)
     st.pool_top = &d_ctr->pool_top;
     struct PoolGuard {

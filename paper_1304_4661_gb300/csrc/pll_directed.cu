@@ -266,7 +266,6 @@ struct Store {
         st.off = off.as<uint64_t>();
         st.len = len.as<uint32_t>();
         st.cap = cap.as<uint32_t>();
-        st.pooled = true;
         st.pool_cap = std::max<uint64_t>((uint64_t)n * 64, 1ull << 20);
         PLL_TRY(pool_malloc(&st.pool, st.pool_cap * 4, s));
         st.pool_top = top;

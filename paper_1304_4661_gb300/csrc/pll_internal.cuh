@@ -180,32 +180,6 @@ struct PoolMem {
     void *release() { void *q = p; p = nullptr; bytes = 0; return q; }
 };
 
-// Device allocation that frees itself; release() hands ownership out (the
-// new owner frees it with dev_free).
-struct DevMem {
-    void *p = nullptr;
-    size_t bytes = 0;
-    DevMem() = default;
-    DevMem(const DevMem &) = delete;
-    DevMem &operator=(const DevMem &) = delete;
-    ~DevMem() { reset(); }
-    int alloc(size_t b) {
-        reset();
-        if (b == 0) b = 16;
-        cudaError_t e = dev_malloc(&p, b);
-        if (e != cudaSuccess) { p = nullptr; (void)cudaGetLastError(); return PLL_E_NOMEM; }
-        bytes = b;
-        return PLL_OK;
-    }
-    void reset() {
-        dev_free(p);
-        p = nullptr;
-        bytes = 0;
-    }
-    template <class T> T *as() const { return static_cast<T *>(p); }
-    void *release() { void *q = p; p = nullptr; bytes = 0; return q; }
-};
-
 // Pinned host memory of one synchronous call: the words its kernels add errors to
 // directly, or the target of its copy back (a pageable target makes the copy a
 // staged one). Blocks of one size are kept per CUDA context (pll_abi.cu) for the
@@ -450,7 +424,7 @@ struct LabelStore {
     uint64_t *off = nullptr;   // [n]
     uint32_t *len = nullptr;   // [n]
     uint32_t *cap = nullptr;   // [n]
-    uint32_t *pool = nullptr;
+    uint32_t *pool = nullptr;        // from pool_malloc
     uint64_t pool_cap = 0;
     unsigned long long *pool_top = nullptr;
     uint32_t *near = nullptr;        // [near_cap] the near copy, or null
@@ -460,7 +434,6 @@ struct LabelStore {
     bool near_given_back = false;    // its memory was needed: no copy any more
     NearLabel *near_lab = nullptr;   // [n]
     uint32_t *near_end = nullptr;    // [NEAR_CLASSES][n] its entries of distance <= c
-    bool pooled = false;  // `pool` comes from pool_malloc (else dev_malloc)
 };
 // radix sort of packed tuples by their bits [begin_bit, end_bit)
 int labels_sort_tuples(uint64_t *d_in, uint64_t *d_out, uint64_t count, int begin_bit, int end_bit,
