@@ -772,6 +772,7 @@ using namespace pll;
 
 struct pll_mlp {
     int device = 0;
+    uint32_t wide = 0;  // blocks of k_mlp_fwd<2> that the device holds at once
     uint32_t max_batch = 0, blocks = 0;
     float *master = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *w16 = nullptr;
@@ -910,7 +911,11 @@ PLL_API int pll_mlp_create(uint32_t max_batch, pll_mlp **out) {
     p->max_batch = max_batch;
     p->blocks = (max_batch + GT - 1) / GT;
     const size_t nf = 4 * (size_t)NP + (NP + 1) + (size_t)p->blocks * NP + p->blocks + 8;
+    int sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&p->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_mlp_fwd<2>, FT, 0);
+    p->wide = (uint32_t)std::max(1, sms * per);
     if (e == cudaSuccess) e = cudaMalloc(&p->mem, nf * sizeof(float));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
@@ -969,9 +974,8 @@ PLL_API int pll_mlp_forward(const pll_mlp *p, const float *x, uint64_t n, float 
     cudaStream_t s = (cudaStream_t)stream;
     // two rows a thread where that still fills the GPU (three blocks an SM)
     const bool vec = reinterpret_cast<uintptr_t>(x) % 16 == 0;
-    const uint64_t wide = 152ull * 3;
-    if (n >= wide * FT * 2)
-        k_mlp_fwd<2><<<(unsigned)wide, FT, 0, s>>>(n, x, vec, p->w16, y);
+    if (n >= (uint64_t)p->wide * FT * 2)
+        k_mlp_fwd<2><<<p->wide, FT, 0, s>>>(n, x, vec, p->w16, y);
     else
         k_mlp_fwd<1><<<(unsigned)((n + FT - 1) / FT), FT, 0, s>>>(n, x, vec, p->w16, y);
     PLL_TRY(cudaGetLastError());
