@@ -637,8 +637,8 @@ PLL_API int64_t pll_test_live_allocs(void);
  * Test hook for the buffer-growth paths of the pruned stage; the paper has no
  * counterpart. pll_test_capacities(cand, out, pool, tables) sets the initial
  * sizes, in entries, of the candidate buffer, the pre-cleanup tuple buffer,
- * the label pool and the root-table pool of every later build (0 keeps the
- * library's own sizing, which is the default). With cand or out set, buffers
+ * the label pools and the root-table pool of every later build, directed ones
+ * included (0 keeps the library's own sizing, which is the default). With cand or out set, buffers
  * are not grown ahead of demand, so a batch that overflows one is run again
  * with a larger one; with tables set, the root-table pool keeps that size for
  * the whole build, so the roots whose tables do not fit have their labels

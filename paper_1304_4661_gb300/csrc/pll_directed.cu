@@ -266,7 +266,8 @@ struct Store {
         st.off = off.as<uint64_t>();
         st.len = len.as<uint32_t>();
         st.cap = cap.as<uint32_t>();
-        st.pool_cap = std::max<uint64_t>((uint64_t)n * 64, 1ull << 20);
+        const uint64_t test_cap = test_caps().pool;
+        st.pool_cap = test_cap ? test_cap : std::max<uint64_t>((uint64_t)n * 64, 1ull << 20);
         PLL_TRY(pool_malloc(&st.pool, st.pool_cap * 4, s));
         st.pool_top = top;
         return PLL_OK;
@@ -324,7 +325,8 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
     PLL_CHECK(vis.alloc((size_t)bmax * NW * 4));
     PLL_CHECK(inX.alloc(n));
     PLL_TRY(cudaMemsetAsync(inX.p, 0, n, s));
-    uint64_t ht_cap = std::max<uint64_t>((uint64_t)bmax * 1024, 1ull << 18);
+    const TestCaps caps = test_caps();
+    uint64_t ht_cap = caps.ht ? caps.ht : std::max<uint64_t>((uint64_t)bmax * 1024, 1ull << 18);
     auto alloc_tables = [&]() -> int {
         PLL_CHECK(ht.alloc(ht_cap * 4));
         return reach.alloc(ht_cap * 4);
@@ -336,10 +338,12 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         (void)cudaGetLastError();
         free_b = 0;
     }
-    const uint64_t slice_cap = slice_entries(ix->nnz, free_b);
+    const uint64_t slice_cap = caps.cand ? std::min<uint64_t>(caps.cand, SLICE_CAP) : slice_entries(ix->nnz, free_b);
     PLL_CHECK(slices.alloc(slice_cap * 16));
-    uint64_t cand_cap = std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 128, free_b / 16 / 24), 1ull << 16);
-    uint64_t out_cap = std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 64, free_b / 16 / 33), 1ull << 16);
+    uint64_t cand_cap = caps.cand ? caps.cand
+                                  : std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 128, free_b / 16 / 24), 1ull << 16);
+    uint64_t out_cap = caps.out ? caps.out
+                                : std::max<uint64_t>(std::min<uint64_t>((uint64_t)n * 64, free_b / 16 / 33), 1ull << 16);
     const int end_bit = 32 + [&] { int b = 1; while (b < 24 && ((n - 1) >> b)) ++b; return b; }();
     constexpr int SORT_BEGIN_BIT = 8;  // (u, k) is unique within a batch and direction
     auto alloc_cand = [&]() -> int {
@@ -428,7 +432,8 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
         const uint32_t err = h->d.c[0].err | h->d.c[1].err;
         if (err & ERR_TABLE) {  // those roots were binary-searched; grow for later batches
             const uint64_t need = std::max(h->d.c[0].ht_top, h->d.c[1].ht_top);
-            PLL_CHECK(grow_if_possible(ht_cap, std::max<uint64_t>(need + need / 4, ht_cap * 2), alloc_tables));
+            if (!caps.ht)  // the test capacity keeps the pool small for the whole build
+                PLL_CHECK(grow_if_possible(ht_cap, std::max<uint64_t>(need + need / 4, ht_cap * 2), alloc_tables));
         }
         if (err & ERR_BUF) {
             const uint64_t nc = std::max(h->d.c[0].cand_n, h->d.c[1].cand_n), no = std::max(h->d.c[0].out_n, h->d.c[1].out_n);
@@ -472,7 +477,7 @@ int directed_labels(pll_dindex *ix, PoolMem *adj_off, PoolMem *adj_col, uint32_t
             PLL_CHECK(labels_compact(sorted[dir].as<uint64_t>(), keep.as<uint8_t>(), P[dir], out[dir].as<uint64_t>(),
                                      &d->c[dir].nkept, temp.p, &tb, s));
             PLL_CHECK(labels_append(st, out[dir].as<uint64_t>(), &d->c[dir].nkept, P[dir], &d->c[dir].err_post, s));
-            PLL_CHECK(labels_near(st, total[dir], s));
+            if (!caps.ht) PLL_CHECK(labels_near(st, total[dir], s));
             pending[dir] = true;
         }
         ++ix->batches;
