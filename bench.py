@@ -366,11 +366,11 @@ def run_ours(args, w, ws, rank, local):
 
     exp_bytes = expand_bytes(units)
     test_bytes = test_bytes_of(units)
-    # the same per-unit bytes over the GPU's own work counts (its root batches'
-    # surplus included; a vertex that the bit-parallel bound prunes is counted
-    # each time it is reached), for comparison with the sequential-count figure
-    gpu_units = {"visited": st["visited"], "labeled": st["pre_cleanup"],
-                 "scanned": st["pruned_scanned"], "labeled_deg": st["pruned_expanded"]}
+    # what the sweeps themselves ask for, by their own work counts (the root
+    # batches' surplus included): an arc's neighbour id and the neighbour's nibble
+    # row (16 bytes for 32 roots), an entry, a label entry
+    gpu_bytes = ((4 + 16 * ((t + 31) // 32)) * st["pruned_expanded"] + 5 * st["pre_cleanup"]
+                 + 4 * st["pruned_scanned"])
     # per pair: ids (8), ranks (8), 2 x t distance bytes, 4 label offsets (32),
     # the result byte, and both labels (4 bytes per entry; Lsz is by vertex id)
     q_bytes = q * (8 + 8 + 2 * t + 32 + 1) + 4 * int(Lsz[s].sum() + Lsz[u].sum())
@@ -424,10 +424,9 @@ def run_ours(args, w, ws, rank, local):
                                "achieved_gbs": round(v["bytes"] / max(v["ms_per_step"], 1e-9) / 1e6, 1)}
                            for k, v in phases.items()}}
     if st["levels_launches"] and dom != "k_query" and seq:
-        gb = expand_bytes(gpu_units) + test_bytes_of(gpu_units)
-        ga = gb / max(kd["ms_per_step"], 1e-9) / 1e6
+        ga = gpu_bytes / max(kd["ms_per_step"], 1e-9) / 1e6
         roofline["with_gpu_counts"] = {"achieved": round(ga, 1), "frac": round(ga / hbm, 4),
-                                       "algorithmic_bytes_per_launch": round(gb / kd["launches"])}
+                                       "bytes_per_launch": round(gpu_bytes / kd["launches"])}
 
     out = {
         "metric": METRIC, "value": round(build_ms / 1e3, 6), "unit": "s", "n_gpus": ws,

@@ -106,8 +106,11 @@ typedef struct pll_stats {
     uint64_t label_entries;      /* sum over v of |L(v)| (normal labels) */
     uint64_t pre_cleanup;        /* entries emitted by batched pruned BFSs
                                     before the redundancy cleanup */
-    uint64_t visited;            /* (root, vertex) pairs that pruned BFSs reached
-                                    and the bit-parallel distances left */
+    uint64_t visited;            /* arcs of the pruned BFSs (to vertices of rank
+                                    >= the batch's first; the others are cut
+                                    off unread) that the bit-parallel distances
+                                    prune, plus, of those they leave, the arcs
+                                    to a vertex not yet marked for the root */
     uint64_t batches;            /* root batches */
     uint64_t index_bytes;        /* device bytes held by the index */
     double ms_prep;              /* order, relabel, root selection */
