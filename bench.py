@@ -45,13 +45,15 @@ WORKLOADS = {
 
 # DRAM bytes per algorithmic byte of a kernel, measured by ncu over every
 # launch of one build of a smaller R-MAT (dram__bytes_read.sum +
-# dram__bytes_write.sum, one pass), valid only for the kernel source with this
-# hash (else traffic is reported as null). The level-loop graph's figure is
-# ncu's per-graph-launch count (--graph-profiling graph) on R-MAT scale 18:
-# 24 launches, 4.955 GB of DRAM against 6.953 GB of algorithmic bytes.
+# dram__bytes_write.sum, one pass), valid only for the sources with this hash,
+# on which the sweeps' traffic depends (else traffic is reported as null). The
+# level-loop graph's figure is ncu's per-graph-launch count (--graph-profiling
+# graph) on R-MAT scale 18: 13 launches, 2.005 GB of DRAM against 6.953 GB of
+# algorithmic bytes.
 PROFILED = {
     "level-loop graph (k_batch_expand_g + k_batch_test_g)": {
-        "src_sha": "2f8ca0172ddd4fd8", "dram_per_alg_byte": 0.289},
+        "src": ["k_pruned.cu", "bp_nibble.h", "build_sizes.h", "k_labels.cu", "pll_internal.cuh"],
+        "src_sha": "946c579aa20c7e3a", "dram_per_alg_byte": 0.288},
 }
 
 
@@ -91,8 +93,12 @@ def sequential_work(w, g):
     return d.get("sequential_work")
 
 
-def file_sha(path):
-    return hashlib.sha256(open(path, "rb").read()).hexdigest()[:16]
+def source_sha(names):
+    h = hashlib.sha256()
+    for name in names:
+        with open(os.path.join(ROOT, "paper_1304_4661_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 class ClockSampler:
@@ -404,13 +410,11 @@ def run_ours(args, w, ws, rank, local):
     dom = max(kern, key=lambda k: kern[k]["ms_per_step"])
     kd = kern[dom]
     achieved = kd["achieved_gbs"]
-    src = os.path.join(ROOT, "paper_1304_4661_gb300", "csrc",
-                       "k_query.cu" if dom == "k_query" else "k_pruned.cu")
     prof = PROFILED.get(dom)
     # DRAM bytes per algorithmic byte, measured by ncu on a smaller graph of the
-    # same family with this kernel source, scaled to this launch's bytes
+    # same family with these sources, scaled to this launch's bytes
     traffic = (round(prof["dram_per_alg_byte"] * kd["bytes_per_launch"])
-               if prof and prof["src_sha"] == file_sha(src) else None)
+               if prof and prof["src_sha"] == source_sha(prof["src"]) else None)
     roofline = {"kernel": dom, "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm,
                 "peak_source": peak_src, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "traffic": traffic,

@@ -74,7 +74,8 @@ __global__ void k_deg_twohop(uint32_t n, const uint32_t *__restrict__ off,
 // few hundred vertices, where peeling by degree takes 488 dependent passes,
 // each a scan of all vertices and a read-back (pll_features with t = 64: 24.0
 // ms so, 4.7 ms with the steps, 1.3 ms of it theirs). Bound by the longest
-// lists of a step and the gathers of their neighbours' values.
+// lists of a step and the gathers of their neighbours' values (which take 64
+// registers and 136 bytes of local memory a thread in lists next to CORE_BIG).
 constexpr uint32_t CORE_BIG = 512;     // lists this long get a block each
 constexpr int CORE_BIG_BLOCKS = 1024;
 constexpr int CORE_CHUNK = 4;          // vertices a warp looks at together; it takes the marked
@@ -210,7 +211,7 @@ __device__ void core_small(const CoreArgs &a, uint32_t v, uint32_t b, uint32_t d
 }
 
 // One step: the marked vertices' values. Blocks below CORE_BIG_BLOCKS take the
-// long lists, the others 32 vertices a warp. Nothing to do (and nothing
+// long lists, the others CORE_CHUNK vertices a warp. Nothing to do (and nothing
 // marked) if the step before changed nothing.
 __global__ void __launch_bounds__(256) k_core_step(CoreArgs a) {
     if (a.prev && *a.prev == 0) return;

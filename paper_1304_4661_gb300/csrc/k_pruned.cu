@@ -502,9 +502,12 @@ __device__ __forceinline__ void expand_open(const BatchArgs &a, const ExpandWarp
     append_cand(a, keep, lane, slot, w, c1, c2);
 }
 
-// entries of at least this many neighbours are taken 32 arcs at a time (32 to 1000:
-// no difference), and threads an SM of the expand sweep (builds of R-MAT-20 and of
-// the batch of 96 graphs: 144.9 and 176.4 ms at 1280, 138.5 and 170.6 at 1024)
+// Entries of at least this many arcs are taken 32 arcs at a time: with slices of as
+// many, whole slices and full first ones (and the long lists of a level whose slices
+// found no room), which leave no lane idle and need no owner search. A line at 32 to
+// 1000 made no difference to the time. And threads an SM of the expand sweep (builds
+// of R-MAT-20 and of the batch of 96 graphs: 144.9 and 176.4 ms at 1280, 138.5 and
+// 170.6 at 1024)
 constexpr uint32_t HEAVY_DEG = 64;
 constexpr int EXPAND_TPS = 1024;
 
@@ -540,7 +543,8 @@ __device__ __forceinline__ unsigned long long next_chunk(const BatchArgs &a, uns
 // memory, so that the rest of the test runs with full warps.
 //
 // Bound by the L1's rate of scattered accesses (one row per arc). 1024 threads
-// per SM (64 registers; 1280 threads spill: 52.9 against 51.4 ms). All of
+// per SM (64 registers; the graph loop's form keeps 100 bytes of its chunk in local
+// memory, the separate launch 12; at 1280 threads more: 52.9 against 51.4 ms). All of
 // R-MAT-20's expand sweeps (t = 64; 3.15G arcs): 95.1 ms with a warp per
 // entry, 64-byte rows and the visited word first; 71.9 ms with chunks, the
 // queue and nibble rows; 55.3 ms with long lists in slices; 51.4 ms with one
@@ -751,8 +755,8 @@ __global__ void k_batch_clear(BatchArgs a) {
 //           of entries laid end to end over the lanes (a quad's candidate found
 //           by a binary search over a warp scan of the lengths). An entry at
 //           distance d >= level can prune nothing (every hub is at least 1 from
-//           the root): 95 of 100 entries on power-law graphs and 6 of 10 on the
-//           high-diameter ones, most of which are not even read (the labels are
+//           the root): 95 of 100 entries on power-law graphs and more than half on
+//           the high-diameter ones, most of which are not even read (the labels are
 //           read from their near copy, k_labels.cu, up to distance level - 1,
 //           and from the store past what the copy holds); an
 //           entry that the table lets through is looked up in the root's hash
@@ -762,7 +766,7 @@ __global__ void k_batch_clear(BatchArgs a) {
 //
 // Bound by instruction issue (0.57 to 0.7 of the slots on the batch's heavy
 // launches) and the latency of the labels. All test sweeps of the batch of 96
-// uneven graphs (t = 16; 33G label entries, 12G of them nearer than the
+// uneven graphs (t = 16; 33G label entries, 15G of them nearer than the
 // candidate): 325 ms with every entry probed in the hash table (gathers from
 // L2), 124 ms with the reach tables and single entries on the lanes, 106.6 ms
 // with quads. R-MAT-20 (t = 64; 7.8G entries, 0.4G nearer): 65.9, 47.0, 43.3
@@ -1139,6 +1143,9 @@ __device__ __forceinline__ bool grid_barrier(const BatchArgs &a, LoopState *ls) 
 // reaches 255, or a barrier times out). Level bounds live in registers, the
 // same in every CTA (they come from the barrier's snapshots), so no level
 // needs the host. Block 0 adds the phases' wall times to the loop state.
+// At blocks of 128 and 256 the bound of 1280 threads an SM leaves 48 registers and
+// spills (R-MAT-20's build 121 ms); at 512 and 1024 it comes to 1024 threads and 64
+// registers (83 ms, the graph loop's 87).
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_batch_levels(BatchArgs a) {
     extern __shared__ uint4 s_dyn[];

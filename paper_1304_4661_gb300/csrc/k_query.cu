@@ -35,7 +35,8 @@ constexpr int QUERY_BLOCKS = 8;
 // in shared memory. PG is 32 for launches that fill the GPU that way and smaller
 // for launches that would otherwise leave warps idle. Bound by the traffic and
 // the latency of scattered loads, so it wants resident warps: eight blocks an
-// SM, 32 registers a thread (six blocks: 10 % slower). 10M uniform pairs of
+// SM, 32 registers a thread, for which 56 bytes of a warp's state go to local memory
+// (six blocks, without: 10 % slower). 10M uniform pairs of
 // R-MAT-20, t = 64: 5.02 ms with the merge join for every pair, 3.22 ms so, of
 // which (by leaving steps out) 0.3 ms for ranks, offsets and lone pairs, 0.3
 // for the rows, 1.0 for the masks and 0.8 for each end's label.

@@ -161,8 +161,8 @@ int pruned_stage(pll_index *ix, const uint32_t *roff, const uint32_t *rcol, cons
     PLL_CHECK(m_bpq.alloc(std::max<size_t>((size_t)n * qn * 16, 16)));
     PLL_CHECK(batch_nibble_rows(ix->d_bp_d, n, ix->tp, qn, m_bpq.as<uint4>(), grid[0], s));
     ix->stats.launches += ix->t ? 2 : 0;
-    // visited bitmap, one row of ceil(n / 32) words per root slot; cleared once
-    // here, then lazily after each batch (only the words the batch set)
+    // visited bitmap, one row of ceil(n / 32) words per root slot; a row is cleared
+    // when it is first used, then lazily after each batch (only the words it set)
     const uint32_t NW = (n + 31) / 32;
     PoolMem m_vis(s), m_ht(s), m_tab(s), m_cand(s), m_candc(s), m_out(s),
         m_sorted(s), m_keep(s), m_temp(s);

@@ -30,7 +30,7 @@
 // lists' offsets; a warp per vertex) and k_dquery (warp per pair).
 // R-MAT-15, arcs one way or both (1.2M): 49.3 ms for the build and 1M queries
 // with a thread-serial merge of two labels per frontier entry, two read-backs a
-// level and batches of 1024; 11.9 ms so. What is left is launches: two
+// level and batches of 1024; 11.7 ms so. What is left is launches: two
 // directions of up to ten levels a batch, and a sort and a cleanup each.
 #include <algorithm>
 #include <new>
@@ -513,8 +513,8 @@ PLL_API int pll_build_directed(const uint32_t *offsets, const uint32_t *cols, ui
     if (o.t != 0 || o.flags != 0 || o.reserved != 0) return PLL_E_INVAL;
     if (n > MAX_N || nnz >= 0xffffffffull) return PLL_E_RANGE;
     if ((n > 0 && !offsets) || (nnz > 0 && !cols) || (n == 0 && nnz != 0)) return PLL_E_INVAL;
-    // default batch: as large as the undirected build's (R-MAT-17: 104 ms at
-    // 1024 roots, 60 ms at 16384; R-MAT-15: 22.0 and 13.6 ms); the visited bits
+    // default batch: as large as the undirected build's (R-MAT-17: 84.8 ms at 1024
+    // roots, 52.0 at 16384, 50.6 at 65536; R-MAT-15: 18.6, 11.4, 11.4); the visited bits
     // of any batch stay within 2 GiB
     uint32_t bmax = std::max(1u, std::min({n, o.root_batch ? o.root_batch : default_batch(n, 2ull << 30, 64), BATCH_MAX}));
     while (bmax > 64 && (uint64_t)n * bmax / 8 > (2ull << 30)) bmax >>= 1;

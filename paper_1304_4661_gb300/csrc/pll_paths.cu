@@ -290,9 +290,9 @@ struct PathLength {
 // ones one by one, then the climbs and walks of all of them side by side (two
 // ends each; a climb is a chain of dependent searches, and a walk's steps wait
 // for one another too). Bound by the latency of those chains: eight blocks an
-// SM (32 registers; five blocks of 47 registers 10 % slower). 1M uniform pairs of
+// SM (32 registers and 106 bytes of local memory; five blocks of 47 registers 10 % slower). 1M uniform pairs of
 // R-MAT-20, t = 64, with the lengths: 2.90 ms with a warp per pair, binary
-// searches for every witness and the climbs on two lanes; 1.72 ms so, of which
+// searches for every witness and the climbs on two lanes; 1.70 ms so, of which
 // (by leaving steps out) 0.6 ms is the witnesses, 0.5 the walks, 0.05 the climbs.
 __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t G) {
     __shared__ uint32_t s_keep[8][PATH_KEEP];

@@ -6,6 +6,7 @@ import gc
 import numpy as np
 import pytest
 
+import oracle
 from paper_1304_4661_gb300 import graphgen as gg
 from paper_1304_4661_gb300 import pll
 
@@ -105,3 +106,21 @@ def test_a_small_graph_needs_little_scratch():
     with_roots = undirected(g, 16)[0]()
     assert 0 < with_roots.stats()["scratch_peak_bytes"] < 0.8e9
     with_roots.close()
+
+
+@pytest.mark.parametrize("root_batch", [8, 13])
+def test_an_older_near_copy_beside_a_store_that_moved(root_batch):
+    """Label pools that start small (a batch of few roots asks for little more) move to larger ones
+    between rebuilds of the near copy, which then covers the labels as they were."""
+    lib, g = pll.load(), gg.ba(20000, 6, 7)
+    d = gg.oriented(g, 3, both=0.3)
+    lib.pll_test_capacities(0, 0, 1 << 18, 0)
+    try:
+        ix = undirected(g, 0, root_batch=root_batch)[0]()
+        dix = directed(d, root_batch=root_batch)[0]()
+    finally:
+        lib.pll_test_capacities(0, 0, 0, 0)
+    assert ix.stats()["pool_regrows"] > 1
+    assert same_labels(ix.labels(), oracle.Index(g.offsets, g.cols, 0).labels())
+    ref = oracle.DirectedIndex(d.offsets, d.cols)
+    assert same_labels(dix.labels_in(), ref.labels_in()) and same_labels(dix.labels_out(), ref.labels_out())
