@@ -188,7 +188,7 @@ struct PoolMem {
 // waited for, also where the call ends early, so nothing in flight can write to
 // another call's words. p is null if no block can be had.
 constexpr size_t HOST_BLOCK_BYTES = 20480;
-constexpr size_t HOST_BLOCKS_KEPT = 16;
+constexpr size_t HOST_BLOCKS_KEPT = 64;
 void *host_block_take(unsigned long long *ctx_id);
 void host_block_give(void *p, unsigned long long ctx_id);
 struct HostBlock {

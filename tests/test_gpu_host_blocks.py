@@ -92,12 +92,12 @@ def test_many_threads_keep_their_statuses_apart():
     gc.collect()  # indices of earlier tests must not be freed mid-count
     live = lib.pll_test_live_allocs()
     good, bad = dev_u32(np.arange(500, dtype=np.uint32)), dev_u32(np.full(500, 500, np.uint32))
-    wrong, gate = [], threading.Barrier(40)
+    wrong, gate = [], threading.Barrier(100)
 
     def work(i):
         stream, out = torch.cuda.Stream(), torch.empty(500, dtype=torch.uint8, device="cuda")
         gate.wait()
-        for _ in range(50):
+        for _ in range(20):
             code = pll.PLL_OK
             try:
                 ix.query(bad if i % 3 == 0 else good, good, out=out, stream=stream)
@@ -105,7 +105,7 @@ def test_many_threads_keep_their_statuses_apart():
                 code = e.code
             if code != (pll.PLL_E_INVAL if i % 3 == 0 else pll.PLL_OK):
                 wrong.append((i, code))
-    threads = [threading.Thread(target=work, args=(i,)) for i in range(40)]
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(100)]
     for th in threads:
         th.start()
     for th in threads:
