@@ -3,9 +3,10 @@
 // d(s, t) = min( bit-parallel query (Sec. 5.3), Query(s, t, L) (Sec. 3.3) ).
 //
 // A persistent grid (a few CTAs per SM) walks the pairs; one warp answers one
-// pair, the bit-parallel part first, which bounds what the labels can add
-// (pair_bounded). Pairs with an end that nothing reaches are settled by one
-// lane each (lone_pair). A launch too small to fill the GPU that way (up to 4 pairs per
+// pair, the labels first (pair_merged) or, where the labels are far larger than the
+// L2, the bit-parallel part, which bounds what the labels can add (pair_bounded).
+// Pairs with an end that nothing reaches are settled by one lane each (lone_pair).
+// A launch too small to fill the GPU that way (up to 4 pairs per
 // resident block) gives each pair 2, 4 or 8 warps instead, which split the
 // label scan and meet in shared memory. Lanes own bit-parallel roots (lane, lane + 32): the t distance bytes
 // of s and of t arrive in one coalesced load each, and d~_i = d(s,r_i) +
@@ -35,20 +36,29 @@ constexpr int QUERY_BLOCKS = 8;
 // in shared memory. PG is 32 for launches that fill the GPU that way and smaller
 // for launches that would otherwise leave warps idle. Bound by the traffic and
 // the latency of scattered loads, so it wants resident warps: eight blocks an
-// SM, 32 registers a thread, for which 56 bytes of a warp's state go to local memory
-// (six blocks, without: 10 % slower). 10M uniform pairs of
-// R-MAT-20, t = 64: 5.02 ms with the merge join for every pair, 3.22 ms so, of
+// SM, 32 registers a thread, for which 28 or 56 bytes of a thread's state go to local
+// memory (six blocks, without: 10 % slower). 10M uniform pairs of
+// R-MAT-20, t = 64: 5.02 ms with the merge join for every pair, 3.28 ms so, of
 // which (by leaving steps out) 0.3 ms for ranks, offsets and lone pairs, 0.3
 // for the rows, 1.0 for the masks and 0.8 for each end's label.
-template <int PG>
+//
+// NEAR: near entries only (pair_bounded), for indices whose labels are well past the
+// L2, where what it leaves unread counts; otherwise the labels first (pair_merged):
+// the near entries are a second reading of what the L2 holds, and the masks they
+// are bounded by are most of the work. 10M uniform pairs, near entries against
+// labels first: R-MAT-17, 18, 19, 20, 21 at t = 64 (labels of 5, 21, 78, 288 and
+// 998 MB) 2.26 and 1.93, 2.51 and 2.24, 2.82 and 2.68, 3.29 and 3.35, 4.01 and 4.54
+// ms; R-MAT-20 at t = 16 (537 MB) 3.97 and 4.57; BA of 10,000 and 50,000
+// vertices at t = 16 (1 and 32 MB) 4.59 and 3.46, 9.57 and 8.26.
+template <int PG, bool NEAR>
 __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
-    __shared__ uint32_t s_keep[8][KEEP];
+    __shared__ uint32_t s_keep[NEAR ? 8 : 1][KEEP];
     __shared__ OpenPair s_pair[8][PG];
     __shared__ uint32_t s_errors[2];
     if (threadIdx.x < 2) s_errors[threadIdx.x] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    uint32_t *keep = s_keep[threadIdx.x >> 5];
+    uint32_t *keep = s_keep[NEAR ? threadIdx.x >> 5 : 0];
     OpenPair *pair = s_pair[threadIdx.x >> 5];
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t q0 = (((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * PG; q0 < a.q;
@@ -81,7 +91,7 @@ __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
         for (uint32_t m = __ballot_sync(FULL, open); m; m &= m - 1) {
             const int j = __ffs(m) - 1;
             const OpenPair p = pair[j];
-            const uint32_t best = pair_bounded(a, p, lane, keep);
+            const uint32_t best = NEAR ? pair_bounded(a, p, lane, keep) : pair_merged(a, p, lane);
             if (lane == j) ans = pair_answer(best);  // best is the same on every lane
         }
         // the group's answers in one coalesced store (the output may be host
@@ -135,6 +145,14 @@ __global__ void __launch_bounds__(256) k_query_wide(QueryArgs a) {
     }
 }
 
+template <bool NEAR>
+void launch_query(const QueryArgs &a, uint64_t per, unsigned blocks, cudaStream_t s) {
+    if (per >= 32) k_query<32, NEAR><<<blocks, 256, 0, s>>>(a);
+    else if (per >= 8) k_query<8, NEAR><<<blocks, 256, 0, s>>>(a);
+    else if (per >= 2) k_query<2, NEAR><<<blocks, 256, 0, s>>>(a);
+    else k_query<1, NEAR><<<blocks, 256, 0, s>>>(a);
+}
+
 }  // namespace
 
 int query_launch(const pll_index *ix, const uint32_t *d_src, const uint32_t *d_dst, uint64_t q,
@@ -146,18 +164,22 @@ int query_launch_strided(const pll_index *ix, const uint32_t *d_src, const uint3
                          uint32_t stride, uint64_t q, uint8_t *d_out, unsigned long long *err,
                          cudaStream_t s) {
     if (q == 0) return PLL_OK;
-    // resident blocks of k_query on this device (SMs x blocks per SM), looked
-    // up once per device: the serving loop launches it thousands of times
-    static std::atomic<int> resident[64];
+    // resident blocks of k_query on this device (SMs x blocks per SM) and its L2,
+    // looked up once per device: the serving loop launches it thousands of times
+    static std::atomic<int> resident[64], l2_bytes[64];
     int dev = 0;
     PLL_TRY(cudaGetDevice(&dev));
+    int l2 = dev < 64 ? l2_bytes[dev].load(std::memory_order_relaxed) : 0;
     int res = dev < 64 ? resident[dev].load(std::memory_order_relaxed) : 0;
-    if (res == 0) {
+    if (res == 0 || l2 == 0) {
         int sms = 0, per = 0;
         PLL_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        PLL_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_query<32>, 256, 0));
+        PLL_TRY(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+        PLL_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_query<32, true>, 256, 0));
         res = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+        l2 = l2 > 0 ? l2 : 1;
         if (dev < 64) resident[dev].store(res, std::memory_order_relaxed);
+        if (dev < 64) l2_bytes[dev].store(l2, std::memory_order_relaxed);
     }
     const QueryArgs a = query_args(ix, d_src, d_dst, stride, q, d_out, err);
     // Pairs one warp each would leave most of the GPU idle: give each pair G
@@ -174,10 +196,8 @@ int query_launch_strided(const pll_index *ix, const uint32_t *d_src, const uint3
         // pairs per warp group: as many as keep every resident warp busy (R
         // blocks of 8 warps), up to 32
         const uint64_t per = q / (R * 8);
-        if (per >= 32) k_query<32><<<(unsigned)R, 256, 0, s>>>(a);
-        else if (per >= 8) k_query<8><<<(unsigned)R, 256, 0, s>>>(a);
-        else if (per >= 2) k_query<2><<<(unsigned)R, 256, 0, s>>>(a);
-        else k_query<1><<<(unsigned)R, 256, 0, s>>>(a);
+        if (ix->entries * 4 > 2 * (uint64_t)l2) launch_query<true>(a, per, (unsigned)R, s);
+        else launch_query<false>(a, per, (unsigned)R, s);
     }
     PLL_TRY(cudaGetLastError());
     return PLL_OK;

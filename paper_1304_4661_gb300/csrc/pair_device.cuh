@@ -266,7 +266,16 @@ __device__ __forceinline__ uint32_t keep_near(const uint32_t *__restrict__ lab, 
     return cnt;
 }
 
-// The distance of an open pair, one warp. The bit-parallel answer ub comes
+// The distance of an open pair, one warp, the labels first: the merge join, then the
+// masks of the bit-parallel roots that can beat its answer.
+__device__ __forceinline__ uint32_t pair_merged(const QueryArgs &a, const OpenPair &p, int lane) {
+    uint32_t td0, td1, dstar;
+    bp_tilde(a, p.s, p.t, lane, &td0, &td1, &dstar);
+    const uint32_t best = label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane);
+    return finish_pair(a, p.s, p.t, lane, td0, td1, dstar, best);
+}
+
+// The same, reading as little of the labels as can be. The bit-parallel answer ub comes
 // first: a common hub of the labels matters only below it. A label's hubs are
 // at most its vertex's own rank, so of the two ends only the one of lower rank,
 // h, can be a hub of the other, v: L(v) is read first, for h itself and for the
@@ -275,16 +284,23 @@ __device__ __forceinline__ uint32_t keep_near(const uint32_t *__restrict__ lab, 
 // The reads are one pass of independent loads; the merge join's windows wait
 // for one another. (Bounded by the least d~ alone, with the masks after the
 // labels, twice as many entries stay: 0.6 ms more on the 10M pairs of
-// R-MAT-20; with both labels loaded along with the rows: 1 ms more.) Without a
-// bound (t = 0, or ends that no root reaches), with too many near entries or
-// where one label is long against the other, the merge join or its binary
-// searches decide.
+// R-MAT-20; with both labels loaded along with the rows: 1 ms more.) With a bound
+// past NEAR_MOST most entries are near, and the labels come first after all, as
+// without a bound (t = 0, or ends that no root reaches); with too many near entries
+// or where one label is long against the other, the merge join or its binary
+// searches decide. 10M pairs with NEAR_MOST = 3, 4, 5 and none: R-MAT-20, t = 64, 3.50,
+// 3.28, 3.30, 3.31 ms; BA of 50,000 vertices, t = 16, 8.43, 8.97, 9.59, 9.59 (8.26 with
+// the labels first throughout).
+constexpr uint32_t NEAR_MOST = 4;
 constexpr uint32_t LONG_LABEL = 256;
 constexpr uint32_t KEEP = 32;
 __device__ __forceinline__ uint32_t pair_bounded(const QueryArgs &a, const OpenPair &p, int lane, uint32_t *keep) {
     uint32_t td0, td1, dstar;
     bp_tilde(a, p.s, p.t, lane, &td0, &td1, &dstar);
-    if (dstar >= BIG) return label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane);
+    if (dstar > NEAR_MOST) {
+        const uint32_t best = label_min_merge_at(a, p.s, p.t, p.os, p.ls, p.ot, p.lt, lane);
+        return finish_pair(a, p.s, p.t, lane, td0, td1, dstar, best);
+    }
     uint32_t ub = finish_pair(a, p.s, p.t, lane, td0, td1, dstar, BIG);
     const bool low = p.s < p.t;  // h = s, v = t
     const uint32_t h = low ? p.s : p.t, v = low ? p.t : p.s, lh = low ? p.ls : p.lt, lv = low ? p.lt : p.ls;
