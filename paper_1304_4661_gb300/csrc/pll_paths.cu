@@ -110,6 +110,7 @@ struct PathArgs {
     QueryArgs x;               // the index and the pairs
     const uint32_t *order, *par;
     const uint32_t *roff, *rcol;
+    const uint32_t *bp_root, *bp_S;  // [graphs][t], [graphs][t][64]
     const uint64_t *path_off;  // slot of pair i is [path_off[i], path_off[i + 1])
     uint64_t cap;
     uint32_t *path;
@@ -239,6 +240,9 @@ __device__ __forceinline__ uint32_t bp_dist_to(const PathArgs &a, uint32_t i, ui
 // dv + 1 vertices at path[pos], path[pos + step], ...; by the WALK lanes of
 // `group` (lane g of them), each step to the first neighbour one hop nearer.
 // Every lane returns the same value: false if some vertex has no nearer neighbour.
+// The last step is to the bit-parallel vertex itself, which a binary search finds in
+// v's list (1M pairs of a complete graph of 1500 vertices, all of whose paths are
+// such steps: 6.6 ms with a scan of the list by these lanes, 6.0 by 32, 0.57 so).
 constexpr int WALK = 8;  // 4 or 16 lanes: 3 % slower
 __device__ bool bp_walk(const PathArgs &a, uint32_t i, uint32_t kind, uint32_t bit, uint32_t v,
                         uint32_t dv, int64_t pos, int step, unsigned group, int g) {
@@ -246,10 +250,21 @@ __device__ bool bp_walk(const PathArgs &a, uint32_t i, uint32_t kind, uint32_t b
     while (dv > 0) {
         const uint32_t b = a.roff[v], e = a.roff[v + 1];
         uint32_t next = NONE;
-        for (uint32_t x = b; x < e; x += WALK) {
-            const uint32_t w = x + g < e ? a.rcol[x + g] : NONE;
-            const unsigned m = __ballot_sync(group, w != NONE && bp_dist_to(a, i, kind, bit, w) == dv - 1) & group;
-            if (m) { next = __shfl_sync(group, w, __ffs(m) - 1); break; }
+        if (dv == 1) {
+            const size_t slot = (size_t)(a.x.graph ? a.x.graph[v] : 0) * a.x.t + i;
+            const uint32_t goal = kind == 2 ? a.bp_root[slot] : a.bp_S[slot * BPW + bit];
+            uint32_t lo = b, hi = e;
+            while (lo < hi) {
+                const uint32_t mid = lo + ((hi - lo) >> 1);
+                if (a.rcol[mid] < goal) lo = mid + 1; else hi = mid;
+            }
+            if (lo < e && a.rcol[lo] == goal) next = goal;
+        } else {
+            for (uint32_t x = b; x < e; x += WALK) {
+                const uint32_t w = x + g < e ? a.rcol[x + g] : NONE;
+                const unsigned m = __ballot_sync(group, w != NONE && bp_dist_to(a, i, kind, bit, w) == dv - 1) & group;
+                if (m) { next = __shfl_sync(group, w, __ffs(m) - 1); break; }
+            }
         }
         if (next == NONE) return false;
         v = next;
@@ -289,11 +304,13 @@ struct PathLength {
 // what each lane can settle about its own pair, then the witnesses of the open
 // ones one by one, then the climbs and walks of all of them side by side (two
 // ends each; a climb is a chain of dependent searches, and a walk's steps wait
-// for one another too). Bound by the latency of those chains: eight blocks an
-// SM (32 registers and 106 bytes of local memory; five blocks of 47 registers 10 % slower). 1M uniform pairs of
-// R-MAT-20, t = 64, with the lengths: 2.90 ms with a warp per pair, binary
-// searches for every witness and the climbs on two lanes; 1.70 ms so, of which
-// (by leaving steps out) 0.6 ms is the witnesses, 0.5 the walks, 0.05 the climbs.
+// for one another too). Bound by the latency of those chains: eight blocks an SM
+// (32 registers and 116 bytes of local memory; five blocks of 47 registers 10 %
+// slower). 1M uniform pairs of R-MAT-20, t = 64, with the lengths: 2.90 ms with a warp
+// per pair, binary searches for every witness and the climbs on two lanes; 1.70 ms
+// so, of which (by leaving steps out) 0.6 ms was the witnesses, 0.5 the walks, 0.05
+// the climbs; 1.45 ms with a search for a walk's last step and one copy each of the
+// climb and the walk for both ends.
 __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t G) {
     __shared__ uint32_t s_keep[8][PATH_KEEP];
     __shared__ OpenPair s_pair[8][32];
@@ -389,8 +406,8 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
             const int j = item[x] & 31;
             const Witness w = wit[j];
             const bool from_t = item[x] & 32;
-            const bool ok = from_t ? climb(a, w.at, pair[j].t, w.d - w.by, (int64_t)(slot[j] + w.d), -1)
-                                   : climb(a, w.at, pair[j].s, w.by, (int64_t)slot[j], 1);
+            const bool ok = climb(a, w.at, from_t ? pair[j].t : pair[j].s, from_t ? w.d - w.by : w.by,
+                                  (int64_t)(from_t ? slot[j] + w.d : slot[j]), from_t ? -1 : 1);
             if (!ok) failed |= 1u << j;
         }
         __syncwarp();
@@ -410,10 +427,8 @@ __global__ void __launch_bounds__(256, PATH_BLOCKS) k_paths(PathArgs a, uint32_t
             const uint32_t i = w.at >> 8, kind = (w.at >> 6) & 3u, bit = w.at & 63u;
             const uint32_t ds = bp_dist_to(a, i, kind, bit, pair[j].s), dt = bp_dist_to(a, i, kind, bit, pair[j].t);
             const bool ok = ds + dt == w.d &&
-                            (from_t ? bp_walk(a, i, kind, bit, pair[j].t, dt, (int64_t)(slot[j] + w.d), -1, group,
-                                              lane & (WALK - 1))
-                                    : bp_walk(a, i, kind, bit, pair[j].s, ds, (int64_t)slot[j], 1, group,
-                                              lane & (WALK - 1)));
+                            bp_walk(a, i, kind, bit, from_t ? pair[j].t : pair[j].s, from_t ? dt : ds,
+                                    (int64_t)(from_t ? slot[j] + w.d : slot[j]), from_t ? -1 : 1, group, lane & (WALK - 1));
             if (!ok) failed |= 1u << j;
         }
         failed = __reduce_or_sync(FULL, failed);
@@ -586,6 +601,7 @@ PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32
     a.x = query_args(p->ix, src, dst, 1, q, nullptr, err.p);
     a.order = p->ix->d_order; a.par = p->d_par;
     a.roff = p->d_roff; a.rcol = p->d_rcol;
+    a.bp_root = p->ix->d_bp_root; a.bp_S = p->ix->d_bp_S;
     a.path_off = path_off;
     a.cap = cap;
     a.path = path;
