@@ -111,6 +111,7 @@ struct PathArgs {
     const uint32_t *order, *par;
     const uint32_t *roff, *rcol;
     const uint32_t *bp_root, *bp_S;  // [graphs][t], [graphs][t][64]
+    uint32_t graphs;
     const uint64_t *path_off;  // slot of pair i is [path_off[i], path_off[i + 1])
     uint64_t cap;
     uint32_t *path;
@@ -251,7 +252,9 @@ __device__ bool bp_walk(const PathArgs &a, uint32_t i, uint32_t kind, uint32_t b
         const uint32_t b = a.roff[v], e = a.roff[v + 1];
         uint32_t next = NONE;
         if (dv == 1) {
-            const size_t slot = (size_t)(a.x.graph ? a.x.graph[v] : 0) * a.x.t + i;
+            const uint32_t gi = a.x.graph ? a.x.graph[v] : 0;
+            if (gi >= a.graphs) return false;  // a file's graph ids are not checked
+            const size_t slot = (size_t)gi * a.x.t + i;
             const uint32_t goal = kind == 2 ? a.bp_root[slot] : a.bp_S[slot * BPW + bit];
             uint32_t lo = b, hi = e;
             while (lo < hi) {
@@ -601,7 +604,7 @@ PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32
     a.x = query_args(p->ix, src, dst, 1, q, nullptr, err.p);
     a.order = p->ix->d_order; a.par = p->d_par;
     a.roff = p->d_roff; a.rcol = p->d_rcol;
-    a.bp_root = p->ix->d_bp_root; a.bp_S = p->ix->d_bp_S;
+    a.bp_root = p->ix->d_bp_root; a.bp_S = p->ix->d_bp_S; a.graphs = p->ix->graphs;
     a.path_off = path_off;
     a.cap = cap;
     a.path = path;

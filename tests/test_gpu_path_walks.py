@@ -48,3 +48,27 @@ def test_each_graph_of_a_batch_has_its_own_roots(t):
     ix = pll.Index.build_batch(dev_u32(off), dev_u32(col), start, t=t)
     with pll.Paths(ix, dev_u32(off), dev_u32(col)) as P:
         check(P, g, brute.apsp(g.offsets, g.cols))
+
+
+def test_a_file_with_wrong_graph_ids(tmp_path):
+    """The graph ids of a batch index's file are taken as they are: paths through roots are refused, as
+    for a graph that is not the index's, and distances inside a graph stay."""
+    parts = [graphs.complete(60), gg.ba(90, 20, 1)]
+    off, col, start = gg.union(parts)
+    t, n = 16, 150
+    ix = pll.Index.build_batch(dev_u32(off), dev_u32(col), start, t=t)
+    path = tmp_path / "i"
+    ix.save(path)
+    data = bytearray(path.read_bytes())
+    at = len(data) - 4 * ix.label_entries() - 8 * (n + 1) - 4 * n
+    ids = np.frombuffer(bytes(data[at:at + 4 * n]), np.uint32)
+    assert sorted(np.bincount(ids).tolist()) == [60, 90]
+    data[at:at + 4 * n] = (ids + 1_000_000).tobytes()
+    path.write_bytes(bytes(data))
+    wrong = pll.Index.load(path)
+    s, u = dev_u32(np.arange(59, dtype=np.uint32)), dev_u32(np.arange(1, 60, dtype=np.uint32))
+    assert bool((wrong.query(s, u) == 1).all())
+    with pll.Paths(wrong, dev_u32(off), dev_u32(col)) as P:
+        with pytest.raises(pll.PLLError) as e:
+            P.query(s, u)
+    assert e.value.code == pll.PLL_E_INVAL
