@@ -668,9 +668,10 @@ PLL_API void pll_test_barrier_timeout(uint64_t ns);
  * eighth of the device's memory) mapped so that the next call does not map
  * and unmap pages again (about 3 ms per GiB). A few 20 KiB blocks of pinned
  * host memory, in which synchronous calls learn their status, are kept the same
- * way (64 at most; a call under way has one of its own). pll_release_cached
- * synchronises the current device and hands what the current context has cached
- * back to the driver; later calls work as before. PLL_E_CUDA if the device
+ * way (one by each thread, which hands it on when it ends, and 64 handed on at
+ * most; a call under way has one of its own). pll_release_cached synchronises the
+ * current device and hands what the current context has cached, but for the
+ * blocks of other threads, back to the driver; later calls work as before. PLL_E_CUDA if the device
  * reports an error.
  */
 PLL_API int pll_release_cached(void);

@@ -773,6 +773,7 @@ using namespace pll;
 
 struct pll_mlp {
     int device = 0;
+    unsigned long long ctx = 0;  // context_id() of its arrays
     uint32_t wide = 0;  // blocks of k_mlp_fwd<2> that the device holds at once
     uint32_t max_batch = 0, blocks = 0;
     float *master = nullptr, *m = nullptr, *v = nullptr;
@@ -940,6 +941,7 @@ PLL_API int pll_mlp_create(uint32_t max_batch, pll_mlp **out) {
         delete p;
         return PLL_E_CUDA;
     }
+    p->ctx = context_id();
     *out = p;
     return PLL_OK;
 }
@@ -1003,7 +1005,7 @@ PLL_API int pll_mlp_read_grad(const pll_mlp *p, float *host_grad, float *host_lo
     // gradient and loss in one copy into pinned memory (two into the caller's
     // pageable arrays are staged ones, a wait each)
     static_assert((NP + 1) * sizeof(float) <= HOST_BLOCK_BYTES, "the gradient fits a host block");
-    HostBlock block(s);
+    HostBlock block(s, p->ctx);
     if (!block.p) {
         if (host_grad) PLL_TRY(cudaMemcpyAsync(host_grad, p->grad, NP * sizeof(float), cudaMemcpyDeviceToHost, s));
         if (host_loss) PLL_TRY(cudaMemcpyAsync(host_loss, p->grad + NP, sizeof(float), cudaMemcpyDeviceToHost, s));

@@ -45,6 +45,7 @@ using namespace pll;
 // The directed index: labels in rank space, [0] = L_IN, [1] = L_OUT.
 struct pll_dindex {
     int device = 0;
+    unsigned long long ctx = 0;   // context_id() of its arrays
     uint32_t n = 0;
     uint64_t nnz = 0;
     uint32_t *d_order = nullptr;  // rank -> caller vertex id
@@ -546,6 +547,7 @@ PLL_API int pll_build_directed(const uint32_t *offsets, const uint32_t *cols, ui
         PLL_CHECK(directed_labels(ix, adj_off, adj_col, bmax, s));
     }
     PLL_TRY(cudaStreamSynchronize(s));
+    ix->ctx = context_id();
     guard.ix = nullptr;
     *out = ix;
     return PLL_OK;
@@ -557,7 +559,7 @@ PLL_API int pll_dquery(const pll_dindex *idx, const uint32_t *src, const uint32_
     if (q == 0) return PLL_OK;
     if (!src || !dst || !out) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    CallErrors err(s);
+    CallErrors err(s, idx->ctx);
     PLL_CHECK(err.begin(idx->d_qerr));
     const DQueryArgs a{idx->n, idx->d_inv, idx->d_off[0], idx->d_off[1], idx->d_lab[0], idx->d_lab[1],
                        src, dst, q, out, err.p};

@@ -57,6 +57,7 @@ __host__ __device__ inline uint64_t pack_tuple(uint32_t u, uint32_t k, uint32_t 
 // The opaque index of the C ABI.
 struct pll_index {
     int device = 0;
+    unsigned long long ctx = 0;    // context_id() of its arrays
     uint32_t n = 0, t = 0;
     uint32_t tp = 0;               // bp_d row stride: t rounded up to 16
     uint32_t graphs = 1;           // graphs built together (disjoint union)
@@ -136,6 +137,9 @@ inline void host_free(void *p) {
 // (pll_abi.cu), which keeps freed memory mapped for later calls; nullptr if
 // the driver cannot name the context (the default pool is used then).
 cudaMemPool_t scratch_pool();
+// the current context's unique id (0 if the driver cannot name it): a context made
+// after a device reset has another
+unsigned long long context_id();
 // Stream-ordered scratch from that pool (counted and failed like dev_malloc).
 template <class T> inline cudaError_t pool_malloc(T **p, size_t b, cudaStream_t s) {
     *p = nullptr;
@@ -182,19 +186,20 @@ struct PoolMem {
 
 // Pinned host memory of one synchronous call: the words its kernels add errors to
 // directly, or the target of its copy back (a pageable target makes the copy a
-// staged one). Blocks of one size are kept per CUDA context (pll_abi.cu) for the
-// calls after it, at most HOST_BLOCKS_KEPT of them, until pll_release_cached; they
-// belong to no thread. A block goes back only once the call's stream has been
-// waited for, also where the call ends early, so nothing in flight can write to
-// another call's words. p is null if no block can be had.
+// staged one). Blocks of one size are kept for later calls of the same CUDA context
+// (pll_abi.cu): one by each thread, until it ends, and at most HOST_BLOCKS_KEPT
+// that threads left, until pll_release_cached. A block goes back only once the
+// call's stream has been waited for, also where the call ends early, so nothing in
+// flight can write to another call's words. p is null if no block can be had.
 constexpr size_t HOST_BLOCK_BYTES = 20480;
 constexpr size_t HOST_BLOCKS_KEPT = 64;
-void *host_block_take(unsigned long long *ctx_id);
+void *host_block_take(unsigned long long ctx_id);
 void host_block_give(void *p, unsigned long long ctx_id);
 struct HostBlock {
     void *p = nullptr;
     cudaStream_t s;
-    explicit HostBlock(cudaStream_t st) : s(st) { p = host_block_take(&ctx_id); }
+    // ctx: the context of the object called, from context_id()
+    HostBlock(cudaStream_t st, unsigned long long ctx) : s(st), ctx_id(ctx) { p = host_block_take(ctx); }
     HostBlock(const HostBlock &) = delete;
     HostBlock &operator=(const HostBlock &) = delete;
     // waits for the stream: what the call's work wrote to the block can be read
@@ -210,7 +215,7 @@ struct HostBlock {
     template <class T> T *as() const { return static_cast<T *>(p); }
 
 private:
-    unsigned long long ctx_id = 0;
+    unsigned long long ctx_id;
     bool waited = false;
 };
 
@@ -488,7 +493,7 @@ struct CallErrors {
     PoolMem dev;
     cudaStream_t s;
     unsigned long long *p = nullptr;
-    explicit CallErrors(cudaStream_t st) : host(st), dev(st), s(st) {}
+    CallErrors(cudaStream_t st, unsigned long long ctx) : host(st, ctx), dev(st), s(st) {}
     int begin(unsigned long long *shared) {
         p = host.as<unsigned long long>();
         if (p) {

@@ -175,6 +175,7 @@ PLL_API int pll_load(const char *path, pll_index **out) {
     PLL_CHECK(get(file.f, &ix->d_lab, h.entries));
     PLL_TRY(pll::dev_malloc(&ix->d_qerr, 16));
     PLL_TRY(cudaMemset(ix->d_qerr, 0, 16));
+    ix->ctx = pll::context_id();
     ix->stats.n = h.n;
     ix->stats.t = h.t;
     ix->stats.nnz = h.nnz;

@@ -574,7 +574,7 @@ PLL_API int pll_path_offsets(const pll_paths *p, const uint32_t *src, const uint
     cudaStream_t s = (cudaStream_t)stream;
     // the pairs' distances, then one scan of the lengths they stand for; the
     // total comes back behind the call's error counters
-    CallErrors err(s);
+    CallErrors err(s, p->ix->ctx);
     PLL_CHECK(err.begin(nullptr));
     PoolMem dist(s), temp(s);
     PLL_CHECK(dist.alloc(q));
@@ -598,7 +598,7 @@ PLL_API int pll_path_query(const pll_paths *p, const uint32_t *src, const uint32
     if (q == 0) return PLL_OK;
     if (!src || !dst || !path_off || (cap > 0 && !path)) return PLL_E_INVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    CallErrors err(s);  // the first word takes the error bits
+    CallErrors err(s, p->ix->ctx);  // the first word takes the error bits
     PLL_CHECK(err.begin(nullptr));
     PathArgs a{};
     a.x = query_args(p->ix, src, dst, 1, q, nullptr, err.p);
