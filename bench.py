@@ -48,12 +48,12 @@ WORKLOADS = {
 # dram__bytes_write.sum, one pass), valid only for the sources with this hash,
 # on which the sweeps' traffic depends (else traffic is reported as null). The
 # level-loop graph's figure is ncu's per-graph-launch count (--graph-profiling
-# graph) on R-MAT scale 18: 13 launches, 2.005 GB of DRAM against 6.953 GB of
+# graph) on R-MAT scale 18: 13 launches, 2.004 GB of DRAM against 6.953 GB of
 # algorithmic bytes.
 PROFILED = {
     "level-loop graph (k_batch_expand_g + k_batch_test_g)": {
         "src": ["k_pruned.cu", "bp_nibble.h", "build_sizes.h", "k_labels.cu", "pll_internal.cuh"],
-        "src_sha": "946c579aa20c7e3a", "dram_per_alg_byte": 0.288},
+        "src_sha": "a4aeafa6b3e20487", "dram_per_alg_byte": 0.288},
 }
 
 
