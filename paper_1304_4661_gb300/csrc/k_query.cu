@@ -100,11 +100,14 @@ __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
         count_errors(s_errors, ans, lane);
         __syncwarp();  // the next group writes pair
     }
-    // the block's errors at once: the counters may be host memory, where an addition
-    // costs 12 ns (10M pairs, every id out of range: 3.6 ms with one a group, 0.07 so)
-    __syncthreads();
-    if (threadIdx.x < 2 && s_errors[threadIdx.x])
-        atomicAdd_system(a.err + threadIdx.x, (unsigned long long)s_errors[threadIdx.x]);
+    // What errors the block has counted, by each warp as it ends (its own are among
+    // them): the counters may be host memory, where an addition costs 12 ns (10M pairs,
+    // every id out of range: 3.6 ms with one a group of pairs, 0.2 so). A barrier at the end
+    // costs the server, whose runs overlap, 4 % on R-MAT-22.
+    if (lane < 2 && s_errors[lane]) {
+        const uint32_t count = atomicExch(&s_errors[lane], 0u);
+        if (count) atomicAdd_system(a.err + lane, (unsigned long long)count);
+    }
 }
 
 // G warps of a block per pair, for launches too small to fill the GPU with

@@ -116,15 +116,12 @@ struct DQueryArgs {
 };
 
 // One warp per pair: lanes take entries of the shorter of L_OUT(s), L_IN(t)
-// and binary-search the other by hub. A block counts its errors and adds them at the
+// and binary-search the other by hub. A warp counts its errors and adds them at the
 // end: the counters may be host memory (10M pairs, every id out of range: 114 ms
 // with an addition for each, 0.4 ms so).
 __global__ void __launch_bounds__(256) k_dquery(DQueryArgs a) {
     const int lane = threadIdx.x & 31;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    __shared__ uint32_t s_errors[2];
-    if (threadIdx.x < 2) s_errors[threadIdx.x] = 0;
-    __syncthreads();
     uint32_t far = 0, bad = 0;
     for (uint64_t qi = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; qi < a.q; qi += warps) {
         const uint32_t sid = a.src[qi], tid = a.dst[qi];
@@ -159,11 +156,8 @@ __global__ void __launch_bounds__(256) k_dquery(DQueryArgs a) {
         if (lane == 0) a.out[qi] = (uint8_t)min(best, (uint32_t)INF8);
         far += best >= INF8 && best < BIG;
     }
-    if (lane == 0 && far) atomicAdd(&s_errors[0], far);
-    if (lane == 0 && bad) atomicAdd(&s_errors[1], bad);
-    __syncthreads();
-    if (threadIdx.x < 2 && s_errors[threadIdx.x])
-        atomicAdd_system(a.err + threadIdx.x, (unsigned long long)s_errors[threadIdx.x]);
+    if (lane == 0 && far) atomicAdd_system(a.err, (unsigned long long)far);
+    if (lane == 0 && bad) atomicAdd_system(a.err + 1, (unsigned long long)bad);
 }
 
 // ------------------------------------------------------------- host
