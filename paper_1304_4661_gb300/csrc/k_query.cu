@@ -3,8 +3,8 @@
 // d(s, t) = min( bit-parallel query (Sec. 5.3), Query(s, t, L) (Sec. 3.3) ).
 //
 // A persistent grid (a few CTAs per SM) walks the pairs; one warp answers one
-// pair, the labels first (pair_merged) or, where the labels are far larger than the
-// L2, the bit-parallel part, which bounds what the labels can add (pair_bounded).
+// pair, the labels first (pair_merged) or, where the labels are larger than the L2,
+// the bit-parallel part, which bounds what the labels can add (pair_bounded).
 // Pairs with an end that nothing reaches are settled by one lane each (lone_pair).
 // A launch too small to fill the GPU that way (up to 4 pairs per
 // resident block) gives each pair 2, 4 or 8 warps instead, which split the
@@ -42,13 +42,14 @@ constexpr int QUERY_BLOCKS = 8;
 // which (by leaving steps out) 0.3 ms for ranks, offsets and lone pairs, 0.3
 // for the rows, 1.0 for the masks and 0.8 for each end's label.
 //
-// NEAR: near entries only (pair_bounded), for indices whose labels are well past the
+// NEAR: near entries only (pair_bounded), for indices whose labels are larger than the
 // L2, where what it leaves unread counts; otherwise the labels first (pair_merged):
 // the near entries are a second reading of what the L2 holds, and the masks they
 // are bounded by are most of the work. 10M uniform pairs, near entries against
-// labels first: R-MAT-17, 18, 19, 20, 21 at t = 64 (labels of 5, 21, 78, 288 and
-// 998 MB) 2.26 and 1.93, 2.51 and 2.24, 2.82 and 2.68, 3.29 and 3.35, 4.01 and 4.54
-// ms; R-MAT-20 at t = 16 (537 MB) 3.97 and 4.57; BA of 10,000 and 50,000
+// labels first: R-MAT-17, 18, 20, 21 at t = 64 (labels of 5, 21, 288 and 998 MB)
+// 2.26 and 1.93, 2.51 and 2.24, 3.27 and 3.37, 4.02 and 4.59 ms; R-MAT-19 at t = 64,
+// 48, 32, 16, 8, 4 (77, 98, 127, 168, 225 and 268 MB) 2.77 and 2.67, 2.87 and 2.83,
+// 2.79 and 2.82, 3.12 and 3.27, 3.77 and 4.08, 4.22 and 4.60; BA of 10,000 and 50,000
 // vertices at t = 16 (1 and 32 MB) 4.59 and 3.46, 9.57 and 8.26.
 template <int PG, bool NEAR>
 __global__ void __launch_bounds__(256, QUERY_BLOCKS) k_query(QueryArgs a) {
@@ -199,7 +200,7 @@ int query_launch_strided(const pll_index *ix, const uint32_t *d_src, const uint3
         // pairs per warp group: as many as keep every resident warp busy (R
         // blocks of 8 warps), up to 32
         const uint64_t per = q / (R * 8);
-        if (ix->entries * 4 > 2 * (uint64_t)l2) launch_query<true>(a, per, (unsigned)R, s);
+        if (ix->entries * 4 > (uint64_t)l2) launch_query<true>(a, per, (unsigned)R, s);
         else launch_query<false>(a, per, (unsigned)R, s);
     }
     PLL_TRY(cudaGetLastError());
